@@ -358,6 +358,9 @@ gbs_status gbs_server_stats_get(gbs_ctx* ctx, gbs_server_stats* out);
  *   mid_e          0..8: levels each first-kernel CTA goes on expanding in
  *                  shared memory after its prefix (replacing that many
  *                  breadth-first level launches; reduced to fit 200 KB).
+ * The fixed-point precisions shape their launches by rules on the batch; of the
+ * above only d_top (an upper limit; at least 5 levels are taken) and q_drop (at
+ * most 3 - q_drop levels per leaf thread) act on them.
  * gbs_autotune times candidate shapes on a synthetic batch of n_trees (1..64)
  * trees of n, n-1, ... modes (6 <= n <= 28; a workload of uneven trees tunes
  * best on a batch that resembles it)

@@ -1,10 +1,9 @@
 // Batched subset-determinant trees, wide fixed-point per-term arithmetic (real basis).
-#include "gbs_fx.cuh"
-#include "gbs_batch_driver.cuh"
+#include "gbs_fxtree_driver.cuh"
 
 namespace gbs {
 gbs_status batch_fxw_real(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots, TreeOut* outs,
                           int* status, const BatchTune& tune) {
-  return batch_run<fxw, 3>(ctx, ntrees, trees, roots, outs, status, tune);
+  return fx_batch_run<fxw>(ctx, ntrees, trees, roots, outs, status, tune);
 }
 }  // namespace gbs

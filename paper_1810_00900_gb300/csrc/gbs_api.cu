@@ -225,13 +225,13 @@ gbs_status gbs_ctx_create(gbs_ctx** out, int device, size_t hbm_budget_bytes) {
     ctx->tune[GBS_PREC_TD][b].sub_e = 6;
     ctx->tune[GBS_PREC_TD][b].d_top = 4;
     ctx->tune[GBS_PREC_FX][b].sub_e = 6;
-    ctx->tune[GBS_PREC_FX][b].d_top = 6;
+    ctx->tune[GBS_PREC_FX][b].d_top = 10;
     ctx->tune[GBS_PREC_FXW][b].sub_e = 6;
-    ctx->tune[GBS_PREC_FXW][b].d_top = 6;
+    ctx->tune[GBS_PREC_FXW][b].d_top = 10;
     ctx->tune[GBS_PREC_FP64P][b].sub_e = 6;
     ctx->tune[GBS_PREC_FP64P][b].d_top = 8;
     ctx->tune[GBS_PREC_FXN][b].sub_e = 6;
-    ctx->tune[GBS_PREC_FXN][b].d_top = 6;
+    ctx->tune[GBS_PREC_FXN][b].d_top = 10;
   }
   *out = ctx;
   return GBS_OK;

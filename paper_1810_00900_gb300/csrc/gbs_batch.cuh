@@ -62,36 +62,6 @@ __device__ __forceinline__ int find_seg(const Seg* segs, int nseg, Key key, Key 
   return lo;
 }
 
-// Node buffers in global memory hold packed lower triangles entry-major: entry
-// e of node i of a region of `count` nodes is element e * count + i.  Multiword
-// entries (node_words > 0) are stored limb-major inside that: limb k of entry e
-// of node i is 32-bit word (e * L + k) * count + i of the region, so every limb
-// load or store of a warp covers one contiguous 128-byte line.
-template <class E>
-__device__ __forceinline__ E ld_node(const E* base, long long e, long long count, long long i) {
-  constexpr int L = node_words<E>::value;
-  if constexpr (L == 0) {
-    return base[e * count + i];
-  } else {
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(base);
-    E r;
-#pragma unroll
-    for (int k = 0; k < L; ++k) r.w[k] = w[(e * L + k) * count + i];
-    return r;
-  }
-}
-template <class E>
-__device__ __forceinline__ void st_node(E* base, long long e, long long count, long long i, const E& v) {
-  constexpr int L = node_words<E>::value;
-  if constexpr (L == 0) {
-    base[e * count + i] = v;
-  } else {
-    uint32_t* w = reinterpret_cast<uint32_t*>(base);
-#pragma unroll
-    for (int k = 0; k < L; ++k) w[(e * L + k) * count + i] = v.w[k];
-  }
-}
-
 // packed index -> (row, col), col <= row
 __device__ __forceinline__ void untri(int e, int& a, int& b) {
   int r = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
@@ -108,13 +78,13 @@ __device__ __forceinline__ void untri(int e, int& a, int& b) {
 // last level and nodes/q describe it.  Scratch: pm10, pq00, pq11 hold one
 // value per node of the level being split.
 template <class E>
-__device__ __forceinline__ void smem_expand(E*& src, E*& dst, typename scale_of<E>::type*& ssrc,
-                                            typename scale_of<E>::type*& sdst, E* pm10,
+__device__ __forceinline__ void smem_expand(E*& src, E*& dst, typename real_of<E>::type*& ssrc,
+                                            typename real_of<E>::type*& sdst, E* pm10,
                                             typename real_of<E>::type* pq00, typename real_of<E>::type* pq11,
                                             int& nodes, int& q, int levels,
                                             bool& bad) {
   typedef typename real_of<E>::type T;
-  typedef typename scale_of<E>::type S;
+  typedef typename real_of<E>::type S;
   const int nthr = blockDim.x;
   for (int lvl = 0; lvl < levels; ++lvl) {
     for (int t = threadIdx.x; t < nodes; t += nthr) {
@@ -163,11 +133,11 @@ __device__ __forceinline__ void smem_expand(E*& src, E*& dst, typename scale_of<
 template <class E>
 __global__ void batch_top_kernel(const TopSeg* __restrict__ segs, int nseg,
                                  const typename root_src<E>::type* __restrict__ roots, E* __restrict__ buf0,
-                                 E* __restrict__ buf1, typename scale_of<E>::type* __restrict__ s0,
-                                 typename scale_of<E>::type* __restrict__ s1, int* __restrict__ status, int capA,
+                                 E* __restrict__ buf1, typename real_of<E>::type* __restrict__ s0,
+                                 typename real_of<E>::type* __restrict__ s1, int* __restrict__ status, int capA,
                                  int capB, int mid_off, int ncap) {
   typedef typename real_of<E>::type T;
-  typedef typename scale_of<E>::type S;
+  typedef typename real_of<E>::type S;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   E* C = reinterpret_cast<E*>(smem_raw);
   const TopSeg sg = segs[find_seg(segs, nseg, (long long)blockIdx.x, &TopSeg::block_begin)];
@@ -220,7 +190,7 @@ __global__ void batch_top_kernel(const TopSeg* __restrict__ segs, int nseg,
     for (int e = threadIdx.x; e < sym(dq); e += blockDim.x) {
       int a, b;
       untri(e, a, b);
-      st_node(out + sg.out_base, e, cnt, node, C[tri(a + o, b + o)]);
+      out[sg.out_base + e * cnt + node] = C[tri(a + o, b + o)];
     }
     if (threadIdx.x == 0) sout[sg.s_base + node] = s;
   } else {
@@ -246,18 +216,18 @@ __global__ void batch_top_kernel(const TopSeg* __restrict__ segs, int nseg,
     const long long first = node << sg.emid;
     for (int i = threadIdx.x; i < sym(2 * q) * nodes; i += blockDim.x) {
       const int e = i / nodes, t = i - e * nodes;
-      st_node(out + sg.out_base, e, cnt, first + t, src[i]);
+      out[sg.out_base + e * cnt + first + t] = src[i];
     }
     for (int t = threadIdx.x; t < nodes; t += blockDim.x) sout[sg.s_base + first + t] = ssrc[t];
   }
-  if (bad) atomicExch(status + sg.tree, bad_status<typename real_of<E>::type>());
+  if (bad) atomicExch(status + sg.tree, (int)kStatusNotPD);
 }
 
 // ---------------------------------------------------------------- level --
 template <class E>
-__global__ void __launch_bounds__(256, level_min_blocks<E>::value) batch_level_kernel(const LevelSeg* __restrict__ segs, int nseg, long long total,
-                                   const E* __restrict__ in, const typename scale_of<E>::type* __restrict__ sin,
-                                   E* __restrict__ out, typename scale_of<E>::type* __restrict__ sout,
+__global__ void __launch_bounds__(256) batch_level_kernel(const LevelSeg* __restrict__ segs, int nseg, long long total,
+                                   const E* __restrict__ in, const typename real_of<E>::type* __restrict__ sin,
+                                   E* __restrict__ out, typename real_of<E>::type* __restrict__ sout,
                                    int* __restrict__ status) {
   typedef typename real_of<E>::type T;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -287,79 +257,53 @@ __global__ void __launch_bounds__(256, level_min_blocks<E>::value) batch_level_k
   const E* par = in + sg.in_base;
   const long long c2 = 2 * count;
   E* chi = out + sg.out_base;
-#define PAR(i, j) ld_node(par, tri(i, j), count, node)
+#define PAR(i, j) par[(long long)tri(i, j) * count + node]
+#define CHI(i, j, c) chi[(long long)tri(i, j) * c2 + 2 * node + (c)]
   const T p00 = re_of(PAR(0, 0));
   const T p11 = re_of(PAR(1, 1));
   const E p10 = PAR(1, 0);
   const T det = p00 * p11 - norm2(p10);
   if (!is_pos(det) || !lead_pos(p00)) {
-    if (grp == 0) atomicExch(status + sg.tree, bad_status<typename real_of<E>::type>());
+    if (grp == 0) atomicExch(status + sg.tree, (int)kStatusNotPD);
     return;
   }
   const T g = rsqrt_(det);
   const T inv = g * g;
   const T q00 = p00 * inv, q11 = p11 * inv;
   const E m10 = neg_(scale_(p10, inv));
-  // Fixed-point entries (level_park): the scaled pivot inverse and g wait in this
-  // thread's shared-memory slot while the rows are formed (read back once per
-  // row), which frees the registers the row loop would otherwise spill.
-  constexpr int LW = node_words<E>::value;
-  constexpr bool PARK = level_park<E>::value && LW > 0;
-  __shared__ uint32_t park[PARK ? 4 * LW : 1][PARK ? 256 : 1];
-  if constexpr (PARK) {
-#pragma unroll
-    for (int k = 0; k < LW; ++k) {
-      park[k][threadIdx.x] = q00.w[k];
-      park[LW + k][threadIdx.x] = q11.w[k];
-      park[2 * LW + k][threadIdx.x] = m10.w[k];
-      park[3 * LW + k][threadIdx.x] = g.w[k];
-    }
-  }
-  auto unpark = [&](int slot, const auto& keep) {
-    typedef typename std::decay<decltype(keep)>::type V;
-    if constexpr (PARK) {
-      V r;
-      const volatile uint32_t* src = &park[slot * LW][threadIdx.x];
-#pragma unroll
-      for (int k = 0; k < LW; ++k) r.w[k] = src[k * 256];
-      return r;
-    } else {
-      return keep;
-    }
-  };
   for (int a = grp; a < rows; a += sg.groups) {
     const E u0 = PAR(a + 2, 0), u1 = PAR(a + 2, 1);
-    const E m10r = unpark(2, m10);
-    const E L0 = lin2(u0, unpark(1, q11), u1, m10r);
-    const E L1 = lin2(u1, unpark(0, q00), u0, conj_(m10r));
+    const E L0 = lin2(u0, q11, u1, m10);
+    const E L1 = lin2(u1, q00, u0, conj_(m10));
     for (int b = 0; b < a; ++b) {
       const E x = PAR(a + 2, b + 2);
       E v = fms_conj(x, L0, PAR(b + 2, 0));
       v = fms_conj(v, L1, PAR(b + 2, 1));
-      st_node(chi, tri(a, b), c2, 2 * node, x);
-      st_node(chi, tri(a, b), c2, 2 * node + 1, v);
+      CHI(a, b, 0) = x;
+      CHI(a, b, 1) = v;
     }
     const E x = PAR(a + 2, a + 2);
     E v = fms_conj_re(x, L0, u0);
     v = fms_conj_re(v, L1, u1);
-    st_node(chi, tri(a, a), c2, 2 * node, x);
-    st_node(chi, tri(a, a), c2, 2 * node + 1, v);
+    CHI(a, a, 0) = x;
+    CHI(a, a, 1) = v;
   }
   if (grp == 0) {
-    const typename scale_of<E>::type s = sin[sg.s_in + node];
+    const typename real_of<E>::type s = sin[sg.s_in + node];
     sout[sg.s_out + 2 * node] = s;
-    sout[sg.s_out + 2 * node + 1] = s * unpark(3, g);
+    sout[sg.s_out + 2 * node + 1] = s * g;
   }
 #undef PAR
+#undef CHI
 }
 
 // ----------------------------------------------------------------- leaf --
 template <class E, int Q, bool PAIR = false>
-__global__ void __launch_bounds__(128, leaf_min_blocks<E>::value) batch_leaf_kernel(const LeafSeg* __restrict__ segs, int nseg,
+__global__ void __launch_bounds__(128) batch_leaf_kernel(const LeafSeg* __restrict__ segs, int nseg,
                                                          long long total_blocks, const E* __restrict__ buf0,
                                                          const E* __restrict__ buf1,
-                                                         const typename scale_of<E>::type* __restrict__ s0,
-                                                         const typename scale_of<E>::type* __restrict__ s1,
+                                                         const typename real_of<E>::type* __restrict__ s0,
+                                                         const typename real_of<E>::type* __restrict__ s1,
                                                          Partial<typename acc_traits<typename real_of<E>::type>::Red>* parts,
                                                          int* __restrict__ status) {
   typedef typename real_of<E>::type T;
@@ -374,10 +318,10 @@ __global__ void __launch_bounds__(128, leaf_min_blocks<E>::value) batch_leaf_ker
         const E* nodes = (sg.buf ? buf1 : buf0) + sg.base;
         E c[sym(2 * Q)];
 #pragma unroll
-        for (int e = 0; e < sym(2 * Q); ++e) c[e] = ld_node(nodes, e, sg.count, node);
-        const typename scale_of<E>::type s = (sg.buf ? s1 : s0)[sg.s_base + node];
-        const bool ok = subtree_run<E, Q, PAIR>(c, s, a);
-        if (!ok || !isfinite((a.ip + a.in) + (a.ep + a.en))) atomicExch(status + sg.tree, bad_status<T>());
+        for (int e = 0; e < sym(2 * Q); ++e) c[e] = nodes[e * sg.count + node];
+        const typename real_of<E>::type s = (sg.buf ? s1 : s0)[sg.s_base + node];
+        Dfs<E, Q, 2 * Q, 0, false, PAIR>::run(c, s, a);
+        if (!isfinite((a.ip + a.in) + (a.ep + a.en))) atomicExch(status + sg.tree, (int)kStatusNotPD);
         if ((sg.depth - __popcll((unsigned long long)node)) & 1) {
           const double t0 = a.ip, t1 = a.ep;
           a.ip = a.in; a.in = t0; a.ep = a.en; a.en = t1;
@@ -391,9 +335,9 @@ __global__ void __launch_bounds__(128, leaf_min_blocks<E>::value) batch_leaf_ker
         const E* nodes = (sg.buf ? buf1 : buf0) + sg.base;
         E c[sym(2 * Q)];
 #pragma unroll
-        for (int e = 0; e < sym(2 * Q); ++e) c[e] = ld_node(nodes, e, sg.count, node);
-        const typename scale_of<E>::type s = (sg.buf ? s1 : s0)[sg.s_base + node];
-        if (!subtree_sums<E, Q, PAIR>(c, s, inc, exc, asum)) atomicExch(status + sg.tree, bad_status<T>());
+        for (int e = 0; e < sym(2 * Q); ++e) c[e] = nodes[e * sg.count + node];
+        const typename real_of<E>::type s = (sg.buf ? s1 : s0)[sg.s_base + node];
+        if (!subtree_sums<E, Q, PAIR>(c, s, inc, exc, asum)) atomicExch(status + sg.tree, (int)kStatusNotPD);
         if ((sg.depth - __popcll((unsigned long long)node)) & 1) {
           inc = red_neg(inc);
           exc = red_neg(exc);
@@ -421,8 +365,8 @@ struct SubSeg {
 template <class E, int Q, bool PAIR = false>
 __global__ void __launch_bounds__(128) batch_subtree_kernel(
     const SubSeg* __restrict__ segs, int nseg, long long total_blocks, const E* __restrict__ buf0,
-    const E* __restrict__ buf1, const typename scale_of<E>::type* __restrict__ s0,
-    const typename scale_of<E>::type* __restrict__ s1, int capA, int capB,
+    const E* __restrict__ buf1, const typename real_of<E>::type* __restrict__ s0,
+    const typename real_of<E>::type* __restrict__ s1, int capA, int capB,
     Partial<typename acc_traits<typename real_of<E>::type>::Red>* parts, int* __restrict__ status) {
   typedef typename real_of<E>::type T;
   typedef typename acc_traits<T>::Acc Acc;
@@ -432,7 +376,7 @@ __global__ void __launch_bounds__(128) batch_subtree_kernel(
   E* bufA = reinterpret_cast<E*>(smem_raw);
   E* bufB = bufA + capA;
   E* pm10 = bufB + capB;                           // per node of the current level
-  typedef typename scale_of<E>::type S;
+  typedef typename real_of<E>::type S;
   S* sA = reinterpret_cast<S*>(pm10 + nthr);       // s of the current level
   S* sB = sA + nthr;
   T* pq00 = reinterpret_cast<T*>(sB + nthr);
@@ -445,7 +389,7 @@ __global__ void __launch_bounds__(128) batch_subtree_kernel(
     int q = sg.q_root;
     for (int i = threadIdx.x; i < sym(2 * q) * nroots; i += nthr) {
       const int e = i / nroots, k = i - e * nroots;
-      bufA[i] = ld_node(rsrc, e, sg.count, root + k);
+      bufA[i] = rsrc[e * sg.count + root + k];
     }
     for (int k = threadIdx.x; k < nroots; k += nthr) sA[k] = (sg.buf ? s1 : s0)[sg.s_base + root + k];
     __syncthreads();
@@ -456,7 +400,7 @@ __global__ void __launch_bounds__(128) batch_subtree_kernel(
     int nodes = nroots;
     bool bad = false;
     smem_expand<E>(src, dst, ssrc, sdst, pm10, pq00, pq11, nodes, q, sg.e_levels, bad);
-    if (bad) atomicExch(status + sg.tree, bad_status<typename real_of<E>::type>());
+    if (bad) atomicExch(status + sg.tree, (int)kStatusNotPD);
     const int t = threadIdx.x;
     if constexpr (std::is_same<Acc, double>::value) {
       Sums<double> a = sums_zero<double>();
@@ -464,8 +408,8 @@ __global__ void __launch_bounds__(128) batch_subtree_kernel(
         E c[sym(2 * Q)];
 #pragma unroll
         for (int e = 0; e < sym(2 * Q); ++e) c[e] = src[e * nodes + t];
-        const bool ok = subtree_run<E, Q, PAIR>(c, ssrc[t], a);
-        if (!ok || !isfinite((a.ip + a.in) + (a.ep + a.en))) atomicExch(status + sg.tree, bad_status<T>());
+        Dfs<E, Q, 2 * Q, 0, false, PAIR>::run(c, ssrc[t], a);
+        if (!isfinite((a.ip + a.in) + (a.ep + a.en))) atomicExch(status + sg.tree, (int)kStatusNotPD);
         const unsigned long long gnode = ((unsigned long long)root << sg.e_levels) + (unsigned long long)t;
         if ((sg.depth_leaf - __popcll(gnode)) & 1) {
           const double t0 = a.ip, t1 = a.ep;
@@ -481,7 +425,7 @@ __global__ void __launch_bounds__(128) batch_subtree_kernel(
 #pragma unroll
         for (int e = 0; e < sym(2 * Q); ++e) c[e] = src[e * nodes + t];
         const S sv = ssrc[t];
-        if (!subtree_sums<E, Q, PAIR>(c, sv, inc, exc, asum)) atomicExch(status + sg.tree, bad_status<T>());
+        if (!subtree_sums<E, Q, PAIR>(c, sv, inc, exc, asum)) atomicExch(status + sg.tree, (int)kStatusNotPD);
         const unsigned long long gnode = ((unsigned long long)root << sg.e_levels) + (unsigned long long)t;
         if ((sg.depth_leaf - __popcll(gnode)) & 1) {
           inc = red_neg(inc);

@@ -533,6 +533,8 @@ extern "C" gbs_status gbs_autotune(gbs_ctx* ctx, int prec, int basis, int n, int
           cand.level_threads = lt;
           cand.q_drop = qd;
           cand.mid_e = me;
+          // only d_top and q_drop act on the fixed-point engine: one candidate for the rest
+          if (is_fixed_point(prec) && (me != mids[0] || se != subs[0] || gr != grids[0] || lt != lts[0])) continue;
           ctx->tune[prec][real ? 1 : 0] = cand;
           float ms_best = 1e30f;
           for (int rep_i = 0; rep_i < 3; ++rep_i) {

@@ -27,7 +27,7 @@ template <class E, int QMAX, bool PAIR = false>
 gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots_dev, TreeOut* outs_dev,
                      int* status_dev, const BatchTune& tune) {
   typedef typename real_of<E>::type T;
-  typedef typename scale_of<E>::type S;
+  typedef typename real_of<E>::type S;
   typedef typename acc_traits<T>::Red Red;
   if (ntrees <= 0) return GBS_OK;
   const int sub_e = std::max(0, std::min(tune.sub_e, 7));  // levels expanded inside a subtree CTA

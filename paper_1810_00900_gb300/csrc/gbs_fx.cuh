@@ -29,13 +29,13 @@
 #include <stdint.h>
 #include <string.h>
 
-#include "gbs_tree_driver.cuh"
+#include "gbs_num.cuh"
 
 namespace gbs {
 
 template <int L, int F>
 struct fxn {
-  static_assert(F >= 3 && L > F, "at least three fraction limbs and one integer limb");
+  static_assert(F >= 2 && L > F, "at least two fraction limbs and one integer limb");
   uint32_t w[L];
 };
 typedef fxn<5, 4> fxn4;  // FXN entries
@@ -89,81 +89,80 @@ GBS_HD fxn<L, F> operator-(const fxn<L, F>& a) {
   r.w[L - 1] = subc(0u, a.w[L - 1]);
   return r;
 }
-// x / 2 (arithmetic shift by one bit)
-template <int L, int F>
-GBS_HD fxn<L, F> fx_half(const fxn<L, F>& a) {
-  fxn<L, F> r;
+// ---------------------------------------------------------------- product --
+// out[0 .. CHI - CLO] receives columns CLO .. CHI (32-bit words of weight
+// 2^(32 c)) of the sum of the partial products a_i b_j with i + j in
+// [CLO, CHI] of two unsigned multiword integers, modulo 2^(32 (CHI + 1)).
+//
+// What bounds a product is the multiply pipe: a 32 x 32 + 64 bit multiply-add
+// holds it for about 4 cycles per warp.  A partial product is a pair of words;
+// pairs that start at columns of equal parity never overlap, so each row of
+// partial products is two carry chains (even and odd columns) of mad.lo.cc /
+// madc.hi.cc pairs, each pair being one wide multiply-add with carry in and out
+// and nothing else; the two accumulators are added once at the end.  A chain's
+// last carry goes to the next pair of its parity, which no earlier row has
+// reached (rows go up, and so do their ends), so it never carries further.
+// Measured on the GB300 (chains of dependent 26-partial-product products, 16
+// warps per SM): 42.5 instructions per product, multiply pipe 90 % busy, 322 G/s,
+// against 97 instructions, 80 % and 219 G/s for 64-bit multiply-adds with a
+// separate running carry (78 adds and moves beside the 26 multiplies).
+#ifdef __CUDA_ARCH__
+#define GBS_ASM3(op, r, a, b, c) asm volatile(op " %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c))
+#else
+#define GBS_ASM3(op, r, a, b, c) (r = 0u)
+#endif
+GBS_HD uint32_t mad_lo_cc(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; GBS_ASM3("mad.lo.cc.u32", r, a, b, c); return r; }
+GBS_HD uint32_t madc_lo_cc(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; GBS_ASM3("madc.lo.cc.u32", r, a, b, c); return r; }
+GBS_HD uint32_t madc_hi_cc(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; GBS_ASM3("madc.hi.cc.u32", r, a, b, c); return r; }
+#undef GBS_ASM3
+
+template <int NA, int NB, int CLO, int CHI>
+GBS_HD void prod_cols(const uint32_t* a, const uint32_t* b, uint32_t* out) {
+  uint32_t acc[2][CHI + 4];
 #pragma unroll
-  for (int k = 0; k < L - 1; ++k) r.w[k] = (a.w[k] >> 1) | (a.w[k + 1] << 31);
-  r.w[L - 1] = (uint32_t)((int32_t)a.w[L - 1] >> 1);
-  return r;
-}
-// The same value with one more integer limb (sign extension).
-template <int L, int F>
-GBS_HD fxn<L + 1, F> fx_widen(const fxn<L, F>& a) {
-  fxn<L + 1, F> r;
+  for (int k = 0; k < CHI + 4; ++k) acc[0][k] = acc[1][k] = 0u;
 #pragma unroll
-  for (int k = 0; k < L; ++k) r.w[k] = a.w[k];
-  r.w[L] = (uint32_t)((int32_t)a.w[L - 1] >> 31);
-  return r;
+  for (int i = 0; i < NA; ++i) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      int end = -1;
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        const int c = i + j;
+        if (c < CLO || c > CHI || (c & 1) != p) continue;
+        acc[p][c] = end < 0 ? mad_lo_cc(a[i], b[j], acc[p][c]) : madc_lo_cc(a[i], b[j], acc[p][c]);
+        if (c < CHI) acc[p][c + 1] = madc_hi_cc(a[i], b[j], acc[p][c + 1]);
+        end = c;
+      }
+      if (end >= 0 && i > 0 && end + 2 <= CHI) acc[p][end + 2] = addc(acc[p][end + 2], 0u);
+    }
+  }
+  // column CLO holds one accumulator only
+  constexpr int P = CLO & 1;
+  out[0] = acc[P][CLO];
+  if constexpr (CHI > CLO) {
+    out[1] = add_cc(acc[0][CLO + 1], acc[1][CLO + 1]);
+#pragma unroll
+    for (int c = CLO + 2; c < CHI; ++c) out[c - CLO] = addc_cc(acc[0][c], acc[1][c]);
+    if constexpr (CHI > CLO + 1) out[CHI - CLO] = addc(acc[0][CHI], acc[1][CHI]);
+  }
 }
 
-// ---------------------------------------------------------------- product --
-// Window of the unsigned product: columns F to F + L - 1, plus a guard column
-// F - 1.  Row by row (operand a_i against the limbs of b that reach the
-// window), each partial product is added to its column together with the
-// running carry as one 64-bit multiply-add, whose high word is the next
-// carry; a row's final carry lands in the column one past its last product,
-// which no earlier row has reached (rows whose last product is the top
-// column drop it: the arithmetic is modulo 2^(32 L)).  Partial products below
-// the guard column are not formed and the guard column is dropped: at most F
-// units of the last place, always toward -inf.  The two's-complement
-// correction subtracts b (resp. a) shifted by L limbs when a (resp. b) is
-// negative.
-template <int L, int F>
-GBS_HD fxn<L, F> operator*(const fxn<L, F>& a, const fxn<L, F>& b) {
-  constexpr int W = L, G = F - 1;  // G: column of r[0] (the guard)
-  uint32_t r[W + 1];
+// a * b of non-negative values (a with LA limbs, the result too): the columns
+// from the fraction point up, formed with one guard column below it whose sum is
+// dropped: at most F units of the last place, always toward -inf.  Every product
+// of the tree is of this kind: a signed factor is shifted by a power of two first
+// (one add in its integer limb), and the shift's effect is separable and folded
+// into constants (fx_pivot below).  A two's-complement correction instead costs
+// 20-25 adds and masks a product (259 against 322 G products/s).
+template <int LA, int LB, int F>
+GBS_HD fxn<LA, F> umul(const fxn<LA, F>& a, const fxn<LB, F>& b) {
+  uint32_t t[LA + 1];
+  prod_cols<LA, LB, F - 1, F + LA - 1>(a.w, b.w, t);
+  fxn<LA, F> r;
 #pragma unroll
-  for (int k = 0; k <= W; ++k) r[k] = 0u;
-#pragma unroll
-  for (int i = 0; i < L; ++i) {
-    const int j0 = (G - i) > 0 ? (G - i) : 0;
-    const int j1 = (G + W - i) < (L - 1) ? (G + W - i) : (L - 1);
-    if (j0 > j1) continue;
-    uint32_t carry = 0u;
-#pragma unroll
-    for (int j = j0; j <= j1; ++j) {
-      const unsigned long long t = (unsigned long long)a.w[i] * b.w[j] + r[i + j - G] + carry;
-      r[i + j - G] = (uint32_t)t;
-      carry = (uint32_t)(t >> 32);
-    }
-    if (i + j1 + 1 - G <= W) r[i + j1 + 1 - G] = carry;
-  }
-  fxn<L, F> out;
-#pragma unroll
-  for (int k = 0; k < L; ++k) out.w[k] = r[k + 1];
-  // signed correction: result limbs S .. L-1 (column L and up) minus masked limbs
-  constexpr int S = L - F;
-  const uint32_t ma = (uint32_t)((int32_t)a.w[L - 1] >> 31), mb = (uint32_t)((int32_t)b.w[L - 1] >> 31);
-  if constexpr (S == L - 1) {
-    out.w[S] -= (b.w[0] & ma) + (a.w[0] & mb);
-  } else {
-    out.w[S] = sub_cc(out.w[S], b.w[0] & ma);
-#pragma unroll
-    for (int k = S + 1; k < L - 1; ++k) out.w[k] = subc_cc(out.w[k], b.w[k - S] & ma);
-    out.w[L - 1] = subc(out.w[L - 1], b.w[L - 1 - S] & ma);
-    out.w[S] = sub_cc(out.w[S], a.w[0] & mb);
-#pragma unroll
-    for (int k = S + 1; k < L - 1; ++k) out.w[k] = subc_cc(out.w[k], a.w[k - S] & mb);
-    out.w[L - 1] = subc(out.w[L - 1], a.w[L - 1 - S] & mb);
-  }
-  return out;
-}
-// s * g: the wide scale type times an entry scalar.
-template <int L, int F>
-GBS_HD fxn<L + 1, F> operator*(const fxn<L + 1, F>& a, const fxn<L, F>& b) {
-  return a * fx_widen(b);
+  for (int k = 0; k < LA; ++k) r.w[k] = t[k + 1];
+  return r;
 }
 
 // ----------------------------------------------------------- conversions --
@@ -189,12 +188,15 @@ GBS_HD fxn<L, F> fx_from_double(double x) {
   }
   return (bits >> 63) ? -r : r;
 }
-template <> GBS_HD fxn4 from_double<fxn4>(double x) { return fx_from_double<5, 4>(x); }
-template <> GBS_HD fxn4s from_double<fxn4s>(double x) { return fx_from_double<6, 4>(x); }
-template <> GBS_HD fx from_double<fx>(double x) { return fx_from_double<6, 5>(x); }
-template <> GBS_HD fxs from_double<fxs>(double x) { return fx_from_double<7, 5>(x); }
-template <> GBS_HD fxw from_double<fxw>(double x) { return fx_from_double<7, 6>(x); }
-template <> GBS_HD fxws from_double<fxws>(double x) { return fx_from_double<8, 6>(x); }
+template <int L, int F>
+GBS_HD fxn<L, F> fx_of_(double x, fxn<L, F>*) {
+  return fx_from_double<L, F>(x);
+}
+// x as the fixed-point type E.
+template <class E>
+GBS_HD E fx_of(double x) {
+  return fx_of_(x, (E*)nullptr);
+}
 
 // Nearest-ish double (a few units of the last place).
 template <int L, int F>
@@ -202,28 +204,17 @@ GBS_HD double to_double(const fxn<L, F>& a) {
   double v = (double)(int32_t)a.w[L - 1];
 #pragma unroll
   for (int k = L - 2; k >= 0; --k) v = fma(v, 4294967296.0, (double)a.w[k]);
-  return v * (F == 4 ? 0x1p-128 : F == 5 ? 0x1p-160 : 0x1p-192);
+  return v * (F == 2 ? 0x1p-64 : F == 4 ? 0x1p-128 : F == 5 ? 0x1p-160 : 0x1p-192);
 }
 static_assert(sizeof(fxn4) == 20 && sizeof(fxn4s) == 24 && sizeof(fx) == 24 && sizeof(fxs) == 28 &&
                   sizeof(fxw) == 28 && sizeof(fxws) == 32,
               "fx widths");
 
-// ------------------------------------------------------ tree interface ----
-template <int L, int F> GBS_HD fxn<L, F> fms(const fxn<L, F>& x, const fxn<L, F>& a, const fxn<L, F>& b) {
-  return x - a * b;
-}
-template <int L, int F> GBS_HD fxn<L, F> fpa(const fxn<L, F>& x, const fxn<L, F>& a, const fxn<L, F>& b) {
-  return x + a * b;
-}
-template <> GBS_HD fxn4 scale_<fxn4, fxn4>(const fxn4& x, const fxn4& s) { return x * s; }
-template <> GBS_HD fx scale_<fx, fx>(const fx& x, const fx& s) { return x * s; }
-template <> GBS_HD fxw scale_<fxw, fxw>(const fxw& x, const fxw& s) { return x * s; }
-template <> GBS_HD fxn4 conv_entry<fxn4>(const double& x) { return from_double<fxn4>(x); }
-template <> GBS_HD fx conv_entry<fx>(const double& x) { return from_double<fx>(x); }
-template <> GBS_HD fxw conv_entry<fxw>(const double& x) { return from_double<fxw>(x); }
-template <> struct scale_of<fxn4> { typedef fxn4s type; };
-template <> struct scale_of<fx> { typedef fxs type; };
-template <> struct scale_of<fxw> { typedef fxws type; };
+// The s type (running product of pivot factors, term sums) of an entry type.
+template <class E> struct fx_sum;
+template <> struct fx_sum<fxn4> { typedef fxn4s type; };
+template <> struct fx_sum<fx> { typedef fxs type; };
+template <> struct fx_sum<fxw> { typedef fxws type; };
 
 // A pivot determinant the fixed-point tree can use: in [2^-20, 2^12), where
 // its inverse square root keeps ~150 bits (the resolution is absolute, so the
@@ -235,145 +226,165 @@ GBS_HD bool fx_det_in_range(const fxn<L, F>& d) {
   for (int k = F + 1; k < L; ++k) high_zero &= d.w[k] == 0u;
   return high_zero && d.w[F] < (1u << 12) && (d.w[F] != 0u || d.w[F - 1] >= (1u << 12));
 }
-template <int L, int F> GBS_HD bool not_positive(const fxn<L, F>& d) { return !fx_det_in_range(d); }
-template <int L, int F> GBS_HD bool is_pos(const fxn<L, F>& d) { return fx_det_in_range(d); }
-// Fixed-point trees run only on matrices the host has bounded (positive definite).
-template <int L, int F> GBS_HD bool lead_pos(const fxn<L, F>&) { return true; }
-template <> constexpr int bad_status<fxn4>() { return kStatusRange; }
-template <> struct level_min_blocks<fxn4> { static const int value = 4; };
-template <> struct level_park<fxn4> { static const bool value = true; };
-template <> constexpr int bad_status<fx>() { return kStatusRange; }
-template <> struct level_min_blocks<fx> { static const int value = 4; };
-template <> struct level_park<fx> { static const bool value = true; };
-template <> struct level_park<fxw> { static const bool value = true; };
-template <int L, int F> struct node_words<fxn<L, F>> { static const int value = L; };
-template <int L, int F> struct leaf_min_blocks<fxn<L, F>> { static const int value = 4; };
-template <> struct level_min_blocks<fxw> { static const int value = 3; };
-template <> constexpr int bad_status<fxw>() { return kStatusRange; }
 
-// a * b where b >= 0 has nonzero limbs only in [JLO, JHI] (and, when ILO/IHI
-// are given, a >= 0 only in [ILO, IHI]), for the inverse square root's short
-// operands: the general product's rows and guard column restricted to those
-// rows and columns (the carry of row i still lands in column i + JHI + 1, which
-// no earlier row reached), then the one correction a negative a needs.
-template <int JLO, int JHI, int L, int F, int ILO = 0, int IHI = L - 1>
-__device__ __forceinline__ fxn<L, F> mul_short(const fxn<L, F>& a, const fxn<L, F>& b) {
-  constexpr int W = L, G = F - 1;
-  uint32_t r[W + 1];
-#pragma unroll
-  for (int k = 0; k <= W; ++k) r[k] = 0u;
-#pragma unroll
-  for (int i = ILO; i <= IHI; ++i) {
-    const int j0 = (G - i) > JLO ? (G - i) : JLO;
-    const int j1 = (G + W - i) < JHI ? (G + W - i) : JHI;
-    if (j0 > j1) continue;
-    uint32_t carry = 0u;
-#pragma unroll
-    for (int j = j0; j <= j1; ++j) {
-      const unsigned long long t = (unsigned long long)a.w[i] * b.w[j] + r[i + j - G] + carry;
-      r[i + j - G] = (uint32_t)t;
-      carry = (uint32_t)(t >> 32);
-    }
-    if (i + j1 + 1 - G <= W) r[i + j1 + 1 - G] = carry;
-  }
-  fxn<L, F> out;
-#pragma unroll
-  for (int k = 0; k < L; ++k) out.w[k] = r[k + 1];
-  constexpr int S = L - F;
-  const uint32_t ma = (uint32_t)((int32_t)a.w[L - 1] >> 31);
-  out.w[S] = sub_cc(out.w[S], b.w[0] & ma);
-#pragma unroll
-  for (int k = S + 1; k < L - 1; ++k) out.w[k] = subc_cc(out.w[k], b.w[k - S] & ma);
-  out.w[L - 1] = subc(out.w[L - 1], b.w[L - 1 - S] & ma);
-  return out;
-}
-
-// The value of a float (exact: 24 significant bits placed in the limbs).
-template <int L, int F>
-__device__ __forceinline__ fxn<L, F> fx_from_float(float v) {
-  const uint32_t bits = __float_as_uint(v);
-  const int e = (int)((bits >> 23) & 0xffu);
-  const uint32_t m = e ? ((bits & 0x7fffffu) | 0x800000u) : 0u;  // no subnormal reaches here
-  const int sh = e - 150 + 32 * F;                              // bit position of m's last bit in X
-  fxn<L, F> r;
-#pragma unroll
-  for (int k = 0; k < L; ++k) {
-    const int s = 32 * k - sh;
-    r.w[k] = s >= 0 ? (s < 32 ? m >> s : 0u) : (s > -32 ? m << (-s) : 0u);
-  }
-  return (bits >> 31) ? -r : r;
-}
-
-// 1/sqrt(x) for x in [2^-20, 2^12), on the integer pipe apart from an FP32
-// seed.  Seed: the single-precision inverse square root of the float of x's
-// two leading limbs (from the integer limb, or from the first fraction limb
-// when x < 1; the limbs left out change x by less than 2^-32 relative), with
-// a relative error below 2^-21; when the seed rounded
-// to 12 significant bits squares exactly to 1/x in single precision it is
-// taken instead, so that exact cases (x = 1, 1/4, 4, ...) stay exact.  The
-// seed lies in (2^-6, 2^11), i.e. in limbs F-1 .. F.  Then two third-order
-// steps y <- y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2:
-//   1. y0^2 is exact (48 bits), e^2 comes from the float of e (|e| < 2^-20);
-//      the result, cut to limbs F-2 .. F (2^-64 resolution), has |e| < 2^-55;
-//   2. y1^2 is exact (192 bits), e^2 is a short product of |e| cut to limbs
-//      F-5 .. F-2; the remaining error 5|e|^3/16 is below 2^-165 relative.
-// Every product has a short nonnegative factor (mul_short).
+// 1/sqrt(x) for x in [2^-20, 2^12), on the integer pipe apart from an FP32 seed.
+// x is normalised to x = m 2^(2h), m in [1, 4), as the integer M = m 2^(32 F + 30)
+// of F + 1 limbs (so its top limb has two integer bits), and y = m^(-1/2) in
+// (1/2, 1] is refined by third-order steps y <- y (1 + e/2 + 3 e^2/8), e = 1 - m y^2:
+//   seed   the single-precision inverse square root of the float of M's top limb,
+//          Y0 = y0 2^31, |e| < 2^-20; if y0 rounded to 12 significant bits squares
+//          exactly to 1/m in single precision it is taken instead, so that exact
+//          cases (x = 1, 1/4, 4, ...) stay exact;
+//   1.     e 2^64 from the exact 128-bit difference 2^124 - (top 64 bits of M) Y0^2;
+//          Y1 = y1 2^63 (64 bits), |e| < 2^-59;
+//   2.     (F > 2) e from the product of M and the exact 128-bit Y1^2, of which only
+//          the columns from just below the wanted resolution up to the one |e| can
+//          reach are formed (the leading ones cancel against the 1); e^2 from the
+//          top 64 bits of e; the result's relative error is below 2^-165 (F >= 5),
+//          2^-150 (F = 4).
+// With F = 2 the value after step 1 is returned (relative error below 2^-61).
+// The normalisation makes every factor short: 39 partial products for F = 5,
+// against 89 for the same steps on the unnormalised limbs.
 template <int L, int F>
 __device__ __forceinline__ fxn<L, F> rsqrt_(const fxn<L, F>& x) {
-  fxn<L, F> one;
+  static_assert(L == F + 1, "one integer limb");
+  const unsigned long long top = ((unsigned long long)x.w[F] << 32) | x.w[F - 1];
+  const int sh = __clzll((long long)top) & ~1;  // 20 .. 50 (garbage in, garbage out beyond)
+  const bool mv = sh >= 32;
+  uint32_t M[F + 1];  // x's limbs << sh
 #pragma unroll
-  for (int k = 0; k < L; ++k) one.w[k] = k == F ? 1u : 0u;
-  const float xf = x.w[F] ? __ull2float_rn(((unsigned long long)x.w[F] << 32) | x.w[F - 1]) * 0x1p-32f
-                          : __ull2float_rn(((unsigned long long)x.w[F - 1] << 32) | x.w[F - 2]) * 0x1p-64f;
-  float yf = rsqrtf(xf);
+  for (int k = F; k >= 0; --k) {
+    const uint32_t hi = mv ? (k >= 1 ? x.w[k >= 1 ? k - 1 : 0] : 0u) : x.w[k];
+    const uint32_t lo = mv ? (k >= 2 ? x.w[k >= 2 ? k - 2 : 0] : 0u) : (k >= 1 ? x.w[k >= 1 ? k - 1 : 0] : 0u);
+    M[k] = __funnelshift_l(lo, hi, sh);
+  }
+  const int h = (30 - sh) / 2;  // -10 .. 5 (sh is even)
+  const float mf = __uint2float_rn(M[F]) * 0x1p-30f;
+  float yf = rsqrtf(mf);
   const float ys = __uint_as_float((__float_as_uint(yf) + 0x800u) & ~0xfffu);
-  if (fmaf(xf * ys, ys, -1.0f) == 0.0f) yf = ys;
-  const fxn<L, F> y0 = fx_from_float<L, F>(yf);
+  if (fmaf(mf * ys, ys, -1.0f) == 0.0f) yf = ys;
+  const uint32_t Y0 = __float2uint_rz(yf * 0x1p31f);
   // step 1
-  const fxn<L, F> y0sq = mul_short<F - 1, F, L, F, F - 1, F>(y0, y0);
-  const fxn<L, F> e0 = one - mul_short<F - 2, F>(x, y0sq);
-  const float e0f = __ll2float_rn((long long)(((unsigned long long)e0.w[F - 1] << 32) | e0.w[F - 2])) * 0x1p-64f;
-  const fxn<L, F> c0 = fx_half(e0) + fx_from_float<L, F>(0.375f * e0f * e0f);
-  fxn<L, F> y1 = y0 + mul_short<F - 1, F>(c0, y0);
+  const unsigned long long q0 = (unsigned long long)Y0 * Y0;
+  const unsigned long long mt = ((unsigned long long)M[F] << 32) | M[F - 1];
+  const unsigned long long plo = mt * q0, phi = __umul64hi(mt, q0);
+  const unsigned long long dhi = (1ull << 60) - phi - (plo != 0ull);
+  const long long e64 = (long long)((dhi << 4) | ((0ull - plo) >> 60));  // e 2^64
+  const int es = (int)(e64 >> 14);                                       // e 2^50
+  const unsigned long long sq = (unsigned long long)((long long)es * es) >> 36;
+  const long long f = (e64 >> 1) + (long long)((sq * 3ull) >> 3);        // (e/2 + 3 e^2/8) 2^64
+  const int fh = (int)(f >> 32);
+  const unsigned long long Y1 = ((unsigned long long)Y0 << 32) + (unsigned long long)((long long)fh * (long long)Y0) +
+                                (((unsigned long long)(uint32_t)f * Y0) >> 32);
+  fxn<L, F> r;
+  const uint32_t yh = (uint32_t)(Y1 >> 32), yl = (uint32_t)Y1;
+  if constexpr (F == 2) {
+    // y 2^(64 + 26), then down by 26 + h (16 .. 31)
+    const uint32_t a0 = yl << 27, a1 = __funnelshift_l(yl, yh, 27), a2 = yh >> 5;
+    r.w[0] = __funnelshift_r(a0, a1, 26 + h);
+    r.w[1] = __funnelshift_r(a1, a2, 26 + h);
+    r.w[2] = a2 >> ((26 + h) & 31);
+    return r;
+  } else {
+    // step 2
+    const unsigned long long ll = (unsigned long long)yl * yl, lh = (unsigned long long)yl * yh,
+                             hh = (unsigned long long)yh * yh;
+    const unsigned long long s0 = ll + (lh << 33);
+    const unsigned long long s1 = hh + (lh >> 31) + (s0 < ll ? 1ull : 0ull);
+    const uint32_t q[4] = {(uint32_t)s0, (uint32_t)(s0 >> 32), (uint32_t)s1, (uint32_t)(s1 >> 32)};
+    // 1 = 2^(32 F + 156) in the product; e needs the columns CLO + 1 .. CHI
+    constexpr int CHI = (32 * F + 156 - 59) / 32;
+    constexpr int CLO = F >= 6 ? 4 : 3;
+    constexpr int NE = CHI - CLO;  // limbs of e 2^U2
+    uint32_t t[NE + 1];
+    prod_cols<F + 1, 4, CLO, CHI>(M, q, t);
+    uint32_t e[NE];
+    e[0] = sub_cc(0u, t[1]);
 #pragma unroll
-  for (int k = 0; k < F - 2; ++k) y1.w[k] = 0u;
-  // step 2
-  constexpr int ELO = F - 5 > 0 ? F - 5 : 0;
-  const fxn<L, F> y1sq = mul_short<F - 2, F, L, F, F - 2, F>(y1, y1);
-  const fxn<L, F> e1 = one - mul_short<F - 4, F>(x, y1sq);
-  const bool neg = (int32_t)e1.w[L - 1] < 0;
-  fxn<L, F> ae = neg ? -e1 : e1;
+    for (int k = 1; k < NE - 1; ++k) e[k] = subc_cc(0u, t[k + 1]);
+    e[NE - 1] = subc(0u, t[NE]);
+    // c = e/2 + 3 e^2/8 in units of 2^-U, U = 32 F + 155 - 32 (CLO + 1); |c| < 2^-60
+    constexpr int NC = NE - 1;  // limbs of c, two's complement
+    uint32_t c[NC];
 #pragma unroll
-  for (int k = 0; k < L; ++k)
-    if (k < ELO || k > F - 2) ae.w[k] = 0u;
-  const fxn<L, F> esq = mul_short<ELO, F - 2, L, F, ELO, F - 2>(ae, ae);
-  const fxn<L, F> q = fx_half(fx_half(esq));
-  const fxn<L, F> c1 = fx_half(e1) + (q + fx_half(q));  // e/2 + 3 e^2 / 8
-  return y1 + mul_short<F - 2, F>(c1, y1);
+    for (int k = 0; k < NC; ++k) c[k] = __funnelshift_r(e[k], e[k + 1], 2);
+    const uint32_t neg = (uint32_t)((int32_t)c[NC - 1] >> 31);
+    // |e/2| 2^(U - 32 (NC - 2)) in two limbs (the truncated rest is below 2^-123)
+    const uint32_t ah = c[NC - 1] ^ neg, al = c[NC - 2] ^ neg;
+    const unsigned long long sll = (unsigned long long)al * al, slh = (unsigned long long)al * ah,
+                             shh = (unsigned long long)ah * ah;
+    const unsigned long long sm = (sll >> 32) + (slh << 1);  // (2 al ah) + carry: below 2^64 as ah < 2^31
+    const unsigned long long sq2 = shh + (sm >> 32);         // (e/2)^2 2^(2U - 64 (NC - 2) - 64)
+    // (e/2)^2 in units of 2^-U: up by U - (2U - 64 (NC - 2) - 64) = 64 (NC - 1) - U
+    constexpr int U = 32 * F + 155 - 32 * (CLO + 1);
+    constexpr int DN = U - 64 * (NC - 1);  // -5 for every F: 64 (NC - 1) - U = 5
+    static_assert(DN == -5 || DN == 27, "alignment of the squared residual");
+    unsigned long long q2;
+    uint32_t q2h;
+    if constexpr (DN == -5) {
+      const unsigned long long w = (sq2 << 5) | ((sm & 0xffffffffull) >> 27);
+      const uint32_t wh = (uint32_t)(sq2 >> 59);
+      q2 = w + ((w >> 1) | ((unsigned long long)wh << 63));  // 3/2 (e/2)^2
+      q2h = wh + (wh >> 1) + (q2 < w ? 1u : 0u);
+    } else {
+      const unsigned long long w = sq2 >> 27;
+      q2 = w + (w >> 1);
+      q2h = 0u;
+    }
+    c[0] = add_cc(c[0], (uint32_t)q2);
+    c[1] = addc_cc(c[1], (uint32_t)(q2 >> 32));
+    if constexpr (NC == 3) {
+      c[2] = addc(c[2], q2h);
+    } else {
+      c[2] = addc_cc(c[2], q2h);
+#pragma unroll
+      for (int k = 3; k < NC - 1; ++k) c[k] = addc_cc(c[k], 0u);
+      c[NC - 1] = addc(c[NC - 1], 0u);
+    }
+    // y 2^(U - 1) = Y1 2^(U - 64) + c Y1 2^-64 (NC + 2 limb product, limbs 2 up)
+    const uint32_t sg = (uint32_t)((int32_t)c[NC - 1] >> 31);
+    const uint32_t yy[2] = {yl, yh};
+    uint32_t d[NC + 1];
+    prod_cols<NC, 2, 1, NC + 1>(c, yy, d);  // d[k]: limb k + 1; d[0] is the guard
+    uint32_t o[NC + 1];                      // limbs 2 .. NC + 1, then the sign
+#pragma unroll
+    for (int k = 0; k < NC; ++k) o[k] = d[k + 1];
+    o[NC - 2] = sub_cc(o[NC - 2], yl & sg);
+    o[NC - 1] = subc_cc(o[NC - 1], yh & sg);
+    // Y1 2^(U - 64) covers the limbs Z .. Z + 2
+    constexpr int ZB = U - 64, Z = ZB / 32, ZS = ZB % 32;
+    constexpr int NO = NC + 2;
+    uint32_t z[NO];
+#pragma unroll
+    for (int k = 0; k < NO; ++k) z[k] = 0u;
+    z[Z] = yl << ZS;
+    z[Z + 1] = __funnelshift_l(yl, yh, ZS);
+    z[Z + 2] = ZS ? yh >> (32 - ZS) : 0u;
+    const uint32_t sx = (uint32_t)((int32_t)o[NC - 1] >> 31);
+    uint32_t v[NO];
+    v[0] = add_cc(z[0], o[0]);
+#pragma unroll
+    for (int k = 1; k < NO - 1; ++k) v[k] = addc_cc(z[k], k < NC ? o[k] : sx);
+    v[NO - 1] = addc(z[NO - 1], sx);
+    // v = y 2^(U - 1); the result is y 2^-h in units of 2^-32F: down by U - 1 - 32 F + h
+    constexpr int SD = U - 1 - 32 * F;  // 26 (F <= 5) or -6 (F = 6: one limb of zeros below)
+    static_assert(SD == 26 || SD == -6, "alignment of the result");
+    constexpr int PADL = SD < 0 ? 1 : 0;
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+      const int a = k - PADL, b = a + 1;
+      const uint32_t lo = a >= 0 && a < NO ? v[a >= 0 && a < NO ? a : 0] : 0u;
+      const uint32_t hi = b >= 0 && b < NO ? v[b >= 0 && b < NO ? b : 0] : 0u;
+      r.w[k] = __funnelshift_r(lo, hi, 26 + h);
+    }
+    return r;
+  }
 }
 
-// ------------------------------------------------------ sums and reduction --
-// The four sign-split sums are exact and non-negative: add them, convert once.
-template <int L, int F>
-struct sums_total<fxn<L, F>> {
-  static GBS_HD double of(const Sums<fxn<L, F>>& a) { return to_double((a.ip + a.in) + (a.ep + a.en)); }
-};
-template <> struct acc_traits<fxn4> { typedef fxn4s Acc; typedef fxn4s Red; };
-template <> struct acc_traits<fx> { typedef fxs Acc; typedef fxs Red; };
-template <> struct acc_traits<fxw> { typedef fxws Acc; typedef fxws Red; };
-template <int L, int F> GBS_HD void acc_add(fxn<L, F>& a, const fxn<L, F>& x) { a = a + x; }
-template <int L, int F>
-GBS_HD void acc_fpa(fxn<L + 1, F>& acc, const fxn<L + 1, F>& s, const fxn<L, F>& g) { acc = acc + s * g; }
-template <int L, int F> GBS_HD fxn<L, F> red_diff(const fxn<L, F>& a, const fxn<L, F>& b, fxn<L, F>*) { return a - b; }
-template <int L, int F> GBS_HD fxn<L, F> red_add(const fxn<L, F>& a, const fxn<L, F>& b) { return a + b; }
-template <int L, int F> GBS_HD fxn<L, F> red_neg(const fxn<L, F>& a) { return -a; }
-template <> GBS_HD fxn4s red_zero<fxn4s>() { return from_double<fxn4s>(0.0); }
-template <> GBS_HD fxs red_zero<fxs>() { return from_double<fxs>(0.0); }
-template <> GBS_HD fxws red_zero<fxws>() { return from_double<fxws>(0.0); }
 // Three doubles whose sum is the value to ~2^-159 relative (each the nearest
 // double of what the previous ones left over; the differences are exact).
 template <int L, int F>
-GBS_HD void red_store(const fxn<L, F>& a, double* o) {
+GBS_HD void fx_store3(const fxn<L, F>& a, double* o) {
   const double x0 = to_double(a);
   const fxn<L, F> r1 = a - fx_from_double<L, F>(x0);
   const double x1 = to_double(r1);

@@ -1,0 +1,591 @@
+// Subset-determinant trees in fixed point (gbs_fx.cuh): kernels.
+//
+// The decision tree of gbs_tree.cuh for the integer entry types, organised so
+// that only *included* children are ever computed or stored: excluding a mode
+// drops two rows, so an excluded child is a view of its parent's matrix.
+//
+// Nodes.  With the first D = n - Q modes of a tree decided, node v in [0, 2^D)
+// has mode j included iff bit j of v is set.  Its matrix is that of its last
+// included mode: v = 0 is the root (all n modes), and v with top bit k is matrix
+// v - 2^k of level k, the Schur complement of the q = n - 1 - k modes after mode
+// k given the included ones; a node at depth d > k is the trailing 2 (n - d) rows
+// of it.  Level k has 2^k matrices, and its parents are exactly the nodes
+// 0 .. 2^k - 1: matrix c of level k includes mode k at node c.  Against storing
+// both children of every node this halves the writes and takes a quarter off the
+// traffic.
+//
+//   top kernel    one CTA per node v < 2^dtop: eliminates the modes of v from the
+//                 root in shared memory and writes that matrix; replaces the
+//                 first levels, where nodes are few.
+//   level kernel  one launch per child size q: a CTA of W warps takes 32
+//                 consecutive children of one tree (lane = child).
+//   leaf kernel   a warp takes tiles of 32 nodes of one tree, one thread per node
+//                 for all 2^Q subsets of its last Q modes.
+//   final kernel  one CTA per tree adds the warps' sums.
+// Measured against the engine it replaced (both children stored, subtrees of 9
+// modes expanded in shared memory, signed products, 2 products per entry), with the
+// default launch shapes: N = 24 (M = 200, AUTO) 8.86 -> 3.32 ms, 256 requests of N =
+// 8 .. 20 23.1 -> 9.2 ms.
+// All sums are exact integers, and every pivot, row and entry is formed by the
+// same functions below wherever it is formed: results do not depend on the launch
+// shape or on the rest of the batch, bit for bit.
+//
+// Including a mode with pivot block P = [[p00, p10], [p10, p11]] and its columns
+// U = (u0, u1): C' = C - L U^T, L = U P^-1.  Products are the cost, so they are
+// saved where exact additions can take their place:
+//   rows     the second pivot coordinate is flipped where p10 > 0, so that with
+//            al = p11/det, be = p00/det, m = |p10|/det >= 0
+//              L0 = (al + m) u0 - m (u0 - u1),  L1 = (be + m) u1 + m (u0 - u1):
+//            three products per row in place of four;
+//   entries  Winograd's inner product (S. Winograd, IEEE Trans. Comp. C-17, 1968):
+//              L0_a u0_b + L1_a u1_b = (L0_a + u1_b)(u0_b + L1_a) - L0_a L1_a - u0_b u1_b:
+//            one product per entry and two per row in place of two per entry.
+// An update of R rows takes R (R + 1) / 2 + 5 R products in place of R (R + 1) +
+// 4 R (R = 4, 6, 8: 30, 51, 76 for 36, 66, 104).  Neither form loses accuracy
+// here: sums are exact and a product's error is absolute, whatever its factors.
+// Signed factors are shifted by K = 2^9 (entries and rows of L stay below 128 in
+// magnitude on every matrix the host admits: |u| <= lambda_max <= 64, and U P^-1 U^T
+// <= C bounds a row of L by |L_a|^2 <= C_aa lambda_max(P^-1) <= lambda_max / lambda_min
+// <= 2^14), so that all products are of
+// non-negative values; the shifts are separable and live in c0, c1, A and B:
+//   U = u0 + K, V = u1 + K, P = L0 + K, Q = L1 + K
+//   P = (al + m) U - m (U - V + 2K) + c0,  c0 = K + 2K m - K (al + m)
+//   Q = (be + m) V + m (U - V + 2K) + c1,  c1 = K - 2K m - K (be + m)
+//   A = (P + K)(Q + K) - 2 K^2,  B = (U + K)(V + K) - 2 K^2
+//   C' = C - (P_a + V_b)(U_b + Q_a) + A_a + B_b
+#pragma once
+#include "gbs_fx.cuh"
+#include "gbs_internal.h"
+#include "gbs_tree.cuh"
+
+namespace gbs {
+
+constexpr uint32_t kFxShift = 1u << 9;  // K
+
+// Scalars of a pivot.
+template <class E>
+struct FxPivot {
+  E g, a, b, m, c0, c1;  // det^(-1/2), al + m, be + m, m and the row constants
+  uint32_t flip;         // all ones: the second coordinate changes sign
+};
+// A row of the update: P, Q, A (as row a) and U, V, B (as column b).
+template <class E>
+struct FxRow {
+  E P, Q, A, U, V, B;
+};
+
+// x + v 2^(32 F): v in the integer limb.
+template <int L, int F>
+GBS_HD fxn<L, F> fx_add_int(fxn<L, F> x, uint32_t v) {
+  x.w[L - 1] += v;
+  return x;
+}
+// x << s (0 < s < 32)
+template <int L, int F>
+__device__ __forceinline__ fxn<L, F> fx_shl(const fxn<L, F>& x, int s) {
+  fxn<L, F> r;
+#pragma unroll
+  for (int k = L - 1; k > 0; --k) r.w[k] = __funnelshift_l(x.w[k - 1], x.w[k], s);
+  r.w[0] = x.w[0] << s;
+  return r;
+}
+// x, or -x where mask is all ones
+template <int L, int F>
+GBS_HD fxn<L, F> fx_flip(const fxn<L, F>& x, uint32_t mask) {
+  fxn<L, F> t, r;
+#pragma unroll
+  for (int k = 0; k < L; ++k) t.w[k] = x.w[k] ^ mask;
+  r.w[0] = sub_cc(t.w[0], mask);
+#pragma unroll
+  for (int k = 1; k < L - 1; ++k) r.w[k] = subc_cc(t.w[k], mask);
+  r.w[L - 1] = subc(t.w[L - 1], mask);
+  return r;
+}
+
+// |x|; mask (all ones where x < 0)
+template <int L, int F>
+GBS_HD fxn<L, F> fx_abs(const fxn<L, F>& x, uint32_t& mask) {
+  mask = (uint32_t)((int32_t)x.w[L - 1] >> 31);
+  return fx_flip(x, mask);
+}
+
+// det(P); the determinant alone is what a one-mode node needs.
+template <class E>
+__device__ __forceinline__ E fx_det(const E& p00, const E& p10, const E& p11) {
+  uint32_t neg;
+  const E n10 = fx_abs(p10, neg);
+  return umul(p00, p11) - umul(n10, n10);
+}
+
+// Returns whether the determinant is in range.
+template <class E>
+__device__ __forceinline__ bool fx_pivot(const E& p00, const E& p10, const E& p11, FxPivot<E>& pv) {
+  uint32_t neg;
+  const E n10 = fx_abs(p10, neg);
+  bool zero = true;
+#pragma unroll
+  for (int k = 0; k < (int)(sizeof(E) / 4); ++k) zero &= p10.w[k] == 0u;
+  pv.flip = (neg == 0u && !zero) ? 0xffffffffu : 0u;  // p10 > 0
+  const E det = umul(p00, p11) - umul(n10, n10);
+  pv.g = rsqrt_(det);
+  const E inv = umul(pv.g, pv.g);
+  pv.m = umul(n10, inv);
+  pv.a = umul(p11, inv) + pv.m;
+  pv.b = umul(p00, inv) + pv.m;
+  const E km = fx_shl(pv.m, 10);  // 2 K m
+  pv.c0 = fx_add_int(km - fx_shl(pv.a, 9), kFxShift);
+  pv.c1 = fx_add_int(-(km + fx_shl(pv.b, 9)), kFxShift);
+  return fx_det_in_range(det);
+}
+
+template <class E>
+__device__ __forceinline__ void fx_row(const FxPivot<E>& pv, const E& u0, const E& u1, FxRow<E>& r) {
+  r.U = fx_add_int(u0, kFxShift);
+  r.V = fx_add_int(fx_flip(u1, pv.flip), kFxShift);
+  const E mt = umul(pv.m, fx_add_int(r.U - r.V, 2 * kFxShift));
+  r.P = umul(pv.a, r.U) - mt + pv.c0;
+  r.Q = umul(pv.b, r.V) + mt + pv.c1;
+  r.A = fx_add_int(umul(fx_add_int(r.P, kFxShift), fx_add_int(r.Q, kFxShift)), 0u - 2u * kFxShift * kFxShift);
+  r.B = fx_add_int(umul(fx_add_int(r.U, kFxShift), fx_add_int(r.V, kFxShift)), 0u - 2u * kFxShift * kFxShift);
+}
+
+// Entry (a, b) of the child.
+template <class E>
+__device__ __forceinline__ E fx_entry(const E& c, const E& Pa, const E& Qa, const E& Aa, const E& Ub, const E& Vb,
+                                      const E& Bb) {
+  return (c + Aa + Bb) - umul(Pa + Vb, Ub + Qa);
+}
+
+// ------------------------------------------------------------- node buffers --
+// Matrices of level k are packed lower triangles.  From level 5 on they lie in
+// tiles of 32: limb l of entry e of matrix c is word ((c / 32) ne + e) 32 L + 32 l +
+// c % 32, so a warp's access is one 128-byte line and the limbs of an entry are at
+// constant distances (immediate offsets).  The root and levels 0 .. 4, less than a
+// tile each, are stored one matrix after another (stride 1 between limbs).
+template <class E, int ST>
+__device__ __forceinline__ E fx_ld(const uint32_t* p, int e) {
+  constexpr int L = sizeof(E) / 4;
+  const uint32_t* q = p + (long long)e * (L * ST);
+  E r;
+#pragma unroll
+  for (int k = 0; k < L; ++k) r.w[k] = q[k * ST];
+  return r;
+}
+template <class E, int ST>
+__device__ __forceinline__ void fx_st(uint32_t* p, int e, const E& v) {
+  constexpr int L = sizeof(E) / 4;
+  uint32_t* q = p + (long long)e * (L * ST);
+#pragma unroll
+  for (int k = 0; k < L; ++k) q[k * ST] = v.w[k];
+}
+
+// One tree of a batch.  Level k of it starts at word lvl_off[tab + k + 1] of the
+// node buffer (k = -1: the root).
+//
+// A tree whose levels would not fit the workspace is taken in chunks: the nodes of
+// depth d0 stay, and the levels from d0 on hold the descendants of 2^cb consecutive
+// ones at a time.  Inside chunk h, index v' >= 2^cb stands for the node with low
+// bits (v' mod 2^cb) + h 2^cb and its bits from d0 on those of v' from cb on; v' <
+// 2^cb for node v' + h 2^cb of depth d0.  Unchunked, cb = d0 = 0 and v' = v.
+// s of it is element s_base + v (v < 2^d0), s_base + 2^d0 - 2^cb + v'.
+struct FxTree {
+  long long root_off, s_base;
+  int n, D, tree, tab, d0, cb;
+};
+struct FxSeg {
+  long long first;  // first CTA (top) / tile (level) / warp unit (leaf) of this tree
+  int idx, tiles_per_unit;
+};
+template <class Sum>
+struct FxPart {
+  Sum inc, exc, abs;
+};
+
+__device__ __forceinline__ int fx_find(const FxSeg* segs, int n, long long key) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (segs[mid].first <= key) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Where the matrix of index v is, and how many modes (p) it holds.  ST = 32 for
+// nodes in tiles, 1 for nodes 0 .. 31 of a tree.
+template <int ST, int L>
+__device__ __forceinline__ const uint32_t* fx_node(const uint32_t* nodes, const long long* lvl_off, const FxTree& t,
+                                                   unsigned v, unsigned chunk, int& p) {
+  int up = 0;  // levels of the tree above bit 0 of v's level
+  if (v < (1u << t.cb)) {
+    v += chunk << t.cb;
+    if (v == 0u) {
+      p = t.n;
+      return nodes + lvl_off[t.tab];
+    }
+  } else {
+    up = t.d0 - t.cb;
+  }
+  const int k = 31 - __clz((int)v);
+  const unsigned c = v - (1u << k);
+  p = t.n - 1 - k - up;
+  const int ne = sym(2 * p);
+  const uint32_t* base = nodes + lvl_off[t.tab + k + up + 1];
+  if constexpr (ST == 1) return base + (long long)c * ne * L;
+  return base + (long long)(c >> 5) * ne * (L * 32) + (c & 31u);
+}
+__device__ __forceinline__ long long fx_sidx(const FxTree& t, unsigned v, unsigned chunk) {
+  return v < (1u << t.cb) ? t.s_base + v + ((long long)chunk << t.cb)
+                          : t.s_base + (1LL << t.d0) - (1LL << t.cb) + v;
+}
+
+// ---------------------------------------------------------------------- top --
+template <class E>
+__global__ void __launch_bounds__(256) fx_top_kernel(const FxSeg* __restrict__ segs, int nseg,
+                                                     const FxTree* __restrict__ trees,
+                                                     const long long* __restrict__ lvl_off,
+                                                     const double* __restrict__ roots, uint32_t* __restrict__ nodes,
+                                                     typename fx_sum<E>::type* __restrict__ sval,
+                                                     int* __restrict__ status) {
+  typedef typename fx_sum<E>::type S;
+  constexpr int L = sizeof(E) / 4;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxPivot<E> pv;
+  const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
+  const FxTree t = trees[sg.idx];
+  const unsigned v = (unsigned)((long long)blockIdx.x - sg.first);  // (the top runs before any chunk: v' = v)
+  const int d = 2 * t.n;
+  E* C = reinterpret_cast<E*>(smem_raw);
+  FxRow<E>* rows = reinterpret_cast<FxRow<E>*>(C + sym(d));
+  for (int i = threadIdx.x; i < sym(d); i += blockDim.x)
+    C[i] = fx_of<E>(roots[t.root_off + i]);
+  S s = fx_of<S>(1.0);
+  bool ok = true;
+  __syncthreads();
+  for (unsigned left = v; left; left &= left - 1u) {
+    const int o = 2 * (__ffs((int)left) - 1);
+    if (threadIdx.x < 32) {  // one warp forms the pivot (every lane the same)
+      FxPivot<E> q;
+      ok &= fx_pivot(C[tri(o, o)], C[tri(o + 1, o)], C[tri(o + 1, o + 1)], q);
+      s = umul(s, q.g);
+      if (threadIdx.x == 0) pv = q;
+    }
+    __syncthreads();
+    const int R = d - o - 2;
+    for (int a = threadIdx.x; a < R; a += blockDim.x) fx_row(pv, C[tri(a + o + 2, o)], C[tri(a + o + 2, o + 1)], rows[a]);
+    __syncthreads();
+    for (int e = threadIdx.x; e < sym(R); e += blockDim.x) {
+      int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+      while (a * (a + 1) / 2 > e) --a;
+      while ((a + 1) * (a + 2) / 2 <= e) ++a;
+      const int b = e - a * (a + 1) / 2;
+      E& c = C[tri(a + o + 2, b + o + 2)];
+      c = fx_entry(c, rows[a].P, rows[a].Q, rows[a].A, rows[b].U, rows[b].V, rows[b].B);
+    }
+    __syncthreads();
+  }
+  int p;
+  uint32_t* out;
+  const bool tiled = v >= 32u;
+  if (tiled) out = const_cast<uint32_t*>(fx_node<32, L>(nodes, lvl_off, t, v, 0u, p));
+  else out = const_cast<uint32_t*>(fx_node<1, L>(nodes, lvl_off, t, v, 0u, p));
+  const int o = d - 2 * p;
+  for (int e = threadIdx.x; e < sym(2 * p); e += blockDim.x) {
+    int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+    while (a * (a + 1) / 2 > e) --a;
+    while ((a + 1) * (a + 2) / 2 <= e) ++a;
+    const int b = e - a * (a + 1) / 2;
+    if (tiled) fx_st<E, 32>(out, e, C[tri(a + o, b + o)]); else fx_st<E, 1>(out, e, C[tri(a + o, b + o)]);
+  }
+  if (threadIdx.x == 0) sval[t.s_base + v] = s;
+  if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
+}
+
+// -------------------------------------------------------------------- level --
+// Children of q = R / 2 modes, one CTA of W warps per tile of 32.  One warp forms
+// the 32 pivots (a chain: the other warps' CTAs hide it), then the rows and then
+// the entries are shared out among the warps; rows wait in shared memory.
+template <class E, int ST>
+__device__ __forceinline__ void fx_level_tile(const FxTree& t, const long long* lvl_off, int q, unsigned tile,
+                                              unsigned chunk, uint32_t* nodes, typename fx_sum<E>::type* sval, int* status,
+                                              uint32_t* sh) {
+  constexpr int L = sizeof(E) / 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const int R = 2 * q;
+  const int k = t.n - 1 - q;
+  const unsigned c = tile * 32u + lane;  // child of level k = parent node
+  int p;
+  const uint32_t* par = fx_node<ST, L>(nodes, lvl_off, t, c, chunk, p);
+  const int o = 2 * (p - q - 1);  // the pivot's first row in the parent
+  uint32_t* out = nodes + lvl_off[t.tab + k + 1] + (long long)tile * sym(R) * (L * 32) + lane;
+  uint32_t* piv = sh + lane;                    // 5 values and the flip of a pivot
+  uint32_t* rowp = sh + (5 * L + 1) * 32 + lane;  // 6 values per row
+  if (warp == 0) {
+    FxPivot<E> pv;
+    const bool ok = fx_pivot(fx_ld<E, ST>(par, tri(o, o)), fx_ld<E, ST>(par, tri(o + 1, o)),
+                             fx_ld<E, ST>(par, tri(o + 1, o + 1)), pv);
+    if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
+    sval[fx_sidx(t, (1u << (k - t.d0 + t.cb)) + c, chunk)] = umul(sval[fx_sidx(t, c, chunk)], pv.g);
+    fx_st<E, 32>(piv, 0, pv.a);
+    fx_st<E, 32>(piv, 1, pv.b);
+    fx_st<E, 32>(piv, 2, pv.m);
+    fx_st<E, 32>(piv, 3, pv.c0);
+    fx_st<E, 32>(piv, 4, pv.c1);
+    piv[5 * L * 32] = pv.flip;
+  }
+  __syncthreads();
+  {
+    FxPivot<E> pv;
+    pv.a = fx_ld<E, 32>(piv, 0);
+    pv.b = fx_ld<E, 32>(piv, 1);
+    pv.m = fx_ld<E, 32>(piv, 2);
+    pv.c0 = fx_ld<E, 32>(piv, 3);
+    pv.c1 = fx_ld<E, 32>(piv, 4);
+    pv.flip = piv[5 * L * 32];
+#pragma unroll 1
+    for (int a = warp; a < R; a += W) {
+      const int e = tri(o + 2 + a, o);
+      FxRow<E> r;
+      fx_row(pv, fx_ld<E, ST>(par, e), fx_ld<E, ST>(par, e + 1), r);
+      uint32_t* w = rowp + a * (6 * L * 32);
+      fx_st<E, 32>(w, 0, r.P);
+      fx_st<E, 32>(w, 1, r.Q);
+      fx_st<E, 32>(w, 2, r.A);
+      fx_st<E, 32>(w, 3, r.U);
+      fx_st<E, 32>(w, 4, r.V);
+      fx_st<E, 32>(w, 5, r.B);
+    }
+  }
+  __syncthreads();
+  const int ne = sym(R);
+  int e = ne * warp / W;
+  const int e1 = ne * (warp + 1) / W;
+  if (e >= e1) return;
+  int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+  while (a * (a + 1) / 2 > e) --a;
+  while ((a + 1) * (a + 2) / 2 <= e) ++a;
+  int b = e - a * (a + 1) / 2;
+  while (e < e1) {
+    const uint32_t* w = rowp + a * (6 * L * 32);
+    const E Pa = fx_ld<E, 32>(w, 0), Qa = fx_ld<E, 32>(w, 1), Aa = fx_ld<E, 32>(w, 2);
+    const int stop = min(e1, e + a + 1 - b);
+    const int src = tri(o + 2 + a, o + 2 + b) - e;
+#pragma unroll 1
+    for (; e < stop; ++e, ++b) {
+      const uint32_t* x = rowp + b * (6 * L * 32);
+      const E cc = fx_ld<E, ST>(par, src + e);
+      fx_st<E, 32>(out, e, fx_entry(cc, Pa, Qa, Aa, fx_ld<E, 32>(x, 3), fx_ld<E, 32>(x, 4), fx_ld<E, 32>(x, 5)));
+    }
+    ++a;
+    b = 0;
+  }
+}
+
+template <class E>
+__global__ void __launch_bounds__(256) fx_level_kernel(const FxSeg* __restrict__ segs, int nseg,
+                                                       const FxTree* __restrict__ trees,
+                                                       const long long* __restrict__ lvl_off, int q, unsigned chunk,
+                                                       uint32_t* nodes, typename fx_sum<E>::type* sval,
+                                                       int* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
+  const FxTree t = trees[sg.idx];
+  const unsigned tile = (unsigned)((long long)blockIdx.x - sg.first);
+  // the first tile's parents are the root and levels 0 .. 4
+  if (tile == 0u && chunk == 0u) fx_level_tile<E, 1>(t, lvl_off, q, tile, chunk, nodes, sval, status, (uint32_t*)smem_raw);
+  else fx_level_tile<E, 32>(t, lvl_off, q, tile, chunk, nodes, sval, status, (uint32_t*)smem_raw);
+}
+
+// --------------------------------------------------------------------- leaf --
+// Signed sums of a thread: terms with / without the last mode, and all magnitudes.
+template <class S>
+struct FxSums {
+  S ip, in, ep, en;  // split by sign: inc = ip - in, exc = ep - en
+};
+
+// The two subsets of a one-mode node: s g and s, signs (-1)^neg and -(-1)^neg.
+template <class E, class S>
+__device__ __forceinline__ bool fx_leaf1(const E& p00, const E& p10, const E& p11, const S& s, bool neg, FxSums<S>& acc) {
+  const E det = fx_det(p00, p10, p11);
+  const S sg = umul(s, rsqrt_(det));
+  if (neg) {
+    acc.in = acc.in + sg;
+    acc.ep = acc.ep + s;
+  } else {
+    acc.ip = acc.ip + sg;
+    acc.en = acc.en + s;
+  }
+  return fx_det_in_range(det);
+}
+
+// The four subsets of a two-mode node c (packed lower triangle, 10 entries).
+template <class E, class S>
+__device__ __forceinline__ bool fx_leaf2(const E (&c)[10], const S& s, bool neg, FxSums<S>& acc) {
+  FxPivot<E> pv;
+  bool ok = fx_pivot(c[0], c[1], c[2], pv);
+  FxRow<E> r0, r1;
+  fx_row(pv, c[3], c[4], r0);
+  fx_row(pv, c[6], c[7], r1);
+  E p00 = fx_entry(c[5], r0.P, r0.Q, r0.A, r0.U, r0.V, r0.B);
+  E p10 = fx_entry(c[8], r1.P, r1.Q, r1.A, r0.U, r0.V, r0.B);
+  E p11 = fx_entry(c[9], r1.P, r1.Q, r1.A, r1.U, r1.V, r1.B);
+  S sv = umul(s, pv.g);
+  // both sides through one copy of the code (the instruction cache is the limit of
+  // an inlined one)
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    ok &= fx_leaf1(p00, p10, p11, sv, neg != (side != 0), acc);
+    p00 = c[5];
+    p10 = c[8];
+    p11 = c[9];
+    sv = s;
+  }
+  return ok;
+}
+
+template <class E, int Q, int ST>
+__device__ __forceinline__ bool fx_leaf_node(const uint32_t* m, int p, const typename fx_sum<E>::type& s,
+                                             FxSums<typename fx_sum<E>::type>& acc) {
+  typedef typename fx_sum<E>::type S;
+  const int o = 2 * (p - Q);
+  if constexpr (Q == 1) {
+    return fx_leaf1(fx_ld<E, ST>(m, tri(o, o)), fx_ld<E, ST>(m, tri(o + 1, o)), fx_ld<E, ST>(m, tri(o + 1, o + 1)), s,
+                    false, acc);
+  } else if constexpr (Q == 2) {
+    E c[10];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int row = tri(o + a, o);
+#pragma unroll
+      for (int b = 0; b <= a; ++b) c[tri(a, b)] = fx_ld<E, ST>(m, row + b);
+    }
+    return fx_leaf2(c, s, false, acc);
+  } else {
+    // three modes: the included child is formed entry by entry from the node's
+    // matrix, which is read where it lies; the excluded one is its last four rows
+    static_assert(Q == 3, "at most three levels per leaf thread");
+    E c[10];
+    S sv;
+    bool ok;
+    {
+      FxPivot<E> pv;
+      ok = fx_pivot(fx_ld<E, ST>(m, tri(o, o)), fx_ld<E, ST>(m, tri(o + 1, o)), fx_ld<E, ST>(m, tri(o + 1, o + 1)), pv);
+      sv = umul(s, pv.g);
+      FxRow<E> r[4];
+#pragma unroll 1
+      for (int a = 0; a < 4; ++a) {
+        const int e = tri(o + 2 + a, o);
+        fx_row(pv, fx_ld<E, ST>(m, e), fx_ld<E, ST>(m, e + 1), r[a]);
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b)
+          c[tri(a, b)] = fx_entry(fx_ld<E, ST>(m, tri(o + 2 + a, o + 2) + b), r[a].P, r[a].Q, r[a].A, r[b].U, r[b].V,
+                                  r[b].B);
+    }
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+      ok &= fx_leaf2(c, sv, side != 0, acc);
+      if (side == 0) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b <= a; ++b) c[tri(a, b)] = fx_ld<E, ST>(m, tri(o + 2 + a, o + 2) + b);
+        sv = s;
+      }
+    }
+    return ok;
+  }
+}
+
+// One warp per unit: tiles_per_unit consecutive tiles of 32 nodes of one tree.
+template <class E, int Q>
+__global__ void __launch_bounds__(128) fx_leaf_kernel(const FxSeg* __restrict__ segs, int nseg, long long units,
+                                                      unsigned chunk, const FxTree* __restrict__ trees,
+                                                      const long long* __restrict__ lvl_off,
+                                                      const uint32_t* __restrict__ nodes,
+                                                      const typename fx_sum<E>::type* __restrict__ sval,
+                                                      FxPart<typename fx_sum<E>::type>* __restrict__ parts,
+                                                      int* __restrict__ status) {
+  typedef typename fx_sum<E>::type S;
+  constexpr int L = sizeof(E) / 4;
+  const int lane = threadIdx.x & 31;
+  const long long unit = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (unit >= units) return;
+  const FxSeg sg = segs[fx_find(segs, nseg, unit)];
+  const FxTree t = trees[sg.idx];
+  const unsigned count = 1u << (t.D - t.d0 + t.cb);
+  const S zero = fx_of<S>(0.0);
+  S inc = zero, exc = zero, mag = zero;
+  bool ok = true;
+  const unsigned tile0 = (unsigned)(unit - sg.first) * (unsigned)sg.tiles_per_unit;
+#pragma unroll 1
+  for (int i = 0; i < sg.tiles_per_unit; ++i) {
+    const unsigned v = (tile0 + i) * 32u + lane;
+    if (v >= count) break;
+    FxSums<S> acc{zero, zero, zero, zero};
+    const S s = sval[fx_sidx(t, v, chunk)];
+    int p;
+    if (v < 32u && chunk == 0u) {
+      const uint32_t* m = fx_node<1, L>(nodes, lvl_off, t, v, chunk, p);
+      ok &= fx_leaf_node<E, Q, 1>(m, p, s, acc);
+    } else {
+      const uint32_t* m = fx_node<32, L>(nodes, lvl_off, t, v, chunk, p);
+      ok &= fx_leaf_node<E, Q, 32>(m, p, s, acc);
+    }
+    mag = mag + ((acc.ip + acc.in) + (acc.ep + acc.en));
+    S di = acc.ip - acc.in, de = acc.ep - acc.en;
+    // sign of the node: (-1)^(exclusions above)
+    const uint32_t odd = ((t.D - __popc(v) - __popc(chunk)) & 1) ? 0xffffffffu : 0u;
+    inc = inc + fx_flip(di, odd);
+    exc = exc + fx_flip(de, odd);
+  }
+  if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
+  __syncwarp();
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    inc = inc + shfl_down(inc, off);
+    exc = exc + shfl_down(exc, off);
+    mag = mag + shfl_down(mag, off);
+  }
+  if (lane == 0) parts[unit] = FxPart<S>{inc, exc, mag};
+}
+
+// -------------------------------------------------------------------- final --
+// One CTA per tree; segs[t].first = the tree's first unit, segs[t + 1].first the end.
+template <class S>
+__global__ void __launch_bounds__(256) fx_final_kernel(const FxPart<S>* __restrict__ parts,
+                                                       const FxSeg* __restrict__ segs,
+                                                       const FxTree* __restrict__ trees, TreeOut* __restrict__ outs) {
+  const int t = blockIdx.x;
+  const S zero = fx_of<S>(0.0);
+  S inc = zero, exc = zero, mag = zero;
+  for (long long i = segs[t].first + threadIdx.x; i < segs[t + 1].first; i += blockDim.x) {
+    inc = inc + parts[i].inc;
+    exc = exc + parts[i].exc;
+    mag = mag + parts[i].abs;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    inc = inc + shfl_down(inc, off);
+    exc = exc + shfl_down(exc, off);
+    mag = mag + shfl_down(mag, off);
+  }
+  __shared__ FxPart<S> sh[8];
+  if (lane == 0) sh[warp] = FxPart<S>{inc, exc, mag};
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const int nw = blockDim.x >> 5;
+  for (int w = 1; w < nw; ++w) {
+    inc = inc + sh[w].inc;
+    exc = exc + sh[w].exc;
+    mag = mag + sh[w].abs;
+  }
+  TreeOut* o = outs + trees[segs[t].idx].tree;
+  fx_store3(inc, o->inc);
+  fx_store3(exc, o->exc);
+  o->abs = to_double(mag);
+}
+
+}  // namespace gbs

@@ -1,0 +1,229 @@
+// Host side of the fixed-point tree engine: plan, workspace, launches.
+#pragma once
+#include <algorithm>
+#include <string>
+#include <vector>
+
+#include "gbs_batch_driver.cuh"
+#include "gbs_fxtree.cuh"
+
+namespace gbs {
+
+// Words of the matrices of level k of a tree over n modes (k = -1: the root), `count`
+// matrices of it at a time.
+inline long long fx_level_words(int n, int k, long long count, int L) {
+  const int q = k < 0 ? n : n - 1 - k;
+  if (k >= 5) count = (count + 31) / 32 * 32;
+  return count * (long long)sym(2 * q) * L;
+}
+
+template <class E>
+gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const void* roots_dev, TreeOut* outs_dev,
+                        int* status_dev, const BatchTune& tune) {
+  typedef typename fx_sum<E>::type S;
+  constexpr int L = sizeof(E) / 4;
+  if (ntrees <= 0) return GBS_OK;
+  // ---------------- plan
+  // Largest tree first: every per-size list below is then a run of trees.
+  std::vector<int> order(ntrees);
+  for (int i = 0; i < ntrees; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return in[a].n > in[b].n; });
+  for (int i = 0; i < ntrees; ++i)
+    if (in[i].n < 1 || in[i].n > 32) return set_error(ctx, GBS_EINVAL, "batch tree size out of range");
+  // Levels per leaf thread.
+  const int Qmax = std::max(1, std::min(2, 3 - tune.q_drop));
+  const int nmax = in[order[0]].n;
+  // Depth of the top kernel: at most tune.d_top and about 1024 CTAs, at least the five
+  // levels that are not kept in tiles, and enough that a level's rows fit shared memory.
+  constexpr int kSmemMax = 220 * 1024;
+  constexpr int kRowBytes = 6 * L * 32 * 4, kPivBytes = (5 * L + 1) * 32 * 4;
+  const int q_fit = (kSmemMax - kPivBytes) / kRowBytes / 2;
+  int d_top = 5;
+  while (d_top < tune.d_top && ((long long)ntrees << (d_top + 1)) <= 1024) ++d_top;
+  d_top = std::max(d_top, nmax - 1 - q_fit);
+  std::vector<FxTree> trees(ntrees);
+  std::vector<int> Q(ntrees);
+  for (int i = 0; i < ntrees; ++i) {
+    const BatchTree& b = in[order[i]];
+    Q[i] = std::min(b.n, Qmax);
+    trees[i] = FxTree{b.root_off, 0, b.n, b.n - Q[i], order[i], 34 * i, 0, 0};
+  }
+  const int D0 = trees[0].D;
+  // A single tree too large for the workspace goes in chunks of 2^cb nodes of depth d0
+  // (FxTree): the deepest split with the fewest chunks that fits.
+  const size_t cap = ctx->batch_cap_bytes ? ctx->batch_cap_bytes : (size_t)64 << 30;
+  auto tree_bytes = [&](int i, int d0, int cb) {
+    const int n = trees[i].n, D = trees[i].D;
+    long long words = fx_level_words(n, -1, 1, L), sv = 1LL << d0;
+    for (int k = 0; k < D; ++k) words += fx_level_words(n, k, k < d0 ? 1LL << k : 1LL << (k - d0 + cb), L);
+    sv += (1LL << (D - d0 + cb)) - (1LL << cb);
+    return (size_t)words * 4 + (size_t)sv * sizeof(S);
+  };
+  size_t need = 0;
+  for (int i = 0; i < ntrees; ++i) need += tree_bytes(i, 0, 0);
+  int d0 = 0, cb = 0;
+  if (need > cap) {
+    if (ntrees > 1) {
+      ctx->batch_split = true;  // the caller evaluates the batch in parts
+      return GBS_ENOMEM;
+    }
+    size_t best = ~(size_t)0;
+    for (int chunk_bits = 1; chunk_bits <= D0 - 5 && best > cap; ++chunk_bits)  // log2 of the number of chunks
+      for (int d = std::max(5 + chunk_bits, std::min(d_top, D0)); d < D0; ++d) {
+        const size_t b = tree_bytes(0, d, d - chunk_bits);
+        if (b < best) best = b, d0 = d, cb = d - chunk_bits;
+      }
+    if (best == ~(size_t)0) d0 = cb = 0;
+  }
+  std::vector<long long> off(34 * (size_t)ntrees, 0);
+  long long words = 0, selems = 0;
+  for (int i = 0; i < ntrees; ++i) {
+    const int n = trees[i].n, D = trees[i].D;
+    long long* o = &off[34 * (size_t)i];
+    o[0] = words;
+    words += (fx_level_words(n, -1, 1, L) + 31) / 32 * 32;
+    for (int k = 0; k < D; ++k) {
+      o[k + 1] = words;
+      words += (fx_level_words(n, k, k < d0 || d0 == 0 ? 1LL << k : 1LL << (k - d0 + cb), L) + 31) / 32 * 32;
+    }
+    trees[i].s_base = selems;
+    selems += d0 ? (1LL << d0) + (1LL << (D - d0 + cb)) - (1LL << cb) : 1LL << D;
+  }
+  const int chunks = d0 ? 1 << (d0 - cb) : 1;
+  std::vector<FxTree> chunked = trees;
+  for (FxTree& t : chunked) t.d0 = d0, t.cb = cb;
+  // top: the levels below min(D, d_top)
+  std::vector<FxSeg> top(ntrees);
+  long long top_blocks = 0;
+  auto dtop_of = [&](int i) { return std::min(trees[i].D, d_top); };
+  for (int i = 0; i < ntrees; ++i) {
+    top[i] = FxSeg{top_blocks, i, 0};
+    top_blocks += 1LL << dtop_of(i);
+  }
+  // levels, by child size q downwards
+  struct Launch {
+    int q, W;
+    std::vector<FxSeg> segs;
+    long long tiles;
+    size_t at;
+    bool in_chunk;
+  };
+  std::vector<Launch> levels;
+  for (int q = nmax - 1; q >= 1; --q) {
+    Launch l{q, 1, {}, 0, 0, false};
+    for (int i = 0; i < ntrees; ++i) {
+      const int k = trees[i].n - 1 - q;
+      if (k < dtop_of(i) || k >= trees[i].D) continue;
+      l.in_chunk = d0 > 0 && k >= d0;
+      l.segs.push_back(FxSeg{l.tiles, i, 0});
+      l.tiles += 1LL << ((l.in_chunk ? k - d0 + cb : k) - 5);
+    }
+    if (l.segs.empty()) continue;
+    // Warps per tile: enough tiles fit an SM's shared memory for ~16 warps, and few
+    // tiles are spread over more warps.
+    const int R = 2 * q;
+    l.W = R >= 16 ? 8 : R >= 10 ? 4 : R >= 6 ? 2 : 1;
+    while (l.W < 8 && l.tiles * l.W < 16LL * ctx->sm_count) l.W *= 2;
+    levels.push_back(l);
+  }
+  // leaves, one launch per Q
+  struct Leaf {
+    int Q;
+    std::vector<FxSeg> segs;
+    long long units;
+    size_t at;
+  };
+  std::vector<Leaf> leaves;
+  std::vector<FxSeg> fin;
+  long long tiles_total = 0, units_total = 0;
+  for (int i = 0; i < ntrees; ++i) tiles_total += ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
+  const int tpu = (int)std::max(1LL, std::min(32LL, tiles_total / (64LL * ctx->sm_count)));
+  for (int i = 0; i < ntrees; ++i) {
+    if (leaves.empty() || leaves.back().Q != Q[i]) leaves.push_back(Leaf{Q[i], {}, 0, 0});
+    Leaf& lf = leaves.back();
+    const long long tiles = ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
+    const long long units = (tiles + tpu - 1) / tpu;
+    lf.segs.push_back(FxSeg{lf.units, i, tpu});
+    lf.units += units;
+    fin.push_back(FxSeg{units_total, i, 0});
+    units_total += units * chunks;
+  }
+  fin.push_back(FxSeg{units_total, 0, 0});
+  // ---------------- memory
+  const size_t part_bytes = (size_t)units_total * sizeof(FxPart<S>);
+  if (ntrees > 1 && need + part_bytes > cap) {
+    ctx->batch_split = true;
+    return GBS_ENOMEM;
+  }
+  gbs_status st;
+  if ((st = dev_reserve(ctx, ctx->lvl[0], (size_t)words * 4)) ||
+      (st = dev_reserve(ctx, ctx->sbuf[0], (size_t)selems * sizeof(S))) ||
+      (st = dev_reserve(ctx, ctx->partials, part_bytes)))
+    return st;
+  Blob blob;
+  const size_t o_trees = blob.put(trees), o_chunked = blob.put(chunked), o_off = blob.put(off), o_top = blob.put(top);
+  for (Launch& l : levels) l.at = blob.put(l.segs);
+  for (Leaf& l : leaves) l.at = blob.put(l.segs);
+  const size_t o_fin = blob.put(fin);
+  const unsigned char* plan = nullptr;
+  if ((st = stage(ctx, blob.bytes.data(), blob.bytes.size(), (const void**)&plan))) return st;
+  uint32_t* nodes = (uint32_t*)ctx->lvl[0].ptr;
+  S* sval = (S*)ctx->sbuf[0].ptr;
+  FxPart<S>* parts = (FxPart<S>*)ctx->partials.ptr;
+  const FxTree* d_trees = (const FxTree*)(plan + o_trees);
+  const FxTree* d_chunked = (const FxTree*)(plan + o_chunked);
+  const long long* d_off = (const long long*)(plan + o_off);
+  cudaStream_t s = ctx->stream;
+
+  // ---------------- launches
+  const int smem_top = sym(2 * nmax) * (int)sizeof(E) + 2 * nmax * (int)sizeof(FxRow<E>);
+  if ((st = check_cuda(ctx, cudaFuncSetAttribute(fx_top_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_top),
+                       "top smem")) ||
+      (st = check_cuda(ctx, cudaFuncSetAttribute(fx_level_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax),
+                       "level smem")))
+    return st;
+  fx_top_kernel<E><<<(unsigned)top_blocks, 256, smem_top, s>>>((const FxSeg*)(plan + o_top), ntrees, d_trees, d_off,
+                                                               (const double*)roots_dev, nodes, sval, status_dev);
+  count_launch(ctx);
+  auto level = [&](const Launch& l, unsigned chunk) {
+    fx_level_kernel<E><<<(unsigned)l.tiles, 32 * l.W, kPivBytes + 2 * l.q * kRowBytes, s>>>(
+        (const FxSeg*)(plan + l.at), (int)l.segs.size(), l.in_chunk ? d_chunked : d_trees, d_off, l.q, chunk, nodes, sval,
+        status_dev);
+    count_launch(ctx);
+  };
+  for (const Launch& l : levels)
+    if (!l.in_chunk) level(l, 0u);
+  if (ctx->timing) {
+    if (!ctx->leaf_timer.start) {
+      cudaEventCreate(&ctx->leaf_timer.start);
+      cudaEventCreate(&ctx->leaf_timer.stop);
+    }
+    cudaEventRecord(ctx->leaf_timer.start, s);
+  }
+  for (int h = 0; h < chunks; ++h) {
+    for (const Launch& l : levels)
+      if (l.in_chunk) level(l, (unsigned)h);
+    long long base = h * leaves[0].units;  // chunks: one tree, one leaf launch each
+    for (const Leaf& l : leaves) {
+      const unsigned grid = (unsigned)((l.units + 3) / 4);
+      const FxSeg* sg = (const FxSeg*)(plan + l.at);
+      const int ns = (int)l.segs.size();
+      switch (l.Q) {
+        case 1: fx_leaf_kernel<E, 1><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        case 2: fx_leaf_kernel<E, 2><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        default: fx_leaf_kernel<E, 3><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+      }
+      count_launch(ctx);
+      base += l.units;
+    }
+  }
+  if (ctx->timing) {
+    cudaEventRecord(ctx->leaf_timer.stop, s);
+    ctx->leaf_timer.pending = true;
+  }
+  fx_final_kernel<S><<<(unsigned)ntrees, 256, 0, s>>>(parts, (const FxSeg*)(plan + o_fin), d_trees, outs_dev);
+  count_launch(ctx);
+  return check_cuda(ctx, cudaGetLastError(), "fixed-point batch launch");
+}
+
+}  // namespace gbs

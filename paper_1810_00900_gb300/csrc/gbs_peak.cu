@@ -37,7 +37,7 @@ __global__ void fx_product_chain_kernel(uint32_t* out, int iters, uint32_t seed)
     }
   for (int it = 0; it < iters; ++it) {
 #pragma unroll
-    for (int i = 0; i < ILP; ++i) x[i] = x[i] * y[i];
+    for (int i = 0; i < ILP; ++i) x[i] = umul(x[i], y[i]);
   }
   uint32_t acc = 0u;
 #pragma unroll

@@ -59,25 +59,6 @@ GBS_HD cplx<dd> scale_<cplx<dd>, dd>(const cplx<dd>& x, const dd& s) { return {x
 template <>
 GBS_HD cplx<td> scale_<cplx<td>, td>(const cplx<td>& x, const td& s) { return {x.re * s, x.im * s}; }
 
-// Type of the running product s of pivot factors: the entry scalar type,
-// except for the fixed-point entries, whose s needs a wider integer part.
-template <class E> struct scale_of { typedef typename real_of<E>::type type; };
-
-// Minimum resident CTAs per SM the compiler keeps registers for in the
-// breadth-first level kernel: the fixed-point levels wait on global loads with
-// too few warps otherwise.
-template <class E> struct level_min_blocks { static const int value = 1; };
-// Level kernel: keep the scaled pivot inverse and g in shared memory while the
-// rows are formed (the fixed-point entry types, whose registers would otherwise
-// spill).
-template <class E> struct level_park { static const bool value = false; };
-// The same for the register-subtree leaf kernel (128-thread CTAs).
-template <class E> struct leaf_min_blocks { static const int value = 1; };
-
-// 32-bit words of a multiword entry stored limb by limb in the global node
-// buffers of the batched engine (0: the entry is stored whole).
-template <class E> struct node_words { static const int value = 0; };
-
 // ------------------------------------------------ accumulation types -----
 // Per-thread accumulators (Acc) and cross-thread reduction values (Red).
 template <class T> struct acc_traits;
@@ -104,28 +85,20 @@ template <class Acc>
 struct Sums {
   Acc ip, in, ep, en;
 };
-// Sum of |terms| of a thread's sign-split sums as a double (specialised where the
-// sums are exact integers: add first, convert once).
+// Sum of |terms| of a thread's sign-split sums as a double.
 template <class Acc>
-struct sums_total {
-  static GBS_HD double of(const Sums<Acc>& a) {
-    return to_double(a.ip) + to_double(a.in) + (to_double(a.ep) + to_double(a.en));
-  }
-};
+GBS_HD double sums_total(const Sums<Acc>& a) {
+  return to_double(a.ip) + to_double(a.in) + (to_double(a.ep) + to_double(a.en));
+}
 template <class Acc>
 GBS_HD Sums<Acc> sums_zero() {
   const Acc z = from_double<Acc>(0.0);
   return Sums<Acc>{z, z, z, z};
 }
 
-// A pivot determinant that is not positive: the floating types need no test
-// on the hot path (the inverse square root of a value <= 0 is NaN or inf and
-// reaches the sums, which are checked once per thread).
-GBS_HD bool not_positive(double) { return false; }
-GBS_HD bool not_positive(float) { return false; }
-GBS_HD bool not_positive(const dd&) { return false; }
-GBS_HD bool not_positive(const td&) { return false; }
-
+// A pivot determinant that is not positive needs no test on the hot path: the
+// inverse square root of a value <= 0 is NaN or inf and reaches the sums, which
+// are checked once per thread.
 GBS_HD dd red_add(const dd& a, const dd& b) { return a + b; }
 GBS_HD td red_add(const td& a, const td& b) { return a + b; }
 GBS_HD dd red_neg(const dd& a) { return -a; }
@@ -161,7 +134,6 @@ struct TreeOut {
 // kStatusRange: a fixed-point tree met a value outside the range it can carry
 // (the caller redoes the tree in floating point).
 enum : int { kStatusOk = 0, kStatusNotPD = 3, kStatusRange = 5 };
-template <class T> constexpr int bad_status() { return kStatusNotPD; }
 
 GBS_HD bool is_pos(double x) { return x > 0.0; }
 GBS_HD bool is_pos(float x) { return x > 0.0f; }
@@ -179,11 +151,10 @@ GBS_HD bool lead_pos(const td& x) { return x.x0 > 0.0; }
 // Children: 2*count nodes with q-1 modes; child 2i excludes the first mode of
 // node i, child 2i+1 includes it.
 template <class E>
-__global__ void tree_level_kernel(const E* __restrict__ par, const typename scale_of<E>::type* __restrict__ spar,
+__global__ void tree_level_kernel(const E* __restrict__ par, const typename real_of<E>::type* __restrict__ spar,
                                   long long count, int q, E* __restrict__ chi,
-                                  typename scale_of<E>::type* __restrict__ schi, int* __restrict__ status) {
+                                  typename real_of<E>::type* __restrict__ schi, int* __restrict__ status) {
   typedef typename real_of<E>::type T;
-  typedef typename scale_of<E>::type S;
   const int rows = 2 * q - 2;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= count * rows) return;
@@ -221,7 +192,7 @@ __global__ void tree_level_kernel(const E* __restrict__ par, const typename scal
     chi[(long long)tri(a, a) * c2 + 2 * node + 1] = v;
   }
   if (a == 0) {
-    const S s = spar[node];
+    const T s = spar[node];
     schi[2 * node] = s;
     schi[2 * node + 1] = s * g;
   }
@@ -311,8 +282,7 @@ template <class E, int Q, int D, int OFF, bool NEG, bool PAIR = false>
 struct Dfs {
   typedef typename real_of<E>::type T;
   typedef typename acc_traits<T>::Acc Acc;
-  typedef typename scale_of<E>::type S;
-  static __device__ __forceinline__ void run(const E (&c)[sym(D)], const S& s, Sums<Acc>& acc, bool& bad) {
+  static __device__ __forceinline__ void run(const E (&c)[sym(D)], const T& s, Sums<Acc>& acc) {
     if constexpr (PAIR && Q <= 2) {
       static_assert(std::is_same<E, double>::value, "the paired last levels are FP64 real-basis only");
       if constexpr (Q == 2) pair_group<D, OFF, NEG>(c, s, acc); else pair_single<D, OFF, NEG>(c, s, acc);
@@ -351,15 +321,14 @@ struct Dfs {
 #pragma unroll
           for (int b = 0; b <= a; ++b)
             cn[tri(a, b)] = fma(-w1[a], w1[b], fma(-w0[a], w0[b], c[tri(OFF + 2 + a, OFF + 2 + b)]));
-        Dfs<E, Q - 1, DN, 0, NEG, PAIR>::run(cn, s * g, acc, bad);
-        Dfs<E, Q - 1, D, OFF + 2, !NEG, PAIR>::run(c, s, acc, bad);
+        Dfs<E, Q - 1, DN, 0, NEG, PAIR>::run(cn, s * g, acc);
+        Dfs<E, Q - 1, D, OFF + 2, !NEG, PAIR>::run(c, s, acc);
       }
     } else {
     const T p00 = re_of(c[tri(OFF, OFF)]);
     const T p11 = re_of(c[tri(OFF + 1, OFF + 1)]);
     const E p10 = c[tri(OFF + 1, OFF)];
     const T det = p00 * p11 - norm2(p10);
-    bad |= not_positive(det);
     const T g = rsqrt_(det);
     if constexpr (Q == 1) {
       // include leaf s*g with sign (-1)^NEG; exclude leaf s with one more exclusion
@@ -383,8 +352,8 @@ struct Dfs {
         E v = fms_conj_re(c[tri(OFF + 2 + a, OFF + 2 + a)], L0, u0);
         cn[tri(a, a)] = fms_conj_re(v, L1, u1);
       }
-      Dfs<E, Q - 1, DN, 0, NEG, PAIR>::run(cn, s * g, acc, bad);
-      Dfs<E, Q - 1, D, OFF + 2, !NEG, PAIR>::run(c, s, acc, bad);
+      Dfs<E, Q - 1, DN, 0, NEG, PAIR>::run(cn, s * g, acc);
+      Dfs<E, Q - 1, D, OFF + 2, !NEG, PAIR>::run(c, s, acc);
     }
     }
   }
@@ -392,7 +361,7 @@ struct Dfs {
 
 // Register subtree of one node (all Q levels below it): the node's signed sums
 // as reduction values and its absolute sum; returns false if a pivot was not
-// positive definite (the sums then carry NaN or inf, or the type flagged it).
+// positive definite (the sums then carry NaN or inf).
 GBS_HD dd red_diff(double a, double b, dd*) {
   dd r;
   two_sum(a, -b, r.hi, r.lo);
@@ -404,12 +373,11 @@ GBS_HD td red_diff(const td& a, const td& b, td*) { return a - b; }
 // PAIR: inc receives the node's Torontonian (every group's v), exc zero, and
 // asum the sum of the group magnitudes.
 template <class E, int Q, bool PAIR = false, class Red>
-__device__ __forceinline__ bool subtree_sums(const E (&c)[sym(2 * Q)], const typename scale_of<E>::type& s, Red& inc,
+__device__ __forceinline__ bool subtree_sums(const E (&c)[sym(2 * Q)], const typename real_of<E>::type& s, Red& inc,
                                              Red& exc, double& asum) {
   typedef typename acc_traits<typename real_of<E>::type>::Acc Acc;
   Sums<Acc> a = sums_zero<Acc>();
-  bool bad = false;
-  Dfs<E, Q, 2 * Q, 0, false, PAIR>::run(c, s, a, bad);
+  Dfs<E, Q, 2 * Q, 0, false, PAIR>::run(c, s, a);
   if constexpr (PAIR) {
     inc = red_diff(a.ip, a.in, (Red*)nullptr);
     exc = red_zero<Red>();
@@ -418,19 +386,9 @@ __device__ __forceinline__ bool subtree_sums(const E (&c)[sym(2 * Q)], const typ
   } else {
     inc = red_diff(a.ip, a.in, (Red*)nullptr);
     exc = red_diff(a.ep, a.en, (Red*)nullptr);
-    asum = sums_total<Acc>::of(a);
-    return !bad && isfinite(asum);
+    asum = sums_total(a);
+    return isfinite(asum);
   }
-}
-
-// Register subtree of one node into per-thread sign-split sums (added to acc);
-// false if a pivot was not positive definite.
-template <class E, int Q, bool PAIR = false>
-__device__ __forceinline__ bool subtree_run(const E (&c)[sym(2 * Q)], const typename scale_of<E>::type& s,
-                                            Sums<typename acc_traits<typename real_of<E>::type>::Acc>& a) {
-  bool bad = false;
-  Dfs<E, Q, 2 * Q, 0, false, PAIR>::run(c, s, a, bad);
-  return !bad;
 }
 
 // Block reduction of per-thread FP64 sign-split sums (ip, in, ep, en) into one
@@ -493,7 +451,7 @@ __device__ __forceinline__ void block_reduce_store(Red inc, Red exc, double asum
 // One thread per node with Q undecided modes; depth = n - Q levels above.
 template <class E, int Q>
 __global__ void __launch_bounds__(128) tree_leaf_kernel(const E* __restrict__ nodes,
-                                                        const typename scale_of<E>::type* __restrict__ snode,
+                                                        const typename real_of<E>::type* __restrict__ snode,
                                                         long long count, int depth,
                                                         Partial<typename acc_traits<typename real_of<E>::type>::Red>* partials,
                                                         int* __restrict__ status) {
@@ -507,7 +465,7 @@ __global__ void __launch_bounds__(128) tree_leaf_kernel(const E* __restrict__ no
     E c[sym(2 * Q)];
 #pragma unroll
     for (int e = 0; e < sym(2 * Q); ++e) c[e] = nodes[(long long)e * count + node];
-    const typename scale_of<E>::type s = snode[node];
+    const typename real_of<E>::type s = snode[node];
     if (!subtree_sums<E, Q>(c, s, inc, exc, asum)) atomicExch(status, (int)kStatusNotPD);
     // sign of the node: (-1)^(exclusions above) = (-1)^(depth - popcount(node))
     if ((depth - __popcll((unsigned long long)node)) & 1) { inc = red_neg(inc); exc = red_neg(exc); }

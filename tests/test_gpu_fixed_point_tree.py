@@ -1,0 +1,73 @@
+"""The fixed-point tree engine where its index arithmetic can go wrong: trees smaller than a tile
+of 32 nodes, one level and one tile more, every depth of the top kernel, batches of uneven trees,
+and a tree taken in chunks because its levels exceed the context's budget.  Sums are exact, so
+every launch shape and split gives the same bits."""
+import numpy as np
+import pytest
+
+import gbs_inputs as gi
+import oracle
+import paper_1810_00900_gb300 as gbs
+from helpers import frac3, oracle_tor, real_basis_block
+
+pytestmark = pytest.mark.gpu
+
+# model units of tests/test_gpu_tree.py: |Tor - exact| <= 8 n u sum|terms|
+U_OF = {"fxn": 2.0 ** -108, "fx": 2.0 ** -140, "fxw": 2.0 ** -158}
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1810_00900_gb300 import build
+    build.build()
+    c = gbs.Context(0)
+    yield c
+    c.close()
+
+
+def block(n, seed, r=0.7, eta=0.8):
+    st = gi.uniform_squeezed_state(80, r, seed=seed, eta=eta)
+    Sig = oracle.sigma(oracle.covariance(st.U, st.r, st.eta))
+    return real_basis_block(oracle.sigma_inv_block(Sig, gi.random_modes(80, n, seed=seed)))
+
+
+@pytest.mark.parametrize("prec", ["fxn", "fx", "fxw"])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 7, 8, 9, 10, 12])
+def test_shapes_give_the_oracles_value_and_the_same_bits(ctx, prec, n):
+    G = block(n, 40 + n)
+    ref, ref_abs = oracle_tor(G)
+    seen = set()
+    for d_top in (0, 6, 7, 10):
+        for q_drop in (0, 1, 2):
+            ctx.set_tuning(prec, "real", 6, d_top, 0, 1 << 18, q_drop, 0)
+            inc, exc, tor, a = gbs.subset_sum(ctx, G, "real", prec)
+            seen.add((tuple(inc), tuple(exc), tuple(tor), a))
+            assert abs(float(frac3(tor) - ref.to_fraction())) <= 8 * n * U_OF[prec] * ref_abs
+            assert abs(a - ref_abs) <= 1e-12 * ref_abs
+    ctx.set_tuning(prec, "real", 6, 10, 0, 1 << 18, 0, 0)
+    assert len(seen) == 1
+
+
+def test_uneven_batch_gives_each_trees_own_bits(ctx):
+    st_p = gi.uniform_squeezed_state(60, 0.7, seed=3, eta=0.7)
+    st = gbs.build_state(ctx, st_p.U, st_p.r, st_p.eta)
+    pats = [gi.random_modes(60, n, seed=100 + i) for i, n in enumerate([9, 1, 14, 2, 8, 3, 11, 9, 1, 16, 5, 7])]
+    alone = [gbs.torontonian(ctx, st, p, "fx") for p in pats]
+    for p, a, b in zip(pats, alone, gbs.torontonian_batch(ctx, [st] * len(pats), pats, "fx")):
+        assert a.tor == b.tor and a.abs_sum == b.abs_sum, len(p)
+    st.free()
+
+
+@pytest.mark.parametrize("prec", ["fxn", "fx", "fxw"])
+def test_chunks_of_a_tree_beyond_the_budget(ctx, prec):
+    # 16 modes need ~10 MB of levels at once; half of a budget of 6 and 10 MB makes chunks
+    G = block(16, 77)
+    want = gbs.subset_sum(ctx, G, "real", prec)
+    for budget in (6 << 20, 10 << 20):
+        for d_top in (6, 10):
+            c = gbs.Context(0, hbm_budget_bytes=budget)
+            c.set_tuning(prec, "real", 6, d_top, 0, 1 << 18, 0, 0)
+            got = gbs.subset_sum(c, G, "real", prec)
+            assert all(tuple(np.atleast_1d(x)) == tuple(np.atleast_1d(y)) for x, y in zip(want, got))
+            assert c.launch_count > 15 and c.bytes_in_use <= budget
+            c.close()
