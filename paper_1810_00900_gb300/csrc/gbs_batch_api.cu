@@ -154,11 +154,13 @@ __global__ void batch_click_block_kernel(const ClickReq* __restrict__ reqs, int 
 // block has g = 1 or is not positive definite).
 __global__ void kappa_estimate_kernel(const BatchTree* __restrict__ trees, int ntrees, const void* __restrict__ roots,
                                       int real_basis, double* __restrict__ log10_kappa) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  // a warp per tree, a lane per mode: the logarithms (FP64, ~1 us each) side by side
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (t >= ntrees) return;
   const BatchTree tr = trees[t];
   double lk = 0.0;
-  for (int j = 0; j < tr.n; ++j) {
+  for (int j = lane; j < tr.n; j += 32) {
     const long long a = (long long)(2 * j) * (2 * j + 1) / 2 + 2 * j;        // tri(2j, 2j)
     const long long b = (long long)(2 * j + 1) * (2 * j + 2) / 2 + 2 * j;    // tri(2j+1, 2j)
     double det;
@@ -172,7 +174,9 @@ __global__ void kappa_estimate_kernel(const BatchTree* __restrict__ trees, int n
     const double g = det > 0.0 ? rsqrt(det) : 0.0;
     lk += det > 0.0 && g != 1.0 ? log10((g + 1.0) / fabs(g - 1.0)) : INFINITY;
   }
-  log10_kappa[t] = lk;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) lk += __shfl_down_sync(0xffffffffu, lk, off);
+  if (lane == 0) log10_kappa[t] = lk;
 }
 
 __global__ void batch_finish_kernel(const TreeOut* __restrict__ outs, const int* __restrict__ status,
@@ -401,7 +405,7 @@ gbs_status probs_batch(gbs_ctx* ctx, int nreq, const gbs_state* const* states, c
     if ((st = stage(ctx, tt.data(), tt.size() * sizeof(BatchTree), &d_tt)) ||
         (st = stage(ctx, est.data(), est.size() * sizeof(double), &d_est)))
       return st;
-    kappa_estimate_kernel<<<(unsigned)((todo.size() + 127) / 128), 128, 0, ctx->stream>>>(
+    kappa_estimate_kernel<<<(unsigned)((todo.size() + 3) / 4), 128, 0, ctx->stream>>>(
         (const BatchTree*)d_tt, (int)todo.size(), ctx->hbuf.ptr, real ? 1 : 0, (double*)d_est);
     count_launch(ctx);
     if ((st = check_cuda(ctx, cudaMemcpyAsync(est.data(), d_est, est.size() * sizeof(double), cudaMemcpyDeviceToHost,

@@ -17,15 +17,15 @@
 //   top kernel    one CTA per node v < 2^dtop: eliminates the modes of v from the
 //                 root in shared memory and writes that matrix; replaces the
 //                 first levels, where nodes are few.
-//   level kernel  one launch per child size q: a CTA of W warps takes 32
-//                 consecutive children of one tree (lane = child).
+//   level kernels one launch per child size q: a warp per 32 consecutive children of a
+//                 tree (lane = child), or, where children are few, a CTA per 1 .. 32.
 //   leaf kernel   a warp takes tiles of 32 nodes of one tree, one thread per node
 //                 for all 2^Q subsets of its last Q modes.
 //   final kernel  one CTA per tree adds the warps' sums.
 // Measured against the engine it replaced (both children stored, subtrees of 9
 // modes expanded in shared memory, signed products, 2 products per entry), with the
-// default launch shapes: N = 24 (M = 200, AUTO) 8.86 -> 3.32 ms, 256 requests of N =
-// 8 .. 20 23.1 -> 9.2 ms.
+// default launch shapes: N = 24 (M = 200, AUTO) 8.86 -> 2.4 ms, 256 requests of N =
+// 8 .. 20 23.0 -> 6.9 ms.
 // All sums are exact integers, and every pivot, row and entry is formed by the
 // same functions below wherever it is formed: results do not depend on the launch
 // shape or on the rest of the batch, bit for bit.
@@ -114,7 +114,7 @@ template <class E>
 __device__ __forceinline__ E fx_det(const E& p00, const E& p10, const E& p11) {
   uint32_t neg;
   const E n10 = fx_abs(p10, neg);
-  return umul(p00, p11) - umul(n10, n10);
+  return umul(p00, p11) - usqr(n10);
 }
 
 // Returns whether the determinant is in range.
@@ -126,9 +126,9 @@ __device__ __forceinline__ bool fx_pivot(const E& p00, const E& p10, const E& p1
 #pragma unroll
   for (int k = 0; k < (int)(sizeof(E) / 4); ++k) zero &= p10.w[k] == 0u;
   pv.flip = (neg == 0u && !zero) ? 0xffffffffu : 0u;  // p10 > 0
-  const E det = umul(p00, p11) - umul(n10, n10);
+  const E det = umul(p00, p11) - usqr(n10);
   pv.g = rsqrt_(det);
-  const E inv = umul(pv.g, pv.g);
+  const E inv = usqr(pv.g);
   pv.m = umul(n10, inv);
   pv.a = umul(p11, inv) + pv.m;
   pv.b = umul(p00, inv) + pv.m;
@@ -301,15 +301,22 @@ __global__ void __launch_bounds__(256) fx_top_kernel(const FxSeg* __restrict__ s
 }
 
 // -------------------------------------------------------------------- level --
-// Children of q = R / 2 modes, one CTA of W warps per tile of 32.  One warp forms
-// the 32 pivots (a chain: the other warps' CTAs hide it), then the rows and then
-// the entries are shared out among the warps; rows wait in shared memory.
-template <class E, int ST>
-__device__ __forceinline__ void fx_level_tile(const FxTree& t, const long long* lvl_off, int q, unsigned tile,
-                                              unsigned chunk, uint32_t* nodes, typename fx_sum<E>::type* sval, int* status,
-                                              uint32_t* sh) {
+// Children of level k with q = R / 2 modes, when there are many: one warp per tile of
+// 32, lane = child, no barrier.  Row a's P, Q, A are used at once, for entries (a, 0)
+// .. (a, a); its U, V, B wait in shared memory for the rows below (2304 R bytes a warp
+// with 6 limbs: 24 / 16 / 12 / 9 warps per SM at R = 4 / 6 / 8 / 10).  Bound by the
+// multiply pipe at R = 4, 6 (70, 64 %, 4.4 TB/s beside it) and, with fewer warps, by
+// the latency of its chains: NB entries at a time (FX, N = 24, q = 5, 4: 244, 278 us
+// with 2, 213, 248 with 4, where 164 registers no longer cost warps; q = 3, 2: 312,
+// 370 with 2, 328, 402 with 4), the next row's head loaded while this one is formed.
+// Four warps sharing rows and entries behind barriers ran 683 us at q = 2 and 440 at q
+// = 4 (one at a time: 371, 248).
+template <class E, int ST, int NB>
+__device__ __forceinline__ void fx_level_warp(const FxTree& t, const long long* lvl_off, int q, unsigned tile,
+                                              unsigned chunk, uint32_t* nodes, typename fx_sum<E>::type* sval,
+                                              int* status, uint32_t* sh) {
   constexpr int L = sizeof(E) / 4;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31;
   const int R = 2 * q;
   const int k = t.n - 1 - q;
   const unsigned c = tile * 32u + lane;  // child of level k = parent node
@@ -317,126 +324,246 @@ __device__ __forceinline__ void fx_level_tile(const FxTree& t, const long long* 
   const uint32_t* par = fx_node<ST, L>(nodes, lvl_off, t, c, chunk, p);
   const int o = 2 * (p - q - 1);  // the pivot's first row in the parent
   uint32_t* out = nodes + lvl_off[t.tab + k + 1] + (long long)tile * sym(R) * (L * 32) + lane;
-  uint32_t* piv = sh + lane;                    // 5 values and the flip of a pivot
-  uint32_t* rowp = sh + (5 * L + 1) * 32 + lane;  // 6 values per row
-  if (warp == 0) {
-    FxPivot<E> pv;
-    const bool ok = fx_pivot(fx_ld<E, ST>(par, tri(o, o)), fx_ld<E, ST>(par, tri(o + 1, o)),
-                             fx_ld<E, ST>(par, tri(o + 1, o + 1)), pv);
-    if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
-    sval[fx_sidx(t, (1u << (k - t.d0 + t.cb)) + c, chunk)] = umul(sval[fx_sidx(t, c, chunk)], pv.g);
-    fx_st<E, 32>(piv, 0, pv.a);
-    fx_st<E, 32>(piv, 1, pv.b);
-    fx_st<E, 32>(piv, 2, pv.m);
-    fx_st<E, 32>(piv, 3, pv.c0);
-    fx_st<E, 32>(piv, 4, pv.c1);
-    piv[5 * L * 32] = pv.flip;
-  }
-  __syncthreads();
-  {
-    FxPivot<E> pv;
-    pv.a = fx_ld<E, 32>(piv, 0);
-    pv.b = fx_ld<E, 32>(piv, 1);
-    pv.m = fx_ld<E, 32>(piv, 2);
-    pv.c0 = fx_ld<E, 32>(piv, 3);
-    pv.c1 = fx_ld<E, 32>(piv, 4);
-    pv.flip = piv[5 * L * 32];
+  uint32_t* rowp = sh + lane;
+  FxPivot<E> pv;
+  const bool ok =
+      fx_pivot(fx_ld<E, ST>(par, tri(o, o)), fx_ld<E, ST>(par, tri(o + 1, o)), fx_ld<E, ST>(par, tri(o + 1, o + 1)), pv);
+  if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
+  sval[fx_sidx(t, (1u << (k - t.d0 + t.cb)) + c, chunk)] = umul(sval[fx_sidx(t, c, chunk)], pv.g);
+  int e = 0;
+  const uint32_t* src = par + (long long)tri(o + 2, o) * (L * ST);
+  E u0 = fx_ld<E, ST>(src, 0), u1 = fx_ld<E, ST>(src, 1), cn = fx_ld<E, ST>(src, 2);
 #pragma unroll 1
-    for (int a = warp; a < R; a += W) {
-      const int e = tri(o + 2 + a, o);
-      FxRow<E> r;
-      fx_row(pv, fx_ld<E, ST>(par, e), fx_ld<E, ST>(par, e + 1), r);
-      uint32_t* w = rowp + a * (6 * L * 32);
-      fx_st<E, 32>(w, 0, r.P);
-      fx_st<E, 32>(w, 1, r.Q);
-      fx_st<E, 32>(w, 2, r.A);
-      fx_st<E, 32>(w, 3, r.U);
-      fx_st<E, 32>(w, 4, r.V);
-      fx_st<E, 32>(w, 5, r.B);
+  for (int a = 0; a < R; ++a) {
+    FxRow<E> r;
+    fx_row(pv, u0, u1, r);
+    E cc = cn;
+    const uint32_t* next = src + (long long)(o + 3 + a) * (L * ST);  // row a + 1 is one entry longer
+    if (a + 1 < R) {  // its head is on its way while this row's entries are formed
+      u0 = fx_ld<E, ST>(next, 0);
+      u1 = fx_ld<E, ST>(next, 1);
+      cn = fx_ld<E, ST>(next, 2);
     }
-  }
-  __syncthreads();
-  const int ne = sym(R);
-  int e = ne * warp / W;
-  const int e1 = ne * (warp + 1) / W;
-  if (e >= e1) return;
-  int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-  while (a * (a + 1) / 2 > e) --a;
-  while ((a + 1) * (a + 2) / 2 <= e) ++a;
-  int b = e - a * (a + 1) / 2;
-  while (e < e1) {
-    const uint32_t* w = rowp + a * (6 * L * 32);
-    const E Pa = fx_ld<E, 32>(w, 0), Qa = fx_ld<E, 32>(w, 1), Aa = fx_ld<E, 32>(w, 2);
-    const int stop = min(e1, e + a + 1 - b);
-    const int src = tri(o + 2 + a, o + 2 + b) - e;
+    const uint32_t* x = rowp;
+    int b = 0;
+    // NB, then two entries at a time: their products' chains overlap
+    if constexpr (NB == 4) {
 #pragma unroll 1
-    for (; e < stop; ++e, ++b) {
-      const uint32_t* x = rowp + b * (6 * L * 32);
-      const E cc = fx_ld<E, ST>(par, src + e);
-      fx_st<E, 32>(out, e, fx_entry(cc, Pa, Qa, Aa, fx_ld<E, 32>(x, 3), fx_ld<E, 32>(x, 4), fx_ld<E, 32>(x, 5)));
+      for (; b + 3 < a; b += 4, e += 4, x += 12 * L * 32) {
+        const E c1 = fx_ld<E, ST>(src, b + 3), c2 = fx_ld<E, ST>(src, b + 4), c3 = fx_ld<E, ST>(src, b + 5);
+        const E v0 = fx_entry(cc, r.P, r.Q, r.A, fx_ld<E, 32>(x, 0), fx_ld<E, 32>(x, 1), fx_ld<E, 32>(x, 2));
+        cc = fx_ld<E, ST>(src, b + 6);
+        const E v1 = fx_entry(c1, r.P, r.Q, r.A, fx_ld<E, 32>(x, 3), fx_ld<E, 32>(x, 4), fx_ld<E, 32>(x, 5));
+        const E v2 = fx_entry(c2, r.P, r.Q, r.A, fx_ld<E, 32>(x, 6), fx_ld<E, 32>(x, 7), fx_ld<E, 32>(x, 8));
+        const E v3 = fx_entry(c3, r.P, r.Q, r.A, fx_ld<E, 32>(x, 9), fx_ld<E, 32>(x, 10), fx_ld<E, 32>(x, 11));
+        fx_st<E, 32>(out, e, v0);
+        fx_st<E, 32>(out, e + 1, v1);
+        fx_st<E, 32>(out, e + 2, v2);
+        fx_st<E, 32>(out, e + 3, v3);
+      }
     }
-    ++a;
-    b = 0;
+#pragma unroll 1
+    for (; b + 1 < a; b += 2, e += 2, x += 6 * L * 32) {
+      const E c1 = fx_ld<E, ST>(src, b + 3);
+      const E v0 = fx_entry(cc, r.P, r.Q, r.A, fx_ld<E, 32>(x, 0), fx_ld<E, 32>(x, 1), fx_ld<E, 32>(x, 2));
+      cc = fx_ld<E, ST>(src, b + 4);
+      const E v1 = fx_entry(c1, r.P, r.Q, r.A, fx_ld<E, 32>(x, 3), fx_ld<E, 32>(x, 4), fx_ld<E, 32>(x, 5));
+      fx_st<E, 32>(out, e, v0);
+      fx_st<E, 32>(out, e + 1, v1);
+    }
+    if (b < a) {
+      const E c1 = fx_ld<E, ST>(src, b + 3);
+      fx_st<E, 32>(out, e, fx_entry(cc, r.P, r.Q, r.A, fx_ld<E, 32>(x, 0), fx_ld<E, 32>(x, 1), fx_ld<E, 32>(x, 2)));
+      cc = c1;
+      ++e;
+    }
+    fx_st<E, 32>(out, e, fx_entry(cc, r.P, r.Q, r.A, r.U, r.V, r.B));
+    ++e;
+    uint32_t* w = rowp + a * (3 * L * 32);
+    fx_st<E, 32>(w, 0, r.U);
+    fx_st<E, 32>(w, 1, r.V);
+    fx_st<E, 32>(w, 2, r.B);
+    src = next;
   }
 }
 
-template <class E>
-__global__ void __launch_bounds__(256) fx_level_kernel(const FxSeg* __restrict__ segs, int nseg,
-                                                       const FxTree* __restrict__ trees,
-                                                       const long long* __restrict__ lvl_off, int q, unsigned chunk,
-                                                       uint32_t* nodes, typename fx_sum<E>::type* sval,
-                                                       int* __restrict__ status) {
+template <class E, int NB>
+__global__ void __launch_bounds__(32) fx_level_warp_kernel(const FxSeg* __restrict__ segs, int nseg,
+                                                           const FxTree* __restrict__ trees,
+                                                           const long long* __restrict__ lvl_off, int q, unsigned chunk,
+                                                           uint32_t* nodes, typename fx_sum<E>::type* sval,
+                                                           int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
   const FxTree t = trees[sg.idx];
   const unsigned tile = (unsigned)((long long)blockIdx.x - sg.first);
   // the first tile's parents are the root and levels 0 .. 4
-  if (tile == 0u && chunk == 0u) fx_level_tile<E, 1>(t, lvl_off, q, tile, chunk, nodes, sval, status, (uint32_t*)smem_raw);
-  else fx_level_tile<E, 32>(t, lvl_off, q, tile, chunk, nodes, sval, status, (uint32_t*)smem_raw);
+  if (tile == 0u && chunk == 0u) fx_level_warp<E, 1, NB>(t, lvl_off, q, tile, chunk, nodes, sval, status, (uint32_t*)smem_raw);
+  else fx_level_warp<E, 32, NB>(t, lvl_off, q, tile, chunk, nodes, sval, status, (uint32_t*)smem_raw);
+}
+
+// The same when children are few or their rows too many for that: a CTA takes TW (1 ..
+// 16) consecutive children, and its 32 / TW x W lane groups share out the rows and then
+// the entries.  One warp forms the pivots; the other CTAs of the SM hide it (q = 6, 7, 8
+// at N = 24: 170, 108, 73 us with 16 children and 4 warps, 196, 123, 78 with 32 and 8).
+// Spreading few children over the chip matters for the first levels: 32 .. 128 tiles
+// of 32 took 42 - 54 us a level, now 14 - 24.
+template <class E, int ST>
+__device__ __forceinline__ void fx_level_cta(const FxTree& t, const long long* lvl_off, int q, unsigned c0, int TW,
+                                             unsigned chunk, uint32_t* nodes, typename fx_sum<E>::type* sval,
+                                             int* status, uint32_t* sh) {
+  constexpr int L = sizeof(E) / 4;
+  const int node = threadIdx.x & (TW - 1), worker = threadIdx.x / TW, workers = blockDim.x / TW;
+  const int R = 2 * q;
+  const int k = t.n - 1 - q;
+  const unsigned c = c0 + node;
+  int p;
+  const uint32_t* par = fx_node<ST, L>(nodes, lvl_off, t, c, chunk, p);
+  const int o = 2 * (p - q - 1);
+  uint32_t* out = nodes + lvl_off[t.tab + k + 1] + (long long)(c >> 5) * sym(R) * (L * 32) + (c & 31u);
+  // shared memory, word w of node i at w TW + i: the pivot's 5 values and flip, then 6
+  // values per row (stride 6 L + 1 words, so that rows a group apart differ in bank)
+  auto put = [&](uint32_t* w, const E& v) {
+#pragma unroll
+    for (int l = 0; l < L; ++l) w[l * TW] = v.w[l];
+  };
+  auto get = [&](const uint32_t* w) {
+    E v;
+#pragma unroll
+    for (int l = 0; l < L; ++l) v.w[l] = w[l * TW];
+    return v;
+  };
+  uint32_t* piv = sh + node;
+  uint32_t* rowp = sh + (5 * L + 1) * TW + node;
+  const int rs = (6 * L + 1) * TW, vs = L * TW;
+  if (threadIdx.x < 32) {
+    FxPivot<E> pv;
+    const bool ok = fx_pivot(fx_ld<E, ST>(par, tri(o, o)), fx_ld<E, ST>(par, tri(o + 1, o)),
+                             fx_ld<E, ST>(par, tri(o + 1, o + 1)), pv);
+    if (worker == 0) {
+      if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
+      sval[fx_sidx(t, (1u << (k - t.d0 + t.cb)) + c, chunk)] = umul(sval[fx_sidx(t, c, chunk)], pv.g);
+      put(piv, pv.a);
+      put(piv + vs, pv.b);
+      put(piv + 2 * vs, pv.m);
+      put(piv + 3 * vs, pv.c0);
+      put(piv + 4 * vs, pv.c1);
+      piv[5 * vs] = pv.flip;
+    }
+  }
+  __syncthreads();
+  {
+    FxPivot<E> pv;
+    pv.a = get(piv);
+    pv.b = get(piv + vs);
+    pv.m = get(piv + 2 * vs);
+    pv.c0 = get(piv + 3 * vs);
+    pv.c1 = get(piv + 4 * vs);
+    pv.flip = piv[5 * vs];
+#pragma unroll 1
+    for (int a = worker; a < R; a += workers) {
+      const int e = tri(o + 2 + a, o);
+      FxRow<E> r;
+      fx_row(pv, fx_ld<E, ST>(par, e), fx_ld<E, ST>(par, e + 1), r);
+      uint32_t* w = rowp + a * rs;
+      put(w, r.P);
+      put(w + vs, r.Q);
+      put(w + 2 * vs, r.A);
+      put(w + 3 * vs, r.U);
+      put(w + 4 * vs, r.V);
+      put(w + 5 * vs, r.B);
+    }
+  }
+  __syncthreads();
+  const int ne = sym(R);
+  int a = 0, b = worker;
+#pragma unroll 1
+  for (int e = worker; e < ne; e += workers, b += workers) {
+    while (b > a) b -= ++a;
+    const E cc = fx_ld<E, ST>(par, tri(o + 2 + a, o + 2) + b);
+    const uint32_t *x = rowp + a * rs, *y = rowp + b * rs;
+    fx_st<E, 32>(out, e, fx_entry(cc, get(x), get(x + vs), get(x + 2 * vs), get(y + 3 * vs), get(y + 4 * vs), get(y + 5 * vs)));
+  }
+}
+
+template <class E>
+__global__ void __launch_bounds__(256) fx_level_cta_kernel(const FxSeg* __restrict__ segs, int nseg,
+                                                           const FxTree* __restrict__ trees,
+                                                           const long long* __restrict__ lvl_off, int q, int TW,
+                                                           unsigned chunk, uint32_t* nodes,
+                                                           typename fx_sum<E>::type* sval, int* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
+  const FxTree t = trees[sg.idx];
+  const unsigned c0 = (unsigned)((long long)blockIdx.x - sg.first) * (unsigned)TW;
+  if (c0 < 32u && chunk == 0u) fx_level_cta<E, 1>(t, lvl_off, q, c0, TW, chunk, nodes, sval, status, (uint32_t*)smem_raw);
+  else fx_level_cta<E, 32>(t, lvl_off, q, c0, TW, chunk, nodes, sval, status, (uint32_t*)smem_raw);
 }
 
 // --------------------------------------------------------------------- leaf --
-// Signed sums of a thread: terms with / without the last mode, and all magnitudes.
+// Sums of a thread: signed terms with (inc) and without (exc) the last mode, and all
+// magnitudes.
 template <class S>
 struct FxSums {
-  S ip, in, ep, en;  // split by sign: inc = ip - in, exc = ep - en
+  S inc, exc, mag;
 };
+// a + x, or a - x where mask is all ones (x ^ mask with the mask's carry).
+template <int L, int F>
+GBS_HD fxn<L, F> fx_add_signed(const fxn<L, F>& a, const fxn<L, F>& x, uint32_t mask) {
+  fxn<L, F> t, r;
+#pragma unroll
+  for (int k = 0; k < L; ++k) t.w[k] = x.w[k] ^ mask;
+  add_cc(mask, mask);  // carry = the mask's lowest bit
+#pragma unroll
+  for (int k = 0; k < L - 1; ++k) r.w[k] = addc_cc(a.w[k], t.w[k]);
+  r.w[L - 1] = addc(a.w[L - 1], t.w[L - 1]);
+  return r;
+}
 
-// The two subsets of a one-mode node: s g and s, signs (-1)^neg and -(-1)^neg.
+// The two subsets of a one-mode node: s g and s, of signs (-1)^neg and -(-1)^neg (neg
+// all ones: odd).
 template <class E, class S>
-__device__ __forceinline__ bool fx_leaf1(const E& p00, const E& p10, const E& p11, const S& s, bool neg, FxSums<S>& acc) {
+__device__ __forceinline__ bool fx_leaf1(const E& p00, const E& p10, const E& p11, const S& s, uint32_t neg,
+                                         FxSums<S>& acc) {
   const E det = fx_det(p00, p10, p11);
   const S sg = umul(s, rsqrt_(det));
-  if (neg) {
-    acc.in = acc.in + sg;
-    acc.ep = acc.ep + s;
-  } else {
-    acc.ip = acc.ip + sg;
-    acc.en = acc.en + s;
-  }
+  acc.inc = fx_add_signed(acc.inc, sg, neg);
+  acc.exc = fx_add_signed(acc.exc, s, ~neg);
+  acc.mag = acc.mag + sg + s;
   return fx_det_in_range(det);
 }
 
-// The four subsets of a two-mode node c (packed lower triangle, 10 entries).
-template <class E, class S>
-__device__ __forceinline__ bool fx_leaf2(const E (&c)[10], const S& s, bool neg, FxSums<S>& acc) {
+// The four subsets of the two-mode node in the four rows from o of a matrix.  Entries
+// are read where they are used (the last block twice), which leaves registers for 16
+// warps per SM.
+template <class E, int ST, class S>
+__device__ __forceinline__ bool fx_leaf2(const uint32_t* m, int o, const S& s, uint32_t neg, FxSums<S>& acc) {
+  constexpr int W = sizeof(E) / 4 * ST;
+  const uint32_t* m0 = m + (long long)tri(o, o) * W;
+  const uint32_t* m1 = m + (long long)tri(o + 1, o) * W;
+  const uint32_t* m2 = m + (long long)tri(o + 2, o) * W;
+  const uint32_t* m3 = m + (long long)tri(o + 3, o) * W;
   FxPivot<E> pv;
-  bool ok = fx_pivot(c[0], c[1], c[2], pv);
-  FxRow<E> r0, r1;
-  fx_row(pv, c[3], c[4], r0);
-  fx_row(pv, c[6], c[7], r1);
-  E p00 = fx_entry(c[5], r0.P, r0.Q, r0.A, r0.U, r0.V, r0.B);
-  E p10 = fx_entry(c[8], r1.P, r1.Q, r1.A, r0.U, r0.V, r0.B);
-  E p11 = fx_entry(c[9], r1.P, r1.Q, r1.A, r1.U, r1.V, r1.B);
+  bool ok = fx_pivot(fx_ld<E, ST>(m0, 0), fx_ld<E, ST>(m1, 0), fx_ld<E, ST>(m1, 1), pv);
+  FxRow<E> r;
+  fx_row(pv, fx_ld<E, ST>(m2, 0), fx_ld<E, ST>(m2, 1), r);
+  E p00 = fx_entry(fx_ld<E, ST>(m2, 2), r.P, r.Q, r.A, r.U, r.V, r.B);
+  E p10, p11;
+  {
+    FxRow<E> r1;
+    fx_row(pv, fx_ld<E, ST>(m3, 0), fx_ld<E, ST>(m3, 1), r1);
+    p10 = fx_entry(fx_ld<E, ST>(m3, 2), r1.P, r1.Q, r1.A, r.U, r.V, r.B);
+    p11 = fx_entry(fx_ld<E, ST>(m3, 3), r1.P, r1.Q, r1.A, r1.U, r1.V, r1.B);
+  }
   S sv = umul(s, pv.g);
   // both sides through one copy of the code (the instruction cache is the limit of
   // an inlined one)
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
-    ok &= fx_leaf1(p00, p10, p11, sv, neg != (side != 0), acc);
-    p00 = c[5];
-    p10 = c[8];
-    p11 = c[9];
+    ok &= fx_leaf1(p00, p10, p11, sv, neg ^ (0u - (uint32_t)side), acc);
+    p00 = fx_ld<E, ST>(m2, 2);
+    p10 = fx_ld<E, ST>(m3, 2);
+    p11 = fx_ld<E, ST>(m3, 3);
     sv = s;
   }
   return ok;
@@ -444,63 +571,20 @@ __device__ __forceinline__ bool fx_leaf2(const E (&c)[10], const S& s, bool neg,
 
 template <class E, int Q, int ST>
 __device__ __forceinline__ bool fx_leaf_node(const uint32_t* m, int p, const typename fx_sum<E>::type& s,
-                                             FxSums<typename fx_sum<E>::type>& acc) {
-  typedef typename fx_sum<E>::type S;
+                                             uint32_t neg, FxSums<typename fx_sum<E>::type>& acc) {
   const int o = 2 * (p - Q);
   if constexpr (Q == 1) {
     return fx_leaf1(fx_ld<E, ST>(m, tri(o, o)), fx_ld<E, ST>(m, tri(o + 1, o)), fx_ld<E, ST>(m, tri(o + 1, o + 1)), s,
-                    false, acc);
-  } else if constexpr (Q == 2) {
-    E c[10];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int row = tri(o + a, o);
-#pragma unroll
-      for (int b = 0; b <= a; ++b) c[tri(a, b)] = fx_ld<E, ST>(m, row + b);
-    }
-    return fx_leaf2(c, s, false, acc);
+                    neg, acc);
   } else {
-    // three modes: the included child is formed entry by entry from the node's
-    // matrix, which is read where it lies; the excluded one is its last four rows
-    static_assert(Q == 3, "at most three levels per leaf thread");
-    E c[10];
-    S sv;
-    bool ok;
-    {
-      FxPivot<E> pv;
-      ok = fx_pivot(fx_ld<E, ST>(m, tri(o, o)), fx_ld<E, ST>(m, tri(o + 1, o)), fx_ld<E, ST>(m, tri(o + 1, o + 1)), pv);
-      sv = umul(s, pv.g);
-      FxRow<E> r[4];
-#pragma unroll 1
-      for (int a = 0; a < 4; ++a) {
-        const int e = tri(o + 2 + a, o);
-        fx_row(pv, fx_ld<E, ST>(m, e), fx_ld<E, ST>(m, e + 1), r[a]);
-      }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b <= a; ++b)
-          c[tri(a, b)] = fx_entry(fx_ld<E, ST>(m, tri(o + 2 + a, o + 2) + b), r[a].P, r[a].Q, r[a].A, r[b].U, r[b].V,
-                                  r[b].B);
-    }
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-      ok &= fx_leaf2(c, sv, side != 0, acc);
-      if (side == 0) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b <= a; ++b) c[tri(a, b)] = fx_ld<E, ST>(m, tri(o + 2 + a, o + 2) + b);
-        sv = s;
-      }
-    }
-    return ok;
+    static_assert(Q == 2, "one or two levels per leaf thread");
+    return fx_leaf2<E, ST>(m, o, s, neg, acc);
   }
 }
 
 // One warp per unit: tiles_per_unit consecutive tiles of 32 nodes of one tree.
 template <class E, int Q>
-__global__ void __launch_bounds__(128) fx_leaf_kernel(const FxSeg* __restrict__ segs, int nseg, long long units,
+__global__ void __launch_bounds__(128, 4) fx_leaf_kernel(const FxSeg* __restrict__ segs, int nseg, long long units,
                                                       unsigned chunk, const FxTree* __restrict__ trees,
                                                       const long long* __restrict__ lvl_off,
                                                       const uint32_t* __restrict__ nodes,
@@ -516,47 +600,43 @@ __global__ void __launch_bounds__(128) fx_leaf_kernel(const FxSeg* __restrict__ 
   const FxTree t = trees[sg.idx];
   const unsigned count = 1u << (t.D - t.d0 + t.cb);
   const S zero = fx_of<S>(0.0);
-  S inc = zero, exc = zero, mag = zero;
+  FxSums<S> acc{zero, zero, zero};
   bool ok = true;
   const unsigned tile0 = (unsigned)(unit - sg.first) * (unsigned)sg.tiles_per_unit;
 #pragma unroll 1
   for (int i = 0; i < sg.tiles_per_unit; ++i) {
     const unsigned v = (tile0 + i) * 32u + lane;
     if (v >= count) break;
-    FxSums<S> acc{zero, zero, zero, zero};
     const S s = sval[fx_sidx(t, v, chunk)];
+    // sign of the node: (-1)^(exclusions above)
+    const uint32_t odd = ((t.D - __popc(v) - __popc(chunk)) & 1) ? 0xffffffffu : 0u;
     int p;
     if (v < 32u && chunk == 0u) {
       const uint32_t* m = fx_node<1, L>(nodes, lvl_off, t, v, chunk, p);
-      ok &= fx_leaf_node<E, Q, 1>(m, p, s, acc);
+      ok &= fx_leaf_node<E, Q, 1>(m, p, s, odd, acc);
     } else {
       const uint32_t* m = fx_node<32, L>(nodes, lvl_off, t, v, chunk, p);
-      ok &= fx_leaf_node<E, Q, 32>(m, p, s, acc);
+      ok &= fx_leaf_node<E, Q, 32>(m, p, s, odd, acc);
     }
-    mag = mag + ((acc.ip + acc.in) + (acc.ep + acc.en));
-    S di = acc.ip - acc.in, de = acc.ep - acc.en;
-    // sign of the node: (-1)^(exclusions above)
-    const uint32_t odd = ((t.D - __popc(v) - __popc(chunk)) & 1) ? 0xffffffffu : 0u;
-    inc = inc + fx_flip(di, odd);
-    exc = exc + fx_flip(de, odd);
   }
   if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
   __syncwarp();
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    inc = inc + shfl_down(inc, off);
-    exc = exc + shfl_down(exc, off);
-    mag = mag + shfl_down(mag, off);
+    acc.inc = acc.inc + shfl_down(acc.inc, off);
+    acc.exc = acc.exc + shfl_down(acc.exc, off);
+    acc.mag = acc.mag + shfl_down(acc.mag, off);
   }
-  if (lane == 0) parts[unit] = FxPart<S>{inc, exc, mag};
+  if (lane == 0) parts[unit] = FxPart<S>{acc.inc, acc.exc, acc.mag};
 }
 
 // -------------------------------------------------------------------- final --
 // One CTA per tree; segs[t].first = the tree's first unit, segs[t + 1].first the end.
+// (Ten thousand units took it 31 us: one wave of leaf warps is what it gets.)
 template <class S>
-__global__ void __launch_bounds__(256) fx_final_kernel(const FxPart<S>* __restrict__ parts,
-                                                       const FxSeg* __restrict__ segs,
-                                                       const FxTree* __restrict__ trees, TreeOut* __restrict__ outs) {
+__global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* __restrict__ parts,
+                                                        const FxSeg* __restrict__ segs,
+                                                        const FxTree* __restrict__ trees, TreeOut* __restrict__ outs) {
   const int t = blockIdx.x;
   const S zero = fx_of<S>(0.0);
   S inc = zero, exc = zero, mag = zero;
@@ -565,23 +645,25 @@ __global__ void __launch_bounds__(256) fx_final_kernel(const FxPart<S>* __restri
     exc = exc + parts[i].exc;
     mag = mag + parts[i].abs;
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __shared__ FxPart<S> sh[32];
+#pragma unroll 1
+  for (int stage = 0; stage < 2; ++stage) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    inc = inc + shfl_down(inc, off);
-    exc = exc + shfl_down(exc, off);
-    mag = mag + shfl_down(mag, off);
+    for (int off = 16; off > 0; off >>= 1) {
+      inc = inc + shfl_down(inc, off);
+      exc = exc + shfl_down(exc, off);
+      mag = mag + shfl_down(mag, off);
+    }
+    if (stage == 1) break;
+    if (lane == 0) sh[warp] = FxPart<S>{inc, exc, mag};
+    __syncthreads();
+    if (warp != 0) return;
+    inc = lane < nw ? sh[lane].inc : zero;
+    exc = lane < nw ? sh[lane].exc : zero;
+    mag = lane < nw ? sh[lane].abs : zero;
   }
-  __shared__ FxPart<S> sh[8];
-  if (lane == 0) sh[warp] = FxPart<S>{inc, exc, mag};
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  const int nw = blockDim.x >> 5;
-  for (int w = 1; w < nw; ++w) {
-    inc = inc + sh[w].inc;
-    exc = exc + sh[w].exc;
-    mag = mag + sh[w].abs;
-  }
+  if (lane != 0) return;
   TreeOut* o = outs + trees[segs[t].idx].tree;
   fx_store3(inc, o->inc);
   fx_store3(exc, o->exc);

@@ -33,14 +33,11 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   // Levels per leaf thread.
   const int Qmax = std::max(1, std::min(2, 3 - tune.q_drop));
   const int nmax = in[order[0]].n;
-  // Depth of the top kernel: at most tune.d_top and about 1024 CTAs, at least the five
-  // levels that are not kept in tiles, and enough that a level's rows fit shared memory.
-  constexpr int kSmemMax = 220 * 1024;
-  constexpr int kRowBytes = 6 * L * 32 * 4, kPivBytes = (5 * L + 1) * 32 * 4;
-  const int q_fit = (kSmemMax - kPivBytes) / kRowBytes / 2;
+  // Depth of the top kernel: at most tune.d_top and about 64 CTAs, at least the five
+  // levels that are not kept in tiles.
   int d_top = 5;
-  while (d_top < tune.d_top && ((long long)ntrees << (d_top + 1)) <= 1024) ++d_top;
-  d_top = std::max(d_top, nmax - 1 - q_fit);
+  while (d_top < tune.d_top && ((long long)ntrees << (d_top + 1)) <= 64) ++d_top;
+  auto cta_smem = [&](int R, int TW) { return (size_t)((5 * L + 1) + R * (6 * L + 1)) * TW * 4; };
   std::vector<FxTree> trees(ntrees);
   std::vector<int> Q(ntrees);
   for (int i = 0; i < ntrees; ++i) {
@@ -102,28 +99,38 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   }
   // levels, by child size q downwards
   struct Launch {
-    int q, W;
+    int q, TW, W;  // TW = 0: a warp per 32 children; else W warps per TW children
     std::vector<FxSeg> segs;
-    long long tiles;
-    size_t at;
+    long long children, blocks;
+    size_t at, smem;
     bool in_chunk;
   };
   std::vector<Launch> levels;
   for (int q = nmax - 1; q >= 1; --q) {
-    Launch l{q, 1, {}, 0, 0, false};
+    Launch l{q, 0, 1, {}, 0, 0, 0, 0, false};
     for (int i = 0; i < ntrees; ++i) {
       const int k = trees[i].n - 1 - q;
       if (k < dtop_of(i) || k >= trees[i].D) continue;
       l.in_chunk = d0 > 0 && k >= d0;
-      l.segs.push_back(FxSeg{l.tiles, i, 0});
-      l.tiles += 1LL << ((l.in_chunk ? k - d0 + cb : k) - 5);
+      l.segs.push_back(FxSeg{l.children, i, 0});
+      l.children += 1LL << (l.in_chunk ? k - d0 + cb : k);
     }
     if (l.segs.empty()) continue;
-    // Warps per tile: enough tiles fit an SM's shared memory for ~16 warps, and few
-    // tiles are spread over more warps.
     const int R = 2 * q;
-    l.W = R >= 16 ? 8 : R >= 10 ? 4 : R >= 6 ? 2 : 1;
-    while (l.W < 8 && l.tiles * l.W < 16LL * ctx->sm_count) l.W *= 2;
+    const long long tiles = l.children / 32;
+    if (tiles >= 8LL * ctx->sm_count && q <= 5) {
+      l.smem = (size_t)3 * R * L * 128;
+    } else {
+      // CTAs of 4 warps for 16 children; where that is too few, more warps for fewer
+      l.TW = 16;
+      while (l.TW > 1 && l.children / l.TW < ctx->sm_count) l.TW /= 2;
+      l.W = l.children / l.TW < 3LL * ctx->sm_count ? 8 : 4;
+      while (l.W > 1 && 32 / l.TW * l.W > std::max(R, sym(R) / 2)) l.W /= 2;
+      l.smem = cta_smem(R, l.TW);
+    }
+    const int per = l.TW ? l.TW : 32;
+    for (FxSeg& sg : l.segs) sg.first /= per;
+    l.blocks = l.children / per;
     levels.push_back(l);
   }
   // leaves, one launch per Q
@@ -137,7 +144,8 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   std::vector<FxSeg> fin;
   long long tiles_total = 0, units_total = 0;
   for (int i = 0; i < ntrees; ++i) tiles_total += ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
-  const int tpu = (int)std::max(1LL, std::min(32LL, tiles_total / (64LL * ctx->sm_count)));
+  // tiles per warp: one wave of the 16 warps an SM holds
+  const int tpu = (int)std::max(1LL, std::min(64LL, (tiles_total + 16LL * ctx->sm_count - 1) / (16LL * ctx->sm_count)));
   for (int i = 0; i < ntrees; ++i) {
     if (leaves.empty() || leaves.back().Q != Q[i]) leaves.push_back(Leaf{Q[i], {}, 0, 0});
     Leaf& lf = leaves.back();
@@ -179,16 +187,24 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   const int smem_top = sym(2 * nmax) * (int)sizeof(E) + 2 * nmax * (int)sizeof(FxRow<E>);
   if ((st = check_cuda(ctx, cudaFuncSetAttribute(fx_top_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_top),
                        "top smem")) ||
-      (st = check_cuda(ctx, cudaFuncSetAttribute(fx_level_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax),
+      (st = check_cuda(ctx, cudaFuncSetAttribute(fx_level_cta_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 cta_smem(62, 16)),
                        "level smem")))
     return st;
   fx_top_kernel<E><<<(unsigned)top_blocks, 256, smem_top, s>>>((const FxSeg*)(plan + o_top), ntrees, d_trees, d_off,
                                                                (const double*)roots_dev, nodes, sval, status_dev);
   count_launch(ctx);
   auto level = [&](const Launch& l, unsigned chunk) {
-    fx_level_kernel<E><<<(unsigned)l.tiles, 32 * l.W, kPivBytes + 2 * l.q * kRowBytes, s>>>(
-        (const FxSeg*)(plan + l.at), (int)l.segs.size(), l.in_chunk ? d_chunked : d_trees, d_off, l.q, chunk, nodes, sval,
-        status_dev);
+    const FxSeg* sg = (const FxSeg*)(plan + l.at);
+    const int ns = (int)l.segs.size();
+    const FxTree* tr = l.in_chunk ? d_chunked : d_trees;
+    if (l.TW)
+      fx_level_cta_kernel<E><<<(unsigned)l.blocks, 32 * l.W, l.smem, s>>>(sg, ns, tr, d_off, l.q, l.TW, chunk, nodes, sval,
+                                                                          status_dev);
+    else if (l.q >= 4)
+      fx_level_warp_kernel<E, 4><<<(unsigned)l.blocks, 32, l.smem, s>>>(sg, ns, tr, d_off, l.q, chunk, nodes, sval, status_dev);
+    else
+      fx_level_warp_kernel<E, 2><<<(unsigned)l.blocks, 32, l.smem, s>>>(sg, ns, tr, d_off, l.q, chunk, nodes, sval, status_dev);
     count_launch(ctx);
   };
   for (const Launch& l : levels)
@@ -210,8 +226,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
       const int ns = (int)l.segs.size();
       switch (l.Q) {
         case 1: fx_leaf_kernel<E, 1><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
-        case 2: fx_leaf_kernel<E, 2><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
-        default: fx_leaf_kernel<E, 3><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        default: fx_leaf_kernel<E, 2><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
       }
       count_launch(ctx);
       base += l.units;
@@ -221,7 +236,8 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     cudaEventRecord(ctx->leaf_timer.stop, s);
     ctx->leaf_timer.pending = true;
   }
-  fx_final_kernel<S><<<(unsigned)ntrees, 256, 0, s>>>(parts, (const FxSeg*)(plan + o_fin), d_trees, outs_dev);
+  const int final_threads = units_total > 256LL * ntrees ? 1024 : 128;
+  fx_final_kernel<S><<<(unsigned)ntrees, final_threads, 0, s>>>(parts, (const FxSeg*)(plan + o_fin), d_trees, outs_dev);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "fixed-point batch launch");
 }
