@@ -2,8 +2,8 @@
 #include "gbs_fxtree_driver.cuh"
 
 namespace gbs {
-gbs_status batch_fxw_real(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots, TreeOut* outs,
-                          int* status, const BatchTune& tune) {
-  return fx_batch_run<fxw>(ctx, ntrees, trees, roots, outs, status, tune);
+gbs_status batch_fxw_real(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots, int* status,
+                         const BatchTune& tune, const FxFinish& fin) {
+  return fx_batch_run<fxw>(ctx, ntrees, trees, roots, status, tune, fin);
 }
 }  // namespace gbs

@@ -488,4 +488,27 @@ __global__ void batch_final_kernel(const Partial<Red>* __restrict__ parts, const
   }
 }
 
+// ------------------------------------------------------------------ finish --
+// Torontonian, probability, cancellation ratio and error estimate of one tree.
+__device__ __forceinline__ ProbOut finish_tree(const TreeOut& o, int status, double logdet, int n, double u,
+                                               double extra) {
+  const td a{o.inc[0], o.inc[1], o.inc[2]};
+  const td b{o.exc[0], o.exc[1], o.exc[2]};
+  const td tor = a + b;
+  const double sc = exp(-0.5 * logdet);
+  const td p = tor * sc;
+  ProbOut r;
+  r.p_hi = p.x0;
+  r.p_lo = p.x1 + p.x2;
+  r.tor[0] = tor.x0; r.tor[1] = tor.x1; r.tor[2] = tor.x2;
+  r.abs_sum = o.abs;
+  const double tv = tor.x0 + (tor.x1 + tor.x2);
+  r.kappa = tv != 0.0 ? o.abs / fabs(tv) : INFINITY;
+  r.err = (4.0 * (n > 0 ? n : 1) + extra) * u * o.abs * sc;
+  for (int i = 0; i < 3; ++i) { r.inc[i] = o.inc[i]; r.exc[i] = o.exc[i]; }
+  r.status = status;
+  r.pad = 0;
+  return r;
+}
+
 }  // namespace gbs

@@ -66,6 +66,21 @@ bool fx_ok_sigma(const gbs_state* st, int n) {
   return sm > 0.0 && sm < 64.0 && n <= 36;
 }
 
+// FP64 trees in 64-bit fixed point (64 fraction bits; s and sums have 95 integer bits).
+// Errors there are absolute, 2^-63 per operation, amplified by at most ~sigma_max^2
+// through a pivot's determinant and inverse; FP64's are 2^-53 of values up to 1 and more.
+// With sigma_max <= 16 the former stay below the latter.  Every term of a physical
+// state's (Sigma^-1)_S tree is at least 1 (det of a conditioned V + I/2 is), so the sum
+// of magnitudes is at least 2^n and the terms' absolute errors vanish against FP64's.
+// The bound needs the closed form (a state built from its factors).
+bool fxd_ok_inverse(const gbs_state* st, int n) {
+  const double sm = st->sigma_max;
+  return st->has_factors && sm > 0.0 && sm <= 16.0 && n * std::log2(1.0 + sm) < 92.0;
+}
+// Sampler trees: terms are at most 1 and their magnitudes add up to at least 1, so the
+// absolute errors of 2^n terms stay below FP64's estimate only for small n.
+bool fxd_ok_sigma(const gbs_state* st, int n) { return fx_ok_sigma(st, n) && n <= 10; }
+
 // ------------------------------------------------------- click blocks ---
 struct ClickReq {
   const cplx<double>* U;      // factor form (or null)
@@ -184,24 +199,7 @@ __global__ void batch_finish_kernel(const TreeOut* __restrict__ outs, const int*
                                     double extra, int ntrees, ProbOut* __restrict__ po) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ntrees) return;
-  const TreeOut& o = outs[t];
-  const td a{o.inc[0], o.inc[1], o.inc[2]};
-  const td b{o.exc[0], o.exc[1], o.exc[2]};
-  const td tor = a + b;
-  const double sc = exp(-0.5 * logdet[t]);
-  const td p = tor * sc;
-  ProbOut r;
-  r.p_hi = p.x0;
-  r.p_lo = p.x1 + p.x2;
-  r.tor[0] = tor.x0; r.tor[1] = tor.x1; r.tor[2] = tor.x2;
-  r.abs_sum = o.abs;
-  const double tv = tor.x0 + (tor.x1 + tor.x2);
-  r.kappa = tv != 0.0 ? o.abs / fabs(tv) : INFINITY;
-  r.err = (4.0 * (nmodes[t] > 0 ? nmodes[t] : 1) + extra) * u * o.abs * sc;
-  for (int i = 0; i < 3; ++i) { r.inc[i] = o.inc[i]; r.exc[i] = o.exc[i]; }
-  r.status = status[t];
-  r.pad = 0;
-  po[t] = r;
+  po[t] = finish_tree(outs[t], status[t], logdet[t], nmodes[t], u, extra);
 }
 
 static double unit_roundoff_b(int prec) {
@@ -230,57 +228,73 @@ static gbs_status batch_variant(gbs_ctx* ctx, int prec, bool real, int nt, const
                                   : batch_td_cplx(ctx, nt, tr, roots, outs, status, tu);
     case GBS_PREC_FP32_DIAG: return real ? batch_fp32_real(ctx, nt, tr, roots, outs, status, tu)
                                          : batch_fp32_cplx(ctx, nt, tr, roots, outs, status, tu);
-    case GBS_PREC_FX: return real ? batch_fx_real(ctx, nt, tr, roots, outs, status, tu)
-                                  : set_error(ctx, GBS_EINVAL, "the fixed-point precision needs the real basis");
-    case GBS_PREC_FXW: return real ? batch_fxw_real(ctx, nt, tr, roots, outs, status, tu)
-                                   : set_error(ctx, GBS_EINVAL, "the fixed-point precision needs the real basis");
-    case GBS_PREC_FXN: return real ? batch_fxn_real(ctx, nt, tr, roots, outs, status, tu)
-                                   : set_error(ctx, GBS_EINVAL, "the fixed-point precision needs the real basis");
     case GBS_PREC_FP64P: return real ? batch_fp64p_real(ctx, nt, tr, roots, outs, status, tu)
                                      : set_error(ctx, GBS_EINVAL, "the paired FP64 precision needs the real basis");
   }
   return set_error(ctx, GBS_EINVAL, "unknown precision");
 }
 
+// The fixed-point engine's instance for prec (FP64: the 64-bit one).
+static gbs_status fixed_variant(gbs_ctx* ctx, int prec, int nt, const BatchTree* tr, const void* roots, int* status,
+                                const FxFinish& fin) {
+  const BatchTune& tu = batch_tune_for(ctx, prec == GBS_PREC_FP64 ? GBS_PREC_FXN : prec, true);
+  switch (prec) {
+    case GBS_PREC_FP64: return batch_fxd_real(ctx, nt, tr, roots, status, tu, fin);
+    case GBS_PREC_FXN: return batch_fxn_real(ctx, nt, tr, roots, status, tu, fin);
+    case GBS_PREC_FX: return batch_fx_real(ctx, nt, tr, roots, status, tu, fin);
+    case GBS_PREC_FXW: return batch_fxw_real(ctx, nt, tr, roots, status, tu, fin);
+  }
+  return set_error(ctx, GBS_EINVAL, "unknown precision");
+}
+
 gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const BatchTree* trees, const void* roots_dev,
-                      const double* logdet, ProbOut* host_out) {
+                      const double* logdet, ProbOut* host_out, bool bounded) {
   if (ntrees <= 0) return GBS_OK;
   gbs_status st;
   // too large for one plan: the two halves in turn (a tree's result does not depend
   // on the rest of its batch, so the split changes no value)
   auto split = [&]() -> gbs_status {
     const int h = ntrees / 2;
-    gbs_status s2 = batch_eval(ctx, prec, real, h, trees, roots_dev, logdet, host_out);
+    gbs_status s2 = batch_eval(ctx, prec, real, h, trees, roots_dev, logdet, host_out, bounded);
     if (s2) return s2;
-    return batch_eval(ctx, prec, real, ntrees - h, trees + h, roots_dev, logdet + h, host_out + h);
+    return batch_eval(ctx, prec, real, ntrees - h, trees + h, roots_dev, logdet + h, host_out + h, bounded);
   };
   const size_t n = (size_t)ntrees;
   auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t bytes = r256(n * sizeof(TreeOut)) + r256(n * sizeof(ProbOut)) + r256(n * sizeof(int));
+  const size_t bytes = r256(n * sizeof(TreeOut)) + r256(n * sizeof(ProbOut)) + r256(2 * n * sizeof(int));
   if ((st = dev_reserve(ctx, ctx->aux_dev, bytes))) return st;
   unsigned char* base = (unsigned char*)ctx->aux_dev.ptr;
   TreeOut* outs = (TreeOut*)base;
   ProbOut* po = (ProbOut*)(base + ((n * sizeof(TreeOut) + 255) / 256) * 256);
   int* status = (int*)((unsigned char*)po + ((n * sizeof(ProbOut) + 255) / 256) * 256);
-  std::vector<int> nm(n);
-  for (size_t t = 0; t < n; ++t) nm[t] = trees[t].n;
-  const void *d_logdet = nullptr, *d_n = nullptr;
-  if ((st = stage(ctx, logdet, n * sizeof(double), &d_logdet)) || (st = stage(ctx, nm.data(), n * sizeof(int), &d_n)))
-    return st;
-  if ((st = check_cuda(ctx, cudaMemsetAsync(status, 0, n * sizeof(int), ctx->stream), "memset"))) return st;
+  if ((st = check_cuda(ctx, cudaMemsetAsync(status, 0, 2 * n * sizeof(int), ctx->stream), "memset"))) return st;
   ctx->batch_split = false;
-  if ((st = batch_variant(ctx, prec, real, ntrees, trees, roots_dev, outs, status))) {
+  const double u = unit_roundoff_b(prec), extra = err_factor(prec, 1) - err_factor(GBS_PREC_TD, 1);
+  const bool fixed64 = bounded && real && prec == GBS_PREC_FP64;
+  if (fixed64 || is_fixed_point(prec)) {
+    if (!real) return set_error(ctx, GBS_EINVAL, "the fixed-point precision needs the real basis");
+    st = fixed_variant(ctx, prec, ntrees, trees, roots_dev, status, FxFinish{logdet, u, extra, po, status + n});
+  } else {
+    st = batch_variant(ctx, prec, real, ntrees, trees, roots_dev, outs, status);
+  }
+  if (st) {
     if (st == GBS_ENOMEM && ctx->batch_split) {
       ctx->batch_split = false;
       return split();
     }
     return st;
   }
-  batch_finish_kernel<<<(ntrees + 127) / 128, 128, 0, ctx->stream>>>(
-      outs, status, (const double*)d_logdet, (const int*)d_n, unit_roundoff_b(prec),
-      err_factor(prec, 1) - err_factor(GBS_PREC_TD, 1), ntrees, po);
-  count_launch(ctx);
-  if ((st = check_cuda(ctx, cudaGetLastError(), "finish"))) return st;
+  if (!fixed64 && !is_fixed_point(prec)) {
+    std::vector<int> nm(n);
+    for (size_t t = 0; t < n; ++t) nm[t] = trees[t].n;
+    const void *d_logdet = nullptr, *d_n = nullptr;
+    if ((st = stage(ctx, logdet, n * sizeof(double), &d_logdet)) || (st = stage(ctx, nm.data(), n * sizeof(int), &d_n)))
+      return st;
+    batch_finish_kernel<<<(ntrees + 127) / 128, 128, 0, ctx->stream>>>(
+        outs, status, (const double*)d_logdet, (const int*)d_n, u, extra, ntrees, po);
+    count_launch(ctx);
+    if ((st = check_cuda(ctx, cudaGetLastError(), "finish"))) return st;
+  }
   if ((st = check_cuda(ctx, cudaMemcpyAsync(host_out, po, n * sizeof(ProbOut), cudaMemcpyDeviceToHost, ctx->stream),
                        "readback")) ||
       (st = stream_sync(ctx)))
@@ -291,6 +305,23 @@ gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const Batch
     ctx->leaf_timer.total_ms += ms;
     ctx->leaf_timer.count += 1;
     ctx->leaf_timer.pending = false;
+  }
+  if (fixed64) {
+    // a tree whose values left the range after all: again in floating point
+    std::vector<BatchTree> again;
+    std::vector<double> ld;
+    std::vector<int> which;
+    for (int t = 0; t < ntrees; ++t)
+      if (host_out[t].status == kStatusRange) {
+        again.push_back(trees[t]);
+        ld.push_back(logdet[t]);
+        which.push_back(t);
+      }
+    if (!again.empty()) {
+      std::vector<ProbOut> r(again.size());
+      if ((st = batch_eval(ctx, prec, real, (int)again.size(), again.data(), roots_dev, ld.data(), r.data()))) return st;
+      for (size_t i = 0; i < which.size(); ++i) host_out[which[i]] = r[i];
+    }
   }
   return GBS_OK;
 }
@@ -445,6 +476,12 @@ gbs_status probs_batch(gbs_ctx* ctx, int nreq, const gbs_state* const* states, c
       }
       run.push_back(i);
     }
+    // FP64: the trees their states bound first, in 64-bit fixed point
+    std::stable_partition(run.begin(), run.end(), [&](int i) {
+      return pr == GBS_PREC_FP64 && real && fxd_ok_inverse(states[i], N[i]);
+    });
+    size_t nb = 0;
+    while (nb < run.size() && pr == GBS_PREC_FP64 && real && fxd_ok_inverse(states[run[nb]], N[run[nb]])) ++nb;
     std::vector<BatchTree> sub(run.size());
     std::vector<double> ld(run.size());
     for (size_t i = 0; i < run.size(); ++i) {
@@ -452,7 +489,9 @@ gbs_status probs_batch(gbs_ctx* ctx, int nreq, const gbs_state* const* states, c
       ld[i] = states[run[i]]->logdet_sigma;
     }
     std::vector<ProbOut> res(run.size());
-    if ((st = batch_eval(ctx, pr, real, (int)run.size(), sub.data(), ctx->hbuf.ptr, ld.data(), res.data())))
+    if ((st = batch_eval(ctx, pr, real, (int)nb, sub.data(), ctx->hbuf.ptr, ld.data(), res.data(), true)) ||
+        (st = batch_eval(ctx, pr, real, (int)(run.size() - nb), sub.data() + nb, ctx->hbuf.ptr, ld.data() + nb,
+                         res.data() + nb)))
       return st;
     for (size_t i = 0; i < run.size(); ++i) {
       fill(&out[run[i]], res[i], pr, real, ld[i]);

@@ -38,6 +38,8 @@ struct fxn {
   static_assert(F >= 2 && L > F, "at least two fraction limbs and one integer limb");
   uint32_t w[L];
 };
+typedef fxn<3, 2> fxd;   // FP64 trees of bounded states: entries (64 fraction bits)
+typedef fxn<5, 2> fxds;  // their s and sums
 typedef fxn<5, 4> fxn4;  // FXN entries
 typedef fxn<6, 4> fxn4s; // FXN s and sums
 typedef fxn<6, 5> fx;    // FX entries
@@ -238,6 +240,7 @@ static_assert(sizeof(fxn4) == 20 && sizeof(fxn4s) == 24 && sizeof(fx) == 24 && s
 
 // The s type (running product of pivot factors, term sums) of an entry type.
 template <class E> struct fx_sum;
+template <> struct fx_sum<fxd> { typedef fxds type; };
 template <> struct fx_sum<fxn4> { typedef fxn4s type; };
 template <> struct fx_sum<fx> { typedef fxs type; };
 template <> struct fx_sum<fxw> { typedef fxws type; };

@@ -21,7 +21,9 @@
 //                 tree (lane = child), or, where children are few, a CTA per 1 .. 32.
 //   leaf kernel   a warp takes tiles of 32 nodes of one tree, one thread per node
 //                 for all 2^Q subsets of its last Q modes.
-//   final kernel  one CTA per tree adds the warps' sums.
+//   final kernel  one CTA per tree adds the warps' sums and finishes the result.
+//   small kernel  a tree of few modes in one launch, in the shared memory of one or a
+//                 few CTAs.
 // Measured against the engine it replaced (both children stored, subtrees of 9
 // modes expanded in shared memory, signed products, 2 products per entry), with the
 // default launch shapes: N = 24 (M = 200, AUTO) 8.86 -> 2.4 ms, 256 requests of N =
@@ -56,7 +58,7 @@
 #pragma once
 #include "gbs_fx.cuh"
 #include "gbs_internal.h"
-#include "gbs_tree.cuh"
+#include "gbs_batch.cuh"
 
 namespace gbs {
 
@@ -190,6 +192,7 @@ __device__ __forceinline__ void fx_st(uint32_t* p, int e, const E& v) {
 // s of it is element s_base + v (v < 2^d0), s_base + 2^d0 - 2^cb + v'.
 struct FxTree {
   long long root_off, s_base;
+  double logdet;
   int n, D, tree, tab, d0, cb;
 };
 struct FxSeg {
@@ -636,7 +639,9 @@ __global__ void __launch_bounds__(128, 4) fx_leaf_kernel(const FxSeg* __restrict
 template <class S>
 __global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* __restrict__ parts,
                                                         const FxSeg* __restrict__ segs,
-                                                        const FxTree* __restrict__ trees, TreeOut* __restrict__ outs) {
+                                                        const FxTree* __restrict__ trees,
+                                                        const int* __restrict__ status, double u, double extra,
+                                                        ProbOut* __restrict__ out) {
   const int t = blockIdx.x;
   const S zero = fx_of<S>(0.0);
   S inc = zero, exc = zero, mag = zero;
@@ -664,10 +669,268 @@ __global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* __restr
     mag = lane < nw ? sh[lane].abs : zero;
   }
   if (lane != 0) return;
-  TreeOut* o = outs + trees[segs[t].idx].tree;
-  fx_store3(inc, o->inc);
-  fx_store3(exc, o->exc);
-  o->abs = to_double(mag);
+  const FxTree tr = trees[segs[t].idx];
+  TreeOut o;
+  fx_store3(inc, o.inc);
+  fx_store3(exc, o.exc);
+  o.abs = to_double(mag);
+  out[tr.tree] = finish_tree(o, status[tr.tree], tr.logdet, tr.n, u, extra);
+}
+
+// -------------------------------------------------------------- small trees --
+// A tree of few modes is latency only, so it takes one launch.  A CTA per setting of
+// the tree's first d0 modes (none for the smallest): it eliminates the included ones
+// from the root in shared memory, and then grows the remaining nsub modes' tree there,
+// breadth first.  A level takes two phases shared out among all threads: the rows, then
+// the entries together with the next level's pivots (a child's three pivot entries are
+// formed twice, which takes the pivots' long chain off the path).  Two threads per node
+// with two modes left form its four terms.  The last CTA of a tree to finish adds the
+// CTAs' sums (exact integers: in any order) and finishes the result.
+struct FxSmall {
+  long long first;  // first CTA (and partial sum) of this tree
+  long long root_off;
+  double logdet;
+  int n, d0, tree, pad;
+};
+
+// Shared memory in words: root, the nsub-mode tree's levels, s of its nodes, pivots and
+// rows of the widest level.
+__host__ __device__ constexpr int fx_small_words(int n, int nsub, int L, int LS) {
+  const int D = nsub > 2 ? nsub - 2 : 0;
+  int words = sym(2 * n) * L + (1 << D) * LS, rows = nsub < n ? 2 * n : 0;
+  for (int k = 0; k < D; ++k) {
+    words += (1 << k) * sym(2 * (nsub - 1 - k)) * L;
+    const int r = (1 << k) * 2 * (nsub - 1 - k);
+    rows = r > rows ? r : rows;
+  }
+  return words + (D > 0 ? (1 << (D - 1)) : 1) * (6 * L + 1) + rows * 6 * L;
+}
+
+// One side of a two-mode node (fx_leaf2): the subsets with (side 0) or without its
+// first mode.
+template <class E, class S>
+__device__ __forceinline__ bool fx_leaf2_side(const uint32_t* m, int o, const S& s, uint32_t neg, int side,
+                                              FxSums<S>& acc) {
+  constexpr int W = sizeof(E) / 4;
+  const uint32_t* m2 = m + tri(o + 2, o) * W;
+  const uint32_t* m3 = m + tri(o + 3, o) * W;
+  E p00 = fx_ld<E, 1>(m2, 2), p10 = fx_ld<E, 1>(m3, 2), p11 = fx_ld<E, 1>(m3, 3);
+  S sv = s;
+  bool ok = true;
+  if (side == 0) {
+    FxPivot<E> pv;
+    ok = fx_pivot(fx_ld<E, 1>(m, tri(o, o)), fx_ld<E, 1>(m, tri(o + 1, o)), fx_ld<E, 1>(m, tri(o + 1, o + 1)), pv);
+    FxRow<E> r0, r1;
+    fx_row(pv, fx_ld<E, 1>(m2, 0), fx_ld<E, 1>(m2, 1), r0);
+    fx_row(pv, fx_ld<E, 1>(m3, 0), fx_ld<E, 1>(m3, 1), r1);
+    p00 = fx_entry(p00, r0.P, r0.Q, r0.A, r0.U, r0.V, r0.B);
+    p10 = fx_entry(p10, r1.P, r1.Q, r1.A, r0.U, r0.V, r0.B);
+    p11 = fx_entry(p11, r1.P, r1.Q, r1.A, r1.U, r1.V, r1.B);
+    sv = umul(s, pv.g);
+  }
+  return fx_leaf1(p00, p10, p11, sv, neg ^ (0u - (uint32_t)side), acc) && ok;
+}
+
+template <class E>
+__global__ void __launch_bounds__(512) fx_small_kernel(const FxSmall* __restrict__ trees, int ntrees,
+                                                       const double* __restrict__ roots, double u, double extra,
+                                                       FxPart<typename fx_sum<E>::type>* __restrict__ parts,
+                                                       int* __restrict__ counts, int* __restrict__ status,
+                                                       ProbOut* __restrict__ out) {
+  typedef typename fx_sum<E>::type S;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int lo = 0, hi = ntrees - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (trees[mid].first <= (long long)blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  const FxSmall t = trees[lo];
+  const unsigned pre = (unsigned)((long long)blockIdx.x - t.first);
+  const int n = t.n, ns = n - t.d0, D = ns > 2 ? ns - 2 : 0, nthr = blockDim.x;
+  E* mats = reinterpret_cast<E*>(smem_raw);
+  __shared__ int lvl[16];  // entries before level k (the root first)
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    int o = sym(2 * n);
+    for (int k = 0; k <= D; ++k) {
+      lvl[k] = o;
+      o += (1 << k) * sym(2 * (ns - 1 - k));
+    }
+  }
+  for (int i = threadIdx.x; i < sym(2 * n); i += nthr) mats[i] = fx_of<E>(roots[t.root_off + i]);
+  __syncthreads();
+  S* sv = reinterpret_cast<S*>(mats + lvl[D]);
+  FxPivot<E>* piv = reinterpret_cast<FxPivot<E>*>(sv + (1 << D));
+  FxRow<E>* rows = reinterpret_cast<FxRow<E>*>(piv + (D > 0 ? 1 << (D - 1) : 1));
+  auto untri = [](int e, int& a, int& b) {
+    a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+    while (a * (a + 1) / 2 > e) --a;
+    while ((a + 1) * (a + 2) / 2 <= e) ++a;
+    b = e - a * (a + 1) / 2;
+  };
+  bool ok = true;
+  // ---- the included modes among the first d0
+  S s0 = fx_of<S>(1.0);
+  for (unsigned left = pre; left; left &= left - 1u) {
+    const int o = 2 * (__ffs((int)left) - 1), R = 2 * n - o - 2;
+    if (threadIdx.x < 32) {
+      FxPivot<E> pv;
+      ok &= fx_pivot(mats[tri(o, o)], mats[tri(o + 1, o)], mats[tri(o + 1, o + 1)], pv);
+      s0 = umul(s0, pv.g);
+      if (threadIdx.x == 0) piv[0] = pv;
+    }
+    __syncthreads();
+    for (int a = threadIdx.x; a < R; a += nthr) fx_row(piv[0], mats[tri(a + o + 2, o)], mats[tri(a + o + 2, o + 1)], rows[a]);
+    __syncthreads();
+    for (int e = threadIdx.x; e < sym(R); e += nthr) {
+      int a, b;
+      untri(e, a, b);
+      E& c = mats[tri(a + o + 2, b + o + 2)];
+      c = fx_entry(c, rows[a].P, rows[a].Q, rows[a].A, rows[b].U, rows[b].V, rows[b].B);
+    }
+    __syncthreads();
+  }
+  // ---- the tree of the other ns modes: node v's matrix, and the first row of its
+  // view with q modes
+  auto node = [&](int v, int q, int& o) {
+    int p = n;
+    E* m = mats;
+    if (v > 0) {
+      const int k = 31 - __clz(v);
+      p = ns - 1 - k;
+      m = mats + lvl[k] + (v - (1 << k)) * sym(2 * p);
+    }
+    o = 2 * (p - q);
+    return m;
+  };
+  if (threadIdx.x == 0) {
+    sv[0] = s0;
+    if (D > 0) {
+      int o;
+      const E* m = node(0, ns, o);
+      FxPivot<E> pv;
+      ok &= fx_pivot(m[tri(o, o)], m[tri(o + 1, o)], m[tri(o + 1, o + 1)], pv);
+      sv[1] = umul(s0, pv.g);
+      piv[0] = pv;
+    }
+  }
+  __syncthreads();
+  for (int k = 0; k < D; ++k) {
+    const int q = ns - 1 - k, R = 2 * q, nc = 1 << k;
+    for (int i = threadIdx.x; i < nc * R; i += nthr) {
+      const int c = i / R, a = i - c * R;
+      int o;
+      const E* m = node(c, q + 1, o);
+      fx_row(piv[c], m[tri(o + 2 + a, o)], m[tri(o + 2 + a, o + 1)], rows[i]);
+    }
+    __syncthreads();
+    // the next level's pivots (nodes 0 .. 2 nc - 1 at depth k + 1) by the first threads
+    const int np = k + 1 < D ? 2 * nc : 0;
+    for (int v = threadIdx.x; v < np; v += nthr) {
+      int o;
+      FxPivot<E> pv;
+      if (v < nc) {
+        const E* m = node(v, q, o);
+        ok &= fx_pivot(m[tri(o, o)], m[tri(o + 1, o)], m[tri(o + 1, o + 1)], pv);
+      } else {
+        const int c = v - nc;
+        const E* m = node(c, q + 1, o);
+        const FxRow<E>&r0 = rows[c * R], &r1 = rows[c * R + 1];
+        ok &= fx_pivot(fx_entry(m[tri(o + 2, o + 2)], r0.P, r0.Q, r0.A, r0.U, r0.V, r0.B),
+                       fx_entry(m[tri(o + 3, o + 2)], r1.P, r1.Q, r1.A, r0.U, r0.V, r0.B),
+                       fx_entry(m[tri(o + 3, o + 3)], r1.P, r1.Q, r1.A, r1.U, r1.V, r1.B), pv);
+      }
+      piv[v] = pv;
+      sv[2 * nc + v] = umul(sv[v], pv.g);
+    }
+    // and the entries by the others
+    const int ne = sym(R);
+    const int skip = min((np + 31) & ~31, nthr / 2);
+    E* dst = mats + lvl[k];
+    if ((int)threadIdx.x >= skip) {
+      for (int i = threadIdx.x - skip; i < nc * ne; i += nthr - skip) {
+        const int c = i / ne;
+        int a, b, o;
+        untri(i - c * ne, a, b);
+        const E* m = node(c, q + 1, o);
+        const FxRow<E>&ra = rows[c * R + a], &rb = rows[c * R + b];
+        dst[i] = fx_entry(m[tri(o + 2 + a, o + 2) + b], ra.P, ra.Q, ra.A, rb.U, rb.V, rb.B);
+      }
+    }
+    __syncthreads();
+  }
+  const S zero = fx_of<S>(0.0);
+  FxSums<S> acc{zero, zero, zero};
+  const int above = n - (ns < 2 ? 1 : 2) - __popc(pre);  // decided modes but the prefix's included ones
+  if (ns == 1) {
+    if (threadIdx.x == 0) {
+      int o;
+      const uint32_t* m = reinterpret_cast<const uint32_t*>(node(0, 1, o));
+      ok &= fx_leaf1(fx_ld<E, 1>(m, tri(o, o)), fx_ld<E, 1>(m, tri(o + 1, o)), fx_ld<E, 1>(m, tri(o + 1, o + 1)), sv[0],
+                     (above & 1) ? 0xffffffffu : 0u, acc);
+    }
+  } else {
+    for (int i = threadIdx.x; i < (2 << D); i += nthr) {
+      const int v = i & ((1 << D) - 1);
+      const uint32_t odd = ((above - __popc(v)) & 1) ? 0xffffffffu : 0u;
+      int o;
+      const uint32_t* m = reinterpret_cast<const uint32_t*>(node(v, 2, o));
+      ok &= fx_leaf2_side<E>(m, o, sv[v], odd, i >> D, acc);
+    }
+  }
+  if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
+  // ---- sums of the CTA, and of the tree by its last CTA
+  __shared__ FxPart<S> sh[16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto warp_sum = [&]() {
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) {
+      acc.inc = acc.inc + shfl_down(acc.inc, off);
+      acc.exc = acc.exc + shfl_down(acc.exc, off);
+      acc.mag = acc.mag + shfl_down(acc.mag, off);
+    }
+  };
+  warp_sum();
+  if (lane == 0) sh[warp] = FxPart<S>{acc.inc, acc.exc, acc.mag};
+  __threadfence();  // a status set above is out before this CTA counts itself
+  __syncthreads();
+  if (warp != 0) return;
+  const int nw = nthr >> 5;
+  acc.inc = lane < nw ? sh[lane].inc : zero;
+  acc.exc = lane < nw ? sh[lane].exc : zero;
+  acc.mag = lane < nw ? sh[lane].abs : zero;
+  warp_sum();
+  if (t.d0 > 0) {
+    if (lane == 0) {
+      parts[blockIdx.x] = FxPart<S>{acc.inc, acc.exc, acc.mag};
+      __threadfence();
+      last = atomicAdd(counts + t.tree, 1) == (1 << t.d0) - 1;
+    }
+    __syncwarp();
+    if (!last) return;
+    __threadfence();
+    acc.inc = acc.exc = acc.mag = zero;
+    for (int i = lane; i < (1 << t.d0); i += 32) {
+      const volatile uint32_t* w = reinterpret_cast<const volatile uint32_t*>(parts + t.first + i);
+      FxPart<S> q;
+#pragma unroll
+      for (int k = 0; k < (int)(sizeof(S) / 4); ++k) {
+        q.inc.w[k] = w[k];
+        q.exc.w[k] = w[sizeof(S) / 4 + k];
+        q.abs.w[k] = w[2 * (sizeof(S) / 4) + k];
+      }
+      acc.inc = acc.inc + q.inc;
+      acc.exc = acc.exc + q.exc;
+      acc.mag = acc.mag + q.abs;
+    }
+    warp_sum();
+  }
+  if (lane != 0) return;
+  TreeOut o;
+  fx_store3(acc.inc, o.inc);
+  fx_store3(acc.exc, o.exc);
+  o.abs = to_double(acc.mag);
+  out[t.tree] = finish_tree(o, *(volatile int*)(status + t.tree), t.logdet, n, u, extra);
 }
 
 }  // namespace gbs

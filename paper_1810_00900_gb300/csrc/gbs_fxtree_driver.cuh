@@ -18,18 +18,73 @@ inline long long fx_level_words(int n, int k, long long count, int L) {
 }
 
 template <class E>
-gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const void* roots_dev, TreeOut* outs_dev,
-                        int* status_dev, const BatchTune& tune) {
+gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const void* roots_dev, int* status_dev,
+                        const BatchTune& tune, const FxFinish& fin) {
   typedef typename fx_sum<E>::type S;
   constexpr int L = sizeof(E) / 4;
+  // Small trees (fx_small_kernel): one CTA for up to kOne modes, whose levels fit its
+  // shared memory twice over; beyond, a CTA per setting of the first modes, as long as
+  // the CTAs of the whole call stay within two per SM: the other trees' rate counts, and
+  // the levels below serve it better.
+  constexpr int LS = sizeof(S) / 4;
+  constexpr int kOne = fx_small_words(10, 10, L, LS) * 4 <= 220 * 1024 ? 10 : 9;
+  constexpr int kSub = kOne - 1;  // modes of a CTA's own tree where it is one of several
+  long long ctas = 0;
+  for (int i = 0; i < ntrees; ++i) {
+    if (in[i].n < 1 || in[i].n > 32) return set_error(ctx, GBS_EINVAL, "batch tree size out of range");
+    if (in[i].n > kOne) ctas += 1LL << std::min(in[i].n - kSub, 20);
+  }
+  const int small_max = ctas <= 2 * ctx->sm_count ? 32 : kOne;
+  std::vector<int> order;  // the others, largest first: every per-size list below is then a run of trees
+  std::vector<FxSmall> small[2];  // in one CTA, in several
+  int small_n[2] = {0, 0};
+  long long blocks[2] = {0, 0};
+  for (int i = 0; i < ntrees; ++i) {
+    const int n = in[i].n, several = n > kOne ? 1 : 0;
+    if (n > small_max) {
+      order.push_back(i);
+      continue;
+    }
+    const int d0 = several ? n - kSub : 0;
+    small[several].push_back(FxSmall{blocks[several], in[i].root_off, fin.logdet[i], n, d0, i, 0});
+    blocks[several] += 1LL << d0;
+    small_n[several] = std::max(small_n[several], n);
+  }
+  // the timer takes the leaf launches, or the small trees' where there are none
+  auto timer = [&](bool stop) {
+    if (!ctx->timing) return;
+    if (!ctx->leaf_timer.start) {
+      cudaEventCreate(&ctx->leaf_timer.start);
+      cudaEventCreate(&ctx->leaf_timer.stop);
+    }
+    cudaEventRecord(stop ? ctx->leaf_timer.stop : ctx->leaf_timer.start, ctx->stream);
+    if (stop) ctx->leaf_timer.pending = true;
+  };
+  if (order.empty()) timer(false);
+  for (int c = 0; c < 2; ++c) {
+    if (small[c].empty()) continue;
+    const void* d_small = nullptr;
+    gbs_status st;
+    if ((st = stage(ctx, small[c].data(), small[c].size() * sizeof(FxSmall), &d_small)) ||
+        (st = dev_reserve(ctx, ctx->sbuf[1], (size_t)blocks[1] * sizeof(FxPart<S>))))
+      return st;
+    const int smem = fx_small_words(small_n[c], c ? kSub : small_n[c], L, LS) * 4;
+    if ((st = check_cuda(ctx, cudaFuncSetAttribute(fx_small_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                         "small tree smem")))
+      return st;
+    int threads = c || small_n[c] >= 8 ? 512 : small_n[c] >= 6 ? 256 : small_n[c] >= 4 ? 128 : 32;
+    if (blocks[c] > ctx->sm_count) threads = std::min(threads, 256);  // two CTAs per SM
+    fx_small_kernel<E><<<(unsigned)blocks[c], threads, smem, ctx->stream>>>(
+        (const FxSmall*)d_small, (int)small[c].size(), (const double*)roots_dev, fin.u, fin.extra,
+        (FxPart<S>*)ctx->sbuf[1].ptr, fin.counts, status_dev, fin.po);
+    count_launch(ctx);
+    if ((st = check_cuda(ctx, cudaGetLastError(), "small trees"))) return st;
+  }
+  if (order.empty()) timer(true);
+  ntrees = (int)order.size();
   if (ntrees <= 0) return GBS_OK;
   // ---------------- plan
-  // Largest tree first: every per-size list below is then a run of trees.
-  std::vector<int> order(ntrees);
-  for (int i = 0; i < ntrees; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return in[a].n > in[b].n; });
-  for (int i = 0; i < ntrees; ++i)
-    if (in[i].n < 1 || in[i].n > 32) return set_error(ctx, GBS_EINVAL, "batch tree size out of range");
   // Levels per leaf thread.
   const int Qmax = std::max(1, std::min(2, 3 - tune.q_drop));
   const int nmax = in[order[0]].n;
@@ -43,7 +98,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   for (int i = 0; i < ntrees; ++i) {
     const BatchTree& b = in[order[i]];
     Q[i] = std::min(b.n, Qmax);
-    trees[i] = FxTree{b.root_off, 0, b.n, b.n - Q[i], order[i], 34 * i, 0, 0};
+    trees[i] = FxTree{b.root_off, 0, fin.logdet[order[i]], b.n, b.n - Q[i], order[i], 34 * i, 0, 0};
   }
   const int D0 = trees[0].D;
   // A single tree too large for the workspace goes in chunks of 2^cb nodes of depth d0
@@ -141,7 +196,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     size_t at;
   };
   std::vector<Leaf> leaves;
-  std::vector<FxSeg> fin;
+  std::vector<FxSeg> sums;
   long long tiles_total = 0, units_total = 0;
   for (int i = 0; i < ntrees; ++i) tiles_total += ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
   // tiles per warp: one wave of the 16 warps an SM holds
@@ -153,10 +208,10 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     const long long units = (tiles + tpu - 1) / tpu;
     lf.segs.push_back(FxSeg{lf.units, i, tpu});
     lf.units += units;
-    fin.push_back(FxSeg{units_total, i, 0});
+    sums.push_back(FxSeg{units_total, i, 0});
     units_total += units * chunks;
   }
-  fin.push_back(FxSeg{units_total, 0, 0});
+  sums.push_back(FxSeg{units_total, 0, 0});
   // ---------------- memory
   const size_t part_bytes = (size_t)units_total * sizeof(FxPart<S>);
   if (ntrees > 1 && need + part_bytes > cap) {
@@ -172,7 +227,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   const size_t o_trees = blob.put(trees), o_chunked = blob.put(chunked), o_off = blob.put(off), o_top = blob.put(top);
   for (Launch& l : levels) l.at = blob.put(l.segs);
   for (Leaf& l : leaves) l.at = blob.put(l.segs);
-  const size_t o_fin = blob.put(fin);
+  const size_t o_sums = blob.put(sums);
   const unsigned char* plan = nullptr;
   if ((st = stage(ctx, blob.bytes.data(), blob.bytes.size(), (const void**)&plan))) return st;
   uint32_t* nodes = (uint32_t*)ctx->lvl[0].ptr;
@@ -209,13 +264,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   };
   for (const Launch& l : levels)
     if (!l.in_chunk) level(l, 0u);
-  if (ctx->timing) {
-    if (!ctx->leaf_timer.start) {
-      cudaEventCreate(&ctx->leaf_timer.start);
-      cudaEventCreate(&ctx->leaf_timer.stop);
-    }
-    cudaEventRecord(ctx->leaf_timer.start, s);
-  }
+  timer(false);
   for (int h = 0; h < chunks; ++h) {
     for (const Launch& l : levels)
       if (l.in_chunk) level(l, (unsigned)h);
@@ -232,12 +281,10 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
       base += l.units;
     }
   }
-  if (ctx->timing) {
-    cudaEventRecord(ctx->leaf_timer.stop, s);
-    ctx->leaf_timer.pending = true;
-  }
+  timer(true);
   const int final_threads = units_total > 256LL * ntrees ? 1024 : 128;
-  fx_final_kernel<S><<<(unsigned)ntrees, final_threads, 0, s>>>(parts, (const FxSeg*)(plan + o_fin), d_trees, outs_dev);
+  fx_final_kernel<S><<<(unsigned)ntrees, final_threads, 0, s>>>(parts, (const FxSeg*)(plan + o_sums), d_trees, status_dev,
+                                                                    fin.u, fin.extra, fin.po);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "fixed-point batch launch");
 }

@@ -166,18 +166,31 @@ gbs_status batch_dd_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*,
 gbs_status batch_dd_cplx(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
 gbs_status batch_td_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
 gbs_status batch_td_cplx(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_fx_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_fxw_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
 gbs_status batch_fp64p_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_fxn_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
 gbs_status batch_fp32_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
 gbs_status batch_fp32_cplx(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
 
+// Fixed-point trees finish their results on the device: log det (host, per tree), unit
+// and extra terms of the error model, where the results go (device), and a zeroed
+// counter per tree (device).
+struct FxFinish {
+  const double* logdet;
+  double u, extra;
+  ProbOut* po;
+  int* counts;
+};
+gbs_status batch_fxd_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
+gbs_status batch_fxn_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
+gbs_status batch_fx_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
+gbs_status batch_fxw_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
+
 // Evaluate ntrees trees whose packed FP64 roots are already in roots_dev
 // (entries at trees[t].root_off); logdet[t] (host) scales p = Tor exp(-logdet/2).
-// Synchronous: fills host_out[0..ntrees).  (gbs_batch_api.cu)
+// Synchronous: fills host_out[0..ntrees).  bounded: FP64 trees in the real basis whose
+// values the caller knows to fit 64-bit fixed point (fxd_ok_*); they run on the integer
+// pipe, and again in floating point if one leaves its range.  (gbs_batch_api.cu)
 gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const BatchTree* trees, const void* roots_dev,
-                      const double* logdet, ProbOut* host_out);
+                      const double* logdet, ProbOut* host_out, bool bounded = false);
 // The tuning in force for (prec, basis) -- the autotuner's choice when one was made.
 const BatchTune& batch_tune_for(gbs_ctx* ctx, int prec, bool real);
 
@@ -213,6 +226,10 @@ double unit_of(int prec);
 // (Sigma^-1)_S, resp. of a conditioned Sigma', keeps every value in range.
 bool fx_ok_inverse(const gbs_state* st, int n);
 bool fx_ok_sigma(const gbs_state* st, int n);
+// The same for FP64 trees in 64-bit fixed point, which must also be at least as
+// accurate there as in FP64.
+bool fxd_ok_inverse(const gbs_state* st, int n);
+bool fxd_ok_sigma(const gbs_state* st, int n);
 
 // Error model of a subset tree over n modes in precision prec: |dTor| <=
 // err_factor * unit * sum|terms|, with 4 n units per term (n rank-2 Schur steps

@@ -384,17 +384,23 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
     if ((e = stage(ctx, gi.data(), gi.size() * sizeof(GatherItem), &dgi))) return e;
     gather_kernel<<<(unsigned)gi.size(), 128, 0, ctx->stream>>>((const GatherItem*)dgi, (double*)ctx->hbuf.ptr);
     count_launch(ctx);
-    for (int pv : {GBS_PREC_FP64, GBS_PREC_DD, GBS_PREC_FXN, GBS_PREC_FX, GBS_PREC_FXW, GBS_PREC_TD}) {
+    // FP64 trees that their states bound run in 64-bit fixed point, apart from the others
+    for (int pass = 0; pass < 7; ++pass) {
+      const int order[7] = {GBS_PREC_FP64, GBS_PREC_FP64, GBS_PREC_DD, GBS_PREC_FXN, GBS_PREC_FX, GBS_PREC_FXW, GBS_PREC_TD};
+      const int pv = order[pass];
+      const bool bounded = pass == 0;
       std::vector<size_t> grp;
       for (size_t i : todo)
-        if (trees[i].prec == pv && trees[i].n > 0) grp.push_back(i);
+        if (trees[i].prec == pv && trees[i].n > 0 &&
+            (pv != GBS_PREC_FP64 || fxd_ok_sigma(trees[i].tj->st, trees[i].n) == bounded))
+          grp.push_back(i);
       if (grp.empty()) continue;
       std::vector<BatchTree> sub(grp.size());
       std::vector<double> zero(grp.size(), 0.0);
       for (size_t j = 0; j < grp.size(); ++j) sub[j] = BatchTree{trees[grp[j]].n, trees[grp[j]].root_off};
       std::vector<ProbOut> r(grp.size());
       const auto tb = std::chrono::steady_clock::now();
-      if ((e = batch_eval(ctx, pv, true, (int)grp.size(), sub.data(), ctx->hbuf.ptr, zero.data(), r.data())))
+      if ((e = batch_eval(ctx, pv, true, (int)grp.size(), sub.data(), ctx->hbuf.ptr, zero.data(), r.data(), bounded)))
         return e;
       stt.tree_seconds[stat_slot(pv)] += std::chrono::duration<double>(std::chrono::steady_clock::now() - tb).count();
       stt.trees[stat_slot(pv)] += (long long)grp.size();

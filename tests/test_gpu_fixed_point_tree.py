@@ -58,12 +58,47 @@ def test_uneven_batch_gives_each_trees_own_bits(ctx):
     st.free()
 
 
+@pytest.mark.parametrize("prec", ["fp64", "fxn", "fx", "fxw"])
+def test_one_launch_and_level_paths_agree(ctx, prec):
+    # alone, trees of up to 16 modes take one launch (one CTA up to 9 or 10 modes, several
+    # beyond); among enough others they go by levels: the same bits
+    st_p = gi.uniform_squeezed_state(60, 0.7, seed=5, eta=0.7)
+    st = gbs.build_state(ctx, st_p.U, st_p.r, st_p.eta)
+    pats = [gi.random_modes(60, n, seed=300 + n) for n in range(1, 17)]
+    many = pats + [gi.random_modes(60, 12, seed=400 + i) for i in range(120)]
+    for p, b in zip(pats, gbs.torontonian_batch(ctx, [st] * len(many), many, prec)):
+        a = gbs.torontonian(ctx, st, p, prec)
+        assert a.tor == b.tor and a.abs_sum == b.abs_sum and a.p == b.p, len(p)
+    st.free()
+
+
+@pytest.mark.parametrize("n", [3, 8, 10, 11, 13, 17])
+def test_fp64_of_a_bounded_state_is_no_worse_than_its_estimate(ctx, n):
+    # FP64 trees of bounded states run in 64-bit fixed point; bright states, where FP64 carries
+    # the cancellation: within the FP64 error model of the exact value of the same block, and
+    # as close to it as the FP64 pipe's own tree (gbs_subset_sum on the block) or 1e-13
+    st_p = gi.uniform_squeezed_state(n + 1, 1.4, seed=60 + n, eta=0.9)
+    st = gbs.build_state(ctx, st_p.U, st_p.r, st_p.eta)
+    modes = gi.random_modes(n + 1, n, seed=n)
+    G = gbs.sigma_inv_block(ctx, st, modes, "real")
+    ref, ref_abs = oracle_tor(G)
+    want = float(ref.to_fraction())
+    pr = gbs.torontonian(ctx, st, modes, "fp64", "real")
+    err = abs(float(frac3(pr.tor) - ref.to_fraction()))
+    assert err <= (4 * n + 24) * 2.0 ** -53 * ref_abs
+    _, _, tor, _ = gbs.subset_sum(ctx, G, "real", "fp64")
+    assert err <= max(abs(float(frac3(tor) - ref.to_fraction())), 1e-13 * abs(want))
+    assert abs(pr.abs_sum - ref_abs) <= 1e-12 * ref_abs
+    st.free()
+
+
 @pytest.mark.parametrize("prec", ["fxn", "fx", "fxw"])
 def test_chunks_of_a_tree_beyond_the_budget(ctx, prec):
-    # 16 modes need ~10 MB of levels at once; half of a budget of 6 and 10 MB makes chunks
-    G = block(16, 77)
+    # 18 modes (beyond the trees that run in one launch) need ~40 MB of levels at once; half
+    # of a budget of 24 and 40 MB makes chunks
+    G = block(18, 77)
     want = gbs.subset_sum(ctx, G, "real", prec)
-    for budget in (6 << 20, 10 << 20):
+    for budget in (24 << 20, 40 << 20):
         for d_top in (6, 10):
             c = gbs.Context(0, hbm_budget_bytes=budget)
             c.set_tuning(prec, "real", 6, d_top, 0, 1 << 18, 0, 0)
