@@ -430,4 +430,12 @@ __device__ __forceinline__ fxn<L, F> shfl_down(const fxn<L, F>& v, int off) {
   return r;
 }
 
+template <int L, int F>
+__device__ __forceinline__ fxn<L, F> shfl_xor(const fxn<L, F>& v, int mask) {
+  fxn<L, F> r;
+#pragma unroll
+  for (int k = 0; k < L; ++k) r.w[k] = __shfl_xor_sync(0xffffffffu, v.w[k], mask);
+  return r;
+}
+
 }  // namespace gbs

@@ -693,6 +693,12 @@ struct FxSmall {
   int n, d0, tree, pad;
 };
 
+// A row in shared memory, an odd number of words long (6 L is even).
+template <class E>
+struct FxRowPad : FxRow<E> {
+  uint32_t pad;
+};
+
 // Shared memory in words: root, the nsub-mode tree's levels, s of its nodes, pivots and
 // rows of the widest level.
 __host__ __device__ constexpr int fx_small_words(int n, int nsub, int L, int LS) {
@@ -703,53 +709,100 @@ __host__ __device__ constexpr int fx_small_words(int n, int nsub, int L, int LS)
     const int r = (1 << k) * 2 * (nsub - 1 - k);
     rows = r > rows ? r : rows;
   }
-  return words + (D > 0 ? (1 << (D - 1)) : 1) * (6 * L + 1) + rows * 6 * L;
+  return words + (D > 0 ? (1 << (D - 1)) : 1) * (6 * L + 1) + rows * (6 * L + 1);
 }
 
-// One side of a two-mode node (fx_leaf2): the subsets with (side 0) or without its
-// first mode.
-template <class E, class S>
-__device__ __forceinline__ bool fx_leaf2_side(const uint32_t* m, int o, const S& s, uint32_t neg, int side,
-                                              FxSums<S>& acc) {
-  constexpr int W = sizeof(E) / 4;
-  const uint32_t* m2 = m + tri(o + 2, o) * W;
-  const uint32_t* m3 = m + tri(o + 3, o) * W;
-  E p00 = fx_ld<E, 1>(m2, 2), p10 = fx_ld<E, 1>(m3, 2), p11 = fx_ld<E, 1>(m3, 3);
-  S sv = s;
-  bool ok = true;
-  if (side == 0) {
-    FxPivot<E> pv;
-    ok = fx_pivot(fx_ld<E, 1>(m, tri(o, o)), fx_ld<E, 1>(m, tri(o + 1, o)), fx_ld<E, 1>(m, tri(o + 1, o + 1)), pv);
-    FxRow<E> r0, r1;
-    fx_row(pv, fx_ld<E, 1>(m2, 0), fx_ld<E, 1>(m2, 1), r0);
-    fx_row(pv, fx_ld<E, 1>(m3, 0), fx_ld<E, 1>(m3, 1), r1);
-    p00 = fx_entry(p00, r0.P, r0.Q, r0.A, r0.U, r0.V, r0.B);
-    p10 = fx_entry(p10, r1.P, r1.Q, r1.A, r0.U, r0.V, r0.B);
-    p11 = fx_entry(p11, r1.P, r1.Q, r1.A, r1.U, r1.V, r1.B);
-    sv = umul(s, pv.g);
-  }
-  return fx_leaf1(p00, p10, p11, sv, neg ^ (0u - (uint32_t)side), acc) && ok;
-}
-
+// The operations on values in memory, inlined (CALL = false) or as functions of their
+// own.  A kernel that holds one type's tree inlines them; one that holds four (the
+// sampler's chain) calls them, or the instruction caches thrash: graph sampling of 100
+// modes 45 ms with calls, 53 without; a tree of 9 modes alone (128 fraction bits) 33 us
+// with, 27 without.
 template <class E>
-__global__ void __launch_bounds__(512) fx_small_kernel(const FxSmall* __restrict__ trees, int ntrees,
-                                                       const double* __restrict__ roots, double u, double extra,
-                                                       FxPart<typename fx_sum<E>::type>* __restrict__ parts,
-                                                       int* __restrict__ counts, int* __restrict__ status,
-                                                       ProbOut* __restrict__ out) {
+__device__ __forceinline__ bool fxm_pivot(const E* p00, const E* p10, const E* p11, FxPivot<E>* pv) {
+  FxPivot<E> r;
+  const bool ok = fx_pivot(*p00, *p10, *p11, r);
+  *pv = r;
+  return ok;
+}
+template <class E>
+__device__ __forceinline__ void fxm_row(const FxPivot<E>* pv, const E* u0, const E* u1, FxRow<E>* out) {
+  FxRow<E> r;
+  fx_row(*pv, *u0, *u1, r);
+  *out = r;
+}
+template <class E>
+__device__ __forceinline__ void fxm_entry(const E* c, const FxRow<E>* a, const FxRow<E>* b, E* out) {
+  *out = fx_entry(*c, a->P, a->Q, a->A, b->U, b->V, b->B);
+}
+template <class E, class S>
+__device__ __forceinline__ bool fxm_leaf1(const E* p00, const E* p10, const E* p11, const S* s, uint32_t neg,
+                                          FxSums<S>* acc) {
+  FxSums<S> t = *acc;
+  const bool ok = fx_leaf1(*p00, *p10, *p11, *s, neg, t);
+  *acc = t;
+  return ok;
+}
+template <class E>
+__device__ __noinline__ bool fxc_pivot(const E* p00, const E* p10, const E* p11, FxPivot<E>* pv) {
+  return fxm_pivot(p00, p10, p11, pv);
+}
+template <class E>
+__device__ __noinline__ void fxc_row(const FxPivot<E>* pv, const E* u0, const E* u1, FxRow<E>* out) {
+  fxm_row(pv, u0, u1, out);
+}
+template <class E>
+__device__ __noinline__ void fxc_entry(const E* c, const FxRow<E>* a, const FxRow<E>* b, E* out) {
+  fxm_entry(c, a, b, out);
+}
+template <class E, class S>
+__device__ __noinline__ bool fxc_leaf1(const E* p00, const E* p10, const E* p11, const S* s, uint32_t neg,
+                                       FxSums<S>* acc) {
+  return fxm_leaf1(p00, p10, p11, s, neg, acc);
+}
+template <class E, bool CALL>
+struct FxOps {
   typedef typename fx_sum<E>::type S;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  int lo = 0, hi = ntrees - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (trees[mid].first <= (long long)blockIdx.x) lo = mid; else hi = mid - 1;
+  static __device__ __forceinline__ bool pivot(const E* p00, const E* p10, const E* p11, FxPivot<E>* pv) {
+    if constexpr (CALL) return fxc_pivot(p00, p10, p11, pv); else return fxm_pivot(p00, p10, p11, pv);
   }
-  const FxSmall t = trees[lo];
-  const unsigned pre = (unsigned)((long long)blockIdx.x - t.first);
-  const int n = t.n, ns = n - t.d0, D = ns > 2 ? ns - 2 : 0, nthr = blockDim.x;
-  E* mats = reinterpret_cast<E*>(smem_raw);
-  __shared__ int lvl[16];  // entries before level k (the root first)
-  __shared__ int last;
+  static __device__ __forceinline__ void row(const FxPivot<E>* pv, const E* u0, const E* u1, FxRow<E>* out) {
+    if constexpr (CALL) fxc_row(pv, u0, u1, out); else fxm_row(pv, u0, u1, out);
+  }
+  static __device__ __forceinline__ void entry(const E* c, const FxRow<E>* a, const FxRow<E>* b, E* out) {
+    if constexpr (CALL) fxc_entry(c, a, b, out); else fxm_entry(c, a, b, out);
+  }
+  static __device__ __forceinline__ bool leaf1(const E* p00, const E* p10, const E* p11, const S* s, uint32_t neg,
+                                               FxSums<S>* acc) {
+    if constexpr (CALL) return fxc_leaf1(p00, p10, p11, s, neg, acc); else return fxm_leaf1(p00, p10, p11, s, neg, acc);
+  }
+};
+
+// Sum over a warp; every lane gets it.
+template <class S>
+__device__ __forceinline__ void fx_warp_sum(FxSums<S>& acc) {
+#pragma unroll 1
+  for (int off = 16; off > 0; off >>= 1) {
+    acc.inc = acc.inc + shfl_xor(acc.inc, off);
+    acc.exc = acc.exc + shfl_xor(acc.exc, off);
+    acc.mag = acc.mag + shfl_xor(acc.mag, off);
+  }
+}
+
+// The tree of a CTA: the n-mode root (root(i): entry i of its packed triangle) with the
+// first d0 modes set to pre, all other subsets enumerated.  Returns the CTA's sums in
+// its first warp (every lane); ok turns false in the threads that met a pivot out of
+// range.  Ends without a barrier: one is needed before smem is used again.
+template <class E, bool CALL, class Root>
+__device__ __forceinline__ FxPart<typename fx_sum<E>::type> fx_cta_tree(unsigned char* smem, int n, int d0, unsigned pre,
+                                                                        const Root& root, bool& ok) {
+  typedef typename fx_sum<E>::type S;
+  typedef FxOps<E, CALL> Op;
+  const int ns = n - d0, D = ns > 2 ? ns - 2 : 0, nthr = blockDim.x;
+  E* mats = reinterpret_cast<E*>(smem);
+  __shared__ int lvl[16];           // entries before level k (the root first)
+  __shared__ uint16_t tab[595];     // packed entry -> (row, column), sym(34) of them
+  __shared__ int base[256];         // node -> first entry of its matrix
+  __shared__ unsigned char held[256];  // node -> modes of its matrix
   if (threadIdx.x == 0) {
     int o = sym(2 * n);
     for (int k = 0; k <= D; ++k) {
@@ -757,104 +810,93 @@ __global__ void __launch_bounds__(512) fx_small_kernel(const FxSmall* __restrict
       o += (1 << k) * sym(2 * (ns - 1 - k));
     }
   }
-  for (int i = threadIdx.x; i < sym(2 * n); i += nthr) mats[i] = fx_of<E>(roots[t.root_off + i]);
+  for (int i = threadIdx.x; i < sym(2 * n); i += nthr) {
+    mats[i] = fx_of<E>(root(i));
+    int a = (int)((sqrtf(8.0f * (float)i + 1.0f) - 1.0f) * 0.5f);
+    while (a * (a + 1) / 2 > i) --a;
+    while ((a + 1) * (a + 2) / 2 <= i) ++a;
+    tab[i] = (uint16_t)(a << 8 | (i - a * (a + 1) / 2));
+  }
   __syncthreads();
+  for (int v = threadIdx.x; v < (1 << D); v += nthr) {
+    const int k = 31 - __clz(v | 1), p = v ? ns - 1 - k : n;
+    base[v] = v ? lvl[k] + (v - (1 << k)) * sym(2 * p) : 0;
+    held[v] = (unsigned char)p;
+  }
   S* sv = reinterpret_cast<S*>(mats + lvl[D]);
   FxPivot<E>* piv = reinterpret_cast<FxPivot<E>*>(sv + (1 << D));
-  FxRow<E>* rows = reinterpret_cast<FxRow<E>*>(piv + (D > 0 ? 1 << (D - 1) : 1));
-  auto untri = [](int e, int& a, int& b) {
-    a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-    while (a * (a + 1) / 2 > e) --a;
-    while ((a + 1) * (a + 2) / 2 <= e) ++a;
-    b = e - a * (a + 1) / 2;
-  };
-  bool ok = true;
+  FxRowPad<E>* rows = reinterpret_cast<FxRowPad<E>*>(piv + (D > 0 ? 1 << (D - 1) : 1));
   // ---- the included modes among the first d0
-  S s0 = fx_of<S>(1.0);
+  if (threadIdx.x == 0) sv[0] = fx_of<S>(1.0);
   for (unsigned left = pre; left; left &= left - 1u) {
     const int o = 2 * (__ffs((int)left) - 1), R = 2 * n - o - 2;
-    if (threadIdx.x < 32) {
-      FxPivot<E> pv;
-      ok &= fx_pivot(mats[tri(o, o)], mats[tri(o + 1, o)], mats[tri(o + 1, o + 1)], pv);
-      s0 = umul(s0, pv.g);
-      if (threadIdx.x == 0) piv[0] = pv;
+    if (threadIdx.x == 0) {
+      ok &= Op::pivot(mats + tri(o, o), mats + tri(o + 1, o), mats + tri(o + 1, o + 1), piv);
+      sv[0] = umul(sv[0], piv[0].g);
     }
     __syncthreads();
-    for (int a = threadIdx.x; a < R; a += nthr) fx_row(piv[0], mats[tri(a + o + 2, o)], mats[tri(a + o + 2, o + 1)], rows[a]);
+    for (int a = threadIdx.x; a < R; a += nthr) {
+      const E* m = mats + tri(a + o + 2, o);
+      Op::row(piv, m, m + 1, rows + a);
+    }
     __syncthreads();
     for (int e = threadIdx.x; e < sym(R); e += nthr) {
-      int a, b;
-      untri(e, a, b);
-      E& c = mats[tri(a + o + 2, b + o + 2)];
-      c = fx_entry(c, rows[a].P, rows[a].Q, rows[a].A, rows[b].U, rows[b].V, rows[b].B);
+      const int a = tab[e] >> 8, b = tab[e] & 255;
+      E* c = mats + tri(a + o + 2, b + o + 2);
+      Op::entry(c, rows + a, rows + b, c);
     }
     __syncthreads();
   }
   // ---- the tree of the other ns modes: node v's matrix, and the first row of its
   // view with q modes
   auto node = [&](int v, int q, int& o) {
-    int p = n;
-    E* m = mats;
-    if (v > 0) {
-      const int k = 31 - __clz(v);
-      p = ns - 1 - k;
-      m = mats + lvl[k] + (v - (1 << k)) * sym(2 * p);
-    }
-    o = 2 * (p - q);
-    return m;
+    o = 2 * ((int)held[v] - q);
+    return mats + base[v];
   };
-  if (threadIdx.x == 0) {
-    sv[0] = s0;
-    if (D > 0) {
-      int o;
-      const E* m = node(0, ns, o);
-      FxPivot<E> pv;
-      ok &= fx_pivot(m[tri(o, o)], m[tri(o + 1, o)], m[tri(o + 1, o + 1)], pv);
-      sv[1] = umul(s0, pv.g);
-      piv[0] = pv;
-    }
-  }
-  __syncthreads();
-  for (int k = 0; k < D; ++k) {
-    const int q = ns - 1 - k, R = 2 * q, nc = 1 << k;
+  // level -1: the pivot of node 0; level k: its rows, then its entries together with the
+  // pivots of nodes 0 .. 2^(k+1) - 1 at depth k + 1, by the first threads, which form the
+  // pivot entries of the new ones themselves
+  for (int k = -1; k < D; ++k) {
+    const int q = ns - 1 - k, R = 2 * q, nc = k < 0 ? 0 : 1 << k;
+    const float inv_r = 1.0f / (float)R;
     for (int i = threadIdx.x; i < nc * R; i += nthr) {
-      const int c = i / R, a = i - c * R;
+      const int c = (int)(((float)i + 0.5f) * inv_r), a = i - c * R;  // exact: i < 2^10
       int o;
-      const E* m = node(c, q + 1, o);
-      fx_row(piv[c], m[tri(o + 2 + a, o)], m[tri(o + 2 + a, o + 1)], rows[i]);
+      const E* m = node(c, q + 1, o) + tri(o + 2 + a, o);
+      Op::row(piv + c, m, m + 1, rows + i);
     }
     __syncthreads();
-    // the next level's pivots (nodes 0 .. 2 nc - 1 at depth k + 1) by the first threads
-    const int np = k + 1 < D ? 2 * nc : 0;
-    for (int v = threadIdx.x; v < np; v += nthr) {
-      int o;
-      FxPivot<E> pv;
-      if (v < nc) {
-        const E* m = node(v, q, o);
-        ok &= fx_pivot(m[tri(o, o)], m[tri(o + 1, o)], m[tri(o + 1, o + 1)], pv);
-      } else {
-        const int c = v - nc;
-        const E* m = node(c, q + 1, o);
-        const FxRow<E>&r0 = rows[c * R], &r1 = rows[c * R + 1];
-        ok &= fx_pivot(fx_entry(m[tri(o + 2, o + 2)], r0.P, r0.Q, r0.A, r0.U, r0.V, r0.B),
-                       fx_entry(m[tri(o + 3, o + 2)], r1.P, r1.Q, r1.A, r0.U, r0.V, r0.B),
-                       fx_entry(m[tri(o + 3, o + 3)], r1.P, r1.Q, r1.A, r1.U, r1.V, r1.B), pv);
-      }
-      piv[v] = pv;
-      sv[2 * nc + v] = umul(sv[v], pv.g);
-    }
-    // and the entries by the others
-    const int ne = sym(R);
+    const int np = k + 1 < D ? max(2 * nc, 1) : 0, ne = sym(R);
     const int skip = min((np + 31) & ~31, nthr / 2);
-    E* dst = mats + lvl[k];
-    if ((int)threadIdx.x >= skip) {
-      for (int i = threadIdx.x - skip; i < nc * ne; i += nthr - skip) {
-        const int c = i / ne;
-        int a, b, o;
-        untri(i - c * ne, a, b);
-        const E* m = node(c, q + 1, o);
-        const FxRow<E>&ra = rows[c * R + a], &rb = rows[c * R + b];
-        dst[i] = fx_entry(m[tri(o + 2 + a, o + 2) + b], ra.P, ra.Q, ra.A, rb.U, rb.V, rb.B);
+    const float inv_e = 1.0f / (float)ne;
+    E* dst = mats + lvl[max(k, 0)];
+    auto entry = [&](int c, int e) {
+      const int ab = tab[e], a = ab >> 8, b = ab & 255;
+      int o;
+      const E* m = node(c, q + 1, o);
+      Op::entry(m + tri(o + 2 + a, o + 2) + b, rows + c * R + a, rows + c * R + b, dst + c * ne + e);
+    };
+    // entries e >= first of a child are the other threads'
+    const int first = np ? 3 : 0, per = ne - first;
+    const float inv_p = 1.0f / (float)per;
+    const bool pivots = (int)threadIdx.x < skip;
+    for (int v = pivots || np > skip ? threadIdx.x : np; v < np; v += nthr) {
+      int o = 0;
+      const E* m;
+      if (v < nc || k < 0) {
+        m = node(v, q, o);
+      } else {
+#pragma unroll 1
+        for (int e = 0; e < 3; ++e) entry(v - nc, e);
+        m = dst + (v - nc) * ne;
+      }
+      ok &= Op::pivot(m + tri(o, o), m + tri(o + 1, o), m + tri(o + 1, o + 1), piv + v);
+      sv[max(2 * nc, 1) + v] = umul(sv[v], piv[v].g);
+    }
+    if (!pivots) {
+      for (int i = threadIdx.x - skip; i < nc * per; i += nthr - skip) {
+        const int c = (int)(((float)i + 0.5f) * inv_p);  // exact: i < 2^11
+        entry(c, i - c * per + first);
       }
     }
     __syncthreads();
@@ -865,51 +907,90 @@ __global__ void __launch_bounds__(512) fx_small_kernel(const FxSmall* __restrict
   if (ns == 1) {
     if (threadIdx.x == 0) {
       int o;
-      const uint32_t* m = reinterpret_cast<const uint32_t*>(node(0, 1, o));
-      ok &= fx_leaf1(fx_ld<E, 1>(m, tri(o, o)), fx_ld<E, 1>(m, tri(o + 1, o)), fx_ld<E, 1>(m, tri(o + 1, o + 1)), sv[0],
-                     (above & 1) ? 0xffffffffu : 0u, acc);
+      const E* m = node(0, 1, o);
+      ok &= Op::leaf1(m + tri(o, o), m + tri(o + 1, o), m + tri(o + 1, o + 1), sv, (above & 1) ? 0xffffffffu : 0u, &acc);
     }
   } else {
+    // two threads per two-mode node: the subsets with its first mode, and those without
     for (int i = threadIdx.x; i < (2 << D); i += nthr) {
-      const int v = i & ((1 << D) - 1);
-      const uint32_t odd = ((above - __popc(v)) & 1) ? 0xffffffffu : 0u;
+      const int v = i & ((1 << D) - 1), side = i >> D;
+      const uint32_t neg = ((above - __popc(v) - side) & 1) ? 0xffffffffu : 0u;
       int o;
-      const uint32_t* m = reinterpret_cast<const uint32_t*>(node(v, 2, o));
-      ok &= fx_leaf2_side<E>(m, o, sv[v], odd, i >> D, acc);
+      const E* m = node(v, 2, o);
+      const E *m2 = m + tri(o + 2, o), *m3 = m + tri(o + 3, o);
+      const E *p00 = m2 + 2, *p10 = m3 + 2, *p11 = m3 + 3;
+      const S* s = sv + v;
+      E p[3];
+      S sg;
+      if (side == 0) {
+        FxPivot<E> pv;
+        FxRow<E> r0, r1;
+        ok &= Op::pivot(m + tri(o, o), m + tri(o + 1, o), m + tri(o + 1, o + 1), &pv);
+        Op::row(&pv, m2, m2 + 1, &r0);
+        Op::row(&pv, m3, m3 + 1, &r1);
+        Op::entry(p00, &r0, &r0, p);
+        Op::entry(p10, &r1, &r0, p + 1);
+        Op::entry(p11, &r1, &r1, p + 2);
+        sg = umul(*s, pv.g);
+        p00 = p;
+        p10 = p + 1;
+        p11 = p + 2;
+        s = &sg;
+      }
+      ok &= Op::leaf1(p00, p10, p11, s, neg, &acc);
     }
   }
-  if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
-  // ---- sums of the CTA, and of the tree by its last CTA
   __shared__ FxPart<S> sh[16];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto warp_sum = [&]() {
-#pragma unroll 1
-    for (int off = 16; off > 0; off >>= 1) {
-      acc.inc = acc.inc + shfl_down(acc.inc, off);
-      acc.exc = acc.exc + shfl_down(acc.exc, off);
-      acc.mag = acc.mag + shfl_down(acc.mag, off);
-    }
-  };
-  warp_sum();
+  fx_warp_sum(acc);
   if (lane == 0) sh[warp] = FxPart<S>{acc.inc, acc.exc, acc.mag};
-  __threadfence();  // a status set above is out before this CTA counts itself
   __syncthreads();
-  if (warp != 0) return;
-  const int nw = nthr >> 5;
-  acc.inc = lane < nw ? sh[lane].inc : zero;
-  acc.exc = lane < nw ? sh[lane].exc : zero;
-  acc.mag = lane < nw ? sh[lane].abs : zero;
-  warp_sum();
+  if (warp == 0) {
+    const int nw = nthr >> 5;
+    acc.inc = lane < nw ? sh[lane].inc : zero;
+    acc.exc = lane < nw ? sh[lane].exc : zero;
+    acc.mag = lane < nw ? sh[lane].abs : zero;
+    fx_warp_sum(acc);
+  }
+  return FxPart<S>{acc.inc, acc.exc, acc.mag};
+}
+
+template <class E>
+__global__ void __launch_bounds__(512) fx_small_kernel(const FxSmall* __restrict__ trees, int ntrees,
+                                                       const double* __restrict__ roots, double u, double extra,
+                                                       FxPart<typename fx_sum<E>::type>* __restrict__ parts,
+                                                       int* __restrict__ counts, int* __restrict__ status,
+                                                       ProbOut* __restrict__ out) {
+  typedef typename fx_sum<E>::type S;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int last, bad;
+  int lo = 0, hi = ntrees - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (trees[mid].first <= (long long)blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  const FxSmall t = trees[lo];
+  const unsigned pre = (unsigned)((long long)blockIdx.x - t.first);
+  bool ok = true;
+  if (threadIdx.x == 0) bad = 0;
+  FxPart<S> sum = fx_cta_tree<E, false>(smem_raw, t.n, t.d0, pre, [&](int i) { return roots[t.root_off + i]; }, ok);
+  if (!ok) bad = 1;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x >= 32) return;
+  int st = bad ? (int)kStatusRange : (int)kStatusOk;
   if (t.d0 > 0) {
     if (lane == 0) {
-      parts[blockIdx.x] = FxPart<S>{acc.inc, acc.exc, acc.mag};
+      if (bad) atomicExch(status + t.tree, (int)kStatusRange);
+      parts[blockIdx.x] = sum;
       __threadfence();
       last = atomicAdd(counts + t.tree, 1) == (1 << t.d0) - 1;
     }
     __syncwarp();
     if (!last) return;
     __threadfence();
-    acc.inc = acc.exc = acc.mag = zero;
+    const S zero = fx_of<S>(0.0);
+    FxSums<S> acc{zero, zero, zero};
     for (int i = lane; i < (1 << t.d0); i += 32) {
       const volatile uint32_t* w = reinterpret_cast<const volatile uint32_t*>(parts + t.first + i);
       FxPart<S> q;
@@ -923,14 +1004,16 @@ __global__ void __launch_bounds__(512) fx_small_kernel(const FxSmall* __restrict
       acc.exc = acc.exc + q.exc;
       acc.mag = acc.mag + q.abs;
     }
-    warp_sum();
+    fx_warp_sum(acc);
+    sum = FxPart<S>{acc.inc, acc.exc, acc.mag};
+    st = *(volatile int*)(status + t.tree);
   }
   if (lane != 0) return;
   TreeOut o;
-  fx_store3(acc.inc, o.inc);
-  fx_store3(acc.exc, o.exc);
-  o.abs = to_double(acc.mag);
-  out[t.tree] = finish_tree(o, *(volatile int*)(status + t.tree), t.logdet, n, u, extra);
+  fx_store3(sum.inc, o.inc);
+  fx_store3(sum.exc, o.exc);
+  o.abs = to_double(sum.abs);
+  out[t.tree] = finish_tree(o, st, t.logdet, t.n, u, extra);
 }
 
 }  // namespace gbs

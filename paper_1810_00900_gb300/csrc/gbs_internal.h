@@ -13,6 +13,12 @@
 
 namespace gbs {
 
+#ifdef __CUDACC__
+#define GBS_HD_INLINE __host__ __device__ inline
+#else
+#define GBS_HD_INLINE inline
+#endif
+
 // The largest gbs_prec value.
 constexpr int kPrecLast = GBS_PREC_FXN;
 
@@ -215,13 +221,18 @@ struct Trajectory {
   std::vector<int> S;
   double kappa_prev = 1.0, relD = 0.0;
   std::vector<double> p0;
+  bool host_step = false;  // the next step goes through sampler_advance's own path
 };
 size_t traj_bytes(int M);
 void traj_bind(Trajectory& tj, gbs_state* st, unsigned char* mem);
 gbs_status traj_start(gbs_ctx* ctx, Trajectory& tj);
 gbs_status ensure_sigma_real(gbs_ctx* ctx, gbs_state* st);
 gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int prec, gbs_sample_stats& stt);
-double unit_of(int prec);
+// Whether the trajectory's next step can run in the one-CTA chain (gbs_chain.cu), and
+// up to kChainSteps steps of such trajectories.
+constexpr int kChainSteps = 24;
+bool chain_eligible(const Trajectory& t, int prec);
+gbs_status chain_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int prec, gbs_sample_stats& stt);
 // Fixed-point eligibility (gbs_batch_api.cu): a tree over n modes of
 // (Sigma^-1)_S, resp. of a conditioned Sigma', keeps every value in range.
 bool fx_ok_inverse(const gbs_state* st, int n);
@@ -236,9 +247,45 @@ bool fxd_ok_sigma(const gbs_state* st, int n);
 // and one inverse square root) and, for the FP64 family, 24 more for the FP64
 // sums of the non-negative sign-split partials (up to 15 within a thread's
 // register subtree, 5 across a warp, margin for the double-double stages).
-inline double err_factor(int prec, int n) {
+GBS_HD_INLINE double err_factor(int prec, int n) {
   const double base = 4.0 * (n > 1 ? n : 1);
   return (prec == GBS_PREC_FP64 || prec == GBS_PREC_FP64P || prec == GBS_PREC_FP32_DIAG) ? base + 24.0 : base;
+}
+
+// Unit of the error model of a precision.
+GBS_HD_INLINE double unit_of(int prec) {
+  switch (prec) {
+    case GBS_PREC_FP64: return 0x1p-53;
+    case GBS_PREC_DD: return 0x1p-102;
+    case GBS_PREC_FXN: return 0x1p-108;
+    case GBS_PREC_FX: return 0x1p-140;
+    case GBS_PREC_FXW: return 0x1p-158;  // limited by the three-double tree output
+  }
+  return 0x1p-152;
+}
+
+// Sampler: bound on |delta p0|, half the near-tie threshold, so that a decision can
+// differ from an exact evaluation only for draws already counted as near ties.
+constexpr double kSampleTol = 5e-10;
+
+// Sampler AUTO ladder: FP64, fixed point with 128, 160 then 192 fraction bits (when the
+// state bounds the tree), triple-double.  The prediction kp of the cancellation, from
+// the previous step, keeps a factor 4 of margin for FP64 and 2 for the narrow fixed
+// point (a miss there costs ~0.7 of the next rung); the wider fixed-point trees are
+// cheap enough relative to the next rung that they are tried without margin (the check
+// after the tree escalates it when needed).
+GBS_HD_INLINE int sampler_pick(bool bounded, double kp, int n) {
+  if (err_factor(GBS_PREC_FP64, n) * unit_of(GBS_PREC_FP64) * kp * 4.0 < kSampleTol) return GBS_PREC_FP64;
+  if (!bounded) return GBS_PREC_TD;
+  if (err_factor(GBS_PREC_FXN, n) * unit_of(GBS_PREC_FXN) * kp * 2.0 < kSampleTol) return GBS_PREC_FXN;
+  if (err_factor(GBS_PREC_FX, n) * unit_of(GBS_PREC_FX) * kp < kSampleTol) return GBS_PREC_FX;
+  if (err_factor(GBS_PREC_FXW, n) * unit_of(GBS_PREC_FXW) * kp < kSampleTol) return GBS_PREC_FXW;
+  return GBS_PREC_TD;
+}
+
+// Slot of a precision in gbs_sample_stats.trees / tree_seconds.
+GBS_HD_INLINE int stat_slot(int prec) {
+  return prec == GBS_PREC_FX ? 3 : prec == GBS_PREC_FXW ? 4 : prec == GBS_PREC_FXN ? 5 : prec - 1;
 }
 
 // Up to 32 click modes passed by value as a kernel argument.

@@ -36,6 +36,7 @@
 
 #include "gbs_internal.h"
 #include "gbs_num.cuh"
+#include "gbs_sampler_dev.cuh"
 #include "gbs_tree.cuh"
 
 namespace gbs {
@@ -67,55 +68,27 @@ __global__ void sigma_real_kernel(const cplx<double>* __restrict__ V, int M, dou
 struct GatherItem {
   const double* sig;
   const int* clicks;
-  double* s0;  // half mode: out, det(Sigma'_k)^(-1/2)
   long long root_off;
   int m, k, M, half;
 };
 
-// Full mode: root = Sigma'[S u {k}] (k last).  Half mode: root = (Sigma'|k)[S],
-// the Schur complement of mode k restricted to the clicked modes.  Packed lower
-// triangle, one block per item.
+// The roots of a step's trees (step_root), one block per item.
 __global__ void gather_kernel(const GatherItem* __restrict__ items, double* __restrict__ roots) {
   const GatherItem it = items[blockIdx.x];
   const int n = it.half ? it.m : it.m + 1, d = 2 * n;
   const long long D = 2LL * it.M;
-  const long long rk = 2LL * it.k;
-  double q00 = 0, q10 = 0, q11 = 0;
-  if (it.half) {
-    const double p00 = it.sig[rk * D + rk], p10 = it.sig[(rk + 1) * D + rk], p11 = it.sig[(rk + 1) * D + rk + 1];
-    const double det = p00 * p11 - p10 * p10;
-    const double inv = 1.0 / det;
-    q00 = p11 * inv;
-    q10 = -p10 * inv;
-    q11 = p00 * inv;
-    if (threadIdx.x == 0) *it.s0 = rsqrt(det);
-  }
-  for (int e = threadIdx.x; e < d * (d + 1) / 2; e += blockDim.x) {
-    int a = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
-    while (a * (a + 1) / 2 > e) --a;
-    while ((a + 1) * (a + 2) / 2 <= e) ++a;
-    const int b = e - a * (a + 1) / 2;
-    const int ma = (a >> 1) < it.m ? it.clicks[a >> 1] : it.k;
-    const int mb = (b >> 1) < it.m ? it.clicks[b >> 1] : it.k;
-    const long long ra = 2LL * ma + (a & 1), rb = 2LL * mb + (b & 1);
-    double x = it.sig[ra * D + rb];
-    if (it.half) {
-      const double ua0 = it.sig[ra * D + rk], ua1 = it.sig[ra * D + rk + 1];
-      const double ub0 = it.sig[rk * D + rb], ub1 = it.sig[(rk + 1) * D + rb];
-      const double l0 = fma(ua0, q00, ua1 * q10), l1 = fma(ua0, q10, ua1 * q11);
-      x = fma(-l0, ub0, fma(-l1, ub1, x));
-    }
-    roots[it.root_off + e] = x;
-  }
+  ModePivot pv{};
+  if (it.half) pv = mode_pivot(it.sig, D, it.k);
+  for (int e = threadIdx.x; e < d * (d + 1) / 2; e += blockDim.x)
+    roots[it.root_off + e] = step_root(it.sig, D, it.clicks, it.m, it.k, it.half, pv, e);
 }
 
 struct DecideItem {
   double inc[3], exc[3];  // full: tree sums; half: inc = Tor_k over S, exc unused
-  double* sig;            // Sigma' of the trajectory
+  const double* sig;      // Sigma' of the trajectory
   int* clicks;
   double* pinv;           // out: scaled inverse of the 2x2 pivot block (3 values)
   double* dcarry;         // in (half) / out: D of the next step, triple-double
-  const double* s0;       // half: det(Sigma'_k)^(-1/2)
   unsigned long long seed;
   int m, k, step, sample, attempt, forced, half, M;
 };
@@ -125,68 +98,20 @@ struct DecideOut {
   int click, near_tie;
 };
 
-__device__ __forceinline__ double splitmix_u(unsigned long long seed, unsigned long long n) {
-  unsigned long long z = seed + n * 0x9E3779B97F4A7C15ull;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  z ^= z >> 31;
-  return (double)(z >> 11) * 0x1p-53;
-}
-
 __global__ void decide_kernel(const DecideItem* __restrict__ items, int nitems, DecideOut* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nitems) return;
   const DecideItem it = items[i];
-  const int M = it.M;
-  const unsigned long long seed = it.seed;
-  const double sgn = (it.m & 1) ? -1.0 : 1.0;  // (-1)^m
-  // Nn (a) and D (b) in triple-double, then p0 = a/b by two correction steps
-  td a, b, xnext;
-  if (it.half) {
-    const td tor{it.inc[0], it.inc[1], it.inc[2]};
-    xnext = tor * sgn;  // (-1)^m Tor_k: D of the next step if k stays dark
-    a = xnext * (*it.s0);
-    b = td{it.dcarry[0], it.dcarry[1], it.dcarry[2]};
-  } else {
-    a = td{it.inc[0], it.inc[1], it.inc[2]} * sgn;
-    b = td{it.exc[0], it.exc[1], it.exc[2]} * (-sgn);
-  }
-  const double q0 = a.x0 / b.x0;
-  const td r1 = a - b * q0;
-  const double q1 = r1.x0 / b.x0;
-  const td r2 = r1 - b * q1;
-  const double q2 = r2.x0 / b.x0;
-  const double p0 = q0 + (q1 + q2);
-  int click;
-  int near = 0;
-  if (it.forced >= 0) {
-    click = it.forced;
-  } else {
-    const unsigned long long n =
-        1ull + (unsigned long long)it.step +
-        (1ull << 20) * ((unsigned long long)it.attempt + (1ull << 12) * (unsigned long long)it.sample);
-    const double u = splitmix_u(seed, n);
-    click = !(u < p0);
-    near = fabs(u - p0) < 1e-9;
-  }
-  out[i] = DecideOut{p0, click, near};
-  if (click) {
+  const ModePivot pv = mode_pivot(it.sig, 2LL * it.M, it.k);
+  const Decision d =
+      decide_step(it.inc, it.exc, it.dcarry, it.half, it.m, pv, it.forced, it.seed, it.step, it.sample, it.attempt);
+  out[i] = DecideOut{d.p0, d.click, d.near_tie};
+  if (d.click) {
     it.clicks[it.m] = it.k;
   } else {
-    // pivot block P = Sigma'[k, k] (2 x 2), its inverse for the conditioning
-    const long long D = 2LL * M;
-    const long long r = 2LL * it.k;
-    const double p00 = it.sig[r * D + r], p10 = it.sig[(r + 1) * D + r], p11 = it.sig[(r + 1) * D + r + 1];
-    const double det = p00 * p11 - p10 * p10;
-    const double inv = 1.0 / det;
-    it.pinv[0] = p11 * inv;   // (P^-1)_00
-    it.pinv[1] = -p10 * inv;  // (P^-1)_10
-    it.pinv[2] = p00 * inv;   // (P^-1)_11
-    // D of the next step = Nn_k / det(P)^(-1/2)
-    if (!it.half) xnext = a * sqrt(det);
-    it.dcarry[0] = xnext.x0;
-    it.dcarry[1] = xnext.x1;
-    it.dcarry[2] = xnext.x2;
+    it.pinv[0] = pv.q00;
+    it.pinv[1] = pv.q10;
+    it.pinv[2] = pv.q11;
   }
 }
 
@@ -195,43 +120,55 @@ struct CondItem {
   const int* clicks;
   const double* pinv;
   double* L;       // 2 x A scratch: L row i at L[2i], L[2i+1]
-  long long entry_begin;
   int m, k, A, M;  // A = 2k + 2m active rows
+  int block_begin, pad;
 };
 
 __device__ __forceinline__ long long active_row(int i, int k, const int* clicks) {
   return i < 2 * k ? (long long)i : 2LL * clicks[(i - 2 * k) >> 1] + ((i - 2 * k) & 1);
 }
 
-// L_i = Sigma'[i, k-block] P^-1 for every active row i.
+// L_i = u_i P^-1, u_i = Sigma'[i, k-block], for every active row i.
 __global__ void cond_L_kernel(const CondItem* __restrict__ items) {
   const CondItem it = items[blockIdx.y];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= it.A) return;
   const long long D = 2LL * it.M;
-  const long long ri = active_row(i, it.k, it.clicks);
-  const double u0 = it.sig[ri * D + 2LL * it.k], u1 = it.sig[ri * D + 2LL * it.k + 1];
+  const long long ri = active_row(i, it.k, it.clicks), rk = 2LL * it.k;
+  const double u0 = sig_at(it.sig, D, ri, rk), u1 = sig_at(it.sig, D, ri, rk + 1);
   it.L[2 * i] = fma(u0, it.pinv[0], u1 * it.pinv[1]);
   it.L[2 * i + 1] = fma(u0, it.pinv[1], u1 * it.pinv[2]);
 }
 
-// Sigma'[i, j] -= L_i . Sigma'[k-block, j] over the active block.
-__global__ void cond_update_kernel(const CondItem* __restrict__ items, int nitems, long long total) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= total) return;
+constexpr int kCondRows = 32;
+
+// Sigma'[i, j] -= L_i . u_j over the lower triangle of the active block, kCondRows rows
+// of a trajectory per CTA (a warp per row: its columns are contiguous but for the
+// clicked modes').
+__global__ void cond_update_kernel(const CondItem* __restrict__ items, int nitems) {
   int lo = 0, hi = nitems - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (items[mid].entry_begin <= t) lo = mid; else hi = mid - 1;
+    if (items[mid].block_begin <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
   }
   const CondItem it = items[lo];
-  const long long e = t - it.entry_begin;
-  const int i = (int)(e / it.A), j = (int)(e % it.A);
+  const int i0 = ((int)blockIdx.x - it.block_begin) * kCondRows;
   const long long D = 2LL * it.M;
-  const long long ri = active_row(i, it.k, it.clicks), rj = active_row(j, it.k, it.clicks);
-  const double w0 = it.sig[(2LL * it.k) * D + rj], w1 = it.sig[(2LL * it.k + 1) * D + rj];
-  double* x = it.sig + ri * D + rj;
-  *x = fma(-it.L[2 * i], w0, fma(-it.L[2 * i + 1], w1, *x));
+  const int lane = threadIdx.x & 31;
+  for (int i = i0 + (threadIdx.x >> 5); i < min(i0 + kCondRows, it.A); i += blockDim.x >> 5) {
+    const long long ri = active_row(i, it.k, it.clicks);
+    const double l0 = it.L[2 * i], l1 = it.L[2 * i + 1];
+    const long long rk = 2LL * it.k;
+    // unmeasured rows: columns up to the diagonal; clicked rows: all unmeasured columns
+    // and the clicked ones above the diagonal
+    const int jmax = i < 2 * it.k ? i + 1 : it.A;
+    for (int j = lane; j < jmax; j += 32) {
+      const long long rj = active_row(j, it.k, it.clicks);
+      if (rj > ri) continue;
+      double* x = it.sig + ri * D + rj;
+      *x = fma(-l0, sig_at(it.sig, D, rj, rk), fma(-l1, sig_at(it.sig, D, rj, rk + 1), *x));
+    }
+  }
 }
 
 }  // namespace
@@ -248,25 +185,6 @@ gbs_status ensure_sigma_real(gbs_ctx* ctx, gbs_state* st) {
   return check_cuda(ctx, cudaGetLastError(), "sigma real");
 }
 
-double unit_of(int prec) {
-  switch (prec) {
-    case GBS_PREC_FP64: return 0x1p-53;
-    case GBS_PREC_DD: return 0x1p-102;
-    case GBS_PREC_FXN: return 0x1p-108;
-    case GBS_PREC_FX: return 0x1p-140;
-    case GBS_PREC_FXW: return 0x1p-158;  // limited by the three-double tree output
-  }
-  return 0x1p-152;
-}
-
-namespace {
-// Slot of a precision in gbs_sample_stats.trees / tree_seconds.
-int stat_slot(int prec) {
-  return prec == GBS_PREC_FX ? 3 : prec == GBS_PREC_FXW ? 4 : prec == GBS_PREC_FXN ? 5 : prec - 1;
-}
-}  // namespace
-
-
 size_t traj_bytes(int M) {
   return (size_t)4 * M * M * sizeof(double) + 64 * sizeof(int) + 8 * sizeof(double) +
          ((size_t)4 * M + 256) * sizeof(double);
@@ -278,7 +196,7 @@ void traj_bind(Trajectory& tj, gbs_state* st, unsigned char* mem) {
   const size_t sig_bytes = (size_t)4 * tj.M * tj.M * sizeof(double);
   tj.sig = (double*)mem;
   tj.clicks = (int*)(mem + sig_bytes);
-  tj.pinv = (double*)(mem + sig_bytes + 64 * sizeof(int));  // [0..2] P^-1, [3] s0
+  tj.pinv = (double*)(mem + sig_bytes + 64 * sizeof(int));  // [0..2] P^-1
   tj.dcarry = tj.pinv + 4;
   tj.L = tj.pinv + 8;
 }
@@ -312,34 +230,25 @@ struct StepTree {
 };
 }  // namespace
 
-// Advance every running trajectory of `jobs` by one measured mode.  The jobs may
+// Advance every running trajectory of `jobs`: those with few clicks by up to
+// kChainSteps measured modes in one CTA each (gbs_chain.cu), the others by one here.
+// The jobs may
 // belong to different states, sizes and step positions; all their trees of a
 // given precision run as one batch.  A trajectory that finishes becomes kDone,
 // one abandoned by postselection kRejected (the caller restarts or drops it).
 gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int prec, gbs_sample_stats& stt) {
-  std::vector<Trajectory*> act;
-  for (Trajectory* t : jobs)
-    if (t->state == Trajectory::kRunning) act.push_back(t);
-  if (act.empty()) return GBS_OK;
+  std::vector<Trajectory*> act, chain;
+  for (Trajectory* t : jobs) {
+    if (t->state != Trajectory::kRunning) continue;
+    (!t->host_step && chain_eligible(*t, prec) ? chain : act).push_back(t);
+    t->host_step = false;
+  }
   gbs_status e;
-  // Bound on |delta p0|: half the near-tie threshold, so that a decision can
-  // differ from an exact evaluation only for draws already counted as near ties.
-  const double TOL = 5e-10;
-  // AUTO ladder: FP64, fixed point with 128, 160 then 192 fraction bits (when
-  // the state bounds the tree), triple-double.  The prediction from the
-  // previous step keeps a factor 4 of margin for FP64 and 2 for the narrow
-  // fixed point (a miss there costs ~0.7 of the next rung); the wider
-  // fixed-point trees are cheap enough relative to the next rung that they are
-  // tried without margin (the check after the tree escalates it when needed).
+  if (!chain.empty() && (e = chain_advance(ctx, chain, prec, stt))) return e;
+  if (act.empty()) return GBS_OK;
+  const double TOL = kSampleTol;
   auto pick = [&](const Trajectory* t, double kp, int n) {
-    if (prec != GBS_PREC_AUTO) return prec;
-    const int ladder[5] = {GBS_PREC_FP64, GBS_PREC_FXN, GBS_PREC_FX, GBS_PREC_FXW, GBS_PREC_TD};
-    const double margin[4] = {4.0, 2.0, 1.0, 1.0};
-    for (int l = 0; l < 4; ++l) {
-      if (is_fixed_point(ladder[l]) && !fx_ok_sigma(t->st, n)) continue;
-      if (err_factor(ladder[l], n) * unit_of(ladder[l]) * kp * margin[l] < TOL) return ladder[l];
-    }
-    return (int)GBS_PREC_TD;
+    return prec != GBS_PREC_AUTO ? prec : sampler_pick(fx_ok_sigma(t->st, n), kp, n);
   };
   // The next rung after a failed check; the wide fixed point is the last one
   // where the state allows it (triple-double's bound is looser), so a half
@@ -375,7 +284,7 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
       StepTree& q = trees[i];
       Trajectory* t = q.tj;
       q.root_off = ent;
-      gi.push_back(GatherItem{t->sig, t->clicks, t->pinv + 3, ent, t->m, t->M - 1 - t->step, t->M, q.half});
+      gi.push_back(GatherItem{t->sig, t->clicks, ent, t->m, t->M - 1 - t->step, t->M, q.half});
       const int d = 2 * std::max(q.n, 1);
       ent += (long long)d * (d + 1) / 2;
     }
@@ -462,7 +371,6 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
     d.clicks = t->clicks;
     d.pinv = t->pinv;
     d.dcarry = t->dcarry;
-    d.s0 = t->pinv + 3;
     d.seed = t->seed;
     d.m = t->m;
     d.k = k;
@@ -499,7 +407,7 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
     return e;
   // ---- bookkeeping, postselection, conditioning of the dark modes
   std::vector<CondItem> ci;
-  long long entries = 0;
+  int blocks = 0;
   for (size_t i = 0; i < act.size(); ++i) {
     Trajectory* t = act[i];
     const int k = t->M - 1 - t->step;
@@ -519,8 +427,8 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
     }
     if (!dec[i].click && k > 0) {
       const int A = 2 * k + 2 * t->m;
-      ci.push_back(CondItem{t->sig, t->clicks, t->pinv, t->L, entries, t->m, k, A, t->M});
-      entries += (long long)A * A;
+      ci.push_back(CondItem{t->sig, t->clicks, t->pinv, t->L, t->m, k, A, t->M, blocks, 0});
+      blocks += (A + kCondRows - 1) / kCondRows;
     }
     t->step++;
     if (k == 0) t->state = Trajectory::kDone;
@@ -532,8 +440,7 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
     for (const CondItem& c : ci) amax = std::max(amax, c.A);
     dim3 gl((amax + 255) / 256, (unsigned)ci.size());
     cond_L_kernel<<<gl, 256, 0, ctx->stream>>>((const CondItem*)dci);
-    cond_update_kernel<<<(unsigned)((entries + 255) / 256), 256, 0, ctx->stream>>>((const CondItem*)dci,
-                                                                                   (int)ci.size(), entries);
+    cond_update_kernel<<<(unsigned)blocks, 256, 0, ctx->stream>>>((const CondItem*)dci, (int)ci.size());
     count_launch(ctx, 2);
     if ((e = check_cuda(ctx, cudaGetLastError(), "conditioning"))) return e;
   }
