@@ -40,6 +40,11 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
     const int n = trees[t].n;
     if (n < 1 || n > 40) return set_error(ctx, GBS_EINVAL, "batch tree size out of range");
     Q[t] = std::max(1, std::min(n, QMAX - tune.q_drop));
+    // A tree that one CTA expands: no more register levels than its threads need to go
+    // on with (two at least: the paired groups), since one thread's levels are a serial
+    // chain (FP64P, N = 6: 70 us with five levels in each of two threads, 25 with two in
+    // each of sixteen).  By n alone: a tree's bits do not depend on its batch.
+    if (sub_e >= 5) Q[t] = std::min(Q[t], std::max(2, n - sub_e));
     qroot[t] = std::min(n, Q[t] + sub_e);
     depth[t] = n - qroot[t];  // levels above the leaf / subtree roots
     dtop[t] = std::min(depth[t], tune.d_top);
