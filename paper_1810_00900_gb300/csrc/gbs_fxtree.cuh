@@ -20,8 +20,8 @@
 //   level kernels one launch per child size q: a warp per 32 consecutive children of a
 //                 tree (lane = child), or, where children are few, a CTA per 1 .. 32.
 //   leaf kernel   a warp takes tiles of 32 nodes of one tree, one thread per node
-//                 for all 2^Q subsets of its last Q modes.
-//   final kernel  one CTA per tree adds the warps' sums and finishes the result.
+//                 for all 2^Q subsets of its last Q modes; a sum per CTA.
+//   final kernel  one CTA per tree adds the CTAs' sums and finishes the result.
 //   small kernel  a tree of few modes in one launch, in the shared memory of one or a
 //                 few CTAs.
 // Measured against the engine it replaced (both children stored, subtrees of 9
@@ -63,6 +63,14 @@
 namespace gbs {
 
 constexpr uint32_t kFxShift = 1u << 9;  // K
+
+// Programmatic dependent launch: the launch after this one may set up its CTAs from
+// here on; wait for the launch before this one to be complete.  Every thread of a kernel
+// launched by fx_launch calls it before it touches memory.
+__device__ __forceinline__ void fx_after() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // Scalars of a pivot.
 template <class E>
@@ -253,6 +261,7 @@ __global__ void __launch_bounds__(256) fx_top_kernel(const FxSeg* __restrict__ s
   constexpr int L = sizeof(E) / 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FxPivot<E> pv;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
   const FxTree t = trees[sg.idx];
   const unsigned v = (unsigned)((long long)blockIdx.x - sg.first);  // (the top runs before any chunk: v' = v)
@@ -397,6 +406,7 @@ __global__ void __launch_bounds__(32) fx_level_warp_kernel(const FxSeg* __restri
                                                            uint32_t* nodes, typename fx_sum<E>::type* sval,
                                                            int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  fx_after();
   const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
   const FxTree t = trees[sg.idx];
   const unsigned tile = (unsigned)((long long)blockIdx.x - sg.first);
@@ -496,6 +506,7 @@ __global__ void __launch_bounds__(256) fx_level_cta_kernel(const FxSeg* __restri
                                                            unsigned chunk, uint32_t* nodes,
                                                            typename fx_sum<E>::type* sval, int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  fx_after();
   const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
   const FxTree t = trees[sg.idx];
   const unsigned c0 = (unsigned)((long long)blockIdx.x - sg.first) * (unsigned)TW;
@@ -579,36 +590,76 @@ __device__ __forceinline__ bool fx_leaf_node(const uint32_t* m, int p, const typ
   if constexpr (Q == 1) {
     return fx_leaf1(fx_ld<E, ST>(m, tri(o, o)), fx_ld<E, ST>(m, tri(o + 1, o)), fx_ld<E, ST>(m, tri(o + 1, o + 1)), s,
                     neg, acc);
-  } else {
-    static_assert(Q == 2, "one or two levels per leaf thread");
+  } else if constexpr (Q == 2) {
     return fx_leaf2<E, ST>(m, o, s, neg, acc);
+  } else {
+    // Three modes, for the narrow type (registers): the included child's ten entries are
+    // formed row by row into local memory, the excluded one is a view.  356 us at N = 24
+    // (64 fraction bits) against 164 + 216 for a level launch that writes them and a
+    // two-mode leaf that reads them back, and a launch less.
+    static_assert(Q == 3, "at most three levels per leaf thread");
+    constexpr int L = sizeof(E) / 4;
+    uint32_t child[10 * L];
+    typename fx_sum<E>::type sv;
+    bool ok;
+    {
+      FxPivot<E> pv;
+      ok = fx_pivot(fx_ld<E, ST>(m, tri(o, o)), fx_ld<E, ST>(m, tri(o + 1, o)), fx_ld<E, ST>(m, tri(o + 1, o + 1)), pv);
+      sv = umul(s, pv.g);
+      E U[4], V[4], B[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const int e = tri(o + 2 + a, o);
+        FxRow<E> r;
+        fx_row(pv, fx_ld<E, ST>(m, e), fx_ld<E, ST>(m, e + 1), r);
+        U[a] = r.U;
+        V[a] = r.V;
+        B[a] = r.B;
+#pragma unroll
+        for (int b = 0; b <= a; ++b)
+          fx_st<E, 1>(child, tri(a, b), fx_entry(fx_ld<E, ST>(m, e + 2 + b), r.P, r.Q, r.A, U[b], V[b], B[b]));
+      }
+    }
+    ok &= fx_leaf2<E, 1>(child, 0, sv, neg, acc);
+    return fx_leaf2<E, ST>(m, o + 2, s, ~neg, acc) && ok;
   }
 }
 
-// One warp per unit: tiles_per_unit consecutive tiles of 32 nodes of one tree.
+// Sum over a warp; every lane gets it.
+template <class S>
+__device__ __forceinline__ void fx_warp_sum(FxSums<S>& acc) {
+#pragma unroll 1
+  for (int off = 16; off > 0; off >>= 1) {
+    acc.inc = acc.inc + shfl_xor(acc.inc, off);
+    acc.exc = acc.exc + shfl_xor(acc.exc, off);
+    acc.mag = acc.mag + shfl_xor(acc.mag, off);
+  }
+}
+
+// One CTA of four warps per unit: 4 x tiles_per_unit consecutive tiles of 32 nodes of one
+// tree, one partial sum.
 template <class E, int Q>
-__global__ void __launch_bounds__(128, 4) fx_leaf_kernel(const FxSeg* __restrict__ segs, int nseg, long long units,
-                                                      unsigned chunk, const FxTree* __restrict__ trees,
-                                                      const long long* __restrict__ lvl_off,
-                                                      const uint32_t* __restrict__ nodes,
-                                                      const typename fx_sum<E>::type* __restrict__ sval,
-                                                      FxPart<typename fx_sum<E>::type>* __restrict__ parts,
-                                                      int* __restrict__ status) {
+__global__ void __launch_bounds__(128, 4) fx_leaf_kernel(const FxSeg* __restrict__ segs, int nseg, unsigned chunk,
+                                                         const FxTree* __restrict__ trees,
+                                                         const long long* __restrict__ lvl_off,
+                                                         const uint32_t* __restrict__ nodes,
+                                                         const typename fx_sum<E>::type* __restrict__ sval,
+                                                         FxPart<typename fx_sum<E>::type>* __restrict__ parts,
+                                                         int* __restrict__ status) {
   typedef typename fx_sum<E>::type S;
   constexpr int L = sizeof(E) / 4;
-  const int lane = threadIdx.x & 31;
-  const long long unit = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (unit >= units) return;
-  const FxSeg sg = segs[fx_find(segs, nseg, unit)];
+  fx_after();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];
   const FxTree t = trees[sg.idx];
   const unsigned count = 1u << (t.D - t.d0 + t.cb);
   const S zero = fx_of<S>(0.0);
   FxSums<S> acc{zero, zero, zero};
   bool ok = true;
-  const unsigned tile0 = (unsigned)(unit - sg.first) * (unsigned)sg.tiles_per_unit;
+  const unsigned tile0 = (unsigned)((long long)blockIdx.x - sg.first) * 4u * (unsigned)sg.tiles_per_unit + warp;
 #pragma unroll 1
   for (int i = 0; i < sg.tiles_per_unit; ++i) {
-    const unsigned v = (tile0 + i) * 32u + lane;
+    const unsigned v = (tile0 + 4u * i) * 32u + lane;
     if (v >= count) break;
     const S s = sval[fx_sidx(t, v, chunk)];
     // sign of the node: (-1)^(exclusions above)
@@ -624,24 +675,30 @@ __global__ void __launch_bounds__(128, 4) fx_leaf_kernel(const FxSeg* __restrict
   }
   if (!ok) atomicExch(status + t.tree, (int)kStatusRange);
   __syncwarp();
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    acc.inc = acc.inc + shfl_down(acc.inc, off);
-    acc.exc = acc.exc + shfl_down(acc.exc, off);
-    acc.mag = acc.mag + shfl_down(acc.mag, off);
+  fx_warp_sum(acc);
+  __shared__ FxPart<S> sh[4];
+  if (lane == 0) sh[warp] = FxPart<S>{acc.inc, acc.exc, acc.mag};
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 4; ++w) {
+      acc.inc = acc.inc + sh[w].inc;
+      acc.exc = acc.exc + sh[w].exc;
+      acc.mag = acc.mag + sh[w].abs;
+    }
+    parts[blockIdx.x] = FxPart<S>{acc.inc, acc.exc, acc.mag};
   }
-  if (lane == 0) parts[unit] = FxPart<S>{acc.inc, acc.exc, acc.mag};
 }
 
 // -------------------------------------------------------------------- final --
 // One CTA per tree; segs[t].first = the tree's first unit, segs[t + 1].first the end.
-// (Ten thousand units took it 31 us: one wave of leaf warps is what it gets.)
+// (Ten thousand partial sums took it 31 us; a sum per leaf CTA leaves it some thousand.)
 template <class S>
 __global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* __restrict__ parts,
                                                         const FxSeg* __restrict__ segs,
                                                         const FxTree* __restrict__ trees,
                                                         const int* __restrict__ status, double u, double extra,
                                                         ProbOut* __restrict__ out) {
+  fx_after();
   const int t = blockIdx.x;
   const S zero = fx_of<S>(0.0);
   S inc = zero, exc = zero, mag = zero;
@@ -776,17 +833,6 @@ struct FxOps {
     if constexpr (CALL) return fxc_leaf1(p00, p10, p11, s, neg, acc); else return fxm_leaf1(p00, p10, p11, s, neg, acc);
   }
 };
-
-// Sum over a warp; every lane gets it.
-template <class S>
-__device__ __forceinline__ void fx_warp_sum(FxSums<S>& acc) {
-#pragma unroll 1
-  for (int off = 16; off > 0; off >>= 1) {
-    acc.inc = acc.inc + shfl_xor(acc.inc, off);
-    acc.exc = acc.exc + shfl_xor(acc.exc, off);
-    acc.mag = acc.mag + shfl_xor(acc.mag, off);
-  }
-}
 
 // The tree of a CTA: the n-mode root (root(i): entry i of its packed triangle) with the
 // first d0 modes set to pre, all other subsets enumerated.  Returns the CTA's sums in

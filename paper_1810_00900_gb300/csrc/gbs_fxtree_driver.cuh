@@ -17,15 +17,36 @@ inline long long fx_level_words(int n, int k, long long count, int L) {
   return count * (long long)sym(2 * q) * L;
 }
 
+// Launch of a kernel that waits (fx_after) for the launch before it.  early: its CTAs may
+// be set up while that launch runs -- where that one leaves the chip room (a few CTAs
+// per SM at most), or they would take it from its own later CTAs.  ~2 us a launch: N =
+// 18, FP64, 14 launches, 163 -> 137 us.
+template <class... P, class... A>
+void fx_launch(bool early, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 template <class E>
 gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const void* roots_dev, int* status_dev,
                         const BatchTune& tune, const FxFinish& fin) {
   typedef typename fx_sum<E>::type S;
   constexpr int L = sizeof(E) / 4;
   // Small trees (fx_small_kernel): one CTA for up to kOne modes, whose levels fit its
-  // shared memory twice over; beyond, a CTA per setting of the first modes, as long as
-  // the CTAs of the whole call stay within two per SM: the other trees' rate counts, and
-  // the levels below serve it better.
+  // shared memory; up to 17 modes a CTA per setting of the first ones, as long as the
+  // call's CTAs are few.  One launch of them against levels, us: 64 fraction bits, 32
+  // trees of 12 .. 15 modes (~640 CTAs) 198 against 231, 4 of 17 (1024) 181 / 173; 128
+  // bits, 8 of 15 (512) 168 / 201, 4 of 17 (1024) 320 / 221; 160 bits, 24 of 12 (384)
+  // 182 / 210, 8 of 15 (1024) 268 / 215; 192 bits, one of 17 (512) 216 / 192.
   constexpr int LS = sizeof(S) / 4;
   constexpr int kOne = fx_small_words(10, 10, L, LS) * 4 <= 220 * 1024 ? 10 : 9;
   constexpr int kSub = kOne - 1;  // modes of a CTA's own tree where it is one of several
@@ -34,7 +55,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     if (in[i].n < 1 || in[i].n > 32) return set_error(ctx, GBS_EINVAL, "batch tree size out of range");
     if (in[i].n > kOne) ctas += 1LL << std::min(in[i].n - kSub, 20);
   }
-  const int small_max = ctas <= 2 * ctx->sm_count ? 32 : kOne;
+  const int small_max = ctas <= ctx->sm_count * (L <= 3 ? 6 : L <= 5 ? 4 : 2.5) ? 17 : kOne;
   std::vector<int> order;  // the others, largest first: every per-size list below is then a run of trees
   std::vector<FxSmall> small[2];  // in one CTA, in several
   int small_n[2] = {0, 0};
@@ -86,12 +107,14 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   // ---------------- plan
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return in[a].n > in[b].n; });
   // Levels per leaf thread.
-  const int Qmax = std::max(1, std::min(2, 3 - tune.q_drop));
+  constexpr int kLeafQ = L <= 3 ? 3 : 2;
+  const int Qmax = std::max(1, std::min(kLeafQ, 3 - tune.q_drop));
   const int nmax = in[order[0]].n;
-  // Depth of the top kernel: at most tune.d_top and about 64 CTAs, at least the five
-  // levels that are not kept in tiles.
+  // Depth of the top kernel: at most tune.d_top and 256 CTAs, at least the five levels
+  // that are not kept in tiles.  (A step of it against a level launch: N = 18 .. 20,
+  // FP64, 171, 203, 233 us with 64 CTAs, 146, 176, 212 with 256, 160, 180, 216 with 1024.)
   int d_top = 5;
-  while (d_top < tune.d_top && ((long long)ntrees << (d_top + 1)) <= 64) ++d_top;
+  while (d_top < tune.d_top && ((long long)ntrees << (d_top + 1)) <= 256) ++d_top;
   auto cta_smem = [&](int R, int TW) { return (size_t)((5 * L + 1) + R * (6 * L + 1)) * TW * 4; };
   std::vector<FxTree> trees(ntrees);
   std::vector<int> Q(ntrees);
@@ -199,13 +222,15 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   std::vector<FxSeg> sums;
   long long tiles_total = 0, units_total = 0;
   for (int i = 0; i < ntrees; ++i) tiles_total += ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
-  // tiles per warp: one wave of the 16 warps an SM holds
-  const int tpu = (int)std::max(1LL, std::min(64LL, (tiles_total + 16LL * ctx->sm_count - 1) / (16LL * ctx->sm_count)));
+  // Tiles per warp: about five waves of the 16 warps an SM holds.  (One wave, and a few
+  // CTAs more than that because every tree ends in a part of one, took twice its time:
+  // 300 trees of 15 .. 17 modes, 64 fraction bits, 685 us.)
+  const int tpu = (int)std::max(1LL, std::min(64LL, tiles_total / (80LL * ctx->sm_count)));
   for (int i = 0; i < ntrees; ++i) {
     if (leaves.empty() || leaves.back().Q != Q[i]) leaves.push_back(Leaf{Q[i], {}, 0, 0});
     Leaf& lf = leaves.back();
     const long long tiles = ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
-    const long long units = (tiles + tpu - 1) / tpu;
+    const long long units = (tiles + 4 * tpu - 1) / (4 * tpu);
     lf.segs.push_back(FxSeg{lf.units, i, tpu});
     lf.units += units;
     sums.push_back(FxSeg{units_total, i, 0});
@@ -249,17 +274,26 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   fx_top_kernel<E><<<(unsigned)top_blocks, 256, smem_top, s>>>((const FxSeg*)(plan + o_top), ntrees, d_trees, d_off,
                                                                (const double*)roots_dev, nodes, sval, status_dev);
   count_launch(ctx);
+  long long before = top_blocks;  // CTAs of the launch before
+  auto early = [&](long long blocks) {
+    const bool e = before <= 2LL * ctx->sm_count;
+    before = blocks;
+    return e;
+  };
   auto level = [&](const Launch& l, unsigned chunk) {
+    const bool el = early(l.blocks);
     const FxSeg* sg = (const FxSeg*)(plan + l.at);
     const int ns = (int)l.segs.size();
     const FxTree* tr = l.in_chunk ? d_chunked : d_trees;
     if (l.TW)
-      fx_level_cta_kernel<E><<<(unsigned)l.blocks, 32 * l.W, l.smem, s>>>(sg, ns, tr, d_off, l.q, l.TW, chunk, nodes, sval,
-                                                                          status_dev);
+      fx_launch(el, fx_level_cta_kernel<E>, (unsigned)l.blocks, 32 * l.W, l.smem, s, sg, ns, tr, d_off, l.q, l.TW, chunk, nodes,
+                sval, status_dev);
     else if (l.q >= 4)
-      fx_level_warp_kernel<E, 4><<<(unsigned)l.blocks, 32, l.smem, s>>>(sg, ns, tr, d_off, l.q, chunk, nodes, sval, status_dev);
+      fx_launch(el, fx_level_warp_kernel<E, 4>, (unsigned)l.blocks, 32, l.smem, s, sg, ns, tr, d_off, l.q, chunk, nodes, sval,
+                status_dev);
     else
-      fx_level_warp_kernel<E, 2><<<(unsigned)l.blocks, 32, l.smem, s>>>(sg, ns, tr, d_off, l.q, chunk, nodes, sval, status_dev);
+      fx_launch(el, fx_level_warp_kernel<E, 2>, (unsigned)l.blocks, 32, l.smem, s, sg, ns, tr, d_off, l.q, chunk, nodes, sval,
+                status_dev);
     count_launch(ctx);
   };
   for (const Launch& l : levels)
@@ -270,12 +304,14 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
       if (l.in_chunk) level(l, (unsigned)h);
     long long base = h * leaves[0].units;  // chunks: one tree, one leaf launch each
     for (const Leaf& l : leaves) {
-      const unsigned grid = (unsigned)((l.units + 3) / 4);
+      const unsigned grid = (unsigned)l.units;
       const FxSeg* sg = (const FxSeg*)(plan + l.at);
       const int ns = (int)l.segs.size();
+      const bool el = early(grid);
       switch (l.Q) {
-        case 1: fx_leaf_kernel<E, 1><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
-        default: fx_leaf_kernel<E, 2><<<grid, 128, 0, s>>>(sg, ns, l.units, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        case 1: fx_launch(el, fx_leaf_kernel<E, 1>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        case 2: fx_launch(el, fx_leaf_kernel<E, 2>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        default: fx_launch(el, fx_leaf_kernel<E, kLeafQ>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
       }
       count_launch(ctx);
       base += l.units;
@@ -283,8 +319,8 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   }
   timer(true);
   const int final_threads = units_total > 256LL * ntrees ? 1024 : 128;
-  fx_final_kernel<S><<<(unsigned)ntrees, final_threads, 0, s>>>(parts, (const FxSeg*)(plan + o_sums), d_trees, status_dev,
-                                                                    fin.u, fin.extra, fin.po);
+  fx_launch(early(0), fx_final_kernel<S>, (unsigned)ntrees, final_threads, 0, s, parts, (const FxSeg*)(plan + o_sums), d_trees,
+            status_dev, fin.u, fin.extra, fin.po);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "fixed-point batch launch");
 }
