@@ -4,7 +4,7 @@
 
 namespace gbs {
 gbs_status batch_fxn_real(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots, int* status,
-                         const BatchTune& tune, const FxFinish& fin) {
+                         const BatchTune& tune, const TreeFinish& fin) {
   return fx_batch_run<fxn4>(ctx, ntrees, trees, roots, status, tune, fin);
 }
 }  // namespace gbs

@@ -3,7 +3,7 @@
 
 namespace gbs {
 gbs_status batch_fxw_real(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots, int* status,
-                         const BatchTune& tune, const FxFinish& fin) {
+                         const BatchTune& tune, const TreeFinish& fin) {
   return fx_batch_run<fxw>(ctx, ntrees, trees, roots, status, tune, fin);
 }
 }  // namespace gbs

@@ -15,8 +15,9 @@
 //   leaf kernel    register depth-first subtrees of the last Q levels (as in
 //                  gbs_tree.cuh); blocks never straddle two trees, so each
 //                  block partial belongs to one tree; optionally persistent.
-//   final kernel   one warp per tree sums its block partials in a fixed order,
-//                  so a tree's result does not depend on the rest of the batch.
+//   final kernel   one CTA per tree sums its block partials in a fixed order (chunks
+//                  of them first where they are many) and finishes the result, which
+//                  does not depend on the rest of the batch.
 //
 // Each tree owns a fixed region of both level buffers (sized for its largest
 // level), so trees at different depths never overwrite each other.
@@ -460,42 +461,13 @@ __global__ void batch_chunk_kernel(const Partial<Red>* __restrict__ parts, const
   block_reduce_store(inc, exc, asum, out + c);
 }
 
-// ---------------------------------------------------------------- final --
-template <class Red>
-__global__ void batch_final_kernel(const Partial<Red>* __restrict__ parts, const PartRange* __restrict__ ranges,
-                                   int ntrees, TreeOut* __restrict__ outs) {
-  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (t >= ntrees) return;
-  const PartRange r = ranges[t];
-  Red inc = red_zero<Red>(), exc = red_zero<Red>();
-  double asum = 0.0;
-  for (long long i = lane; i < r.count; i += 32) {
-    inc = red_add(inc, parts[r.first + i].inc);
-    exc = red_add(exc, parts[r.first + i].exc);
-    asum += parts[r.first + i].abs;
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    inc = red_add(inc, shfl_down(inc, off));
-    exc = red_add(exc, shfl_down(exc, off));
-    asum += __shfl_down_sync(0xffffffffu, asum, off);
-  }
-  if (lane == 0) {
-    red_store(inc, outs[t].inc);
-    red_store(exc, outs[t].exc);
-    outs[t].abs = asum;
-  }
-}
-
 // ------------------------------------------------------------------ finish --
-// Torontonian, probability, cancellation ratio and error estimate of one tree.
-__device__ __forceinline__ ProbOut finish_tree(const TreeOut& o, int status, double logdet, int n, double u,
-                                               double extra) {
+// Torontonian, probability, cancellation ratio and error estimate of one tree; sc =
+// det(Sigma)^(-1/2).
+__device__ __forceinline__ ProbOut finish_tree(const TreeOut& o, int status, double sc, int n, double u, double extra) {
   const td a{o.inc[0], o.inc[1], o.inc[2]};
   const td b{o.exc[0], o.exc[1], o.exc[2]};
   const td tor = a + b;
-  const double sc = exp(-0.5 * logdet);
   const td p = tor * sc;
   ProbOut r;
   r.p_hi = p.x0;
@@ -509,6 +481,37 @@ __device__ __forceinline__ ProbOut finish_tree(const TreeOut& o, int status, dou
   r.status = status;
   r.pad = 0;
   return r;
+}
+
+// ---------------------------------------------------------------- final --
+// Sum of a tree's partials (or of their chunks' sums) in a fixed order and its finished
+// result, one CTA per tree: thread i sums partials i, i + 256, ... (the same ones in a
+// smaller block, whose ranges are no longer than it), then shuffle trees; threads without
+// one add zeros.  Chains of dependent double-double additions are what it costs, and the
+// launches that it saves (the chunks' and the finish's) what it gives: a torontonian of 9
+// modes under AUTO takes 117 us, 160 with three launches per precision.
+template <class Red>
+__global__ void batch_final_kernel(const Partial<Red>* __restrict__ parts, const PartRange* __restrict__ ranges,
+                                   const int* __restrict__ status, const double* __restrict__ scale,
+                                   const int* __restrict__ nmodes, double u, double extra, ProbOut* __restrict__ po) {
+  const int t = blockIdx.x;
+  const PartRange r = ranges[t];
+  Red inc = red_zero<Red>(), exc = red_zero<Red>();
+  double asum = 0.0;
+  for (long long i = threadIdx.x; i < r.count; i += blockDim.x) {
+    inc = red_add(inc, parts[r.first + i].inc);
+    exc = red_add(exc, parts[r.first + i].exc);
+    asum += parts[r.first + i].abs;
+  }
+  __shared__ Partial<Red> res;
+  block_reduce_store(inc, exc, asum, &res);
+  if (threadIdx.x == 0) {
+    TreeOut o;
+    red_store(res.inc, o.inc);
+    red_store(res.exc, o.exc);
+    o.abs = res.abs;
+    po[t] = finish_tree(o, status[t], scale[t], nmodes[t], u, extra);
+  }
 }
 
 }  // namespace gbs

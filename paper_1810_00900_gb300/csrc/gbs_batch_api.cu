@@ -194,14 +194,6 @@ __global__ void kappa_estimate_kernel(const BatchTree* __restrict__ trees, int n
   if (lane == 0) log10_kappa[t] = lk;
 }
 
-__global__ void batch_finish_kernel(const TreeOut* __restrict__ outs, const int* __restrict__ status,
-                                    const double* __restrict__ logdet, const int* __restrict__ nmodes, double u,
-                                    double extra, int ntrees, ProbOut* __restrict__ po) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= ntrees) return;
-  po[t] = finish_tree(outs[t], status[t], logdet[t], nmodes[t], u, extra);
-}
-
 static double unit_roundoff_b(int prec) {
   switch (prec) {
     case GBS_PREC_FP64:
@@ -216,35 +208,28 @@ static double unit_roundoff_b(int prec) {
   return 1.0;
 }
 
-static gbs_status batch_variant(gbs_ctx* ctx, int prec, bool real, int nt, const BatchTree* tr, const void* roots,
-                                TreeOut* outs, int* status) {
-  const BatchTune& tu = batch_tune_for(ctx, prec, real);
+// The engine of a precision and basis (fixed64: FP64 in 64-bit fixed point).
+static gbs_status batch_variant(gbs_ctx* ctx, int prec, bool real, bool fixed64, int nt, const BatchTree* tr,
+                                const void* roots, int* status, const TreeFinish& fin) {
+  BatchEngine* e = nullptr;
   switch (prec) {
-    case GBS_PREC_FP64: return real ? batch_fp64_real(ctx, nt, tr, roots, outs, status, tu)
-                                    : batch_fp64_cplx(ctx, nt, tr, roots, outs, status, tu);
-    case GBS_PREC_DD: return real ? batch_dd_real(ctx, nt, tr, roots, outs, status, tu)
-                                  : batch_dd_cplx(ctx, nt, tr, roots, outs, status, tu);
-    case GBS_PREC_TD: return real ? batch_td_real(ctx, nt, tr, roots, outs, status, tu)
-                                  : batch_td_cplx(ctx, nt, tr, roots, outs, status, tu);
-    case GBS_PREC_FP32_DIAG: return real ? batch_fp32_real(ctx, nt, tr, roots, outs, status, tu)
-                                         : batch_fp32_cplx(ctx, nt, tr, roots, outs, status, tu);
-    case GBS_PREC_FP64P: return real ? batch_fp64p_real(ctx, nt, tr, roots, outs, status, tu)
-                                     : set_error(ctx, GBS_EINVAL, "the paired FP64 precision needs the real basis");
+    case GBS_PREC_FP64: e = fixed64 ? batch_fxd_real : real ? batch_fp64_real : batch_fp64_cplx; break;
+    case GBS_PREC_DD: e = real ? batch_dd_real : batch_dd_cplx; break;
+    case GBS_PREC_TD: e = real ? batch_td_real : batch_td_cplx; break;
+    case GBS_PREC_FP32_DIAG: e = real ? batch_fp32_real : batch_fp32_cplx; break;
+    case GBS_PREC_FP64P:
+      if (!real) return set_error(ctx, GBS_EINVAL, "the paired FP64 precision needs the real basis");
+      e = batch_fp64p_real;
+      break;
+    case GBS_PREC_FXN:
+    case GBS_PREC_FX:
+    case GBS_PREC_FXW:
+      if (!real) return set_error(ctx, GBS_EINVAL, "the fixed-point precision needs the real basis");
+      e = prec == GBS_PREC_FXN ? batch_fxn_real : prec == GBS_PREC_FX ? batch_fx_real : batch_fxw_real;
+      break;
+    default: return set_error(ctx, GBS_EINVAL, "unknown precision");
   }
-  return set_error(ctx, GBS_EINVAL, "unknown precision");
-}
-
-// The fixed-point engine's instance for prec (FP64: the 64-bit one).
-static gbs_status fixed_variant(gbs_ctx* ctx, int prec, int nt, const BatchTree* tr, const void* roots, int* status,
-                                const FxFinish& fin) {
-  const BatchTune& tu = batch_tune_for(ctx, prec == GBS_PREC_FP64 ? GBS_PREC_FXN : prec, true);
-  switch (prec) {
-    case GBS_PREC_FP64: return batch_fxd_real(ctx, nt, tr, roots, status, tu, fin);
-    case GBS_PREC_FXN: return batch_fxn_real(ctx, nt, tr, roots, status, tu, fin);
-    case GBS_PREC_FX: return batch_fx_real(ctx, nt, tr, roots, status, tu, fin);
-    case GBS_PREC_FXW: return batch_fxw_real(ctx, nt, tr, roots, status, tu, fin);
-  }
-  return set_error(ctx, GBS_EINVAL, "unknown precision");
+  return e(ctx, nt, tr, roots, status, batch_tune_for(ctx, fixed64 ? (int)GBS_PREC_FXN : prec, real), fin);
 }
 
 gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const BatchTree* trees, const void* roots_dev,
@@ -261,39 +246,23 @@ gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const Batch
   };
   const size_t n = (size_t)ntrees;
   auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t bytes = r256(n * sizeof(TreeOut)) + r256(n * sizeof(ProbOut)) + r256(2 * n * sizeof(int));
+  const size_t bytes = r256(n * sizeof(ProbOut)) + r256(2 * n * sizeof(int));
   if ((st = dev_reserve(ctx, ctx->aux_dev, bytes))) return st;
-  unsigned char* base = (unsigned char*)ctx->aux_dev.ptr;
-  TreeOut* outs = (TreeOut*)base;
-  ProbOut* po = (ProbOut*)(base + ((n * sizeof(TreeOut) + 255) / 256) * 256);
-  int* status = (int*)((unsigned char*)po + ((n * sizeof(ProbOut) + 255) / 256) * 256);
+  ProbOut* po = (ProbOut*)ctx->aux_dev.ptr;
+  int* status = (int*)((unsigned char*)po + r256(n * sizeof(ProbOut)));  // then the counters
   if ((st = check_cuda(ctx, cudaMemsetAsync(status, 0, 2 * n * sizeof(int), ctx->stream), "memset"))) return st;
   ctx->batch_split = false;
   const double u = unit_roundoff_b(prec), extra = err_factor(prec, 1) - err_factor(GBS_PREC_TD, 1);
   const bool fixed64 = bounded && real && prec == GBS_PREC_FP64;
-  if (fixed64 || is_fixed_point(prec)) {
-    if (!real) return set_error(ctx, GBS_EINVAL, "the fixed-point precision needs the real basis");
-    st = fixed_variant(ctx, prec, ntrees, trees, roots_dev, status, FxFinish{logdet, u, extra, po, status + n});
-  } else {
-    st = batch_variant(ctx, prec, real, ntrees, trees, roots_dev, outs, status);
-  }
-  if (st) {
+  std::vector<double> scale(n);
+  for (size_t t = 0; t < n; ++t) scale[t] = std::exp(-0.5 * logdet[t]);
+  if ((st = batch_variant(ctx, prec, real, fixed64, ntrees, trees, roots_dev, status,
+                          TreeFinish{scale.data(), u, extra, po, status + n}))) {
     if (st == GBS_ENOMEM && ctx->batch_split) {
       ctx->batch_split = false;
       return split();
     }
     return st;
-  }
-  if (!fixed64 && !is_fixed_point(prec)) {
-    std::vector<int> nm(n);
-    for (size_t t = 0; t < n; ++t) nm[t] = trees[t].n;
-    const void *d_logdet = nullptr, *d_n = nullptr;
-    if ((st = stage(ctx, logdet, n * sizeof(double), &d_logdet)) || (st = stage(ctx, nm.data(), n * sizeof(int), &d_n)))
-      return st;
-    batch_finish_kernel<<<(ntrees + 127) / 128, 128, 0, ctx->stream>>>(
-        outs, status, (const double*)d_logdet, (const int*)d_n, u, extra, ntrees, po);
-    count_launch(ctx);
-    if ((st = check_cuda(ctx, cudaGetLastError(), "finish"))) return st;
   }
   if ((st = check_cuda(ctx, cudaMemcpyAsync(host_out, po, n * sizeof(ProbOut), cudaMemcpyDeviceToHost, ctx->stream),
                        "readback")) ||

@@ -24,8 +24,8 @@ struct Blob {
 // PAIR: the last two levels of every tree as cancellation-free groups (FP64
 // real basis; the tree's inc output then carries the whole Torontonian).
 template <class E, int QMAX, bool PAIR = false>
-gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots_dev, TreeOut* outs_dev,
-                     int* status_dev, const BatchTune& tune) {
+gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const void* roots_dev, int* status_dev,
+                     const BatchTune& tune, const TreeFinish& fin) {
   typedef typename real_of<E>::type T;
   typedef typename real_of<E>::type S;
   typedef typename acc_traits<T>::Red Red;
@@ -147,14 +147,20 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
     parts_total += grp_blocks[qv];
   }
   for (int t = 0; t < ntrees; ++t) ranges[t].first += part_base[Q[t]];
-  // two-stage reduction: chunks of <= 128 partials of one tree, then one warp per tree
+  // reduction: one CTA per tree over its partials, or over the sums of chunks of <= 128
+  // of them (behind the partials) where it has thousands; by the tree alone, so that its
+  // sum does not depend on its batch
   std::vector<PartChunk> chunks;
-  std::vector<PartRange> ranges2(ntrees);
+  std::vector<PartRange> ranges2 = ranges;
+  long long part_max = 0;  // the longest range
   for (int t = 0; t < ntrees; ++t) {
-    ranges2[t].first = (long long)chunks.size();
-    for (long long i = 0; i < ranges[t].count; i += 128)
-      chunks.push_back(PartChunk{ranges[t].first + i, std::min<long long>(128, ranges[t].count - i)});
-    ranges2[t].count = (long long)chunks.size() - ranges2[t].first;
+    if (ranges[t].count > 2048) {
+      ranges2[t].first = parts_total + (long long)chunks.size();
+      for (long long i = 0; i < ranges[t].count; i += 128)
+        chunks.push_back(PartChunk{ranges[t].first + i, std::min<long long>(128, ranges[t].count - i)});
+      ranges2[t].count = (ranges[t].count + 127) / 128;
+    }
+    part_max = std::max(part_max, ranges2[t].count);
   }
 
   // ---------------- memory
@@ -179,6 +185,10 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
   for (int qv = 1; qv <= QMAX; ++qv) o_leaf[qv] = sub_e > 0 ? blob.put(subs[qv]) : blob.put(leaf[qv]);
   const size_t o_chk = blob.put(chunks);
   const size_t o_rng = blob.put(ranges2);
+  std::vector<int> nm(ntrees);
+  for (int t = 0; t < ntrees; ++t) nm[t] = trees[t].n;
+  const size_t o_n = blob.put(nm);
+  const size_t o_sc = blob.put(std::vector<double>(fin.scale, fin.scale + ntrees));
   const unsigned char* plan = nullptr;
   if ((st = stage(ctx, blob.bytes.data(), blob.bytes.size(), (const void**)&plan))) return st;
 
@@ -186,7 +196,6 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
   E* buf[2] = {(E*)ctx->lvl[0].ptr, (E*)ctx->lvl[1].ptr};
   S* sb[2] = {(S*)ctx->sbuf[0].ptr, (S*)ctx->sbuf[1].ptr};
   Partial<Red>* parts = (Partial<Red>*)ctx->partials.ptr;
-  Partial<Red>* parts2 = parts + parts_total;
 
   // ---------------- top
   // The opt-in limit is set whatever the size: the kernels' static shared
@@ -257,12 +266,16 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
     cudaEventRecord(ctx->leaf_timer.stop, s);
     ctx->leaf_timer.pending = true;
   }
-  // ---------------- per-tree reduction in two fixed-order stages
-  batch_chunk_kernel<Red><<<(unsigned)chunks.size(), 128, 0, s>>>(parts, (const PartChunk*)(plan + o_chk),
-                                                                 (int)chunks.size(), parts2);
-  batch_final_kernel<Red><<<(ntrees * 32 + 255) / 256, 256, 0, s>>>(parts2, (const PartRange*)(plan + o_rng), ntrees,
-                                                                     outs_dev);
-  count_launch(ctx, 2);
+  // ---------------- per-tree reduction
+  if (!chunks.empty()) {
+    batch_chunk_kernel<Red><<<(unsigned)chunks.size(), 128, 0, s>>>(parts, (const PartChunk*)(plan + o_chk),
+                                                                   (int)chunks.size(), parts + parts_total);
+    count_launch(ctx);
+  }
+  batch_final_kernel<Red><<<(unsigned)ntrees, part_max > 128 ? 256 : part_max > 32 ? 128 : 32, 0, s>>>(
+      parts, (const PartRange*)(plan + o_rng), status_dev, (const double*)(plan + o_sc), (const int*)(plan + o_n),
+      fin.u, fin.extra, fin.po);
+  count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "batch launch");
 }
 

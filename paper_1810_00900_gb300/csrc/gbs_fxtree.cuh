@@ -200,7 +200,7 @@ __device__ __forceinline__ void fx_st(uint32_t* p, int e, const E& v) {
 // s of it is element s_base + v (v < 2^d0), s_base + 2^d0 - 2^cb + v'.
 struct FxTree {
   long long root_off, s_base;
-  double logdet;
+  double scale;  // det(Sigma)^(-1/2)
   int n, D, tree, tab, d0, cb;
 };
 struct FxSeg {
@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* __restr
   fx_store3(inc, o.inc);
   fx_store3(exc, o.exc);
   o.abs = to_double(mag);
-  out[tr.tree] = finish_tree(o, status[tr.tree], tr.logdet, tr.n, u, extra);
+  out[tr.tree] = finish_tree(o, status[tr.tree], tr.scale, tr.n, u, extra);
 }
 
 // -------------------------------------------------------------- small trees --
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* __restr
 struct FxSmall {
   long long first;  // first CTA (and partial sum) of this tree
   long long root_off;
-  double logdet;
+  double scale;  // det(Sigma)^(-1/2)
   int n, d0, tree, pad;
 };
 
@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(512) fx_small_kernel(const FxSmall* __restrict
   fx_store3(sum.inc, o.inc);
   fx_store3(sum.exc, o.exc);
   o.abs = to_double(sum.abs);
-  out[t.tree] = finish_tree(o, st, t.logdet, t.n, u, extra);
+  out[t.tree] = finish_tree(o, st, t.scale, t.n, u, extra);
 }
 
 }  // namespace gbs

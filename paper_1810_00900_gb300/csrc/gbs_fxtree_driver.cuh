@@ -38,7 +38,7 @@ void fx_launch(bool early, void (*kernel)(P...), unsigned grid, unsigned block, 
 
 template <class E>
 gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const void* roots_dev, int* status_dev,
-                        const BatchTune& tune, const FxFinish& fin) {
+                        const BatchTune& tune, const TreeFinish& fin) {
   typedef typename fx_sum<E>::type S;
   constexpr int L = sizeof(E) / 4;
   // Small trees (fx_small_kernel): one CTA for up to kOne modes, whose levels fit its
@@ -67,7 +67,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
       continue;
     }
     const int d0 = several ? n - kSub : 0;
-    small[several].push_back(FxSmall{blocks[several], in[i].root_off, fin.logdet[i], n, d0, i, 0});
+    small[several].push_back(FxSmall{blocks[several], in[i].root_off, fin.scale[i], n, d0, i, 0});
     blocks[several] += 1LL << d0;
     small_n[several] = std::max(small_n[several], n);
   }
@@ -121,7 +121,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   for (int i = 0; i < ntrees; ++i) {
     const BatchTree& b = in[order[i]];
     Q[i] = std::min(b.n, Qmax);
-    trees[i] = FxTree{b.root_off, 0, fin.logdet[order[i]], b.n, b.n - Q[i], order[i], 34 * i, 0, 0};
+    trees[i] = FxTree{b.root_off, 0, fin.scale[order[i]], b.n, b.n - Q[i], order[i], 34 * i, 0, 0};
   }
   const int D0 = trees[0].D;
   // A single tree too large for the workspace goes in chunks of 2^cb nodes of depth d0

@@ -27,8 +27,6 @@ constexpr bool is_fixed_point(int prec) {
   return prec == GBS_PREC_FXN || prec == GBS_PREC_FX || prec == GBS_PREC_FXW;
 }
 
-struct TreeOut;
-
 // One tree of a batch: n modes, packed FP64 root starting at entry root_off.
 struct BatchTree {
   int n;
@@ -166,29 +164,22 @@ struct ProbOut {
   int pad;
 };
 
-gbs_status batch_fp64_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_fp64_cplx(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_dd_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_dd_cplx(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_td_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_td_cplx(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_fp64p_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_fp32_real(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
-gbs_status batch_fp32_cplx(gbs_ctx*, int, const BatchTree*, const void*, TreeOut*, int*, const BatchTune&);
 
-// Fixed-point trees finish their results on the device: log det (host, per tree), unit
-// and extra terms of the error model, where the results go (device), and a zeroed
-// counter per tree (device).
-struct FxFinish {
-  const double* logdet;
+// The engines finish their results on the device: det(Sigma)^(-1/2) (host, per tree), unit and
+// extra terms of the error model, where the results go (device), and a zeroed counter per
+// tree (device).
+struct TreeFinish {
+  const double* scale;
   double u, extra;
   ProbOut* po;
   int* counts;
 };
-gbs_status batch_fxd_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
-gbs_status batch_fxn_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
-gbs_status batch_fx_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
-gbs_status batch_fxw_real(gbs_ctx*, int, const BatchTree*, const void*, int*, const BatchTune&, const FxFinish&);
+typedef gbs_status BatchEngine(gbs_ctx*, int ntrees, const BatchTree*, const void* roots, int* status, const BatchTune&,
+                               const TreeFinish&);
+BatchEngine batch_fp64_real, batch_fp64_cplx, batch_dd_real, batch_dd_cplx, batch_td_real, batch_td_cplx, batch_fp32_real,
+    batch_fp32_cplx, batch_fp64p_real;
+// the fixed-point engine (fxd: FP64 precision with 64 fraction bits)
+BatchEngine batch_fxd_real, batch_fxn_real, batch_fx_real, batch_fxw_real;
 
 // Evaluate ntrees trees whose packed FP64 roots are already in roots_dev
 // (entries at trees[t].root_off); logdet[t] (host) scales p = Tor exp(-logdet/2).

@@ -426,25 +426,31 @@ __device__ __forceinline__ void block_reduce_sums(double ip, double in, double e
   }
 }
 
+// Sums over a block into *out: a shuffle tree per warp, then one over the warps (a serial
+// loop over them was 8 dependent double-double additions).
 template <class Red>
 __device__ __forceinline__ void block_reduce_store(Red inc, Red exc, double asum, Partial<Red>* out) {
   __shared__ Red s_inc[32], s_exc[32];
   __shared__ double s_abs[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto warp_sum = [&]() {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    inc = red_add(inc, shfl_down(inc, off));
-    exc = red_add(exc, shfl_down(exc, off));
-    asum += __shfl_down_sync(0xffffffffu, asum, off);
-  }
+    for (int off = 16; off > 0; off >>= 1) {
+      inc = red_add(inc, shfl_down(inc, off));
+      exc = red_add(exc, shfl_down(exc, off));
+      asum += __shfl_down_sync(0xffffffffu, asum, off);
+    }
+  };
+  warp_sum();
   if (lane == 0) { s_inc[warp] = inc; s_exc[warp] = exc; s_abs[warp] = asum; }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (warp == 0) {
     const int nw = (blockDim.x + 31) >> 5;
-    Red a = s_inc[0], b = s_exc[0];
-    double c = s_abs[0];
-    for (int w = 1; w < nw; ++w) { a = red_add(a, s_inc[w]); b = red_add(b, s_exc[w]); c += s_abs[w]; }
-    out->inc = a; out->exc = b; out->abs = c;
+    inc = lane < nw ? s_inc[lane] : red_zero<Red>();
+    exc = lane < nw ? s_exc[lane] : red_zero<Red>();
+    asum = lane < nw ? s_abs[lane] : 0.0;
+    if (nw > 1) warp_sum();
+    if (lane == 0) { out->inc = inc; out->exc = exc; out->abs = asum; }
   }
 }
 
