@@ -87,78 +87,176 @@ struct ClickReq {
   const double* alpha;
   const double* beta;
   const cplx<double>* Sinv;   // dense form (when U is null)
-  long long pair_begin;
   long long root_off;
   int M, N;
   ModeList S;
 };
 
-// One warp per (request, mode pair j >= k); writes the packed lower triangle.
-__global__ void batch_click_block_kernel(const ClickReq* __restrict__ reqs, int nreq, long long total_pairs,
-                                         int real_basis, void* __restrict__ roots) {
-  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= total_pairs) return;
-  int lo = 0, hi = nreq - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (reqs[mid].pair_begin <= w) lo = mid; else hi = mid - 1;
-  }
-  const ClickReq& q = reqs[lo];
-  const int p = (int)(w - q.pair_begin);
-  int j = 0;
-  while ((j + 1) * (j + 2) / 2 <= p) ++j;
-  const int k = p - j * (j + 1) / 2;
-  const int M = q.M;
-  double ar = 0, ai = 0, br = 0, bi = 0;  // A = (Sigma^-1)_{a_j a_k}, B = (Sigma^-1)_{a_j a^+_k}
-  cplx<double> h10{0, 0}, h11{0, 0};
-  if (q.U) {
-    const cplx<double>* uj = q.U + (long long)q.S.m[j] * M;
-    const cplx<double>* uk = q.U + (long long)q.S.m[k] * M;
-    for (int l = lane; l < M; l += 32) {
-      const cplx<double> x = uj[l], y = uk[l];
-      const double pr = x.re * y.re + x.im * y.im, pi = x.im * y.re - x.re * y.im;
-      const double qr = x.re * y.re - x.im * y.im, qi = x.re * y.im + x.im * y.re;
-      ar = fma(pr, q.alpha[l], ar);
-      ai = fma(pi, q.alpha[l], ai);
-      br = fma(qr, q.beta[l], br);
-      bi = fma(qi, q.beta[l], bi);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      ar += __shfl_down_sync(0xffffffffu, ar, off);
-      ai += __shfl_down_sync(0xffffffffu, ai, off);
-      br += __shfl_down_sync(0xffffffffu, br, off);
-      bi += __shfl_down_sync(0xffffffffu, bi, off);
-    }
-    h10 = {br, -bi};
-    h11 = {ar, -ai};
-  } else if (lane == 0) {
-    const long long D = 2LL * M;
-    const long long rj = q.S.m[j], rk = q.S.m[k];
-    const cplx<double> h00 = q.Sinv[rj * D + rk], h01 = q.Sinv[rj * D + rk + M];
-    h10 = q.Sinv[(rj + M) * D + rk];
-    h11 = q.Sinv[(rj + M) * D + rk + M];
-    ar = h00.re; ai = h00.im; br = h01.re; bi = h01.im;
-  }
-  if (lane != 0) return;
-  if (j == k) { ai = 0.0; h11.im = 0.0; }
+// The 2 x 2 block of (Sigma^-1) between two modes: [[h00, h01], [h10, h11]] in (a, a^+).
+struct ClickEntry {
+  cplx<double> h00, h01, h10, h11;
+};
+__device__ __forceinline__ ClickEntry click_entry_dense(const ClickReq& q, int j, int k) {
+  const long long M = q.M, D = 2 * M;
+  const long long rj = q.S.m[j], rk = q.S.m[k];
+  return ClickEntry{q.Sinv[rj * D + rk], q.Sinv[rj * D + rk + M], q.Sinv[(rj + M) * D + rk], q.Sinv[(rj + M) * D + rk + M]};
+}
+// Writes the block of mode pair (j, k) into the request's packed root.
+__device__ __forceinline__ void click_store(const ClickReq& q, int j, int k, ClickEntry h, int real_basis,
+                                            void* __restrict__ roots) {
+  if (j == k) h.h00.im = h.h11.im = 0.0;
   const int a0 = 2 * j, b0 = 2 * k;
   auto T3 = [](int a, int b) { return a * (a + 1) / 2 + b; };
   if (real_basis) {
-    // q^+ h q with q = [[1, i], [1, -i]]/sqrt2, h = [[h00, h01], [h10, h11]]
+    // q^+ h q with q = [[1, i], [1, -i]]/sqrt2
     double* o = (double*)roots + q.root_off;
-    o[T3(a0, b0)] = 0.5 * (ar + br + h10.re + h11.re);
-    o[T3(a0 + 1, b0)] = 0.5 * ((ai + bi) - (h10.im + h11.im));
-    o[T3(a0 + 1, b0 + 1)] = 0.5 * ((ar - br) - (h10.re - h11.re));
-    if (j != k) o[T3(a0, b0 + 1)] = -0.5 * (ai - bi + h10.im - h11.im);
+    o[T3(a0, b0)] = 0.5 * (h.h00.re + h.h01.re + h.h10.re + h.h11.re);
+    o[T3(a0 + 1, b0)] = 0.5 * ((h.h00.im + h.h01.im) - (h.h10.im + h.h11.im));
+    o[T3(a0 + 1, b0 + 1)] = 0.5 * ((h.h00.re - h.h01.re) - (h.h10.re - h.h11.re));
+    if (j != k) o[T3(a0, b0 + 1)] = -0.5 * (h.h00.im - h.h01.im + h.h10.im - h.h11.im);
   } else {
     cplx<double>* o = (cplx<double>*)roots + q.root_off;
-    o[T3(a0, b0)] = {ar, ai};
-    o[T3(a0 + 1, b0)] = h10;
-    o[T3(a0 + 1, b0 + 1)] = h11;
-    if (j != k) o[T3(a0, b0 + 1)] = {br, bi};
+    o[T3(a0, b0)] = h.h00;
+    o[T3(a0 + 1, b0)] = h.h10;
+    o[T3(a0 + 1, b0 + 1)] = h.h11;
+    if (j != k) o[T3(a0, b0 + 1)] = h.h01;
   }
+}
+
+// Mode pair (j, k) of index p in the packed triangle.
+__device__ __forceinline__ void click_pair(int p, int* j, int* k) {
+  int r = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
+  while (r * (r + 1) / 2 > p) --r;
+  while ((r + 1) * (r + 2) / 2 <= p) ++r;
+  *j = r;
+  *k = p - r * (r + 1) / 2;
+}
+// The sums over l of A = (Sigma^-1)_{a_j a_k}, B = (Sigma^-1)_{a_j a^+_k}: runs of kClickL
+// in kClickS strided parts of 8, the parts summed over the runs and joined in pairs.  Both
+// kernels below add the same numbers in this order, so a request's root does not depend
+// on its batch; its rounding is that of a sum over 32 lanes.
+constexpr int kClickS = 4, kClickL = 32;
+struct ClickSum {
+  double ar = 0, ai = 0, br = 0, bi = 0;
+  __device__ __forceinline__ void step(cplx<double> x, cplx<double> v, double alpha, double beta) {
+    const double rr = x.re * v.re, ri = x.re * v.im;
+    ar = fma(fma(x.im, v.im, rr), alpha, ar);
+    ai = fma(fma(x.im, v.re, -ri), alpha, ai);
+    br = fma(fma(-x.im, v.im, rr), beta, br);
+    bi = fma(fma(x.im, v.re, ri), beta, bi);
+  }
+  __device__ __forceinline__ void add(const ClickSum& o) {
+    ar += o.ar;
+    ai += o.ai;
+    br += o.br;
+    bi += o.bi;
+  }
+  // lane i's of each 16 lanes
+  __device__ __forceinline__ ClickSum from(int i) const {
+    return ClickSum{__shfl_sync(0xffffffffu, ar, i, 16), __shfl_sync(0xffffffffu, ai, i, 16),
+                    __shfl_sync(0xffffffffu, br, i, 16), __shfl_sync(0xffffffffu, bi, i, 16)};
+  }
+  __device__ __forceinline__ ClickEntry entry() const { return ClickEntry{{ar, ai}, {br, bi}, {br, -bi}, {ar, -ai}}; }
+};
+
+// Few requests: kClickG groups of kClickS lanes per (request, mode pair j >= k), a run a
+// group, blockIdx.x the request; writes the packed lower triangle.  Bound by the latency
+// of the loads, which a lane issues together.
+constexpr int kClickG = 4, kClickPair = kClickG * kClickS;
+__global__ void __launch_bounds__(128) batch_click_block_kernel(const ClickReq* __restrict__ reqs, int real_basis,
+                                                                void* __restrict__ roots) {
+  __shared__ ClickReq q;
+  for (int i = threadIdx.x; i < (int)(sizeof(ClickReq) / 4); i += blockDim.x)
+    reinterpret_cast<int*>(&q)[i] = reinterpret_cast<const int*>(reqs + blockIdx.x)[i];
+  __syncthreads();
+  const int M = q.M, lane = threadIdx.x % kClickPair, pairs = q.N * (q.N + 1) / 2;
+  const int p = blockIdx.y * (blockDim.x / kClickPair) + threadIdx.x / kClickPair;
+  int j, k;
+  click_pair(min(p, pairs - 1), &j, &k);
+  ClickEntry h{};
+  if (q.U) {
+    const cplx<double>* uj = q.U + (long long)q.S.m[j] * M;
+    const cplx<double>* uk = q.U + (long long)q.S.m[k] * M;
+    const int l_first = lane / kClickS * kClickL + lane % kClickS;
+    ClickSum t;
+    for (int l0 = 0; l0 < M; l0 += kClickG * kClickL) {
+      constexpr int kT = kClickL / kClickS;
+      cplx<double> x[kT], v[kT];
+      double wa[kT], wb[kT];
+#pragma unroll
+      for (int i = 0; i < kT; ++i) {
+        const int l = min(l0 + l_first + i * kClickS, M - 1);
+        x[i] = uj[l];
+        v[i] = uk[l];
+        wa[i] = q.alpha[l];
+        wb[i] = q.beta[l];
+      }
+      ClickSum run;
+#pragma unroll
+      for (int i = 0; i < kT; ++i)
+        if (l0 + l_first + i * kClickS < M) run.step(x[i], v[i], wa[i], wb[i]);
+      // the groups' runs in order (one beyond the last is zero)
+#pragma unroll
+      for (int g = 0; g < kClickG; ++g) t.add(run.from(g * kClickS + lane % kClickS));
+    }
+#pragma unroll
+    for (int off = kClickS / 2; off > 0; off >>= 1) t.add(t.from(lane % kClickS + off));
+    h = t.entry();
+  } else {
+    h = click_entry_dense(q, j, k);
+  }
+  if (lane == 0 && p < pairs) click_store(q, j, k, h, real_basis, roots);
+}
+
+// Many requests: a CTA per request and 128 pairs, a thread per pair, the rows of U staged
+// in shared memory: nothing is summed across lanes (a warp per pair spends 20 of its FP64
+// additions on that, more than on the products of a small state).  1500 requests of
+// 5 .. 17 of 17 modes: 314 us with a warp per pair, 90 so.  From a request per SM on;
+// fewer fill the chip better with lanes per pair.
+__global__ void __launch_bounds__(128) batch_click_tile_kernel(const ClickReq* __restrict__ reqs, int real_basis,
+                                                               void* __restrict__ roots) {
+  __shared__ ClickReq q;
+  __shared__ cplx<double> x[32][kClickL + 1];
+  __shared__ double wa[kClickL], wb[kClickL];
+  for (int i = threadIdx.x; i < (int)(sizeof(ClickReq) / 4); i += blockDim.x)
+    reinterpret_cast<int*>(&q)[i] = reinterpret_cast<const int*>(reqs + blockIdx.x)[i];
+  __syncthreads();
+  const int p = blockIdx.y * blockDim.x + threadIdx.x, pairs = q.N * (q.N + 1) / 2, M = q.M;
+  if ((int)(blockIdx.y * blockDim.x) >= pairs) return;
+  int j, k;
+  click_pair(min(p, pairs - 1), &j, &k);
+  ClickEntry h{};
+  if (q.U) {
+    ClickSum t[kClickS];
+    for (int l0 = 0; l0 < M; l0 += kClickL) {
+      const int len = min(kClickL, M - l0);
+      for (int e = threadIdx.x; e < q.N * kClickL; e += blockDim.x) {
+        const int r = e / kClickL, c = e % kClickL;
+        if (c < len) x[r][c] = q.U[(long long)q.S.m[r] * M + l0 + c];
+      }
+      if ((int)threadIdx.x < len) {
+        wa[threadIdx.x] = q.alpha[l0 + threadIdx.x];
+        wb[threadIdx.x] = q.beta[l0 + threadIdx.x];
+      }
+      __syncthreads();
+      ClickSum run[kClickS];
+      for (int c = 0; c < len; c += kClickS)
+#pragma unroll
+        for (int s = 0; s < kClickS; ++s)
+          if (c + s < len) run[s].step(x[j][c + s], x[k][c + s], wa[c + s], wb[c + s]);
+#pragma unroll
+      for (int s = 0; s < kClickS; ++s) t[s].add(run[s]);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int off = kClickS / 2; off > 0; off >>= 1)
+#pragma unroll
+      for (int s = 0; s < off; ++s) t[s].add(t[s + off]);
+    h = t[0].entry();
+  } else {
+    h = click_entry_dense(q, j, k);
+  }
+  if (p < pairs) click_store(q, j, k, h, real_basis, roots);
 }
 
 // A-priori cancellation estimate of each tree: the ratio sum|t| / |Tor| the
@@ -300,7 +398,8 @@ gbs_status batch_click_blocks(gbs_ctx* ctx, int nreq, const gbs_state* const* st
                               const int* N, bool real, std::vector<BatchTree>& trees) {
   std::vector<ClickReq> reqs;
   trees.resize(nreq);
-  long long pairs = 0, ent = 0;
+  long long ent = 0;
+  int n_max = 0;
   for (int i = 0; i < nreq; ++i) {
     ClickReq q{};
     const gbs_state* st = states[i];
@@ -311,10 +410,9 @@ gbs_status batch_click_blocks(gbs_ctx* ctx, int nreq, const gbs_state* const* st
     q.M = st->M;
     q.N = N[i];
     for (int j = 0; j < 32; ++j) q.S.m[j] = j < N[i] ? modes[i][j] : 0;
-    q.pair_begin = pairs;
     q.root_off = ent;
     trees[i] = BatchTree{N[i], ent};
-    pairs += (long long)N[i] * (N[i] + 1) / 2;
+    n_max = std::max(n_max, N[i]);
     ent += (long long)N[i] * (2 * N[i] + 1);  // sym(2N)
     if (N[i] > 0) reqs.push_back(q);
   }
@@ -323,9 +421,12 @@ gbs_status batch_click_blocks(gbs_ctx* ctx, int nreq, const gbs_state* const* st
   if (reqs.empty()) return GBS_OK;
   const void* d = nullptr;
   if ((st = stage(ctx, reqs.data(), reqs.size() * sizeof(ClickReq), &d))) return st;
-  const long long threads = pairs * 32;
-  batch_click_block_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, ctx->stream>>>(
-      (const ClickReq*)d, (int)reqs.size(), pairs, real ? 1 : 0, ctx->hbuf.ptr);
+  const int pairs = n_max * (n_max + 1) / 2;
+  const bool many = (int)reqs.size() >= ctx->sm_count;
+  const int per_cta = many ? 128 : 128 / kClickPair;
+  (many ? batch_click_tile_kernel : batch_click_block_kernel)<<<
+      dim3((unsigned)reqs.size(), (unsigned)((pairs + per_cta - 1) / per_cta)), 128, 0, ctx->stream>>>(
+      (const ClickReq*)d, real ? 1 : 0, ctx->hbuf.ptr);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "click blocks");
 }

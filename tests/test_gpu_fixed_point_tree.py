@@ -106,3 +106,24 @@ def test_chunks_of_a_tree_beyond_the_budget(ctx, prec):
             assert all(tuple(np.atleast_1d(x)) == tuple(np.atleast_1d(y)) for x, y in zip(want, got))
             assert c.launch_count > 15 and c.bytes_in_use <= budget
             c.close()
+
+
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("M", [1, 2, 15, 16, 17, 33, 66])
+def test_many_requests_get_the_roots_of_each_alone(ctx, M, dense):
+    """Enough requests for a CTA each: the bits of a few of them alone, whose mode pairs are
+    spread over lanes."""
+    p = gi.uniform_squeezed_state(M, 0.5, seed=M, eta=0.8)
+    st = gbs.build_state(ctx, p.U, p.r, p.eta)
+    if dense:
+        st.free()
+        st = gbs.state_from_V(ctx, oracle.covariance(p.U, p.r, p.eta))
+    rng = np.random.default_rng(M)
+    pats = [rng.permutation(M)[:rng.integers(1, min(M, 20 if i < 4 else 9) + 1)] for i in range(640)]
+    many = gbs.torontonian_batch(ctx, [st] * len(pats), pats, "fp64")
+    for i in list(range(4)) + [5, 639]:
+        for basis in ("real", "complex"):
+            a = gbs.torontonian(ctx, st, pats[i], "fp64", basis)
+            b = many[i] if basis == "real" else gbs.torontonian_batch(ctx, [st] * 320, [pats[i]] * 320, "fp64", basis)[7]
+            assert (a.tor, a.abs_sum, a.p) == (b.tor, b.abs_sum, b.p), (len(pats[i]), basis)
+    st.free()
