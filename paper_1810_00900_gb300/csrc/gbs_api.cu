@@ -3,7 +3,6 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <set>
 #include <vector>
 
 #include "gbs_internal.h"
@@ -103,13 +102,14 @@ gbs_status dev_reserve(gbs_ctx* ctx, DevBuf& b, size_t bytes) {
   return dev_alloc(ctx, b, bytes);
 }
 
-static gbs_status validate_modes(gbs_ctx* ctx, const int* modes, int N, int M) {
+gbs_status validate_modes(gbs_ctx* ctx, const int* modes, int N, int M) {
   if (N < 0 || N > 32) return set_error(ctx, GBS_EINVAL, "N must be in [0, 32]");
   if (N > 0 && !modes) return set_error(ctx, GBS_EINVAL, "modes is NULL");
-  std::set<int> seen;
   for (int i = 0; i < N; ++i) {
     if (modes[i] < 0 || modes[i] >= M) return set_error(ctx, GBS_EINVAL, "mode out of range");
-    if (!seen.insert(modes[i]).second) return set_error(ctx, GBS_EINVAL, "repeated mode");
+    bool seen = false;
+    for (int j = 0; j < i; ++j) seen |= modes[j] == modes[i];
+    if (seen) return set_error(ctx, GBS_EINVAL, "repeated mode");
   }
   return GBS_OK;
 }

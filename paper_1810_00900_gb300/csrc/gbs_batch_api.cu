@@ -5,7 +5,6 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
-#include <set>
 #include <vector>
 
 #include "gbs_batch_driver.cuh"
@@ -727,15 +726,8 @@ extern "C" gbs_status gbs_torontonian_batch(gbs_ctx* ctx, int n_req, const gbs_s
   long long off = 0;
   for (int i = 0; i < n_req; ++i) {
     if (!states[i] || states[i]->ctx != ctx) return set_error(ctx, GBS_EINVAL, "state of another context");
-    if (N_per[i] < 0 || N_per[i] > 32) return set_error(ctx, GBS_EINVAL, "N must be in [0, 32]");
-    if (N_per[i] > 0 && !modes) return set_error(ctx, GBS_EINVAL, "modes is NULL");
     mp[i] = modes ? modes + off : nullptr;
-    std::set<int> seen;
-    for (int j = 0; j < N_per[i]; ++j) {
-      const int m = mp[i][j];
-      if (m < 0 || m >= states[i]->M) return set_error(ctx, GBS_EINVAL, "mode out of range");
-      if (!seen.insert(m).second) return set_error(ctx, GBS_EINVAL, "repeated mode");
-    }
+    if (const gbs_status st = validate_modes(ctx, mp[i], N_per[i], states[i]->M)) return st;
     off += N_per[i];
   }
   if (n_req == 0) return GBS_OK;

@@ -136,6 +136,8 @@ gbs_status set_error(gbs_ctx* ctx, gbs_status st, const std::string& msg);
 gbs_status check_cuda(gbs_ctx* ctx, cudaError_t e, const char* what);
 gbs_status dev_alloc(gbs_ctx* ctx, DevBuf& b, size_t bytes);
 gbs_status dev_reserve(gbs_ctx* ctx, DevBuf& b, size_t bytes);  // grow-only
+// At most 32 modes in [0, M), none twice.
+gbs_status validate_modes(gbs_ctx* ctx, const int* modes, int N, int M);
 void dev_free(gbs_ctx* ctx, DevBuf& b);
 void cache_release(gbs_ctx* ctx);  // return cached device blocks to CUDA (cudaFree)
 inline void count_launch(gbs_ctx* ctx, long long n = 1) {
