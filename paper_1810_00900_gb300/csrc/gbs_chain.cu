@@ -10,13 +10,15 @@
 // for it: too many modes, another precision, a bound that misses the tolerance or a
 // value out of range; the next call then takes that step the other way.
 //
-// What bounds it is latency: at M = 100 a step takes ~22 us, about 10 in the tree's
-// phases, 8 in the conditioning (~A^2/2 FP64 updates of two FMAs each, at 2 per clock on
-// the one SM), 4 in the decision's chains of FP64 operations.  8 postselected samples of
-// a 100-mode graph state: 131 ms with a launch per operation, 45 here; 64 free samples
-// of 30 modes: 5.4 and 3.1.  At M = 200 the conditioning is up to 40 us a step, where
-// spreading it over the chip costs two launches and a wait: both ways took 45 ms for 24
-// trajectories of 200 modes, so kChainMaxM lies just beyond.
+// What bounds it is latency: at M = 100 a step takes ~20 us, about 10 in the tree's
+// phases, 4 in the decision's chains of FP64 operations, the rest in the conditioning
+// (~A^2/2 FP64 updates of two FMAs each, at 2 per clock and SM: 8 us on one SM, so the
+// CTAs of a cluster share it).  8 postselected samples of a 100-mode graph state: 131 ms
+// with a launch per operation, 39 here; 64 free samples of 30 modes: 5.4 and 3.2.  At M =
+// 200 the conditioning on one SM is up to 40 us a step; with a cluster 24 trajectories of
+// 200 modes take 39.4 ms, 42.8 without.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <chrono>
 #include <cstring>
@@ -61,7 +63,7 @@ struct ChainOut {
 
 // The trajectory's state between steps and what thread 0 tells the others.
 struct ChainShared {
-  int step, m, need_full, prec, stop, click, bad;
+  int step, m, need_full, prec, stop, click, bad, go, k;
   double kappa_prev, relD, dcarry[3];
   int clicks[40];
   ModePivot pv;
@@ -85,14 +87,79 @@ __device__ __noinline__ void chain_tree(unsigned char* smem, const double* sig, 
   __syncthreads();
 }
 
+// Conditions the active rows on mode k dark (its clicked modes are those before it): this
+// CTA's share of the rows, one of `parts`.  No row or column of mode k changes, so every CTA
+// forms the factors from Sigma' itself.
+__device__ __forceinline__ void chain_condition(unsigned char* smem, double* sig, long long D, const ChainShared& st,
+                                                int k, int m, int part, int parts) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int A = 2 * k + 2 * m;
+  const long long rk = 2LL * k;
+  double* u0 = reinterpret_cast<double*>(smem);
+  double *u1 = u0 + A, *l0 = u1 + A, *l1 = l0 + A;
+  int* row = reinterpret_cast<int*>(l1 + A);
+  const ModePivot pv = st.pv;
+  for (int i = tid; i < A; i += blockDim.x) {
+    const int ri = i < 2 * k ? i : 2 * st.clicks[(i - 2 * k) >> 1] + ((i - 2 * k) & 1);
+    const double a0 = sig_at(sig, D, ri, rk), a1 = sig_at(sig, D, ri, rk + 1);
+    row[i] = ri;
+    u0[i] = a0;
+    u1[i] = a1;
+    l0[i] = fma(a0, pv.q00, a1 * pv.q10);
+    l1[i] = fma(a0, pv.q10, a1 * pv.q11);
+  }
+  __syncthreads();
+  // a warp per row; four of its entries are in flight at a time (one at a time, the
+  // loads' latency was most of a step)
+  for (int i = (tid >> 5) * parts + part; i < A; i += (blockDim.x >> 5) * parts) {
+    const int ri = row[i];
+    const double x0 = l0[i], x1 = l1[i];
+    double* dst = sig + (long long)ri * D;
+    const int jmax = i < 2 * k ? i + 1 : A;
+    for (int c0 = lane; c0 < jmax; c0 += 128) {
+      double x[4];
+      int rc[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int c = c0 + 32 * q;
+        rc[q] = c < jmax ? row[c] : ri + 1;
+        if (rc[q] <= ri) x[q] = dst[rc[q]];
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int c = c0 + 32 * q;
+        if (rc[q] <= ri) dst[rc[q]] = fma(-x0, u0[c], fma(-x1, u1[c], x[q]));
+      }
+    }
+  }
+}
+
+// A cluster per trajectory: its first CTA takes the steps, the others (chain_cluster) only
+// their share of the conditioning.  All of a cluster's CTAs pass the same barriers: two per
+// conditioning, two at the end.
 __global__ void __launch_bounds__(512) chain_kernel(const ChainJob* __restrict__ jobs, ChainOut* __restrict__ outs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ ChainShared st;
   __shared__ TreeOut tree;
-  const ChainJob j = jobs[blockIdx.x];
-  ChainOut* out = outs + blockIdx.x;
+  const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int job = (int)(blockIdx.x / cluster.num_blocks());
+  const ChainJob j = jobs[job];
+  ChainOut* out = outs + job;
   const long long D = 2LL * j.M;
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x;
+  if (cluster.block_rank() != 0) {
+    const int* lead = reinterpret_cast<const int*>(cluster.map_shared_rank(&st, 0));
+    for (;;) {
+      cluster.sync();
+      for (int i = tid; i < (int)(sizeof(ChainShared) / 4); i += blockDim.x) reinterpret_cast<int*>(&st)[i] = lead[i];
+      __syncthreads();
+      if (!st.go) break;
+      chain_condition(smem_raw, j.sig, D, st, st.k, st.m, (int)cluster.block_rank(), (int)cluster.num_blocks());
+      cluster.sync();
+    }
+    cluster.sync();
+    return;
+  }
   int trees[6] = {0, 0, 0, 0, 0, 0}, near_ties = 0, uncertified = 0, steps = 0, code = kChainMore;  // thread 0's
   unsigned clicked = 0u;
   if (tid < j.m) st.clicks[tid] = j.clicks[tid];
@@ -197,47 +264,20 @@ __global__ void __launch_bounds__(512) chain_kernel(const ChainJob* __restrict__
     __syncthreads();
     if (st.stop) break;
     if (!st.click) {
-      // condition the active rows on mode k dark (its clicked modes are those before it)
-      const int A = 2 * k + 2 * m;
-      const long long rk = 2LL * k;
-      double* u0 = reinterpret_cast<double*>(smem_raw);
-      double *u1 = u0 + A, *l0 = u1 + A, *l1 = l0 + A;
-      int* row = reinterpret_cast<int*>(l1 + A);
-      const ModePivot pv = st.pv;
-      for (int i = tid; i < A; i += blockDim.x) {
-        const int ri = i < 2 * k ? i : 2 * st.clicks[(i - 2 * k) >> 1] + ((i - 2 * k) & 1);
-        const double a0 = sig_at(j.sig, D, ri, rk), a1 = sig_at(j.sig, D, ri, rk + 1);
-        row[i] = ri;
-        u0[i] = a0;
-        u1[i] = a1;
-        l0[i] = fma(a0, pv.q00, a1 * pv.q10);
-        l1[i] = fma(a0, pv.q10, a1 * pv.q11);
-      }
-      __syncthreads();
-      // a warp per row; four of its entries are in flight at a time (one at a time, the
-      // loads' latency was most of a step)
-      for (int i = tid >> 5; i < A; i += blockDim.x >> 5) {
-        const int ri = row[i];
-        const double x0 = l0[i], x1 = l1[i];
-        double* dst = j.sig + (long long)ri * D;
-        const int jmax = i < 2 * k ? i + 1 : A;
-        for (int c0 = lane; c0 < jmax; c0 += 128) {
-          double x[4];
-          int rc[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int c = c0 + 32 * q;
-            rc[q] = c < jmax ? row[c] : ri + 1;
-            if (rc[q] <= ri) x[q] = dst[rc[q]];
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int c = c0 + 32 * q;
-            if (rc[q] <= ri) dst[rc[q]] = fma(-x0, u0[c], fma(-x1, u1[c], x[q]));
-          }
+      if (cluster.num_blocks() > 1) {
+        if (tid == 0) {
+          st.go = 1;
+          st.k = k;
         }
+        cluster.sync();
       }
+      chain_condition(smem_raw, j.sig, D, st, k, m, 0, (int)cluster.num_blocks());
+      if (cluster.num_blocks() > 1) cluster.sync();
     }
+  }
+  if (cluster.num_blocks() > 1) {
+    if (tid == 0) st.go = 0;
+    cluster.sync();
   }
   if (tid == 0) {
     out->kappa_prev = st.kappa_prev;
@@ -251,6 +291,7 @@ __global__ void __launch_bounds__(512) chain_kernel(const ChainJob* __restrict__
     for (int i = 0; i < 6; ++i) out->trees[i] = trees[i];
     out->clicked = clicked;
   }
+  if (cluster.num_blocks() > 1) cluster.sync();  // the others have read st.go
 }
 
 }  // namespace
@@ -305,7 +346,23 @@ gbs_status chain_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int
                       "chain smem")))
     return e;
   const auto t0 = std::chrono::steady_clock::now();
-  chain_kernel<<<(unsigned)T, 512, smem, ctx->stream>>>((const ChainJob*)d_in, d_out);
+  // CTAs per trajectory: as many as the chip has room for, up to a portable cluster's 8.
+  // 8 trajectories of a 100-mode graph state, ms: 44.7 with one, 43.7, 41.5, 40.5 with 2, 4,
+  // 8; 24 of 200 modes 42.8, 41.4, 40.1; 64 of 30 modes 3.3 with one and two.
+  int parts = 1;
+  while (parts < 8 && (int)T * parts * 2 <= ctx->sm_count) parts *= 2;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = parts;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(T * parts));
+  cfg.blockDim = dim3(512);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, chain_kernel, (const ChainJob*)d_in, d_out);
   count_launch(ctx);
   std::vector<ChainOut> out(T);
   if ((e = check_cuda(ctx, cudaGetLastError(), "chain")) ||
