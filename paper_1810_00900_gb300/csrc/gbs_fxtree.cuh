@@ -798,6 +798,17 @@ template <class E>
 __device__ __forceinline__ void fxm_entry(const E* c, const FxRow<E>* a, const FxRow<E>* b, E* out) {
   *out = fx_entry(*c, a->P, a->Q, a->A, b->U, b->V, b->B);
 }
+// The pivot block of a child, entries (0, 0), (1, 0), (1, 1): c and d are the parent's
+// (0, 0) and (1, 0).  Together, so that their chains overlap.
+template <class E>
+__device__ __forceinline__ void fxm_block(const E* c, const E* d, const FxRowPad<E>* r, E* out) {
+  const E x = fx_entry(*c, r[0].P, r[0].Q, r[0].A, r[0].U, r[0].V, r[0].B);
+  const E y = fx_entry(d[0], r[1].P, r[1].Q, r[1].A, r[0].U, r[0].V, r[0].B);
+  const E z = fx_entry(d[1], r[1].P, r[1].Q, r[1].A, r[1].U, r[1].V, r[1].B);
+  out[0] = x;
+  out[1] = y;
+  out[2] = z;
+}
 template <class E, class S>
 __device__ __forceinline__ bool fxm_leaf1(const E* p00, const E* p10, const E* p11, const S* s, uint32_t neg,
                                           FxSums<S>* acc) {
@@ -818,6 +829,10 @@ template <class E>
 __device__ __noinline__ void fxc_entry(const E* c, const FxRow<E>* a, const FxRow<E>* b, E* out) {
   fxm_entry(c, a, b, out);
 }
+template <class E>
+__device__ __noinline__ void fxc_block(const E* c, const E* d, const FxRowPad<E>* r, E* out) {
+  fxm_block(c, d, r, out);
+}
 template <class E, class S>
 __device__ __noinline__ bool fxc_leaf1(const E* p00, const E* p10, const E* p11, const S* s, uint32_t neg,
                                        FxSums<S>* acc) {
@@ -834,6 +849,9 @@ struct FxOps {
   }
   static __device__ __forceinline__ void entry(const E* c, const FxRow<E>* a, const FxRow<E>* b, E* out) {
     if constexpr (CALL) fxc_entry(c, a, b, out); else fxm_entry(c, a, b, out);
+  }
+  static __device__ __forceinline__ void block(const E* c, const E* d, const FxRowPad<E>* r, E* out) {
+    if constexpr (CALL) fxc_block(c, d, r, out); else fxm_block(c, d, r, out);
   }
   static __device__ __forceinline__ bool leaf1(const E* p00, const E* p10, const E* p11, const S* s, uint32_t neg,
                                                FxSums<S>* acc) {
@@ -939,8 +957,9 @@ __device__ __forceinline__ FxPart<typename fx_sum<E>::type> fx_cta_tree(unsigned
       if (v < nc || k < 0) {
         m = node(v, q, o);
       } else {
-#pragma unroll 1
-        for (int e = 0; e < 3; ++e) entry(v - nc, e);
+        const E* par = node(v - nc, q + 1, o);
+        Op::block(par + tri(o + 2, o + 2), par + tri(o + 3, o + 2), rows + (v - nc) * R, dst + (v - nc) * ne);
+        o = 0;
         m = dst + (v - nc) * ne;
       }
       ok &= Op::pivot(m + tri(o, o), m + tri(o + 1, o), m + tri(o + 1, o + 1), piv + v);
