@@ -10,9 +10,10 @@ from the host each step.
 Output: one JSON line (rank 0).  `value` is device time (CUDA events around
 each step on the library's stream); `e2e` runs the same step through the public
 API from pinned host buffers (state build from U, r included) with wall-clock
-timing; `roofline` is the dominant kernel (the register depth-first leaf
-kernel) against the FP64 rate measured in the same run; `cpu_baseline` is the
-oracle timed on this host's cores on a bounded sample.
+timing; `roofline` is the leaf kernel against the rate, measured in the same run,
+of the pipe that it works on (the state bounds this tree, so FP64 evaluates it in
+64-bit fixed point: 32-bit multiply-adds); `cpu_baseline` is the oracle timed on
+this host's cores on a bounded sample.
 
 `--impl reference` times the oracle itself (the only reference there is: the
 paper's code is not available and ran on Titan CPUs) on a bounded sample.
@@ -77,8 +78,9 @@ def executed_flops(q: int, Q: int, complex_basis: bool = False) -> float:
 
 
 def fx_products(n: int) -> float:
-    """Fixed-point products of a whole tree of n modes, in units of one product of two
-    FX entries (six 32-bit limbs: 26 partial products of 32 x 32 bits).  Every node
+    """Fixed-point products of a whole tree of n modes in the plain form of its steps, in
+    units of one product of two FX entries (six 32-bit limbs: 26 partial products of 32 x 32
+    bits); what the kernels execute is fx_macs.  Every node
     with m >= 2 undecided modes forms its include child: pivot determinant (2),
     inverse square root (89 partial products of short operands: 3.42), 1/det (1),
     the scaled inverse (3), s g (a 7-limb scale: 39 partial products, 1.5),
@@ -90,6 +92,45 @@ def fx_products(n: int) -> float:
         t = n - d - 1
         total += 2.0 ** d * (2.0 + R + 1.0 + 3.0 + SG + 8.0 * t + 2.0 * t * (2 * t + 1))
     return total + 2.0 ** (n - 1) * (2.0 + R + SG)
+
+
+# fraction limbs F of the fixed-point types (entries have F + 1 limbs, s and the sums LS), and the
+# multiply-adds of an inverse square root
+FX_TYPES = {"fp64": (2, 5, 12), "fxn": (4, 6, 33), "fx": (5, 7, 39), "fxw": (6, 8, 45)}
+
+
+def fx_macs(n: int, prec: str) -> float:
+    """32 x 32-bit multiply-adds that the kernels execute for all subsets of n modes.  Every node
+    with m >= 2 undecided modes forms its include child: the pivot (two products and two squares
+    for det and 1/det = g^2, three products for the scaled inverse, the inverse square root, s g),
+    five products per row of 2(m-1) rows and one per lower-triangle entry (Winograd's inner
+    product); a one-mode node forms det, its inverse square root and s g."""
+    F, LS, R = FX_TYPES[prec]
+    L = F + 1
+    lo = F - 1  # columns lo .. F + (limbs of the result) - 1 are formed
+
+    def product(la):
+        return sum(1 for i in range(la) for j in range(L) if lo <= i + j < F + la)
+
+    square = sum(1 for i in range(L) for j in range(i, L) if lo <= i + j < F + L)
+    p, sg = product(L), product(LS)
+    total = 2.0 ** (n - 1) * (p + square + R + sg)
+    for d in range(n - 1):
+        t = n - d - 1
+        total += 2.0 ** d * (4 * p + 2 * square + R + sg + (10 * t + sym(2 * t)) * p)
+    return total
+
+
+FX_PRODUCT_MACS = 26.0  # of the product that gbs_measure_fx_peak times
+
+
+def fixed_point(prec: str, complex_basis: bool, N: int, r: float) -> bool:
+    """Whether the tree of N click modes of the uniformly squeezed pure state runs on the
+    fixed-point engine: FP64 does where the state bounds the tree."""
+    sigma_max = (math.exp(2 * r) + 1) / 2
+    if complex_basis or prec not in FX_TYPES:
+        return False
+    return prec != "fp64" or (sigma_max <= 16 and N * math.log2(1 + sigma_max) < 92)
 
 
 class ClockSampler:
@@ -217,19 +258,15 @@ def other_accountings(n: int, step_s: float):
 
 def captured_traffic(args, tuning):
     """DRAM bytes (read + write) per launch of the dominant kernel, from an ncu capture of the same
-    kernel code and launch shape (FP64 real basis, N = 24, the shared-memory levels and register
-    depth given here); None for any other shape, or once the kernel changed since the capture."""
-    return CAPTURED_TRAFFIC.get((args.prec, args.basis, args.N, tuning["sub_e"], tuning["q_drop"],
-                                 tuning["grid_per_sm"]))
+    kernel code (FP64 real basis, N = 24); None for any other shape, or once the kernel changed
+    since the capture."""
+    return CAPTURED_TRAFFIC.get((args.prec, args.basis, args.N))
 
 
-# (prec, basis, N, sub_e, q_drop, grid_per_sm) -> bytes per launch of the subtree kernel,
-# dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of the current kernel code
+# (prec, basis, N) -> bytes per launch of the leaf kernel, dram__bytes_read.sum +
+# dram__bytes_write.sum of one ncu capture of the current kernel code
 CAPTURED_TRAFFIC = {
-    # 2^15 depth-15 roots of 171 entries (44.8 MB of input) into one-warp CTAs of two roots each;
-    # one CTA per pair of roots (16,384 partials, which stay in L2) or 8 persistent CTAs per SM
-    ("fp64", "real", 24, 4, 0, 0): 45235456 + 39424,
-    ("fp64", "real", 24, 4, 0, 8): 45235456 + 4096000,
+    ("fp64", "real", 24): 572865024 + 5093632,
 }
 
 
@@ -300,7 +337,7 @@ def sampler_block(ctx, gbs, gi, n_traj, ws, local, autotune=True):
             # the late steps batch 64 trees of ~13..21 modes: tune on such a batch
             ctx.autotune(prec, "real", 21, n_trees=9)
         else:
-            ctx.set_tuning(prec, "real", sub_e=0, d_top=6, grid_per_sm=0, level_threads=1 << 17, q_drop=1, mid_e=0)
+            ctx.set_tuning(prec, "real", sub_e=0, d_top=10, grid_per_sm=0, level_threads=1 << 17, q_drop=0, mid_e=0)
     # the library draws the forced positions from the seed (the same as the workload's `clicks`)
     gbs.sample_forced_random(ctx, st, 2, seed=2, n_clicks=20)  # warm-up
     l0 = ctx.launch_count  # also locates the timed run in a launch list of the whole process
@@ -342,14 +379,15 @@ def certified_block(ctx, gbs, st, modes, steps, stream):
            "fx_tuning": ctx.tuning("fx", "real")}
     if res[-1].prec == "fx":
         peak = ctx.measure_fx_peak()
-        products = fx_products(24)
+        macs, per_s = fx_macs(24, "fx"), 1.0 / (ms * 1e-3)
         out["roofline"] = {
-            "bound": "alu", "unit": "G products/s", "achieved": products / (ms * 1e-3) / 1e9,
-            "peak": peak / 1e9, "frac": products / (ms * 1e-3) / peak,
+            "bound": "alu", "unit": "G 32-bit multiply-adds/s", "achieved": macs * per_s / 1e9,
+            "peak": peak * FX_PRODUCT_MACS / 1e9, "frac": macs * per_s / (peak * FX_PRODUCT_MACS),
             "scope": "the whole certified evaluation (click block, tree, reduction, readback)",
-            "products_per_term": products / 2.0 ** 24,
-            "model": "fx_products: 192-bit fixed-point products of the tree's Schur steps, "
-                     "inverse square roots and scale updates",
+            "multiply_adds_per_term": macs / 2.0 ** 24,
+            "plain_products_per_s": fx_products(24) * per_s / 1e9,
+            "model": "fx_macs: the multiply-adds the kernels execute; plain_products_per_s: G products/s of the "
+                     "tree's steps in their plain form (fx_products)",
             "peak_source": "independent chains of FX products, 16 warps per SM, measured in this run "
                            "(gbs_measure_fx_peak)"}
     return out
@@ -784,6 +822,16 @@ def main():
     kernel_name = ("batch_subtree_kernel (%d levels expanded in shared memory, then register depth-first %d levels)"
                    % (q_root - Q, Q)) if tuning["sub_e"] else "batch_leaf_kernel (register depth-first, %d levels)" % Q
 
+    fixed = fixed_point(args.prec, complex_basis, args.N, float(st_p.r[0]))
+    if fixed:
+        # one launch for up to 17 modes; else the leaf kernel takes the last Q levels of every node above them
+        one = args.N <= 17
+        q_root = args.N if one else min(args.N, max(1, min(3 if args.prec == "fp64" else 2, 3 - tuning["q_drop"])))
+        depth = args.N - q_root
+        leaf_flops = (2 ** depth) * leading_flops(q_root)
+        leaf_macs = (2 ** depth) * fx_macs(q_root, args.prec)
+        kernel_name = "fx_small_kernel (the whole tree)" if one else "fx_leaf_kernel (the last %d levels)" % q_root
+        mac_peak = ctx.measure_fx_peak() * FX_PRODUCT_MACS
     # L2 flush buffer (larger than the 129 MB L2), written between timed steps.
     flush = torch.empty(256 * 2 ** 20 // 4, dtype=torch.float32, device="cuda:%d" % dev)
 
@@ -845,6 +893,39 @@ def main():
     h2d = st_p.M * st_p.M * 16 + st_p.M * 8 + modes.nbytes
     d2h = 8 * 16  # the probability record
 
+    roofline = {
+        "bound": "alu", "kernel": kernel_name,
+        "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+        "peak_source": "FP64 DFMA-chain kernel measured in this run (gbs_measure_fp64_peak)",
+        "traffic": captured_traffic(args, tuning), "traffic_unit": "bytes per launch",
+        "traffic_source": "stored ncu capture of this kernel code and launch shape (not measured in this run)",
+        "flop_model": "8 t^2 flops per rank-2 update of 2t rows (real basis) + rsqrt and add per subset term",
+        "flops_per_launch": leaf_flops, "leaf_ms_avg": leaf_avg_s * 1e3,
+        "executed": {"flops_per_launch": leaf_exec, "achieved": achieved_exec, "frac": achieved_exec / peak,
+                     "model": "every FP64 operation the kernel executes (FMA = 2, other = 1; the inverse "
+                              "square roots run on the integer pipes)"},
+        "step_flops": total_flops,
+        "step_tflops": total_flops * args.steps / (dev_ms * 1e-3) / 1e12,
+        "other_accountings": other_accountings(args.N, dev_ms * 1e-3 / args.steps),
+    }
+    if fixed:
+        macs_per_s = leaf_macs / leaf_avg_s
+        roofline = {
+            "bound": "alu", "kernel": kernel_name, "unit": "G 32-bit multiply-adds/s",
+            "achieved": macs_per_s / 1e9, "peak": mac_peak / 1e9, "frac": macs_per_s / mac_peak,
+            "peak_source": "independent chains of FX products (26 multiply-adds each) measured in this run "
+                           "(gbs_measure_fx_peak)",
+            "traffic": captured_traffic(args, tuning), "traffic_unit": "bytes per launch",
+            "traffic_source": "stored ncu capture of this kernel code (not measured in this run)",
+            "multiply_adds_per_launch": leaf_macs, "leaf_ms_avg": leaf_avg_s * 1e3,
+            "flops_per_launch": leaf_flops,
+            "flop_model": "8 t^2 flops per rank-2 update of 2t rows (real basis) + rsqrt and add per subset term",
+            "fp64_pipe_equivalent": {"achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak},
+            "step_flops": total_flops,
+            "step_tflops": total_flops * args.steps / (dev_ms * 1e-3) / 1e12,
+            "other_accountings": other_accountings(args.N, dev_ms * 1e-3 / args.steps),
+        }
+
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": dev_ms / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -852,8 +933,9 @@ def main():
         "config": {
             "workload": "single Torontonian, N=%d clicks of the M=200 pure state (r=0.8, Haar seed 1): "
                         "2^%d subset determinants per step" % (args.N, args.N),
-            "M": 200, "N": args.N, "basis": args.basis, "per_term_arithmetic": args.prec,
-            "sum": {"fp64": "double-double", "fp64p": "double-double", "dd": "double-double",
+            "M": 200, "N": args.N, "basis": args.basis, "per_term_arithmetic": args.prec + (
+                " (64-bit fixed point, error model of FP64)" if fixed and args.prec == "fp64" else ""),
+            "sum": "exact fixed point" if fixed else {"fp64": "double-double", "fp64p": "double-double", "dd": "double-double",
                     "fp32": "double-double", "td": "triple-double", "fxn": "exact fixed point",
                     "fx": "exact fixed point", "fxw": "exact fixed point"}[args.prec],
             "l2": "flushed between steps (256 MB write); tree level buffers also exceed L2",
@@ -861,21 +943,7 @@ def main():
             "tuning": tuning, "autotune_candidates": len(tune_report),
             "autotune_fastest": sorted(tune_report, key=lambda c: c["ms"])[:5] if tune_report else [],
         },
-        "roofline": {
-            "bound": "alu", "kernel": kernel_name,
-            "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "peak_source": "FP64 DFMA-chain kernel measured in this run (gbs_measure_fp64_peak)",
-            "traffic": captured_traffic(args, tuning), "traffic_unit": "bytes per launch",
-            "traffic_source": "stored ncu capture of this kernel code and launch shape (not measured in this run)",
-            "flop_model": "8 t^2 flops per rank-2 update of 2t rows (real basis) + rsqrt and add per subset term",
-            "flops_per_launch": leaf_flops, "leaf_ms_avg": leaf_avg_s * 1e3,
-            "executed": {"flops_per_launch": leaf_exec, "achieved": achieved_exec, "frac": achieved_exec / peak,
-                         "model": "every FP64 operation the kernel executes (FMA = 2, other = 1; the inverse "
-                                  "square roots run on the integer pipes)"},
-            "step_flops": total_flops,
-            "step_tflops": total_flops * args.steps / (dev_ms * 1e-3) / 1e12,
-            "other_accountings": other_accountings(args.N, dev_ms * 1e-3 / args.steps),
-        },
+        "roofline": roofline,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         "gpu_launches": launches,
         "clocks": clk,

@@ -66,6 +66,21 @@ def test_state_from_V(ctx, basis):
     assert np.abs(H - Ho).max() <= 1e-11
 
 
+@pytest.mark.parametrize("M", [1, 7, 8, 9, 16, 17, 37])
+def test_dense_inverse_at_the_edges_of_its_blocks(ctx, M):
+    """2M around multiples of the 16 rows a block of the inverse takes.  Sigma's condition number is
+    below 10, so both inverses are within 2M 10^2 2^-52 < 2e-12 of the exact one."""
+    U = gi.haar_unitary(M, 6)
+    r = gi.uniform_range(6, "squeezing", M, 0.3, 0.9)
+    V = oracle.covariance(U, r, 0.9)
+    st = gbs.state_from_V(ctx, V)
+    Sig = oracle.sigma(V)
+    assert abs(st.logdet_sigma - oracle.logdet_sigma(Sig)) <= 1e-11
+    modes = sorted({0, M // 3, M // 2, M - 1})
+    assert np.abs(gbs.sigma_inv_block(ctx, st, modes, "complex") - oracle.sigma_inv_block(Sig, modes)).max() <= 1e-11
+    st.free()
+
+
 def test_bad_inputs_rejected(ctx):
     U = gi.haar_unitary(4, 1)
     with pytest.raises(gbs.GbsError) as e:
