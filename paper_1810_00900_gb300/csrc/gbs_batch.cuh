@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(128) batch_leaf_kernel(const LeafSeg* __restri
                                                          const typename real_of<E>::type* __restrict__ s1,
                                                          Partial<typename acc_traits<typename real_of<E>::type>::Red>* parts,
                                                          int* __restrict__ status) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // another Q's launch may run beside this one
   typedef typename real_of<E>::type T;
   typedef typename acc_traits<T>::Acc Acc;
   typedef typename acc_traits<T>::Red Red;
@@ -348,6 +349,7 @@ __global__ void __launch_bounds__(128) batch_leaf_kernel(const LeafSeg* __restri
     }
     __syncthreads();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // this launch ends after the one before it
 }
 
 // -------------------------------------------------------------- subtree --
@@ -369,6 +371,7 @@ __global__ void __launch_bounds__(128) batch_subtree_kernel(
     const E* __restrict__ buf1, const typename real_of<E>::type* __restrict__ s0,
     const typename real_of<E>::type* __restrict__ s1, int capA, int capB,
     Partial<typename acc_traits<typename real_of<E>::type>::Red>* parts, int* __restrict__ status) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // another Q's launch may run beside this one
   typedef typename real_of<E>::type T;
   typedef typename acc_traits<T>::Acc Acc;
   typedef typename acc_traits<T>::Red Red;
@@ -437,6 +440,7 @@ __global__ void __launch_bounds__(128) batch_subtree_kernel(
     }
     __syncthreads();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // this launch ends after the one before it
 }
 
 // Stage one of the per-tree reduction: chunk c sums partials [first, first+count)
@@ -485,11 +489,12 @@ __device__ __forceinline__ ProbOut finish_tree(const TreeOut& o, int status, dou
 
 // ---------------------------------------------------------------- final --
 // Sum of a tree's partials (or of their chunks' sums) in a fixed order and its finished
-// result, one CTA per tree: thread i sums partials i, i + 256, ... (the same ones in a
+// result, one CTA per tree: thread i sums partials i, i + 128, ... (the same ones in a
 // smaller block, whose ranges are no longer than it), then shuffle trees; threads without
-// one add zeros.  Chains of dependent double-double additions are what it costs, and the
-// launches that it saves (the chunks' and the finish's) what it gives: a torontonian of 9
-// modes under AUTO takes 117 us, 160 with three launches per precision.
+// one add zeros.  Wide additions on one SM's FP64 pipe are what it costs, so it has a warp
+// per scheduler and the ranges are short; the launches that it saves (the finish's, and the
+// chunks' below 512 partials) are what it gives: a torontonian of 9 modes under AUTO takes
+// 117 us, 160 with three launches per precision.
 template <class Red>
 __global__ void batch_final_kernel(const Partial<Red>* __restrict__ parts, const PartRange* __restrict__ ranges,
                                    const int* __restrict__ status, const double* __restrict__ scale,
@@ -505,6 +510,7 @@ __global__ void batch_final_kernel(const Partial<Red>* __restrict__ parts, const
   }
   __shared__ Partial<Red> res;
   block_reduce_store(inc, exc, asum, &res);
+  __syncthreads();
   if (threadIdx.x == 0) {
     TreeOut o;
     red_store(res.inc, o.inc);

@@ -21,6 +21,25 @@ struct Blob {
 };
 
 
+// Launch of a kernel that itself waits for the launch before it (programmatic dependent
+// launch).  early: its CTAs may be set up while that launch runs -- where that one leaves
+// the chip room (a few CTAs per SM at most), or they would take it from its own later
+// CTAs.  ~2 us a launch: N = 18, FP64, 14 launches, 163 -> 137 us.
+template <class... P, class... A>
+void launch_early(bool early, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // PAIR: the last two levels of every tree as cancellation-free groups (FP64
 // real basis; the tree's inc output then carries the whole Torontonian).
 template <class E, int QMAX, bool PAIR = false>
@@ -148,13 +167,14 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
   }
   for (int t = 0; t < ntrees; ++t) ranges[t].first += part_base[Q[t]];
   // reduction: one CTA per tree over its partials, or over the sums of chunks of <= 128
-  // of them (behind the partials) where it has thousands; by the tree alone, so that its
-  // sum does not depend on its batch
+  // of them (behind the partials) where it has more than 512: that many cost its SM's FP64
+  // pipes as much as the chunks' launch (2048 in triple-double ~80 us); by the tree alone,
+  // so that its sum does not depend on its batch
   std::vector<PartChunk> chunks;
   std::vector<PartRange> ranges2 = ranges;
   long long part_max = 0;  // the longest range
   for (int t = 0; t < ntrees; ++t) {
-    if (ranges[t].count > 2048) {
+    if (ranges[t].count > 512) {
       ranges2[t].first = parts_total + (long long)chunks.size();
       for (long long i = 0; i < ranges[t].count; i += 128)
         chunks.push_back(PartChunk{ranges[t].first + i, std::min<long long>(128, ranges[t].count - i)});
@@ -226,6 +246,10 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
     cudaEventRecord(ctx->leaf_timer.start, s);
   }
   const size_t smem_sub = (size_t)(capA + capB + nthr) * sizeof(E) + (size_t)nthr * (2 * sizeof(S) + 2 * sizeof(T));
+  // The launches of different Q run side by side: each lets the next one in when its CTAs
+  // have started, and ends after the one before it (trees of 6 .. 9 modes, eight of them,
+  // triple-double: 1490 us in turn, 943 so).
+  bool beside = false;
   for (int qv = QMAX; qv >= 1; --qv) {
     const long long nb = grp_blocks[qv];
     if (nb == 0) continue;
@@ -243,12 +267,12 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sub),         \
                              "subtree smem")))                                                                         \
           return st;                                                                                                   \
-        batch_subtree_kernel<E, QQ, PAIR><<<(unsigned)grid, nthr, smem_sub, s>>>(                                      \
-            (const SubSeg*)(plan + o_leaf[qv]), ns, nb, buf[0], buf[1], sb[0], sb[1], capA, capB, pp,                  \
-            status_dev);                                                                                               \
+        launch_early(beside, batch_subtree_kernel<E, QQ, PAIR>, (unsigned)grid, (unsigned)nthr, smem_sub, s,           \
+                     (const SubSeg*)(plan + o_leaf[qv]), ns, nb, buf[0], buf[1], sb[0], sb[1], capA, capB, pp,         \
+                     status_dev);                                                                                      \
       } else {                                                                                                         \
-        batch_leaf_kernel<E, QQ, PAIR><<<(unsigned)grid, 128, 0, s>>>((const LeafSeg*)(plan + o_leaf[qv]), ns, nb,     \
-                                                                buf[0], buf[1], sb[0], sb[1], pp, status_dev);         \
+        launch_early(beside, batch_leaf_kernel<E, QQ, PAIR>, (unsigned)grid, 128u, 0, s,                               \
+                     (const LeafSeg*)(plan + o_leaf[qv]), ns, nb, buf[0], buf[1], sb[0], sb[1], pp, status_dev);       \
       }                                                                                                                \
     }                                                                                                                  \
     break;
@@ -260,6 +284,7 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
       GBS_LEAF_CASE(6)
 #undef GBS_LEAF_CASE
     }
+    beside = true;
     count_launch(ctx);
   }
   if (ctx->timing) {
@@ -272,7 +297,7 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
                                                                    (int)chunks.size(), parts + parts_total);
     count_launch(ctx);
   }
-  batch_final_kernel<Red><<<(unsigned)ntrees, part_max > 128 ? 256 : part_max > 32 ? 128 : 32, 0, s>>>(
+  batch_final_kernel<Red><<<(unsigned)ntrees, part_max > 32 ? 128 : 32, 0, s>>>(
       parts, (const PartRange*)(plan + o_rng), status_dev, (const double*)(plan + o_sc), (const int*)(plan + o_n),
       fin.u, fin.extra, fin.po);
   count_launch(ctx);

@@ -66,7 +66,7 @@ constexpr uint32_t kFxShift = 1u << 9;  // K
 
 // Programmatic dependent launch: the launch after this one may set up its CTAs from
 // here on; wait for the launch before this one to be complete.  Every thread of a kernel
-// launched by fx_launch calls it before it touches memory.
+// launched by launch_early calls it before it touches memory.
 __device__ __forceinline__ void fx_after() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -17,25 +17,6 @@ inline long long fx_level_words(int n, int k, long long count, int L) {
   return count * (long long)sym(2 * q) * L;
 }
 
-// Launch of a kernel that waits (fx_after) for the launch before it.  early: its CTAs may
-// be set up while that launch runs -- where that one leaves the chip room (a few CTAs
-// per SM at most), or they would take it from its own later CTAs.  ~2 us a launch: N =
-// 18, FP64, 14 launches, 163 -> 137 us.
-template <class... P, class... A>
-void fx_launch(bool early, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = early ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-
 template <class E>
 gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const void* roots_dev, int* status_dev,
                         const BatchTune& tune, const TreeFinish& fin) {
@@ -286,13 +267,13 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     const int ns = (int)l.segs.size();
     const FxTree* tr = l.in_chunk ? d_chunked : d_trees;
     if (l.TW)
-      fx_launch(el, fx_level_cta_kernel<E>, (unsigned)l.blocks, 32 * l.W, l.smem, s, sg, ns, tr, d_off, l.q, l.TW, chunk, nodes,
+      launch_early(el, fx_level_cta_kernel<E>, (unsigned)l.blocks, 32 * l.W, l.smem, s, sg, ns, tr, d_off, l.q, l.TW, chunk, nodes,
                 sval, status_dev);
     else if (l.q >= 4)
-      fx_launch(el, fx_level_warp_kernel<E, 4>, (unsigned)l.blocks, 32, l.smem, s, sg, ns, tr, d_off, l.q, chunk, nodes, sval,
+      launch_early(el, fx_level_warp_kernel<E, 4>, (unsigned)l.blocks, 32, l.smem, s, sg, ns, tr, d_off, l.q, chunk, nodes, sval,
                 status_dev);
     else
-      fx_launch(el, fx_level_warp_kernel<E, 2>, (unsigned)l.blocks, 32, l.smem, s, sg, ns, tr, d_off, l.q, chunk, nodes, sval,
+      launch_early(el, fx_level_warp_kernel<E, 2>, (unsigned)l.blocks, 32, l.smem, s, sg, ns, tr, d_off, l.q, chunk, nodes, sval,
                 status_dev);
     count_launch(ctx);
   };
@@ -309,9 +290,9 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
       const int ns = (int)l.segs.size();
       const bool el = early(grid);
       switch (l.Q) {
-        case 1: fx_launch(el, fx_leaf_kernel<E, 1>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
-        case 2: fx_launch(el, fx_leaf_kernel<E, 2>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
-        default: fx_launch(el, fx_leaf_kernel<E, kLeafQ>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        case 1: launch_early(el, fx_leaf_kernel<E, 1>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        case 2: launch_early(el, fx_leaf_kernel<E, 2>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
+        default: launch_early(el, fx_leaf_kernel<E, kLeafQ>, grid, 128, 0, s, sg, ns, (unsigned)h, d_chunked, d_off, nodes, sval, parts + base, status_dev); break;
       }
       count_launch(ctx);
       base += l.units;
@@ -319,7 +300,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   }
   timer(true);
   const int final_threads = units_total > 256LL * ntrees ? 1024 : 128;
-  fx_launch(early(0), fx_final_kernel<S>, (unsigned)ntrees, final_threads, 0, s, parts, (const FxSeg*)(plan + o_sums), d_trees,
+  launch_early(early(0), fx_final_kernel<S>, (unsigned)ntrees, final_threads, 0, s, parts, (const FxSeg*)(plan + o_sums), d_trees,
             status_dev, fin.u, fin.extra, fin.po);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "fixed-point batch launch");

@@ -116,6 +116,13 @@ __device__ __forceinline__ td shfl_down(const td& v, int off) {
   return td{__shfl_down_sync(0xffffffffu, v.x0, off), __shfl_down_sync(0xffffffffu, v.x1, off),
             __shfl_down_sync(0xffffffffu, v.x2, off)};
 }
+__device__ __forceinline__ dd shfl_xor(const dd& v, int mask) {
+  return dd{__shfl_xor_sync(0xffffffffu, v.hi, mask), __shfl_xor_sync(0xffffffffu, v.lo, mask)};
+}
+__device__ __forceinline__ td shfl_xor(const td& v, int mask) {
+  return td{__shfl_xor_sync(0xffffffffu, v.x0, mask), __shfl_xor_sync(0xffffffffu, v.x1, mask),
+            __shfl_xor_sync(0xffffffffu, v.x2, mask)};
+}
 
 template <class Red>
 struct Partial {
@@ -426,31 +433,39 @@ __device__ __forceinline__ void block_reduce_sums(double ip, double in, double e
   }
 }
 
-// Sums over a block into *out: a shuffle tree per warp, then one over the warps (a serial
-// loop over them was 8 dependent double-double additions).
+// Sums over a warp: inc in lane 0, exc in lane 16, asum in lane 0.  Lanes below 16 take
+// inc and the others exc, one wide addition a stage for both: a warp's FP64
+// instruction holds its scheduler's pipe for 64 cycles, a double-double addition ~0.7 us
+// and a triple-double one ~2.
+template <class Red>
+__device__ __forceinline__ void warp_reduce_pair(Red& inc, Red& exc, double& asum) {
+  const bool low = (threadIdx.x & 31) < 16;
+  const Red got = shfl_xor(low ? exc : inc, 16);
+  Red v = low ? red_add(inc, got) : red_add(got, exc);
+#pragma unroll
+  for (int off = 8; off > 0; off >>= 1) v = red_add(v, shfl_down(v, off));
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) asum += __shfl_down_sync(0xffffffffu, asum, off);
+  inc = v;
+  exc = v;
+}
+
+// Sums over a block into *out: a shuffle tree per warp, then the warps in order.
 template <class Red>
 __device__ __forceinline__ void block_reduce_store(Red inc, Red exc, double asum, Partial<Red>* out) {
   __shared__ Red s_inc[32], s_exc[32];
   __shared__ double s_abs[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto warp_sum = [&]() {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      inc = red_add(inc, shfl_down(inc, off));
-      exc = red_add(exc, shfl_down(exc, off));
-      asum += __shfl_down_sync(0xffffffffu, asum, off);
-    }
-  };
-  warp_sum();
-  if (lane == 0) { s_inc[warp] = inc; s_exc[warp] = exc; s_abs[warp] = asum; }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  warp_reduce_pair(inc, exc, asum);
+  if (lane == 0) { s_inc[warp] = inc; s_abs[warp] = asum; }
+  if (lane == 16) s_exc[warp] = exc;
   __syncthreads();
-  if (warp == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    inc = lane < nw ? s_inc[lane] : red_zero<Red>();
-    exc = lane < nw ? s_exc[lane] : red_zero<Red>();
-    asum = lane < nw ? s_abs[lane] : 0.0;
-    if (nw > 1) warp_sum();
-    if (lane == 0) { out->inc = inc; out->exc = exc; out->abs = asum; }
+  if (warp == 0 && (lane & 15) == 0) {  // lane 0 joins inc, lane 16 exc
+    const Red* r = lane == 0 ? s_inc : s_exc;
+    Red a = r[0];
+    double c = s_abs[0];
+    for (int w = 1; w < nw; ++w) { a = red_add(a, r[w]); c += s_abs[w]; }
+    if (lane == 0) { out->inc = a; out->abs = c; } else { out->exc = a; }
   }
 }
 
