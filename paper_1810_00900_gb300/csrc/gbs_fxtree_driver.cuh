@@ -225,10 +225,10 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     return GBS_ENOMEM;
   }
   gbs_status st;
-  if ((st = dev_reserve(ctx, ctx->lvl[0], (size_t)words * 4)) ||
-      (st = dev_reserve(ctx, ctx->sbuf[0], (size_t)selems * sizeof(S))) ||
-      (st = dev_reserve(ctx, ctx->partials, part_bytes)))
-    return st;
+  // one allocation: a context's first call pays for each
+  auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t node_bytes = r256((size_t)words * 4), s_bytes = r256((size_t)selems * sizeof(S));
+  if ((st = dev_reserve(ctx, ctx->lvl[0], node_bytes + s_bytes + part_bytes))) return st;
   Blob blob;
   const size_t o_trees = blob.put(trees), o_chunked = blob.put(chunked), o_off = blob.put(off), o_top = blob.put(top);
   for (Launch& l : levels) l.at = blob.put(l.segs);
@@ -237,8 +237,8 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   const unsigned char* plan = nullptr;
   if ((st = stage(ctx, blob.bytes.data(), blob.bytes.size(), (const void**)&plan))) return st;
   uint32_t* nodes = (uint32_t*)ctx->lvl[0].ptr;
-  S* sval = (S*)ctx->sbuf[0].ptr;
-  FxPart<S>* parts = (FxPart<S>*)ctx->partials.ptr;
+  S* sval = (S*)((unsigned char*)nodes + node_bytes);
+  FxPart<S>* parts = (FxPart<S>*)((unsigned char*)nodes + node_bytes + s_bytes);
   const FxTree* d_trees = (const FxTree*)(plan + o_trees);
   const FxTree* d_chunked = (const FxTree*)(plan + o_chunked);
   const long long* d_off = (const long long*)(plan + o_off);
