@@ -493,7 +493,7 @@ __device__ __forceinline__ ProbOut finish_tree(const TreeOut& o, int status, dou
 // smaller block, whose ranges are no longer than it), then shuffle trees; threads without
 // one add zeros.  Wide additions on one SM's FP64 pipe are what it costs, so it has a warp
 // per scheduler and the ranges are short; the launches that it saves (the finish's, and the
-// chunks' below 512 partials) are what it gives: a torontonian of 9 modes under AUTO takes
+// chunks' below 512 partials) are what it gives: a torontonian of 6 modes under AUTO takes
 // 117 us, 160 with three launches per precision.
 template <class Red>
 __global__ void batch_final_kernel(const Partial<Red>* __restrict__ parts, const PartRange* __restrict__ ranges,
