@@ -218,11 +218,9 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
   Partial<Red>* parts = (Partial<Red>*)ctx->partials.ptr;
 
   // ---------------- top
-  // The opt-in limit is set whatever the size: the kernels' static shared
-  // memory (reduction scratch) counts against the default 48 KB as well.
-  if ((st = check_cuda(ctx, cudaFuncSetAttribute(batch_top_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem_top),
-                       "top smem")))
+  // (whatever the size: the kernels' static shared memory, reduction scratch, counts against
+  // the default 48 KB as well)
+  if ((st = allow_smem(ctx, batch_top_kernel<E>, (size_t)smem_top, "top smem")))
     return st;
   batch_top_kernel<E><<<(unsigned)top_blocks, tune.top_threads, smem_top, s>>>(
       (const TopSeg*)(plan + o_top), ntrees, (const typename root_src<E>::type*)roots_dev, buf[0], buf[1], sb[0], sb[1],
@@ -262,10 +260,7 @@ gbs_status batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* trees, const voi
   case QQ:                                                                                                             \
     if constexpr (QQ <= QMAX) {                                                                                        \
       if (sub_e > 0) {                                                                                                 \
-        if ((st = check_cuda(ctx,                                                                                      \
-                             cudaFuncSetAttribute(batch_subtree_kernel<E, QQ, PAIR>,                                   \
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sub),         \
-                             "subtree smem")))                                                                         \
+        if ((st = allow_smem(ctx, batch_subtree_kernel<E, QQ, PAIR>, smem_sub, "subtree smem")))                       \
           return st;                                                                                                   \
         launch_early(beside, batch_subtree_kernel<E, QQ, PAIR>, (unsigned)grid, (unsigned)nthr, smem_sub, s,           \
                      (const SubSeg*)(plan + o_leaf[qv]), ns, nb, buf[0], buf[1], sb[0], sb[1], capA, capB, pp,         \

@@ -342,9 +342,7 @@ gbs_status chain_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int
   const int tree_words = std::max(std::max(fx_small_words(10, 10, 3, 5), fx_small_words(10, 10, 5, 6)),
                                   std::max(fx_small_words(9, 9, 6, 7), fx_small_words(9, 9, 7, 8)));
   const size_t smem = std::max((size_t)tree_words * 4, (size_t)(2 * M_max + 2) * (4 * sizeof(double) + sizeof(int)));
-  if ((e = check_cuda(ctx, cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                      "chain smem")))
-    return e;
+  if ((e = allow_smem(ctx, chain_kernel, smem, "chain smem"))) return e;
   const auto t0 = std::chrono::steady_clock::now();
   // CTAs per trajectory: as many as the chip has room for, up to a portable cluster's 8.
   // 8 trajectories of a 100-mode graph state, ms: 44.7 with one, 43.7, 41.5, 40.5 with 2, 4,

@@ -71,9 +71,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
         (st = dev_reserve(ctx, ctx->sbuf[1], (size_t)blocks[1] * sizeof(FxPart<S>))))
       return st;
     const int smem = fx_small_words(small_n[c], c ? kSub : small_n[c], L, LS) * 4;
-    if ((st = check_cuda(ctx, cudaFuncSetAttribute(fx_small_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
-                         "small tree smem")))
-      return st;
+    if ((st = allow_smem(ctx, fx_small_kernel<E>, (size_t)smem, "small tree smem"))) return st;
     int threads = c || small_n[c] >= 8 ? 512 : small_n[c] >= 6 ? 256 : small_n[c] >= 4 ? 128 : 32;
     if (blocks[c] > ctx->sm_count) threads = std::min(threads, 256);  // two CTAs per SM
     fx_small_kernel<E><<<(unsigned)blocks[c], threads, smem, ctx->stream>>>(
@@ -246,11 +244,11 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
 
   // ---------------- launches
   const int smem_top = sym(2 * nmax) * (int)sizeof(E) + 2 * nmax * (int)sizeof(FxRow<E>);
-  if ((st = check_cuda(ctx, cudaFuncSetAttribute(fx_top_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_top),
-                       "top smem")) ||
-      (st = check_cuda(ctx, cudaFuncSetAttribute(fx_level_cta_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 cta_smem(62, 16)),
-                       "level smem")))
+  size_t smem_cta = 0;
+  for (const Launch& l : levels)
+    if (l.TW) smem_cta = std::max(smem_cta, l.smem);
+  if ((st = allow_smem(ctx, fx_top_kernel<E>, (size_t)smem_top, "top smem")) ||
+      (st = allow_smem(ctx, fx_level_cta_kernel<E>, smem_cta, "level smem")))
     return st;
   fx_top_kernel<E><<<(unsigned)top_blocks, 256, smem_top, s>>>((const FxSeg*)(plan + o_top), ntrees, d_trees, d_off,
                                                                (const double*)roots_dev, nodes, sval, status_dev);

@@ -136,6 +136,22 @@ gbs_status set_error(gbs_ctx* ctx, gbs_status st, const std::string& msg);
 gbs_status check_cuda(gbs_ctx* ctx, cudaError_t e, const char* what);
 gbs_status dev_alloc(gbs_ctx* ctx, DevBuf& b, size_t bytes);
 gbs_status dev_reserve(gbs_ctx* ctx, DevBuf& b, size_t bytes);  // grow-only
+// Lets a kernel take `need` bytes of dynamic shared memory: up to the device's limit, always
+// the same, since the setting is the process's and another thread's launch may lie between
+// it and the launch here.
+template <class K>
+gbs_status allow_smem(gbs_ctx* ctx, K* kernel, size_t need, const char* what) {
+  int limit = 0;
+  cudaFuncAttributes fa;
+  gbs_status st;
+  if ((st = check_cuda(ctx, cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device), what)) ||
+      (st = check_cuda(ctx, cudaFuncGetAttributes(&fa, kernel), what)))
+    return st;
+  limit -= (int)fa.sharedSizeBytes;
+  if (need > (size_t)limit) return check_cuda(ctx, cudaErrorInvalidValue, what);
+  if (fa.maxDynamicSharedSizeBytes >= limit) return GBS_OK;
+  return check_cuda(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit), what);
+}
 // At most 32 modes in [0, M), none twice.
 gbs_status validate_modes(gbs_ctx* ctx, const int* modes, int N, int M);
 void dev_free(gbs_ctx* ctx, DevBuf& b);

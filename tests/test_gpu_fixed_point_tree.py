@@ -2,6 +2,8 @@
 of 32 nodes, one level and one tile more, every depth of the top kernel, batches of uneven trees,
 and a tree taken in chunks because its levels exceed the context's budget.  Sums are exact, so
 every launch shape and split gives the same bits."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -127,3 +129,33 @@ def test_many_requests_get_the_roots_of_each_alone(ctx, M, dense):
             b = many[i] if basis == "real" else gbs.torontonian_batch(ctx, [st] * 320, [pats[i]] * 320, "fp64", basis)[7]
             assert (a.tor, a.abs_sum, a.p) == (b.tor, b.abs_sum, b.p), (len(pats[i]), basis)
     st.free()
+
+
+def test_threads_with_trees_of_different_sizes_at_once():
+    """Four contexts in four threads, each with trees of other sizes in turn: the same kernels launched
+    with different amounts of shared memory at the same time give every thread its own results."""
+    p = gi.uniform_squeezed_state(40, 0.8, seed=5, eta=0.8)
+    sizes = [1, 3, 6, 8, 9, 10, 12, 14]
+
+    def run(ctx, order):
+        st = gbs.build_state(ctx, p.U, p.r, p.eta)
+        out = {}
+        for _ in range(6):
+            for prec in ("fp64", "fx", "dd"):
+                for n in order:
+                    out[n, prec] = gbs.torontonian(ctx, st, gi.random_modes(40, n, n), prec).tor
+        st.free()
+        return out
+
+    with gbs.Context(0) as ctx:
+        ref = run(ctx, sizes)
+    got = [None] * 4
+
+    def work(i):
+        with gbs.Context(0) as ctx:
+            got[i] = run(ctx, sizes[2 * i:] + sizes[:2 * i])
+
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    [t.start() for t in ts]
+    [t.join() for t in ts]
+    assert all(g == ref for g in got)
