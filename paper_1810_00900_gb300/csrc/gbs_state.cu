@@ -71,7 +71,8 @@ __global__ void sum_dd_kernel(const double* __restrict__ x, int n, double* __res
 // per (pair, l), with the rows of U weighted by cosh and sinh once per tile as they are
 // staged (a thread per pair of the full square with the weights applied to each product
 // took 16 operations per (j, k, l), and read U's rows a thread apart).  Small tiles, so
-// that the triangle's CTAs fill the SMs evenly.  M = 333: 648 -> 290 us, of which 243
+// that the triangle's CTAs fill the SMs evenly.  The sums go in runs of kVL, whose rounding
+// is below that of one chain (M = 333, relative to a wider sum: 5.2e-16, 8.9e-16 with one).  M = 333: 648 -> 290 us, of which 243
 // are the FMAs.
 constexpr int kVT = 8, kVL = 32;
 __global__ void __launch_bounds__(64) build_V_kernel(const cplx<double>* __restrict__ U, const double* __restrict__ ch2,
@@ -97,15 +98,20 @@ __global__ void __launch_bounds__(64) build_V_kernel(const cplx<double>* __restr
       sy[r][c] = okl && rk < M ? U[(long long)rk * M + l] : cplx<double>{0, 0};
     }
     __syncthreads();
+    double car = 0, cai = 0, cbr = 0, cbi = 0;  // this run's sums
 #pragma unroll 4
     for (int c = 0; c < kVL; ++c) {
       const cplx<double> y = sy[lk][c], p = sc[lj][c], q = ss[lj][c];
       // x conj(y) cosh(2r)/2 and x y sinh(2r)/2
-      ar = fma(p.re, y.re, fma(p.im, y.im, ar));
-      ai = fma(p.im, y.re, fma(-p.re, y.im, ai));
-      br = fma(q.re, y.re, fma(-q.im, y.im, br));
-      bi = fma(q.re, y.im, fma(q.im, y.re, bi));
+      car = fma(p.re, y.re, fma(p.im, y.im, car));
+      cai = fma(p.im, y.re, fma(-p.re, y.im, cai));
+      cbr = fma(q.re, y.re, fma(-q.im, y.im, cbr));
+      cbi = fma(q.re, y.im, fma(q.im, y.re, cbi));
     }
+    ar += car;
+    ai += cai;
+    br += cbr;
+    bi += cbi;
     __syncthreads();
   }
   if (j >= M || k > j) return;
