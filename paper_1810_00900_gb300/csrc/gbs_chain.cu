@@ -32,7 +32,12 @@ namespace gbs {
 
 namespace {
 
-constexpr int kChainMaxM = 224;
+// Up to kChainAnyM modes with any number of trajectories, up to kChainMaxM with at most one
+// per two SMs: beyond, the chip's SMs are not all busy conditioning where the launches spread
+// every trajectory over all of them.  10 forced clicks, ms with launches / here: 448 modes, 1, 8, 64,
+// 160 trajectories 45 / 17, 54 / 22, 84 / 44, 119 / 105; 800 modes 90 / 47, 110 / 54, 222 / 166,
+// 372 / 481; 1000 modes, 64: 349 / 291.
+constexpr int kChainAnyM = 448, kChainMaxM = 1024;
 
 // Modes a CTA's tree may have in the type of a precision.
 GBS_HD_INLINE int chain_modes(int prec) { return prec == GBS_PREC_FP64 || prec == GBS_PREC_FXN ? 10 : 9; }
@@ -296,8 +301,8 @@ __global__ void __launch_bounds__(512) chain_kernel(const ChainJob* __restrict__
 
 }  // namespace
 
-bool chain_eligible(const Trajectory& t, int prec) {
-  if (t.M > kChainMaxM || !fx_ok_sigma(t.st, 32)) return false;
+bool chain_eligible(const gbs_ctx* ctx, const Trajectory& t, int prec, size_t n_traj) {
+  if (t.M > (2 * n_traj <= (size_t)ctx->sm_count ? kChainMaxM : kChainAnyM) || !fx_ok_sigma(t.st, 32)) return false;
   const bool half = !t.need_full;
   const int n = half ? t.m : t.m + 1;
   const int p = prec != GBS_PREC_AUTO ? prec : sampler_pick(true, t.kappa_prev * (half ? 1.5 : 8.0), n);
@@ -344,22 +349,34 @@ gbs_status chain_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int
   const size_t smem = std::max((size_t)tree_words * 4, (size_t)(2 * M_max + 2) * (4 * sizeof(double) + sizeof(int)));
   if ((e = allow_smem(ctx, chain_kernel, smem, "chain smem"))) return e;
   const auto t0 = std::chrono::steady_clock::now();
-  // CTAs per trajectory: as many as the chip has room for, up to a portable cluster's 8.
+  // CTAs per trajectory: as many as are resident at once, up to a portable cluster's 8 (18
+  // trajectories of 230 modes: 14.8 ms with clusters of 8, which do not all fit, 11.6 with 4).
   // 8 trajectories of a 100-mode graph state, ms: 44.7 with one, 43.7, 41.5, 40.5 with 2, 4,
   // 8; 24 of 200 modes 42.8, 41.4, 40.1; 64 of 30 modes 3.3 with one and two.
-  int parts = 1;
-  while (parts < 8 && (int)T * parts * 2 <= ctx->sm_count) parts *= 2;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = parts;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  attr.val.clusterDim.x = attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(T * parts));
   cfg.blockDim = dim3(512);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = ctx->stream;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
+  int parts = 1;
+  for (int i = 0; i < 3 && (long long)T * (2 << i) <= ctx->sm_count; ++i) {
+    if (ctx->chain_fit[i] < 0) {  // ~20 us a query; its shared memory allows one CTA per SM whatever M
+      attr.val.clusterDim.x = 2 << i;
+      cfg.gridDim = dim3(2u << i);
+      if (cudaOccupancyMaxActiveClusters(&ctx->chain_fit[i], chain_kernel, &cfg) != cudaSuccess) {
+        ctx->chain_fit[i] = 0;  // without an answer the smaller clusters do
+        (void)cudaGetLastError();
+      }
+    }
+    if (ctx->chain_fit[i] < (int)T) break;
+    parts = 2 << i;
+  }
+  attr.val.clusterDim.x = parts;
+  cfg.gridDim = dim3((unsigned)(T * parts));
   cudaLaunchKernelEx(&cfg, chain_kernel, (const ChainJob*)d_in, d_out);
   count_launch(ctx);
   std::vector<ChainOut> out(T);

@@ -92,6 +92,7 @@ struct gbs_ctx {
   gbs::KernelTimer leaf_timer;
   std::atomic<long long> launches{0};
   int sm_count = 0;
+  int chain_fit[3] = {-1, -1, -1};  // clusters of 2, 4, 8 of the sampler's CTAs that are resident at once
   // host gaps: time from the return of a host wait on the stream (stream_sync)
   // to the next kernel launch, while the stream sits empty
   bool gap_open = false;
@@ -240,7 +241,7 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
 // Whether the trajectory's next step can run in the one-CTA chain (gbs_chain.cu), and
 // up to kChainSteps steps of such trajectories.
 constexpr int kChainSteps = 24;
-bool chain_eligible(const Trajectory& t, int prec);
+bool chain_eligible(const gbs_ctx* ctx, const Trajectory& t, int prec, size_t n_traj);
 gbs_status chain_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int prec, gbs_sample_stats& stt);
 // Fixed-point eligibility (gbs_batch_api.cu): a tree over n modes of
 // (Sigma^-1)_S, resp. of a conditioned Sigma', keeps every value in range.

@@ -238,9 +238,11 @@ struct StepTree {
 // one abandoned by postselection kRejected (the caller restarts or drops it).
 gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, int prec, gbs_sample_stats& stt) {
   std::vector<Trajectory*> act, chain;
+  size_t running = 0;
+  for (const Trajectory* t : jobs) running += t->state == Trajectory::kRunning;
   for (Trajectory* t : jobs) {
     if (t->state != Trajectory::kRunning) continue;
-    (!t->host_step && chain_eligible(*t, prec) ? chain : act).push_back(t);
+    (!t->host_step && chain_eligible(ctx, *t, prec, running) ? chain : act).push_back(t);
     t->host_step = false;
   }
   gbs_status e;

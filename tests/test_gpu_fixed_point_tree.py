@@ -159,3 +159,17 @@ def test_threads_with_trees_of_different_sizes_at_once():
     [t.start() for t in ts]
     [t.join() for t in ts]
     assert all(g == ref for g in got)
+
+
+@pytest.mark.parametrize("M", [30, 230])
+@pytest.mark.parametrize("n", [1, 3, 20, 40, 80])
+def test_sampler_steps_give_the_same_bits_with_any_number_of_trajectories(ctx, M, n):
+    """1, 2, 4 or 8 CTAs condition a trajectory, by how many there are: sample 0's bits alone and
+    among n."""
+    p = gi.uniform_squeezed_state(M, 0.6, seed=M, eta=0.8)
+    st = gbs.build_state(ctx, p.U, p.r, p.eta)
+    clicks = [sorted(np.random.default_rng(i).permutation(M)[:6].tolist()) for i in range(n)]
+    one = gbs.sample(ctx, st, 1, 9, 6, 1, forced_clicks=clicks[:1], want_p0=True)
+    many = gbs.sample(ctx, st, n, 9, 6, 1, forced_clicks=clicks, want_p0=True)
+    assert np.array_equal(one[0][0], many[0][0]) and np.array_equal(one[1][0], many[1][0])
+    st.free()
