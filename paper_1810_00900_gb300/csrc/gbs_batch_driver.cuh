@@ -22,7 +22,8 @@ struct Blob {
 
 
 // Launch of a kernel that itself waits for the launch before it (programmatic dependent
-// launch).  early: its CTAs may be set up while that launch runs -- where that one leaves
+// launch): before it touches what that one writes (fx_after), or, where the two touch nothing
+// in common (leaf launches of different Q), at its end.  early: its CTAs may be set up while that launch runs -- where that one leaves
 // the chip room (a few CTAs per SM at most), or they would take it from its own later
 // CTAs.  ~2 us a launch: N = 18, FP64, 14 launches, 163 -> 137 us.
 template <class... P, class... A>

@@ -65,8 +65,13 @@ namespace gbs {
 constexpr uint32_t kFxShift = 1u << 9;  // K
 
 // Programmatic dependent launch: the launch after this one may set up its CTAs from
-// here on; wait for the launch before this one to be complete.  Every thread of a kernel
-// launched by launch_early calls it before it touches memory.
+// here on; wait for the launch before this one to be complete.  Every thread of a kernel of
+// the chain calls it before it touches memory that an earlier launch of the chain writes.
+// Only the plan (segs, trees, lvl_off), uploaded before the chain's first launch, may be read
+// ahead of it, and only the plan's pointers are const __restrict__: nodes, s, partial sums
+// and status change while such a kernel is already running, so a load from them must not be
+// taken for one of memory that is read-only throughout, which a compiler may move above the
+// wait or through the non-coherent path.
 __device__ __forceinline__ void fx_after() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -411,7 +416,7 @@ __global__ void __launch_bounds__(32) fx_level_warp_kernel(const FxSeg* __restri
                                                            const FxTree* __restrict__ trees,
                                                            const long long* __restrict__ lvl_off, int q, unsigned chunk,
                                                            uint32_t* nodes, typename fx_sum<E>::type* sval,
-                                                           int* __restrict__ status) {
+                                                           int* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];  // the plan is older than the top kernel
   const FxTree t = trees[sg.idx];
@@ -511,7 +516,7 @@ __global__ void __launch_bounds__(256) fx_level_cta_kernel(const FxSeg* __restri
                                                            const FxTree* __restrict__ trees,
                                                            const long long* __restrict__ lvl_off, int q, int TW,
                                                            unsigned chunk, uint32_t* nodes,
-                                                           typename fx_sum<E>::type* sval, int* __restrict__ status) {
+                                                           typename fx_sum<E>::type* sval, int* status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const FxSeg sg = segs[fx_find(segs, nseg, (long long)blockIdx.x)];  // the plan is older than the top kernel
   const FxTree t = trees[sg.idx];
@@ -649,10 +654,10 @@ template <class E, int Q>
 __global__ void __launch_bounds__(128, 4) fx_leaf_kernel(const FxSeg* __restrict__ segs, int nseg, unsigned chunk,
                                                          const FxTree* __restrict__ trees,
                                                          const long long* __restrict__ lvl_off,
-                                                         const uint32_t* __restrict__ nodes,
-                                                         const typename fx_sum<E>::type* __restrict__ sval,
-                                                         FxPart<typename fx_sum<E>::type>* __restrict__ parts,
-                                                         int* __restrict__ status) {
+                                                         const uint32_t* nodes,
+                                                         const typename fx_sum<E>::type* sval,
+                                                         FxPart<typename fx_sum<E>::type>* parts,
+                                                         int* status) {
   typedef typename fx_sum<E>::type S;
   constexpr int L = sizeof(E) / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -700,11 +705,11 @@ __global__ void __launch_bounds__(128, 4) fx_leaf_kernel(const FxSeg* __restrict
 // One CTA per tree; segs[t].first = the tree's first unit, segs[t + 1].first the end.
 // (Ten thousand partial sums took it 31 us; a sum per leaf CTA leaves it some thousand.)
 template <class S>
-__global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* __restrict__ parts,
+__global__ void __launch_bounds__(1024) fx_final_kernel(const FxPart<S>* parts,
                                                         const FxSeg* __restrict__ segs,
                                                         const FxTree* __restrict__ trees,
-                                                        const int* __restrict__ status, double u, double extra,
-                                                        ProbOut* __restrict__ out) {
+                                                        const int* status, double u, double extra,
+                                                        ProbOut* out) {
   fx_after();
   const int t = blockIdx.x;
   const S zero = fx_of<S>(0.0);
