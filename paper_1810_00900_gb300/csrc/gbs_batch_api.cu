@@ -47,12 +47,12 @@ const BatchTune& batch_tune_for(gbs_ctx* ctx, int prec, bool real) {
   return ctx->tune[prec < 0 || prec > kPrecLast ? 1 : prec][real ? 1 : 0];
 }
 
-// Every value of a tree over n modes of (Sigma^-1)_S fits the fixed-point
-// range: Sigma >= I/2 bounds the entries by 2, the pivot determinants lie in
-// [1/sigma_max^2, 4] (so the scaled pivot inverses and the products formed with
-// them stay below 2^23, inside the entries' 31-bit integer part), each included
-// pivot multiplies s by at most sigma_max, and the sums are bounded by
-// (1 + sigma_max)^n (inside the 63-bit integer part of s and the sums).
+// Every value of a tree over n modes of (Sigma^-1)_S fits the fixed-point range: its
+// eigenvalues are at least 1/sigma_max, which bounds the scaled pivot inverses by
+// sigma_max, each included pivot's factor of s by sigma_max and the sums by
+// (1 + sigma_max)^n (inside the 63-bit integer part of s and the sums).  Entries and pivot
+// determinants are bounded where Sigma >= I/2 (a physical state: 2 and 4); a covariance
+// given as such promises Sigma > 0 only, so the engine checks the root itself.
 bool fx_ok_inverse(const gbs_state* st, int n) {
   const double sm = st->sigma_max;
   return sm > 0.0 && sm <= 1024.0 && n * std::log2(1.0 + sm) < 60.0;

@@ -45,16 +45,23 @@
 // An update of R rows takes R (R + 1) / 2 + 5 R products in place of R (R + 1) +
 // 4 R (R = 4, 6, 8: 30, 51, 76 for 36, 66, 104).  Neither form loses accuracy
 // here: sums are exact and a product's error is absolute, whatever its factors.
-// Signed factors are shifted by K = 2^9 (entries and rows of L stay below 128 in
-// magnitude on every matrix the host admits: |u| <= lambda_max <= 64, and U P^-1 U^T
-// <= C bounds a row of L by |L_a|^2 <= C_aa lambda_max(P^-1) <= lambda_max / lambda_min
-// <= 2^14), so that all products are of
+// Signed factors are shifted by K = 2^29, so that all products are of
 // non-negative values; the shifts are separable and live in c0, c1, A and B:
 //   U = u0 + K, V = u1 + K, P = L0 + K, Q = L1 + K
 //   P = (al + m) U - m (U - V + 2K) + c0,  c0 = K + 2K m - K (al + m)
 //   Q = (be + m) V + m (U - V + 2K) + c1,  c1 = K - 2K m - K (be + m)
 //   A = (P + K)(Q + K) - 2 K^2,  B = (U + K)(V + K) - 2 K^2
 //   C' = C - (P_a + V_b)(U_b + Q_a) + A_a + B_b
+// All of it holds modulo 2^32, the range of the integer limb, so only the factors need a
+// bound: |u| and |L| below K.  K costs no accuracy: it lies in the integer limb, whose
+// partial products are all kept, so the bits do not depend on it.  The roots are checked
+// (fx_root_entry_ok, fx_root_mode_ok): entries below 2^29, and by positive definiteness all
+// entries of the tree; and the product of a mode's diagonal entries below 2^31, so that no
+// determinant wraps past the check of its range.  A row of L is bounded by |L_a|^2 <= C_aa
+// lambda_max(P^-1): below 2^20 over (Sigma^-1)_S, whose eigenvalues are at least 1 / sigma_max
+// >= 2^-10 whether V is physical or not, and below 2^17 over a conditioned Sigma', with
+// entries up to 64 and det P >= 2^-20.  (K = 2^9, enough where Sigma >= I/2, lost states
+// given by a V whose Sigma has eigenvalues down to 1/2000.)
 #pragma once
 #include "gbs_fx.cuh"
 #include "gbs_internal.h"
@@ -62,7 +69,8 @@
 
 namespace gbs {
 
-constexpr uint32_t kFxShift = 1u << 9;  // K
+constexpr int kFxShiftBits = 29;
+constexpr uint32_t kFxShift = 1u << kFxShiftBits;  // K
 
 // Programmatic dependent launch: the launch after this one may set up its CTAs from
 // here on; wait for the launch before this one to be complete.  Every thread of a kernel of
@@ -75,6 +83,16 @@ constexpr uint32_t kFxShift = 1u << 9;  // K
 __device__ __forceinline__ void fx_after() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Whether a root fits the engine (see above): |x| < 2^29 for every entry (NaN and infinities
+// are not), and p00 p11 < 2^31 for every mode, from the integer limbs of its diagonal.
+__device__ __forceinline__ bool fx_root_entry_ok(double x) {
+  return (__double2hiint(x) & 0x7fffffff) < ((1023 + 29) << 20);
+}
+template <int L, int F>
+__device__ __forceinline__ bool fx_root_mode_ok(const fxn<L, F>& p00, const fxn<L, F>& p11) {
+  return ((unsigned long long)p00.w[L - 1] + 1ull) * ((unsigned long long)p11.w[L - 1] + 1ull) <= (1ull << 31);
 }
 
 // Scalars of a pivot.
@@ -147,9 +165,9 @@ __device__ __forceinline__ bool fx_pivot(const E& p00, const E& p10, const E& p1
   pv.m = umul(n10, inv);
   pv.a = umul(p11, inv) + pv.m;
   pv.b = umul(p00, inv) + pv.m;
-  const E km = fx_shl(pv.m, 10);  // 2 K m
-  pv.c0 = fx_add_int(km - fx_shl(pv.a, 9), kFxShift);
-  pv.c1 = fx_add_int(-(km + fx_shl(pv.b, 9)), kFxShift);
+  const E km = fx_shl(pv.m, kFxShiftBits + 1);  // 2 K m
+  pv.c0 = fx_add_int(km - fx_shl(pv.a, kFxShiftBits), kFxShift);
+  pv.c1 = fx_add_int(-(km + fx_shl(pv.b, kFxShiftBits)), kFxShift);
   return fx_det_in_range(det);
 }
 
@@ -280,11 +298,18 @@ __global__ void __launch_bounds__(256) fx_top_kernel(const FxSeg* __restrict__ s
   const int d = 2 * t.n;
   E* C = reinterpret_cast<E*>(smem_raw);
   FxRow<E>* rows = reinterpret_cast<FxRow<E>*>(C + sym(d));
-  for (int i = threadIdx.x; i < sym(d); i += blockDim.x)
-    C[i] = fx_of<E>(roots[t.root_off + i]);
   S s = fx_of<S>(1.0);
   bool ok = true;
+  for (int i = threadIdx.x; i < sym(d); i += blockDim.x) {
+    const double x = roots[t.root_off + i];
+    ok &= fx_root_entry_ok(x);
+    C[i] = fx_of<E>(x);
+  }
   __syncthreads();
+  if (v == 0u && (int)threadIdx.x < t.n) {
+    const int o = 2 * threadIdx.x;
+    ok &= fx_root_mode_ok(C[tri(o, o)], C[tri(o + 1, o + 1)]);
+  }
   for (unsigned left = v; left; left &= left - 1u) {
     const int o = 2 * (__ffs((int)left) - 1);
     if (threadIdx.x < 32) {  // one warp forms the pivot (every lane the same)
@@ -887,7 +912,9 @@ __device__ __forceinline__ FxPart<typename fx_sum<E>::type> fx_cta_tree(unsigned
     }
   }
   for (int i = threadIdx.x; i < sym(2 * n); i += nthr) {
-    mats[i] = fx_of<E>(root(i));
+    const double x = root(i);
+    ok &= fx_root_entry_ok(x);
+    mats[i] = fx_of<E>(x);
     int a = (int)((sqrtf(8.0f * (float)i + 1.0f) - 1.0f) * 0.5f);
     while (a * (a + 1) / 2 > i) --a;
     while ((a + 1) * (a + 2) / 2 <= i) ++a;
@@ -898,6 +925,10 @@ __device__ __forceinline__ FxPart<typename fx_sum<E>::type> fx_cta_tree(unsigned
     const int k = 31 - __clz(v | 1), p = v ? ns - 1 - k : n;
     base[v] = v ? lvl[k] + (v - (1 << k)) * sym(2 * p) : 0;
     held[v] = (unsigned char)p;
+  }
+  if ((int)threadIdx.x < n) {
+    const int o = 2 * threadIdx.x;
+    ok &= fx_root_mode_ok(mats[tri(o, o)], mats[tri(o + 1, o + 1)]);
   }
   S* sv = reinterpret_cast<S*>(mats + lvl[D]);
   FxPivot<E>* piv = reinterpret_cast<FxPivot<E>*>(sv + (1 << D));
