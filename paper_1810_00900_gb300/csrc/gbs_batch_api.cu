@@ -359,6 +359,8 @@ gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const Batch
       ctx->batch_split = false;
       return split();
     }
+    // the floating engine keeps two levels where the fixed-point one keeps all of a chunk
+    if (st == GBS_ENOMEM && fixed64) return batch_eval(ctx, prec, real, ntrees, trees, roots_dev, logdet, host_out);
     return st;
   }
   if ((st = check_cuda(ctx, cudaMemcpyAsync(host_out, po, n * sizeof(ProbOut), cudaMemcpyDeviceToHost, ctx->stream),

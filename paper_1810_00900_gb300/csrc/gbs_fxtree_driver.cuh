@@ -52,6 +52,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     blocks[several] += 1LL << d0;
     small_n[several] = std::max(small_n[several], n);
   }
+  ntrees = (int)order.size();
   // the timer takes the leaf launches, or the small trees' where there are none
   auto timer = [&](bool stop) {
     if (!ctx->timing) return;
@@ -62,27 +63,35 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     cudaEventRecord(stop ? ctx->leaf_timer.stop : ctx->leaf_timer.start, ctx->stream);
     if (stop) ctx->leaf_timer.pending = true;
   };
-  if (order.empty()) timer(false);
-  for (int c = 0; c < 2; ++c) {
-    if (small[c].empty()) continue;
-    const void* d_small = nullptr;
-    gbs_status st;
-    if ((st = stage(ctx, small[c].data(), small[c].size() * sizeof(FxSmall), &d_small)) ||
-        (st = dev_reserve(ctx, ctx->sbuf[1], (size_t)blocks[1] * sizeof(FxPart<S>))))
-      return st;
-    const int smem = fx_small_words(small_n[c], c ? kSub : small_n[c], L, LS) * 4;
-    if ((st = allow_smem(ctx, fx_small_kernel<E>, (size_t)smem, "small tree smem"))) return st;
-    int threads = c || small_n[c] >= 8 ? 512 : small_n[c] >= 6 ? 256 : small_n[c] >= 4 ? 128 : 32;
-    if (blocks[c] > ctx->sm_count) threads = std::min(threads, 256);  // two CTAs per SM
-    fx_small_kernel<E><<<(unsigned)blocks[c], threads, smem, ctx->stream>>>(
-        (const FxSmall*)d_small, (int)small[c].size(), (const double*)roots_dev, fin.u, fin.extra,
-        (FxPart<S>*)ctx->sbuf[1].ptr, fin.counts, status_dev, fin.po);
-    count_launch(ctx);
-    if ((st = check_cuda(ctx, cudaGetLastError(), "small trees"))) return st;
+  // Launched once the others have their workspace: a batch that is evaluated in parts for
+  // want of it has not run its small trees yet.
+  auto launch_small = [&]() -> gbs_status {
+    for (int c = 0; c < 2; ++c) {
+      if (small[c].empty()) continue;
+      const void* d_small = nullptr;
+      gbs_status st;
+      if ((st = stage(ctx, small[c].data(), small[c].size() * sizeof(FxSmall), &d_small)) ||
+          (st = dev_reserve(ctx, ctx->sbuf[1], (size_t)blocks[1] * sizeof(FxPart<S>))))
+        return st;
+      const int smem = fx_small_words(small_n[c], c ? kSub : small_n[c], L, LS) * 4;
+      if ((st = allow_smem(ctx, fx_small_kernel<E>, (size_t)smem, "small tree smem"))) return st;
+      int threads = c || small_n[c] >= 8 ? 512 : small_n[c] >= 6 ? 256 : small_n[c] >= 4 ? 128 : 32;
+      if (blocks[c] > ctx->sm_count) threads = std::min(threads, 256);  // two CTAs per SM
+      fx_small_kernel<E><<<(unsigned)blocks[c], threads, smem, ctx->stream>>>(
+          (const FxSmall*)d_small, (int)small[c].size(), (const double*)roots_dev, fin.u, fin.extra,
+          (FxPart<S>*)ctx->sbuf[1].ptr, fin.counts, status_dev, fin.po);
+      count_launch(ctx);
+      if ((st = check_cuda(ctx, cudaGetLastError(), "small trees"))) return st;
+    }
+    return GBS_OK;
+  };
+  gbs_status st;
+  if (ntrees == 0) {
+    timer(false);
+    if ((st = launch_small())) return st;
+    timer(true);
+    return GBS_OK;
   }
-  if (order.empty()) timer(true);
-  ntrees = (int)order.size();
-  if (ntrees <= 0) return GBS_OK;
   // ---------------- plan
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return in[a].n > in[b].n; });
   // Levels per leaf thread.
@@ -103,47 +112,92 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     trees[i] = FxTree{b.root_off, 0, fin.scale[order[i]], b.n, b.n - Q[i], order[i], 34 * i, 0, 0};
   }
   const int D0 = trees[0].D;
-  // A single tree too large for the workspace goes in chunks of 2^cb nodes of depth d0
-  // (FxTree): the deepest split with the fewest chunks that fits.
-  const size_t cap = ctx->batch_cap_bytes ? ctx->batch_cap_bytes : (size_t)64 << 30;
-  auto tree_bytes = [&](int i, int d0, int cb) {
-    const int n = trees[i].n, D = trees[i].D;
-    long long words = fx_level_words(n, -1, 1, L), sv = 1LL << d0;
-    for (int k = 0; k < D; ++k) words += fx_level_words(n, k, k < d0 ? 1LL << k : 1LL << (k - d0 + cb), L);
-    sv += (1LL << (D - d0 + cb)) - (1LL << cb);
-    return (size_t)words * 4 + (size_t)sv * sizeof(S);
+  // Workspace: all levels of all trees, and a partial sum per leaf CTA (N = 20, 24, 26, 28:
+  // 63 MB, 1.0, 3.9, 15.6 GB with 64 fraction bits, 157 MB, 2.5, 9.8, 39 GB with 160).  A
+  // single tree beyond its limit, a sixteenth of the device, goes in chunks of 2^cb nodes of
+  // depth d0 (FxTree).  Where the device or the context's budget has less than the limit
+  // left, a batch is evaluated in parts and a single tree in more chunks.
+  // Tiles per warp: about five waves of the 16 warps an SM holds.  (One wave, and a few
+  // CTAs more than that because every tree ends in a part of one, took twice its time:
+  // 300 trees of 15 .. 17 modes, 64 fraction bits, 685 us.)
+  auto tiles_of = [&](int i, int d0, int cb) { return ((1LL << (trees[i].D - d0 + cb)) + 31) / 32; };
+  auto tpu_of = [&](int d0, int cb) {
+    long long tiles = 0;
+    for (int i = 0; i < ntrees; ++i) tiles += tiles_of(i, d0, cb);
+    return (int)std::max(1LL, std::min(64LL, tiles / (80LL * ctx->sm_count)));
   };
-  size_t need = 0;
-  for (int i = 0; i < ntrees; ++i) need += tree_bytes(i, 0, 0);
-  int d0 = 0, cb = 0;
-  if (need > cap) {
-    if (ntrees > 1) {
-      ctx->batch_split = true;  // the caller evaluates the batch in parts
-      return GBS_ENOMEM;
+  auto units_of = [&](int i, int d0, int cb, int tpu) { return (tiles_of(i, d0, cb) + 4 * tpu - 1) / (4 * tpu); };
+  auto level_count = [](int k, int d0, int cb) { return d0 == 0 || k < d0 ? 1LL << k : 1LL << (k - d0 + cb); };
+  auto s_count = [&](int i, int d0, int cb) {
+    const int D = trees[i].D;
+    return d0 ? (1LL << d0) + (1LL << (D - d0 + cb)) - (1LL << cb) : 1LL << D;
+  };
+  auto r32 = [](long long w) { return (w + 31) / 32 * 32; };
+  auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
+  struct Space {
+    int d0, cb;
+    size_t nodes, s, total;
+  };
+  auto space_of = [&](int d0, int cb) {
+    const int tpu = tpu_of(d0, cb);
+    long long words = 0, sv = 0, units = 0;
+    for (int i = 0; i < ntrees; ++i) {
+      const int n = trees[i].n;
+      words += r32(fx_level_words(n, -1, 1, L));
+      for (int k = 0; k < trees[i].D; ++k) words += r32(fx_level_words(n, k, level_count(k, d0, cb), L));
+      sv += s_count(i, d0, cb);
+      units += units_of(i, d0, cb, tpu) << (d0 - cb);
     }
-    size_t best = ~(size_t)0;
-    for (int chunk_bits = 1; chunk_bits <= D0 - 5 && best > cap; ++chunk_bits)  // log2 of the number of chunks
-      for (int d = std::max(5 + chunk_bits, std::min(d_top, D0)); d < D0; ++d) {
-        const size_t b = tree_bytes(0, d, d - chunk_bits);
-        if (b < best) best = b, d0 = d, cb = d - chunk_bits;
+    const size_t nodes = r256((size_t)words * 4), s = r256((size_t)sv * sizeof(S));
+    return Space{d0, cb, nodes, s, nodes + s + (size_t)units * sizeof(FxPart<S>)};
+  };
+  // The fewest chunks that fit, from the deepest level on, since each chunk repeats the
+  // launches below it (160 bits, N = 24 in 2 GB: 2.41 ms, 2.52 from the shallowest level on,
+  // 2.37 whole; N = 26 in 8, 4, 1 GB 8.62, 8.84, 10.2 ms, 8.61 whole); the least there is where
+  // nothing fits.
+  auto fit = [&](size_t limit) {
+    Space least = space_of(0, 0);
+    if (least.total <= limit) return least;
+    for (int chunk_bits = 1; chunk_bits <= D0 - 5; ++chunk_bits)  // log2 of the number of chunks
+      for (int d = D0 - 1; d >= std::max(5 + chunk_bits, std::min(d_top, D0)); --d) {
+        const Space c = space_of(d, d - chunk_bits);
+        if (c.total <= limit) return c;
+        if (c.total < least.total) least = c;
       }
-    if (best == ~(size_t)0) d0 = cb = 0;
+    return least;
+  };
+  Space space = ntrees > 1 ? space_of(0, 0) : fit(ctx->tree_cap_bytes);
+  if (ntrees > 1 && space.total > ctx->batch_cap_bytes) {
+    ctx->batch_split = true;  // the caller evaluates the batch in parts
+    return GBS_ENOMEM;
   }
+  // one allocation: a context's first call pays for each
+  while ((st = dev_reserve(ctx, ctx->lvl[0], space.total)) == GBS_ENOMEM) {
+    if (ntrees > 1) {
+      ctx->batch_split = true;
+      return st;
+    }
+    const Space less = fit(space.total / 2);
+    if (less.total >= space.total) return st;
+    space = less;
+  }
+  if (st || (st = launch_small())) return st;
+  const int d0 = space.d0, cb = space.cb;
   std::vector<long long> off(34 * (size_t)ntrees, 0);
   long long words = 0, selems = 0;
   for (int i = 0; i < ntrees; ++i) {
     const int n = trees[i].n, D = trees[i].D;
     long long* o = &off[34 * (size_t)i];
     o[0] = words;
-    words += (fx_level_words(n, -1, 1, L) + 31) / 32 * 32;
+    words += r32(fx_level_words(n, -1, 1, L));
     for (int k = 0; k < D; ++k) {
       o[k + 1] = words;
-      words += (fx_level_words(n, k, k < d0 || d0 == 0 ? 1LL << k : 1LL << (k - d0 + cb), L) + 31) / 32 * 32;
+      words += r32(fx_level_words(n, k, level_count(k, d0, cb), L));
     }
     trees[i].s_base = selems;
-    selems += d0 ? (1LL << d0) + (1LL << (D - d0 + cb)) - (1LL << cb) : 1LL << D;
+    selems += s_count(i, d0, cb);
   }
-  const int chunks = d0 ? 1 << (d0 - cb) : 1;
+  const int chunks = 1 << (d0 - cb);
   std::vector<FxTree> chunked = trees;
   for (FxTree& t : chunked) t.d0 = d0, t.cb = cb;
   // top: the levels below min(D, d_top)
@@ -199,34 +253,19 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   };
   std::vector<Leaf> leaves;
   std::vector<FxSeg> sums;
-  long long tiles_total = 0, units_total = 0;
-  for (int i = 0; i < ntrees; ++i) tiles_total += ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
-  // Tiles per warp: about five waves of the 16 warps an SM holds.  (One wave, and a few
-  // CTAs more than that because every tree ends in a part of one, took twice its time:
-  // 300 trees of 15 .. 17 modes, 64 fraction bits, 685 us.)
-  const int tpu = (int)std::max(1LL, std::min(64LL, tiles_total / (80LL * ctx->sm_count)));
+  long long units_total = 0;
+  const int tpu = tpu_of(d0, cb);
   for (int i = 0; i < ntrees; ++i) {
     if (leaves.empty() || leaves.back().Q != Q[i]) leaves.push_back(Leaf{Q[i], {}, 0, 0});
     Leaf& lf = leaves.back();
-    const long long tiles = ((1LL << (trees[i].D - d0 + cb)) + 31) / 32;
-    const long long units = (tiles + 4 * tpu - 1) / (4 * tpu);
+    const long long units = units_of(i, d0, cb, tpu);
     lf.segs.push_back(FxSeg{lf.units, i, tpu});
     lf.units += units;
     sums.push_back(FxSeg{units_total, i, 0});
     units_total += units * chunks;
   }
   sums.push_back(FxSeg{units_total, 0, 0});
-  // ---------------- memory
-  const size_t part_bytes = (size_t)units_total * sizeof(FxPart<S>);
-  if (ntrees > 1 && need + part_bytes > cap) {
-    ctx->batch_split = true;
-    return GBS_ENOMEM;
-  }
-  gbs_status st;
-  // one allocation: a context's first call pays for each
-  auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t node_bytes = r256((size_t)words * 4), s_bytes = r256((size_t)selems * sizeof(S));
-  if ((st = dev_reserve(ctx, ctx->lvl[0], node_bytes + s_bytes + part_bytes))) return st;
+  // ---------------- upload
   Blob blob;
   const size_t o_trees = blob.put(trees), o_chunked = blob.put(chunked), o_off = blob.put(off), o_top = blob.put(top);
   for (Launch& l : levels) l.at = blob.put(l.segs);
@@ -235,8 +274,8 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   const unsigned char* plan = nullptr;
   if ((st = stage(ctx, blob.bytes.data(), blob.bytes.size(), (const void**)&plan))) return st;
   uint32_t* nodes = (uint32_t*)ctx->lvl[0].ptr;
-  S* sval = (S*)((unsigned char*)nodes + node_bytes);
-  FxPart<S>* parts = (FxPart<S>*)((unsigned char*)nodes + node_bytes + s_bytes);
+  S* sval = (S*)((unsigned char*)nodes + space.nodes);
+  FxPart<S>* parts = (FxPart<S>*)((unsigned char*)nodes + space.nodes + space.s);
   const FxTree* d_trees = (const FxTree*)(plan + o_trees);
   const FxTree* d_chunked = (const FxTree*)(plan + o_chunked);
   const long long* d_off = (const long long*)(plan + o_off);

@@ -110,7 +110,8 @@ struct gbs_ctx {
   // A batch whose tree workspace (level buffers, s values, partials) would
   // exceed batch_cap_bytes is refused by the planner before anything is
   // allocated or launched (batch_split set) and evaluated in parts instead.
-  size_t batch_cap_bytes = 0;
+  // A single tree of the fixed-point engine keeps to tree_cap_bytes in chunks.
+  size_t batch_cap_bytes = 0, tree_cap_bytes = 0;
   bool batch_split = false;
 };
 
