@@ -14,32 +14,38 @@ namespace gbs {
 
 gbs_status stage_begin(gbs_ctx* ctx, size_t bytes) {
   bytes = (bytes + 4096 + 255) / 256 * 256;
-  if (bytes > ctx->stage_cap) {
-    gbs_status st;
+  StageArena& a = ctx->stage;
+  gbs_status st;
+  if (bytes > a.cap) {
     if ((st = stream_sync(ctx))) return st;
-    size_t cap = std::max(bytes, ctx->stage_cap * 2);
+    size_t cap = std::max(bytes, a.cap * 2);
     cap = std::max(cap, (size_t)1 << 20);
     if (ctx->stage_host) cudaFreeHost(ctx->stage_host);
     ctx->stage_host = nullptr;
-    ctx->stage_cap = 0;
+    a.cap = 0;
     if ((st = check_cuda(ctx, cudaMallocHost(&ctx->stage_host, cap), "pinned staging"))) return st;
     dev_free(ctx, ctx->stage_dev);
     if ((st = dev_alloc(ctx, ctx->stage_dev, cap))) return st;
-    ctx->stage_cap = cap;
+    a.cap = cap;
   }
-  ctx->stage_off = 0;
+  if (a.begin()) {
+    if ((st = stream_sync(ctx))) return st;
+    a.begin();
+  }
   return GBS_OK;
 }
 
 gbs_status stage(gbs_ctx* ctx, const void* data, size_t bytes, const void** dev) {
-  const size_t off = (ctx->stage_off + 255) / 256 * 256;
-  if (off + bytes > ctx->stage_cap) return set_error(ctx, GBS_ENOMEM, "staging arena too small for this call");
+  StageArena& a = ctx->stage;
+  if (!a.fits(bytes)) return set_error(ctx, GBS_ENOMEM, "staging arena too small for this call");
+  gbs_status st;
+  if (!a.clear(bytes) && (st = stream_sync(ctx))) return st;
+  const size_t off = a.take(bytes);
   unsigned char* h = (unsigned char*)ctx->stage_host + off;
   unsigned char* d = (unsigned char*)ctx->stage_dev.ptr + off;
-  if (bytes) memcpy(h, data, bytes);
-  ctx->stage_off = off + bytes;
   *dev = d;
   if (!bytes) return GBS_OK;
+  memcpy(h, data, bytes);
   return check_cuda(ctx, cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, ctx->stream), "stage copy");
 }
 

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/gbs.h"
+#include "gbs_stage.h"
 
 namespace gbs {
 
@@ -79,11 +80,10 @@ struct gbs_ctx {
   // tree workspace (grown on demand)
   gbs::DevBuf lvl[2], sbuf[2], partials, out, status, hbuf;
   // batched engine: small tables staged host -> device through a bump arena
-  // (pinned host + device, reset at the start of each synchronous call) and
-  // the per-tree results
+  // (pinned host + device, reset at the start of each call) and the per-tree results
   gbs::DevBuf stage_dev, aux_dev;
   void* stage_host = nullptr;
-  size_t stage_cap = 0, stage_off = 0;
+  gbs::StageArena stage;
   // host-pinned readback
   void* host_out = nullptr;
 
@@ -170,7 +170,8 @@ gbs_status stream_sync(gbs_ctx* ctx);
 
 // Staging arena: stage_begin() makes room for `bytes` (synchronising first if it
 // must grow) and resets it; stage() copies host data into the next region and
-// queues the host -> device copy on the context stream.  (gbs_batch_api.cu)
+// queues the host -> device copy on the context stream.  Both wait for the stream where
+// they would write over bytes whose copy may still be queued.  (gbs_batch_api.cu)
 gbs_status stage_begin(gbs_ctx* ctx, size_t bytes);
 gbs_status stage(gbs_ctx* ctx, const void* data, size_t bytes, const void** dev);
 
