@@ -43,6 +43,15 @@ void cache_release(gbs_ctx* ctx) {
   ctx->cached = 0;
 }
 
+// An allocation would fail: what no queued work needs.
+static void memory_release(gbs_ctx* ctx) {
+  if (ctx->side_nodes.ptr && !ctx->side_batch) {
+    cudaStreamSynchronize(ctx->stream);  // which has been joined with the side stream
+    dev_free(ctx, ctx->side_nodes);
+  }
+  cache_release(ctx);
+}
+
 gbs_status dev_alloc(gbs_ctx* ctx, DevBuf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   bytes = (bytes + 255) / 256 * 256;
@@ -58,14 +67,14 @@ gbs_status dev_alloc(gbs_ctx* ctx, DevBuf& b, size_t bytes) {
       return GBS_OK;
     }
   }
-  if (ctx->budget && ctx->in_use.load() + bytes > ctx->budget) cache_release(ctx);
+  if (ctx->budget && ctx->in_use.load() + bytes > ctx->budget) memory_release(ctx);
   if (ctx->budget && ctx->in_use.load() + bytes > ctx->budget)
     return set_error(ctx, GBS_ENOMEM, "device memory budget of the context exceeded");
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    cache_release(ctx);  // CUDA may have been short of memory held in the cache
+    memory_release(ctx);  // CUDA may have been short of memory held here
     e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -249,15 +258,19 @@ void gbs_ctx_destroy(gbs_ctx* ctx) {
   server_shutdown(ctx);
   cudaStreamSynchronize(ctx->stream);
   DevBuf* bufs[] = {&ctx->lvl[0], &ctx->lvl[1], &ctx->sbuf[0], &ctx->sbuf[1], &ctx->partials,
-                    &ctx->out,    &ctx->status, &ctx->hbuf,    &ctx->stage_dev, &ctx->aux_dev};
+                    &ctx->out,    &ctx->status, &ctx->hbuf,    &ctx->stage_dev, &ctx->aux_dev, &ctx->side_nodes, &ctx->small_parts};
   for (DevBuf* b : bufs) dev_free(ctx, *b);
   cache_release(ctx);
-  if (ctx->leaf_timer.start) {
-    cudaEventDestroy(ctx->leaf_timer.start);
-    cudaEventDestroy(ctx->leaf_timer.stop);
-  }
+  for (KernelTimer* t : {&ctx->leaf_timer, &ctx->fx_leaf_timer})
+    if (t->start) {
+      cudaEventDestroy(t->start);
+      cudaEventDestroy(t->stop);
+    }
   if (ctx->host_out) cudaFreeHost(ctx->host_out);
   if (ctx->stage_host) cudaFreeHost(ctx->stage_host);
+  if (ctx->side_go) cudaEventDestroy(ctx->side_go);
+  if (ctx->side_done) cudaEventDestroy(ctx->side_done);
+  if (ctx->side) cudaStreamDestroy(ctx->side);
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }

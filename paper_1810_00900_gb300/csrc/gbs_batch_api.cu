@@ -336,17 +336,9 @@ static gbs_status batch_variant(gbs_ctx* ctx, int prec, bool real, bool fixed64,
 }
 
 gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const BatchTree* trees, const void* roots_dev,
-                      const double* logdet, ProbOut* host_out, bool bounded) {
+                      const double* logdet, ProbOut* host_out, int n_bounded) {
   if (ntrees <= 0) return GBS_OK;
   gbs_status st;
-  // too large for one plan: the two halves in turn (a tree's result does not depend
-  // on the rest of its batch, so the split changes no value)
-  auto split = [&]() -> gbs_status {
-    const int h = ntrees / 2;
-    gbs_status s2 = batch_eval(ctx, prec, real, h, trees, roots_dev, logdet, host_out, bounded);
-    if (s2) return s2;
-    return batch_eval(ctx, prec, real, ntrees - h, trees + h, roots_dev, logdet + h, host_out + h, bounded);
-  };
   const size_t n = (size_t)ntrees;
   auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t bytes = r256(n * sizeof(ProbOut)) + r256(2 * n * sizeof(int));
@@ -354,48 +346,78 @@ gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const Batch
   ProbOut* po = (ProbOut*)ctx->aux_dev.ptr;
   int* status = (int*)((unsigned char*)po + r256(n * sizeof(ProbOut)));  // then the counters
   if ((st = check_cuda(ctx, cudaMemsetAsync(status, 0, 2 * n * sizeof(int), ctx->stream), "memset"))) return st;
-  ctx->batch_split = false;
   const double u = unit_roundoff_b(prec), extra = err_factor(prec, 1) - err_factor(GBS_PREC_TD, 1);
-  const bool fixed64 = bounded && real && prec == GBS_PREC_FP64;
   std::vector<double> scale(n);
   for (size_t t = 0; t < n; ++t) scale[t] = std::exp(-0.5 * logdet[t]);
-  if ((st = batch_variant(ctx, prec, real, fixed64, ntrees, trees, roots_dev, status,
-                          TreeFinish{scale.data(), u, extra, po, status + n}))) {
+  // The bounded trees and the others, each on its engine, side by side and with one wait for
+  // both: few trees are latency on either (16 FP64 requests of 8 .. 17 modes, half of them of
+  // a state without a bound: 275 us in turn with a wait each, 264 with one, 186 side by side).
+  struct Part {
+    int first, count;
+    bool fixed64;
+    enum { kRun, kSplit, kFloat } todo;
+  };
+  const int nb = real && prec == GBS_PREC_FP64 ? n_bounded : 0;
+  Part parts[2] = {{0, nb, true, Part::kRun}, {nb, ntrees - nb, false, Part::kRun}};
+  gbs_status failed = GBS_OK;
+  ctx->side_batch = nb > 0 && nb < ntrees;
+  for (Part& p : parts) {
+    if (p.count == 0 || failed) continue;
+    ctx->batch_split = false;
+    st = batch_variant(ctx, prec, real, p.fixed64, p.count, trees + p.first, roots_dev, status + p.first,
+                       TreeFinish{scale.data() + p.first, u, extra, po + p.first, status + n + p.first,
+                                  p.fixed64 && ctx->side_batch});
     if (st == GBS_ENOMEM && ctx->batch_split) {
-      ctx->batch_split = false;
-      return split();
+      p.todo = Part::kSplit;
+    } else if (st == GBS_ENOMEM && (p.fixed64 || ctx->side_batch)) {
+      // by itself, on the floating engine: that keeps two levels where the fixed-point one
+      // keeps all of a chunk, and the other part's workspace is free then
+      p.todo = Part::kFloat;
+    } else {
+      failed = st;
     }
-    // the floating engine keeps two levels where the fixed-point one keeps all of a chunk
-    if (st == GBS_ENOMEM && fixed64) return batch_eval(ctx, prec, real, ntrees, trees, roots_dev, logdet, host_out);
-    return st;
   }
+  ctx->side_batch = false;
+  if ((st = side_join(ctx))) return st;
+  if (failed) return failed;
   if ((st = check_cuda(ctx, cudaMemcpyAsync(host_out, po, n * sizeof(ProbOut), cudaMemcpyDeviceToHost, ctx->stream),
                        "readback")) ||
       (st = stream_sync(ctx)))
     return st;
-  if (ctx->timing && ctx->leaf_timer.pending) {
+  for (KernelTimer* t : {&ctx->leaf_timer, &ctx->fx_leaf_timer}) {
+    if (!t->pending) continue;
     float ms = 0.f;
-    cudaEventElapsedTime(&ms, ctx->leaf_timer.start, ctx->leaf_timer.stop);
+    cudaEventElapsedTime(&ms, t->start, t->stop);
     ctx->leaf_timer.total_ms += ms;
     ctx->leaf_timer.count += 1;
-    ctx->leaf_timer.pending = false;
+    t->pending = false;
   }
-  if (fixed64) {
-    // a tree whose values left the range after all: again in floating point
-    std::vector<BatchTree> again;
-    std::vector<double> ld;
-    std::vector<int> which;
-    for (int t = 0; t < ntrees; ++t)
-      if (host_out[t].status == kStatusRange) {
-        again.push_back(trees[t]);
-        ld.push_back(logdet[t]);
-        which.push_back(t);
-      }
-    if (!again.empty()) {
-      std::vector<ProbOut> r(again.size());
-      if ((st = batch_eval(ctx, prec, real, (int)again.size(), again.data(), roots_dev, ld.data(), r.data()))) return st;
-      for (size_t i = 0; i < which.size(); ++i) host_out[which[i]] = r[i];
+  for (const Part& p : parts) {
+    if (p.todo == Part::kRun) continue;
+    // too large for one plan: the two halves in turn (a tree's result does not depend
+    // on the rest of its batch, so the split changes no value)
+    const int half = p.todo == Part::kSplit ? p.count / 2 : p.count;
+    for (int i = 0, c = half; i < p.count; i += c, c = p.count - half) {
+      const int k = p.first + i;
+      if ((st = batch_eval(ctx, prec, real, c, trees + k, roots_dev, logdet + k, host_out + k,
+                           p.fixed64 && p.todo == Part::kSplit ? c : 0)))
+        return st;
     }
+  }
+  // a bounded tree whose values left the range after all: again in floating point
+  std::vector<BatchTree> again;
+  std::vector<double> ld;
+  std::vector<int> which;
+  for (int t = 0; t < nb; ++t)
+    if (host_out[t].status == kStatusRange) {
+      again.push_back(trees[t]);
+      ld.push_back(logdet[t]);
+      which.push_back(t);
+    }
+  if (!again.empty()) {
+    std::vector<ProbOut> r(again.size());
+    if ((st = batch_eval(ctx, prec, real, (int)again.size(), again.data(), roots_dev, ld.data(), r.data()))) return st;
+    for (size_t i = 0; i < which.size(); ++i) host_out[which[i]] = r[i];
   }
   return GBS_OK;
 }
@@ -566,9 +588,7 @@ gbs_status probs_batch(gbs_ctx* ctx, int nreq, const gbs_state* const* states, c
       ld[i] = states[run[i]]->logdet_sigma;
     }
     std::vector<ProbOut> res(run.size());
-    if ((st = batch_eval(ctx, pr, real, (int)nb, sub.data(), ctx->hbuf.ptr, ld.data(), res.data(), true)) ||
-        (st = batch_eval(ctx, pr, real, (int)(run.size() - nb), sub.data() + nb, ctx->hbuf.ptr, ld.data() + nb,
-                         res.data() + nb)))
+    if ((st = batch_eval(ctx, pr, real, (int)run.size(), sub.data(), ctx->hbuf.ptr, ld.data(), res.data(), (int)nb)))
       return st;
     for (size_t i = 0; i < run.size(); ++i) {
       fill(&out[run[i]], res[i], pr, real, ld[i]);

@@ -21,6 +21,27 @@ struct Blob {
 };
 
 
+// Work queued on ctx->side from here on follows what is on the context's stream so far.
+// Whoever forks joins on every path (side_join): the stream's later work then follows the side's.
+inline gbs_status side_fork(gbs_ctx* ctx) {
+  gbs_status st = GBS_OK;
+  if (!ctx->side &&
+      ((st = check_cuda(ctx, cudaEventCreateWithFlags(&ctx->side_go, cudaEventDisableTiming), "side event")) ||
+       (st = check_cuda(ctx, cudaEventCreateWithFlags(&ctx->side_done, cudaEventDisableTiming), "side event")) ||
+       (st = check_cuda(ctx, cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking), "side stream"))))
+    return st;
+  if ((st = check_cuda(ctx, cudaEventRecord(ctx->side_go, ctx->stream), "side fork"))) return st;
+  ctx->on_side = true;
+  return check_cuda(ctx, cudaStreamWaitEvent(ctx->side, ctx->side_go, 0), "side fork");
+}
+inline gbs_status side_join(gbs_ctx* ctx) {
+  gbs_status st;
+  if (!ctx->on_side) return GBS_OK;
+  ctx->on_side = false;
+  if ((st = check_cuda(ctx, cudaEventRecord(ctx->side_done, ctx->side), "side join"))) return st;
+  return check_cuda(ctx, cudaStreamWaitEvent(ctx->stream, ctx->side_done, 0), "side join");
+}
+
 // Launch of a kernel that itself waits for the launch before it (programmatic dependent
 // launch): before it touches what that one writes (fx_after), or, where the two touch nothing
 // in common (leaf launches of different Q), at its end.  early: its CTAs may be set up while that launch runs -- where that one leaves

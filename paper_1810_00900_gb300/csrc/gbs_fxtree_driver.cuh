@@ -54,44 +54,52 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   }
   ntrees = (int)order.size();
   // the timer takes the leaf launches, or the small trees' where there are none
+  cudaStream_t s = ctx->stream;
   auto timer = [&](bool stop) {
     if (!ctx->timing) return;
-    if (!ctx->leaf_timer.start) {
-      cudaEventCreate(&ctx->leaf_timer.start);
-      cudaEventCreate(&ctx->leaf_timer.stop);
+    KernelTimer& tm = ctx->fx_leaf_timer;
+    if (!tm.start) {
+      cudaEventCreate(&tm.start);
+      cudaEventCreate(&tm.stop);
     }
-    cudaEventRecord(stop ? ctx->leaf_timer.stop : ctx->leaf_timer.start, ctx->stream);
-    if (stop) ctx->leaf_timer.pending = true;
+    cudaEventRecord(stop ? tm.stop : tm.start, s);
+    if (stop) tm.pending = true;
+  };
+  // Everything uploaded: what follows may go beside what the caller queues next.
+  auto fork = [&]() -> gbs_status {
+    if (!fin.beside) return GBS_OK;
+    if (const gbs_status e = side_fork(ctx)) return e;
+    s = ctx->side;
+    return GBS_OK;
   };
   // Launched once the others have their workspace: a batch that is evaluated in parts for
   // want of it has not run its small trees yet.
+  gbs_status st;
   auto launch_small = [&]() -> gbs_status {
+    const void* d_small[2] = {};
+    for (int c = 0; c < 2; ++c)
+      if ((st = stage(ctx, small[c].data(), small[c].size() * sizeof(FxSmall), &d_small[c]))) return st;
+    if ((st = dev_reserve(ctx, ctx->small_parts, (size_t)blocks[1] * sizeof(FxPart<S>)))) return st;
+    if (ntrees == 0) {
+      if ((st = fork())) return st;
+      timer(false);
+    }
     for (int c = 0; c < 2; ++c) {
       if (small[c].empty()) continue;
-      const void* d_small = nullptr;
-      gbs_status st;
-      if ((st = stage(ctx, small[c].data(), small[c].size() * sizeof(FxSmall), &d_small)) ||
-          (st = dev_reserve(ctx, ctx->sbuf[1], (size_t)blocks[1] * sizeof(FxPart<S>))))
-        return st;
       const int smem = fx_small_words(small_n[c], c ? kSub : small_n[c], L, LS) * 4;
       if ((st = allow_smem(ctx, fx_small_kernel<E>, (size_t)smem, "small tree smem"))) return st;
       int threads = c || small_n[c] >= 8 ? 512 : small_n[c] >= 6 ? 256 : small_n[c] >= 4 ? 128 : 32;
       if (blocks[c] > ctx->sm_count) threads = std::min(threads, 256);  // two CTAs per SM
-      fx_small_kernel<E><<<(unsigned)blocks[c], threads, smem, ctx->stream>>>(
-          (const FxSmall*)d_small, (int)small[c].size(), (const double*)roots_dev, fin.u, fin.extra,
-          (FxPart<S>*)ctx->sbuf[1].ptr, fin.counts, status_dev, fin.po);
+      fx_small_kernel<E><<<(unsigned)blocks[c], threads, smem, s>>>(
+          (const FxSmall*)d_small[c], (int)small[c].size(), (const double*)roots_dev, fin.u, fin.extra,
+          (FxPart<S>*)ctx->small_parts.ptr, fin.counts, status_dev, fin.po);
       count_launch(ctx);
       if ((st = check_cuda(ctx, cudaGetLastError(), "small trees"))) return st;
     }
+    if (ntrees == 0) timer(true);
     return GBS_OK;
   };
-  gbs_status st;
-  if (ntrees == 0) {
-    timer(false);
-    if ((st = launch_small())) return st;
-    timer(true);
-    return GBS_OK;
-  }
+  if (ntrees == 0) return launch_small();
   // ---------------- plan
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return in[a].n > in[b].n; });
   // Levels per leaf thread.
@@ -172,7 +180,8 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     return GBS_ENOMEM;
   }
   // one allocation: a context's first call pays for each
-  while ((st = dev_reserve(ctx, ctx->lvl[0], space.total)) == GBS_ENOMEM) {
+  DevBuf& buf = fin.beside ? ctx->side_nodes : ctx->lvl[0];
+  while ((st = dev_reserve(ctx, buf, space.total)) == GBS_ENOMEM) {
     if (ntrees > 1) {
       ctx->batch_split = true;
       return st;
@@ -273,13 +282,12 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   const size_t o_sums = blob.put(sums);
   const unsigned char* plan = nullptr;
   if ((st = stage(ctx, blob.bytes.data(), blob.bytes.size(), (const void**)&plan))) return st;
-  uint32_t* nodes = (uint32_t*)ctx->lvl[0].ptr;
+  uint32_t* nodes = (uint32_t*)buf.ptr;
   S* sval = (S*)((unsigned char*)nodes + space.nodes);
   FxPart<S>* parts = (FxPart<S>*)((unsigned char*)nodes + space.nodes + space.s);
   const FxTree* d_trees = (const FxTree*)(plan + o_trees);
   const FxTree* d_chunked = (const FxTree*)(plan + o_chunked);
   const long long* d_off = (const long long*)(plan + o_off);
-  cudaStream_t s = ctx->stream;
 
   // ---------------- launches
   const int smem_top = sym(2 * nmax) * (int)sizeof(E) + 2 * nmax * (int)sizeof(FxRow<E>);
@@ -289,6 +297,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
   if ((st = allow_smem(ctx, fx_top_kernel<E>, (size_t)smem_top, "top smem")) ||
       (st = allow_smem(ctx, fx_level_cta_kernel<E>, smem_cta, "level smem")))
     return st;
+  if ((st = fork())) return st;
   fx_top_kernel<E><<<(unsigned)top_blocks, 256, smem_top, s>>>((const FxSeg*)(plan + o_top), ntrees, d_trees, d_off,
                                                                (const double*)roots_dev, nodes, sval, status_dev);
   count_launch(ctx);

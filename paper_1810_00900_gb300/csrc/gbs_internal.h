@@ -79,6 +79,15 @@ struct gbs_ctx {
 
   // tree workspace (grown on demand)
   gbs::DevBuf lvl[2], sbuf[2], partials, out, status, hbuf;
+  gbs::DevBuf small_parts;  // partial sums of one-launch fixed-point trees
+  // Second stream of a batch whose trees run on both engines (batch_eval): forked from
+  // `stream` by side_go, joined to it by side_done before the call returns (on_side between
+  // the two).  side_nodes: levels of the trees that run there, given back when an allocation
+  // would fail outside of such a batch (side_batch).
+  cudaStream_t side = nullptr;
+  cudaEvent_t side_go = nullptr, side_done = nullptr;
+  bool side_batch = false, on_side = false;
+  gbs::DevBuf side_nodes;
   // batched engine: small tables staged host -> device through a bump arena
   // (pinned host + device, reset at the start of each call) and the per-tree results
   gbs::DevBuf stage_dev, aux_dev;
@@ -89,7 +98,7 @@ struct gbs_ctx {
 
   // instrumentation
   bool timing = false;
-  gbs::KernelTimer leaf_timer;
+  gbs::KernelTimer leaf_timer, fx_leaf_timer;  // totals in the first
   std::atomic<long long> launches{0};
   int sm_count = 0;
   int chain_fit[3] = {-1, -1, -1};  // clusters of 2, 4, 8 of the sampler's CTAs that are resident at once
@@ -194,6 +203,9 @@ struct TreeFinish {
   double u, extra;
   ProbOut* po;
   int* counts;
+  // Fixed-point engine: its launches go on ctx->side, beside what the caller queues next
+  // (which shares no memory with them); the caller joins.
+  bool beside = false;
 };
 typedef gbs_status BatchEngine(gbs_ctx*, int ntrees, const BatchTree*, const void* roots, int* status, const BatchTune&,
                                const TreeFinish&);
@@ -204,11 +216,11 @@ BatchEngine batch_fxd_real, batch_fxn_real, batch_fx_real, batch_fxw_real;
 
 // Evaluate ntrees trees whose packed FP64 roots are already in roots_dev
 // (entries at trees[t].root_off); logdet[t] (host) scales p = Tor exp(-logdet/2).
-// Synchronous: fills host_out[0..ntrees).  bounded: FP64 trees in the real basis whose
-// values the caller knows to fit 64-bit fixed point (fxd_ok_*); they run on the integer
-// pipe, and again in floating point if one leaves its range.  (gbs_batch_api.cu)
+// Synchronous: fills host_out[0..ntrees).  The first n_bounded are FP64 trees in the real
+// basis whose values the caller knows to fit 64-bit fixed point (fxd_ok_*); they run on the
+// integer pipe, and again in floating point if one leaves its range.  (gbs_batch_api.cu)
 gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const BatchTree* trees, const void* roots_dev,
-                      const double* logdet, ProbOut* host_out, bool bounded = false);
+                      const double* logdet, ProbOut* host_out, int n_bounded = 0);
 // The tuning in force for (prec, basis) -- the autotuner's choice when one was made.
 const BatchTune& batch_tune_for(gbs_ctx* ctx, int prec, bool real);
 

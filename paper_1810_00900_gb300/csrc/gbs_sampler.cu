@@ -295,16 +295,15 @@ gbs_status sampler_advance(gbs_ctx* ctx, const std::vector<Trajectory*>& jobs, i
     if ((e = stage(ctx, gi.data(), gi.size() * sizeof(GatherItem), &dgi))) return e;
     gather_kernel<<<(unsigned)gi.size(), 128, 0, ctx->stream>>>((const GatherItem*)dgi, (double*)ctx->hbuf.ptr);
     count_launch(ctx);
-    // FP64 trees that their states bound run in 64-bit fixed point, apart from the others
-    for (int pass = 0; pass < 7; ++pass) {
-      const int order[7] = {GBS_PREC_FP64, GBS_PREC_FP64, GBS_PREC_DD, GBS_PREC_FXN, GBS_PREC_FX, GBS_PREC_FXW, GBS_PREC_TD};
-      const int pv = order[pass];
-      const bool bounded = pass == 0;
+    for (int pv : {GBS_PREC_FP64, GBS_PREC_DD, GBS_PREC_FXN, GBS_PREC_FX, GBS_PREC_FXW, GBS_PREC_TD}) {
       std::vector<size_t> grp;
       for (size_t i : todo)
-        if (trees[i].prec == pv && trees[i].n > 0 &&
-            (pv != GBS_PREC_FP64 || fxd_ok_sigma(trees[i].tj->st, trees[i].n) == bounded))
-          grp.push_back(i);
+        if (trees[i].prec == pv && trees[i].n > 0) grp.push_back(i);
+      // FP64 trees that their states bound first: they run in 64-bit fixed point
+      const auto rest = std::stable_partition(grp.begin(), grp.end(), [&](size_t i) {
+        return pv == GBS_PREC_FP64 && fxd_ok_sigma(trees[i].tj->st, trees[i].n);
+      });
+      const int bounded = (int)(rest - grp.begin());
       if (grp.empty()) continue;
       std::vector<BatchTree> sub(grp.size());
       std::vector<double> zero(grp.size(), 0.0);
