@@ -99,8 +99,9 @@ __global__ void __launch_bounds__(64) build_V_kernel(const cplx<double>* __restr
     }
     __syncthreads();
     double car = 0, cai = 0, cbr = 0, cbi = 0;  // this run's sums
+    const int len = min(kVL, M - l0);  // (all of a run for M = 2 as well took 8 us more)
 #pragma unroll 4
-    for (int c = 0; c < kVL; ++c) {
+    for (int c = 0; c < len; ++c) {
       const cplx<double> y = sy[lk][c], p = sc[lj][c], q = ss[lj][c];
       // x conj(y) cosh(2r)/2 and x y sinh(2r)/2
       car = fma(p.re, y.re, fma(p.im, y.im, car));
