@@ -258,7 +258,8 @@ void gbs_ctx_destroy(gbs_ctx* ctx) {
   server_shutdown(ctx);
   cudaStreamSynchronize(ctx->stream);
   DevBuf* bufs[] = {&ctx->lvl[0], &ctx->lvl[1], &ctx->sbuf[0], &ctx->sbuf[1], &ctx->partials,
-                    &ctx->out,    &ctx->status, &ctx->hbuf,    &ctx->stage_dev, &ctx->aux_dev, &ctx->side_nodes, &ctx->small_parts};
+                    &ctx->out,    &ctx->hbuf,   &ctx->stage_dev, &ctx->aux_dev,
+                    &ctx->side_nodes, &ctx->small_parts};
   for (DevBuf* b : bufs) dev_free(ctx, *b);
   cache_release(ctx);
   for (KernelTimer* t : {&ctx->leaf_timer, &ctx->fx_leaf_timer})

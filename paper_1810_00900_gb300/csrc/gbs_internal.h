@@ -78,7 +78,7 @@ struct gbs_ctx {
   size_t cached = 0;
 
   // tree workspace (grown on demand)
-  gbs::DevBuf lvl[2], sbuf[2], partials, out, status, hbuf;
+  gbs::DevBuf lvl[2], sbuf[2], partials, out, hbuf;
   gbs::DevBuf small_parts;  // partial sums of one-launch fixed-point trees
   // Second stream of a batch whose trees run on both engines (batch_eval): forked from
   // `stream` by side_go, joined to it by side_done before the call returns (on_side between

@@ -18,6 +18,7 @@
 //    log det Sigma is the sum of the logs of the pivots.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "gbs_internal.h"
@@ -43,12 +44,13 @@ __global__ void state_params_kernel(const double* __restrict__ r, double eta, in
   logd[l] = log(dp) + log(dm);
 }
 
-// Fixed-order double-double sum of x[0..n) by one block.
+// Fixed-order double-double sum of x[0..n), or of the logarithms (LOG), by one block.
+template <bool LOG>
 __global__ void sum_dd_kernel(const double* __restrict__ x, int n, double* __restrict__ out) {
   // strided per-thread sums, then a fixed-order shuffle tree within each warp
   // and across the (at most 32) warps: deterministic, and no serial loop
   dd acc = dd_make(0.0);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) acc = acc + x[i];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) acc = acc + (LOG ? log(x[i]) : x[i]);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1)
@@ -303,15 +305,18 @@ __device__ __forceinline__ void invert_block(cplx<double> (*S)[kSW + 1], int b, 
   __syncthreads();
 }
 
-// The first pivot block's inverse (Pinv: kSW x kSW, full).
-__global__ void __launch_bounds__(256) sweep_first_kernel(const cplx<double>* __restrict__ X, int D,
+// The first pivot block's inverse (Pinv: kSW x kSW, full); X is swept where that is all of it.
+__global__ void __launch_bounds__(256) sweep_first_kernel(cplx<double>* __restrict__ X, int D,
                                                           cplx<double>* __restrict__ Pinv, double* __restrict__ piv,
                                                           int* __restrict__ status) {
   __shared__ cplx<double> S[kSW][kSW + 1];
   const int b = min(kSW, D), i = threadIdx.x / kSW, j = threadIdx.x % kSW;
   if (i < b && j <= i) S[i][j] = X[(long long)i * D + j];
   invert_block(S, b, piv, status);
-  if (i < b && j < b) Pinv[i * kSW + j] = j <= i ? S[i][j] : cplx<double>{S[j][i].re, -S[j][i].im};
+  if (i >= b || j >= b) return;
+  const cplx<double> p = j <= i ? S[i][j] : cplx<double>{S[j][i].re, -S[j][i].im};
+  Pinv[i * kSW + j] = p;
+  if (D <= kSW && j <= i) X[(long long)i * D + j] = {-p.re, -p.im};
 }
 
 // Panel of pivot block k0: C = X[:, K] and G = C P^-1 for 16 rows per CTA; and a copy
@@ -427,12 +432,6 @@ __global__ void sweep_negate_kernel(const cplx<double>* __restrict__ X, int D, c
   }
 }
 
-__global__ void log_kernel(const double* __restrict__ x, int n, double* __restrict__ y) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = log(x[i]);
-}
-
-
 // ------------------------------------------------------------ host side --
 
 static gbs_status alloc_state(gbs_ctx* ctx, int M, gbs_state** out) {
@@ -511,7 +510,7 @@ gbs_status state_build(gbs_ctx* ctx, int M, const double* U, const double* r, do
   double* ld_out = logd + M;
   state_params_kernel<<<(M + 127) / 128, 128, 0, s>>>((const double*)st->r.ptr, eta, M, (double*)st->alpha.ptr,
                                                       (double*)st->beta.ptr, ch2, sh2, logd);
-  sum_dd_kernel<<<1, 256, 0, s>>>(logd, M, ld_out);
+  sum_dd_kernel<false><<<1, 256, 0, s>>>(logd, M, ld_out);
   count_launch(ctx, 2);
   if ((e = check_cuda(ctx, cudaGetLastError(), "state kernels"))) return fail(e);
   if ((e = check_cuda(ctx, cudaMemcpyAsync(&st->logdet_sigma, ld_out, 8, cudaMemcpyDeviceToHost, s), "copy logdet")))
@@ -541,49 +540,51 @@ gbs_status state_from_V(gbs_ctx* ctx, int M, const double* V, gbs_state** out) {
     gbs_state_free(st);
     return code;
   };
-  // panels C and G, two inverses and a copy of a pivot block, then pivots, their
-  // logarithms and sum, and the row sums
-  const size_t zc = 2 * (size_t)D * kSW + 3 * kSW * kSW, zd = 3 * (size_t)D + 2;
+  // panels C and G, two inverses and a copy of a pivot block, then the pivots, and what the
+  // host reads in one copy: their logarithms' sum, the status words and the row sums
+  const size_t zc = 2 * (size_t)D * kSW + 3 * kSW * kSW, zd = 2 * (size_t)D + 2;
   if ((e = dev_alloc(ctx, st->V, D * D * 16)) || (e = dev_alloc(ctx, st->Sinv, D * D * 16)) ||
-      (e = dev_alloc(ctx, X, D * D * 16)) || (e = dev_alloc(ctx, work, zc * 16 + zd * 8)) ||
-      (e = dev_reserve(ctx, ctx->status, 2 * sizeof(int))))
+      (e = dev_alloc(ctx, X, D * D * 16)) || (e = dev_alloc(ctx, work, zc * 16 + zd * 8)))
     return fail(e);
   cudaStream_t s = ctx->stream;
-  int* status = (int*)ctx->status.ptr;  // [0] not positive definite, [1] not finite
-  if ((e = check_cuda(ctx, cudaMemcpyAsync(st->V.ptr, V, D * D * 16, cudaMemcpyHostToDevice, s), "copy V")) ||
-      (e = check_cuda(ctx, cudaMemsetAsync(status, 0, 2 * sizeof(int), s), "memset")))
-    return fail(e);
   cplx<double>* x = (cplx<double>*)X.ptr;
   cplx<double>* C = (cplx<double>*)work.ptr;
   cplx<double>* G = C + D * kSW;
   cplx<double>* P[2] = {G + D * kSW, G + D * kSW + kSW * kSW};
   cplx<double>* Xk = P[1] + kSW * kSW;
   double* pv = (double*)(Xk + kSW * kSW);
-  double* rowsum = pv + 2 * D + 2;
+  double* result = pv + D;
+  int* status = (int*)(result + 1);  // [0] not positive definite, [1] not finite
+  double* rowsum = result + 2;
+  if ((e = check_cuda(ctx, cudaMemcpyAsync(st->V.ptr, V, D * D * 16, cudaMemcpyHostToDevice, s), "copy V")) ||
+      (e = check_cuda(ctx, cudaMemsetAsync(status, 0, 2 * sizeof(int), s), "memset")))
+    return fail(e);
   sigma_from_V_kernel<<<(unsigned)((D + 7) / 8), 256, 0, s>>>((const cplx<double>*)st->V.ptr, (int)D, x, rowsum, status + 1);
   sweep_first_kernel<<<1, 256, 0, s>>>(x, (int)D, P[0], pv, status);
   const int nb = (int)((D + kSW - 1) / kSW), ntiles = nb * (nb + 1) / 2;
-  for (int k = 0; k < nb; ++k) {
-    sweep_panel_kernel<<<nb, 256, 0, s>>>(x, (int)D, k * kSW, P[k & 1], C, G, Xk);
-    sweep_update_kernel<<<ntiles + (k + 1 < nb ? 1 : 0), 256, 0, s>>>(x, (int)D, k * kSW, ntiles, P[k & 1], C, G, Xk,
-                                                                     P[(k + 1) & 1], pv, status);
+  if (nb > 1) {
+    for (int k = 0; k < nb; ++k) {
+      sweep_panel_kernel<<<nb, 256, 0, s>>>(x, (int)D, k * kSW, P[k & 1], C, G, Xk);
+      sweep_update_kernel<<<ntiles + (k + 1 < nb ? 1 : 0), 256, 0, s>>>(x, (int)D, k * kSW, ntiles, P[k & 1], C, G, Xk,
+                                                                       P[(k + 1) & 1], pv, status);
+    }
+    count_launch(ctx, 2 * nb);
   }
   sweep_negate_kernel<<<(unsigned)((D * D + 255) / 256), 256, 0, s>>>(x, (int)D, (cplx<double>*)st->Sinv.ptr);
-  log_kernel<<<(unsigned)((D + 255) / 256), 256, 0, s>>>(pv, (int)D, pv + D);
-  sum_dd_kernel<<<1, 256, 0, s>>>(pv + D, (int)D, pv + 2 * D);
-  count_launch(ctx, 2 * nb + 5);
+  sum_dd_kernel<true><<<1, 256, 0, s>>>(pv, (int)D, result);
+  count_launch(ctx, 4);
   if ((e = check_cuda(ctx, cudaGetLastError(), "sigma inverse"))) return fail(e);
-  int hstatus[2] = {0, 0};
-  std::vector<double> rows(D);
-  if ((e = check_cuda(ctx, cudaMemcpyAsync(&st->logdet_sigma, pv + 2 * D, 8, cudaMemcpyDeviceToHost, s), "copy")) ||
-      (e = check_cuda(ctx, cudaMemcpyAsync(rows.data(), rowsum, D * 8, cudaMemcpyDeviceToHost, s), "copy")) ||
-      (e = check_cuda(ctx, cudaMemcpyAsync(hstatus, status, 8, cudaMemcpyDeviceToHost, s), "copy")) ||
+  std::vector<double> got(D + 2);
+  if ((e = check_cuda(ctx, cudaMemcpyAsync(got.data(), result, (D + 2) * 8, cudaMemcpyDeviceToHost, s), "copy")) ||
       (e = stream_sync(ctx)))
     return fail(e);
+  int hstatus[2];
+  memcpy(hstatus, &got[1], sizeof hstatus);
   if (hstatus[1]) return fail(set_error(ctx, GBS_EINVAL, "gbs_state_from_V: non-finite V"));
   if (hstatus[0]) return fail(set_error(ctx, GBS_ENOTPD, "gbs_state_from_V: Sigma = V + I/2 is not positive definite"));
+  st->logdet_sigma = got[0];
   // Gershgorin bound on the largest eigenvalue of Sigma = V + I/2
-  for (double r : rows) st->sigma_max = std::max(st->sigma_max, r);
+  for (long long i = 0; i < D; ++i) st->sigma_max = std::max(st->sigma_max, got[2 + i]);
   dev_free(ctx, X);
   dev_free(ctx, work);
   *out = st;
