@@ -500,8 +500,8 @@ def batched_block(ctx, gbs, gi, n_req, n_err, autotune=True):
     reqs = gi.batched_requests(4096)[:n_req]
     if autotune:
         # launch shapes for a batch of uneven trees like this one (22 .. 8 modes), not the single
-        # 24-mode tree of the headline
-        ctx.autotune("fp64", "real", 22, n_trees=15)
+        # 24-mode tree of the headline; every state here bounds its FP64 trees (sigma_max below 4.2)
+        ctx.autotune("fp64_fixed", "real", 22, n_trees=15)
     t0 = time.perf_counter()
     Us = haar_unitaries([(q.M, q.seed) for q in reqs])
     states = [gbs.build_state(ctx, U, np.full(q.M, q.r), q.eta) for U, q in zip(Us, reqs)]
@@ -552,7 +552,7 @@ def batched_block(ctx, gbs, gi, n_req, n_err, autotune=True):
             "batch_seconds": t_batch, "batch_requests_per_s": n_req / t_batch, "batch_terms_per_s": terms / t_batch,
             "one_at_a_time_seconds": t_single, "one_at_a_time_requests_per_s": n_req / t_single,
             "speedup_vs_one_at_a_time": t_single / t_batch, "batch_gpu_launches": launches,
-            "fp64_tuning": ctx.tuning("fp64", "real"),
+            "fp64_tuning": {k: v for k, v in ctx.tuning("fp64_fixed", "real").items() if k in ("d_top", "q_drop")},
             "certified": {"seconds": t_cert, "requests_per_s": n_req / t_cert, "precisions": prec_counts,
                           "max_rel_err_bound": worst_bound, "status": cert_status,
                           "above_1e-10": sum(1 for c in cert if c.p and c.err_bound > 1e-10 * abs(c.p))},
@@ -804,12 +804,14 @@ def main():
     modes = np.ascontiguousarray(modes24, dtype=np.int32)
     st = gbs.build_state(ctx, st_p.U, st_p.r, st_p.eta)
     complex_basis = args.basis == "complex"
+    fixed = fixed_point(args.prec, complex_basis, args.N, float(st_p.r[0]))
+    shape = "fp64_fixed" if fixed and args.prec == "fp64" else args.prec  # of the engine that runs the tree
     if args.tuning:
-        ctx.set_tuning(args.prec, args.basis, *(int(x) for x in args.tuning.split(",")))
+        ctx.set_tuning(shape, args.basis, *(int(x) for x in args.tuning.split(",")))
         tune_report = []
     else:
-        tune_report = ctx.autotune(args.prec, args.basis, min(args.N, 22)) if not args.no_autotune else []
-    tuning = ctx.tuning(args.prec, args.basis)
+        tune_report = ctx.autotune(shape, args.basis, min(args.N, 22)) if not args.no_autotune else []
+    tuning = ctx.tuning(shape, args.basis)
     Q = {("fp64", False): 5, ("fp64", True): 4, ("dd", False): 4, ("dd", True): 3, ("td", False): 3,
          ("td", True): 2, ("fp32", False): 5, ("fp32", True): 4, ("fx", False): 3,
          ("fxw", False): 3, ("fp64p", False): 5, ("fxn", False): 3}[(args.prec, complex_basis)]
@@ -822,8 +824,8 @@ def main():
     kernel_name = ("batch_subtree_kernel (%d levels expanded in shared memory, then register depth-first %d levels)"
                    % (q_root - Q, Q)) if tuning["sub_e"] else "batch_leaf_kernel (register depth-first, %d levels)" % Q
 
-    fixed = fixed_point(args.prec, complex_basis, args.N, float(st_p.r[0]))
     if fixed:
+        tuning = {k: tuning[k] for k in ("d_top", "q_drop")}  # what acts on this engine
         # one launch for up to 17 modes; else the leaf kernel takes the last Q levels of every node above them
         one = args.N <= 17
         q_root = args.N if one else min(args.N, max(1, min(3 if args.prec == "fp64" else 2, 3 - tuning["q_drop"])))
@@ -940,7 +942,7 @@ def main():
                     "fx": "exact fixed point", "fxw": "exact fixed point"}[args.prec],
             "l2": "flushed between steps (256 MB write); tree level buffers also exceed L2",
             "parallelism": "replicas" if ws > 1 else "single GPU",
-            "tuning": tuning, "autotune_candidates": len(tune_report),
+            "tuned_shape": shape, "tuning": tuning, "autotune_candidates": len(tune_report),
             "autotune_fastest": sorted(tune_report, key=lambda c: c["ms"])[:5] if tune_report else [],
         },
         "roofline": roofline,

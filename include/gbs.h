@@ -360,13 +360,21 @@ gbs_status gbs_server_stats_get(gbs_ctx* ctx, gbs_server_stats* out);
  *                  breadth-first level launches; reduced to fit 200 KB).
  * The fixed-point precisions shape their launches by rules on the batch; of the
  * above only d_top (an upper limit; at least 5 levels are taken) and q_drop (at
- * most 3 - q_drop levels per leaf thread) act on them.
+ * most 3 - q_drop levels per leaf thread) act on them, and neither on trees that
+ * take one launch (up to 9 or 10 modes; up to 17 where they are few).
+ * FP64 trees in the real basis run on one of two engines, each with a shape of
+ * its own: in 64-bit fixed point where a state built from its factors bounds the
+ * tree, else in floating point (also explicit matrices and states given by V).
+ * GBS_PREC_FP64 names the floating-point engine's shape here and
+ * GBS_TUNE_FP64_FIXED the other's; gbs_autotune of GBS_PREC_FP64 in the real
+ * basis times and keeps both (its report is the floating-point engine's).
  * gbs_autotune times candidate shapes on a synthetic batch of n_trees (1..64)
  * trees of n, n-1, ... modes (6 <= n <= 28; a workload of uneven trees tunes
  * best on a batch that resembles it)
  * on the context stream and keeps the fastest for later calls; report (may be
  * NULL) receives the timings as a JSON array, truncated to report_len bytes.
  * The paper has no counterpart (its Titan runs used MPI + OpenMP, Sec. III). */
+#define GBS_TUNE_FP64_FIXED 9 /* in place of prec, in these three calls only (real basis) */
 gbs_status gbs_autotune(gbs_ctx* ctx, int prec, int basis, int n, int n_trees, char* report, size_t report_len);
 gbs_status gbs_get_tuning(gbs_ctx* ctx, int prec, int basis, int* sub_e, int* d_top, int* grid_per_sm,
                           long long* level_threads, int* q_drop, int* mid_e);

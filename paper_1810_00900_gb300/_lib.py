@@ -20,6 +20,8 @@ HEADER = os.path.join(HERE, "..", "include", "gbs.h")
 
 OK, EINVAL, ENOMEM, ENOTPD, EPRECISION, EREJECT, ETIMEDOUT, ECUDA, PENDING, ENOTFOUND = range(10)
 PREC = {"auto": 0, "fp64": 1, "dd": 2, "td": 3, "fp32": 4, "fx": 5, "fxw": 6, "fp64p": 7, "fxn": 8}
+# launch shapes: a precision's, or that of the 64-bit fixed-point engine of FP64 trees
+SHAPE = {**PREC, "fp64_fixed": 9}
 PREC_NAME = {v: k for k, v in PREC.items()}
 BASIS = {"auto": 0, "real": 1, "complex": 2}
 BASIS_NAME = {v: k for k, v in BASIS.items()}
@@ -211,23 +213,24 @@ class Context:
 
     def autotune(self, prec: str = "fp64", basis: str = "real", n: int = 22, n_trees: int = 1):
         """Time candidate launch shapes on a batch of n_trees trees of n, n-1, ... modes and keep the
-        fastest; returns the timings."""
+        fastest; returns the timings.  prec: a precision, or "fp64_fixed" for FP64 trees in 64-bit
+        fixed point (tuned with "fp64" too), here and in tuning() and set_tuning()."""
         import json
         buf = ctypes.create_string_buffer(1 << 18)
-        self.check(self.L.gbs_autotune(self.h, PREC[prec], BASIS[basis], int(n), int(n_trees), buf, len(buf)))
+        self.check(self.L.gbs_autotune(self.h, SHAPE[prec], BASIS[basis], int(n), int(n_trees), buf, len(buf)))
         return json.loads(buf.value.decode() or "[]")
 
     def tuning(self, prec: str = "fp64", basis: str = "real") -> dict:
         a, b, c, e, f = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         d = ctypes.c_longlong()
-        self.check(self.L.gbs_get_tuning(self.h, PREC[prec], BASIS[basis], ctypes.byref(a), ctypes.byref(b),
+        self.check(self.L.gbs_get_tuning(self.h, SHAPE[prec], BASIS[basis], ctypes.byref(a), ctypes.byref(b),
                                          ctypes.byref(c), ctypes.byref(d), ctypes.byref(e), ctypes.byref(f)))
         return {"sub_e": a.value, "d_top": b.value, "grid_per_sm": c.value, "level_threads": d.value,
                 "q_drop": e.value, "mid_e": f.value}
 
     def set_tuning(self, prec: str = "fp64", basis: str = "real", sub_e: int = 5, d_top: int = 10,
                    grid_per_sm: int = 0, level_threads: int = 1 << 18, q_drop: int = 0, mid_e: int = 0):
-        self.check(self.L.gbs_set_tuning(self.h, PREC[prec], BASIS[basis], sub_e, d_top, grid_per_sm,
+        self.check(self.L.gbs_set_tuning(self.h, SHAPE[prec], BASIS[basis], sub_e, d_top, grid_per_sm,
                                          level_threads, q_drop, mid_e))
 
     def kernel_time(self):

@@ -229,7 +229,8 @@ gbs_status gbs_ctx_create(gbs_ctx** out, int device, size_t hbm_budget_bytes) {
     }
   }
   // Launch shapes before any autotuning: wider arithmetic makes the redundant
-  // prefix elimination of the top kernel dearer, so it stops earlier.
+  // prefix elimination of the top kernel dearer, so it stops earlier.  (The fixed-point
+  // engine's own rules go no deeper than BatchTune's default.)
   for (int b = 0; b < 2; ++b) {
     ctx->tune[GBS_PREC_FP64][b].sub_e = 6;
     ctx->tune[GBS_PREC_FP64][b].d_top = 8;
@@ -239,14 +240,8 @@ gbs_status gbs_ctx_create(gbs_ctx** out, int device, size_t hbm_budget_bytes) {
     ctx->tune[GBS_PREC_DD][b].d_top = 5;
     ctx->tune[GBS_PREC_TD][b].sub_e = 6;
     ctx->tune[GBS_PREC_TD][b].d_top = 4;
-    ctx->tune[GBS_PREC_FX][b].sub_e = 6;
-    ctx->tune[GBS_PREC_FX][b].d_top = 10;
-    ctx->tune[GBS_PREC_FXW][b].sub_e = 6;
-    ctx->tune[GBS_PREC_FXW][b].d_top = 10;
     ctx->tune[GBS_PREC_FP64P][b].sub_e = 6;
     ctx->tune[GBS_PREC_FP64P][b].d_top = 8;
-    ctx->tune[GBS_PREC_FXN][b].sub_e = 6;
-    ctx->tune[GBS_PREC_FXN][b].d_top = 10;
   }
   *out = ctx;
   return GBS_OK;

@@ -50,7 +50,7 @@ gbs_status stage(gbs_ctx* ctx, const void* data, size_t bytes, const void** dev)
 }
 
 const BatchTune& batch_tune_for(gbs_ctx* ctx, int prec, bool real) {
-  return ctx->tune[prec < 0 || prec > kPrecLast ? 1 : prec][real ? 1 : 0];
+  return ctx->tune[prec < 0 || prec > kTuneLast ? 1 : prec][real ? 1 : 0];
 }
 
 // Every value of a tree over n modes of (Sigma^-1)_S fits the fixed-point range: its
@@ -332,7 +332,7 @@ static gbs_status batch_variant(gbs_ctx* ctx, int prec, bool real, bool fixed64,
       break;
     default: return set_error(ctx, GBS_EINVAL, "unknown precision");
   }
-  return e(ctx, nt, tr, roots, status, batch_tune_for(ctx, fixed64 ? (int)GBS_PREC_FXN : prec, real), fin);
+  return e(ctx, nt, tr, roots, status, batch_tune_for(ctx, fixed64 ? GBS_TUNE_FP64_FIXED : prec, real), fin);
 }
 
 gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const BatchTree* trees, const void* roots_dev,
@@ -622,36 +622,19 @@ gbs_status probs_batch(gbs_ctx* ctx, int nreq, const gbs_state* const* states, c
 
 using namespace gbs;
 
-extern "C" gbs_status gbs_autotune(gbs_ctx* ctx, int prec, int basis, int n, int n_trees, char* report,
-                                   size_t report_len) {
-  if (!ctx || prec < GBS_PREC_FP64 || prec > kPrecLast || n < 6 || n > 28 || n_trees < 1 || n_trees > 64)
-    return GBS_EINVAL;
-  if (prec >= GBS_PREC_FX && basis == GBS_BASIS_COMPLEX) return GBS_EINVAL;
-  std::lock_guard<std::mutex> g(ctx->mu);
-  cudaSetDevice(ctx->device);
-  const bool real = basis != GBS_BASIS_COMPLEX;
-  // A synthetic well-conditioned positive-definite root (the timing does not
-  // depend on the values): identity plus a small symmetric perturbation.
-  const int D = 2 * n, ne = D * (D + 1) / 2;
-  std::vector<double> root(ne * (real ? 1 : 2), 0.0);
-  unsigned long long x = 0x9E3779B97F4A7C15ull;
-  for (int a = 0; a < D; ++a)
-    for (int b = 0; b <= a; ++b) {
-      const int t = a * (a + 1) / 2 + b;
-      x ^= x << 13; x ^= x >> 7; x ^= x << 17;
-      const double v = (a == b) ? 1.0 : 0.02 * ((double)(x >> 11) * 0x1p-53 - 0.5);
-      if (real) root[t] = v; else { root[2 * t] = v; root[2 * t + 1] = (a == b) ? 0.0 : 0.5 * v; }
-    }
-  gbs_status st;
-  // n_trees trees of n, n-1, ... modes (at least 6), all on leading blocks of the one root
-  std::vector<BatchTree> trees(n_trees);
-  for (int i = 0; i < n_trees; ++i) trees[i] = BatchTree{std::max(6, n - i), 0};
+// Times the candidate shapes of tune[shape][real] on the trees (all on leading blocks of one
+// host root) and keeps the fastest.
+static gbs_status autotune_shape(gbs_ctx* ctx, int shape, bool real, const std::vector<double>& root,
+                                 const std::vector<BatchTree>& trees, std::string* rep) {
+  const bool fixed64 = shape == GBS_TUNE_FP64_FIXED, fixed = fixed64 || is_fixed_point(shape);
+  const int prec = fixed64 ? (int)GBS_PREC_FP64 : shape, n_trees = (int)trees.size();
   const std::vector<double> zeros(n_trees, 0.0);
   std::vector<ProbOut> outs(n_trees);
-  const BatchTune saved = ctx->tune[prec][real ? 1 : 0];
+  BatchTune& slot = ctx->tune[shape][real ? 1 : 0];
+  const BatchTune saved = slot;
   BatchTune best = saved;
   double best_ms = 1e30;
-  std::string rep = "[";
+  gbs_status st;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -674,15 +657,17 @@ extern "C" gbs_status gbs_autotune(gbs_ctx* ctx, int prec, int basis, int n, int
           cand.q_drop = qd;
           cand.mid_e = me;
           // only d_top and q_drop act on the fixed-point engine: one candidate for the rest
-          if (is_fixed_point(prec) && (me != mids[0] || se != subs[0] || gr != grids[0] || lt != lts[0])) continue;
-          ctx->tune[prec][real ? 1 : 0] = cand;
+          if (fixed && (me != mids[0] || se != subs[0] || gr != grids[0] || lt != lts[0])) continue;
+          slot = cand;
           float ms_best = 1e30f;
           for (int rep_i = 0; rep_i < 3; ++rep_i) {
             if ((st = stage_begin(ctx, root.size() * 8 + (1 << 16)))) goto done;
             const void* d = nullptr;
             if ((st = stage(ctx, root.data(), root.size() * 8, &d))) goto done;
             cudaEventRecord(e0, ctx->stream);
-            if ((st = batch_eval(ctx, prec, real, n_trees, trees.data(), d, zeros.data(), outs.data()))) goto done;
+            if ((st = batch_eval(ctx, prec, real, n_trees, trees.data(), d, zeros.data(), outs.data(),
+                                 fixed64 ? n_trees : 0)))
+              goto done;
             cudaEventRecord(e1, ctx->stream);
             cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -693,8 +678,8 @@ extern "C" gbs_status gbs_autotune(gbs_ctx* ctx, int prec, int basis, int n, int
           snprintf(buf, sizeof buf,
                    "%s{\"sub_e\":%d,\"d_top\":%d,\"grid_per_sm\":%d,\"level_threads\":%lld,\"q_drop\":%d,"
                    "\"mid_e\":%d,\"ms\":%.4f}",
-                   rep.size() > 1 ? "," : "", se, dt, gr, lt, qd, me, ms_best);
-          rep += buf;
+                   rep->empty() ? "" : ",", se, dt, gr, lt, qd, me, ms_best);
+          *rep += buf;
           if (ms_best < best_ms) {
             best_ms = ms_best;
             best = cand;
@@ -704,18 +689,49 @@ extern "C" gbs_status gbs_autotune(gbs_ctx* ctx, int prec, int basis, int n, int
 done:
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  ctx->tune[prec][real ? 1 : 0] = st == GBS_OK ? best : saved;
-  if (st == GBS_OK) ctx->tuned[prec][real ? 1 : 0] = true;
-  rep += "]";
-  if (report && report_len) {
-    snprintf(report, report_len, "%s", rep.c_str());
-  }
+  slot = st == GBS_OK ? best : saved;
+  return st;
+}
+
+// Whether (prec, basis) names a launch shape.
+static bool valid_shape(int prec, int basis) {
+  return prec >= GBS_PREC_FP64 && prec <= kTuneLast && !(prec == GBS_TUNE_FP64_FIXED && basis == GBS_BASIS_COMPLEX);
+}
+
+extern "C" gbs_status gbs_autotune(gbs_ctx* ctx, int prec, int basis, int n, int n_trees, char* report,
+                                   size_t report_len) {
+  if (!ctx || !valid_shape(prec, basis) || n < 6 || n > 28 || n_trees < 1 || n_trees > 64) return GBS_EINVAL;
+  if (prec >= GBS_PREC_FX && basis == GBS_BASIS_COMPLEX) return GBS_EINVAL;
+  std::lock_guard<std::mutex> g(ctx->mu);
+  cudaSetDevice(ctx->device);
+  const bool real = basis != GBS_BASIS_COMPLEX;
+  // A synthetic well-conditioned positive-definite root (the timing does not
+  // depend on the values): identity plus a small symmetric perturbation.
+  const int D = 2 * n, ne = D * (D + 1) / 2;
+  std::vector<double> root(ne * (real ? 1 : 2), 0.0);
+  unsigned long long x = 0x9E3779B97F4A7C15ull;
+  for (int a = 0; a < D; ++a)
+    for (int b = 0; b <= a; ++b) {
+      const int t = a * (a + 1) / 2 + b;
+      x ^= x << 13; x ^= x >> 7; x ^= x << 17;
+      const double v = (a == b) ? 1.0 : 0.02 * ((double)(x >> 11) * 0x1p-53 - 0.5);
+      if (real) root[t] = v; else { root[2 * t] = v; root[2 * t + 1] = (a == b) ? 0.0 : 0.5 * v; }
+    }
+  // n_trees trees of n, n-1, ... modes (at least 6), all on leading blocks of the one root
+  std::vector<BatchTree> trees(n_trees);
+  for (int i = 0; i < n_trees; ++i) trees[i] = BatchTree{std::max(6, n - i), 0};
+  std::string rep, rep64;
+  gbs_status st = autotune_shape(ctx, prec, real, root, trees, &rep);
+  // FP64 calls run on either engine
+  if (st == GBS_OK && prec == GBS_PREC_FP64 && real)
+    st = autotune_shape(ctx, GBS_TUNE_FP64_FIXED, real, root, trees, &rep64);
+  if (report && report_len) snprintf(report, report_len, "[%s]", rep.c_str());
   return st;
 }
 
 extern "C" gbs_status gbs_get_tuning(gbs_ctx* ctx, int prec, int basis, int* sub_e, int* d_top, int* grid_per_sm,
                                      long long* level_threads, int* q_drop, int* mid_e) {
-  if (!ctx || prec < GBS_PREC_FP64 || prec > kPrecLast) return GBS_EINVAL;
+  if (!ctx || !valid_shape(prec, basis)) return GBS_EINVAL;
   const BatchTune& t = ctx->tune[prec][basis != GBS_BASIS_COMPLEX ? 1 : 0];
   if (sub_e) *sub_e = t.sub_e;
   if (d_top) *d_top = t.d_top;
@@ -728,9 +744,7 @@ extern "C" gbs_status gbs_get_tuning(gbs_ctx* ctx, int prec, int basis, int* sub
 
 extern "C" gbs_status gbs_set_tuning(gbs_ctx* ctx, int prec, int basis, int sub_e, int d_top, int grid_per_sm,
                                      long long level_threads, int q_drop, int mid_e) {
-  if (!ctx || prec < GBS_PREC_FP64 || prec > kPrecLast || sub_e < 0 || sub_e > 7 ||
-      d_top < 0 ||
-      d_top > 16 || grid_per_sm < 0 || level_threads < 1 || q_drop < 0 || q_drop > 2 || mid_e < 0 || mid_e > 8)
+  if (!ctx || !valid_shape(prec, basis) || sub_e < 0 || sub_e > 7 || d_top < 0 || d_top > 16 || grid_per_sm < 0 || level_threads < 1 || q_drop < 0 || q_drop > 2 || mid_e < 0 || mid_e > 8)
     return GBS_EINVAL;
   std::lock_guard<std::mutex> g(ctx->mu);
   BatchTune& t = ctx->tune[prec][basis != GBS_BASIS_COMPLEX ? 1 : 0];

@@ -23,6 +23,11 @@ namespace gbs {
 // The largest gbs_prec value.
 constexpr int kPrecLast = GBS_PREC_FXN;
 
+// Launch shapes are kept per precision, and for the 64-bit fixed-point engine of FP64 trees
+// apart from the floating-point one's.
+constexpr int kTuneLast = GBS_TUNE_FP64_FIXED;
+static_assert(kTuneLast == kPrecLast + 1, "shapes are indexed by precision");
+
 // The fixed-point precisions (real basis; need a state that bounds the tree).
 constexpr bool is_fixed_point(int prec) {
   return prec == GBS_PREC_FXN || prec == GBS_PREC_FX || prec == GBS_PREC_FXW;
@@ -110,8 +115,7 @@ struct gbs_ctx {
   long long gap_waits = 0;
 
   // batched-engine launch parameters per (precision, basis): [prec][real]
-  gbs::BatchTune tune[gbs::kPrecLast + 1][2];  // [gbs_prec][basis is real]
-  bool tuned[gbs::kPrecLast + 1][2] = {};
+  gbs::BatchTune tune[gbs::kTuneLast + 1][2];  // [gbs_prec or GBS_TUNE_FP64_FIXED][basis is real]
 
   // request loop (see gbs_server.cu)
   void* server = nullptr;
@@ -221,7 +225,7 @@ BatchEngine batch_fxd_real, batch_fxn_real, batch_fx_real, batch_fxw_real;
 // integer pipe, and again in floating point if one leaves its range.  (gbs_batch_api.cu)
 gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const BatchTree* trees, const void* roots_dev,
                       const double* logdet, ProbOut* host_out, int n_bounded = 0);
-// The tuning in force for (prec, basis) -- the autotuner's choice when one was made.
+// The tuning in force for (prec or GBS_TUNE_FP64_FIXED, basis) -- the autotuner's choice when one was made.
 const BatchTune& batch_tune_for(gbs_ctx* ctx, int prec, bool real);
 
 // One chain-rule trajectory (gbs_sampler.cu): host bookkeeping plus device
