@@ -72,18 +72,27 @@ bool fx_ok_sigma(const gbs_state* st, int n) {
 }
 
 // FP64 trees in 64-bit fixed point (64 fraction bits; s and sums have 95 integer bits).
-// Errors there are absolute, 2^-63 per operation, amplified by at most ~sigma_max^2
-// through a pivot's determinant and inverse; FP64's are 2^-53 of values up to 1 and more.
-// With sigma_max <= 16 the former stay below the latter.  Every term of a physical
-// state's (Sigma^-1)_S tree is at least 1 (det of a conditioned V + I/2 is), so the sum
-// of magnitudes is at least 2^n and the terms' absolute errors vanish against FP64's.
-// The bound needs the closed form (a state built from its factors).
+// A Schur step rounds an entry by up to 2^-60 of what it takes off it (the inverse square
+// root's 2^-61, squared) and some products' 2^-64 each, all low; FP64 by 2^-53 of the entry
+// and of what is taken off it.  Whatever either leaves goes through the same later steps: a
+// factor of up to 1 + |L|^2 <= 1 + 2 sigma_max in an entry, and of 2 sigma_max from an entry
+// to a relative determinant.  With sigma_max <= 16 entries lie in [1/16, 2] on the diagonal, so
+// a step here rounds by less than 2^-59 where FP64 rounds by 2^-57 at least, and the tree keeps
+// FP64's error estimate.  (That estimate, 4 n + 24 units per term, is a model for either: the
+// worst case over all steps, n 2^-59 (1 + 2 sigma_max) sigma_max relative, would pass it 30-fold
+// at sigma_max = 16, n = 22, and FP64's by more.  Measured there, n = 4 .. 22: at most 4e-4 of
+// the estimate, 0.13 in FP64; 5e-5 and 0.06 at sigma_max = 8.)
+// Every term of a physical state's (Sigma^-1)_S tree is at least 1 (det of a conditioned V +
+// I/2 is), so the sum of magnitudes is at least 2^n and the terms' absolute errors vanish
+// against FP64's.  The bound needs the closed form (a state built from its factors).
 bool fxd_ok_inverse(const gbs_state* st, int n) {
   const double sm = st->sigma_max;
   return st->has_factors && sm > 0.0 && sm <= 16.0 && n * std::log2(1.0 + sm) < 92.0;
 }
-// Sampler trees: terms are at most 1 and their magnitudes add up to at least 1, so the
-// absolute errors of 2^n terms stay below FP64's estimate only for small n.
+// Sampler trees: entries up to 64, rounded relative to what a step takes off them as above.
+// Terms are at most 1, and their magnitudes add up to at least 1; a term's s is a product of
+// factors in [1/64, 2], truncated to 2^-64 at each, so 2^10 terms of 10 factors are off by less
+// than 2^-50 together, against an estimate of 64 2^-53 of the sum of magnitudes at least.
 bool fxd_ok_sigma(const gbs_state* st, int n) { return fx_ok_sigma(st, n) && n <= 10; }
 
 // ------------------------------------------------------- click blocks ---
