@@ -79,7 +79,7 @@ bool fx_ok_sigma(const gbs_state* st, int n) {
 // to a relative determinant.  With sigma_max <= 16 entries lie in [1/16, 2] on the diagonal, so
 // a step here rounds by less than 2^-59 where FP64 rounds by 2^-57 at least, and the tree keeps
 // FP64's error estimate.  (That estimate, 4 n + 24 units per term, is a model for either: the
-// worst case over all steps, n 2^-59 (1 + 2 sigma_max) sigma_max relative, would pass it 30-fold
+// worst case over all steps, n^2 2^-59 (1 + 2 sigma_max) sigma_max relative, would pass it 30-fold
 // at sigma_max = 16, n = 22, and FP64's by more.  Measured there, n = 4 .. 22: at most 4e-4 of
 // the estimate, 0.13 in FP64; 5e-5 and 0.06 at sigma_max = 8.)
 // Every term of a physical state's (Sigma^-1)_S tree is at least 1 (det of a conditioned V +
@@ -306,20 +306,6 @@ __global__ void kappa_estimate_kernel(const BatchTree* __restrict__ trees, int n
   if (lane == 0) log10_kappa[t] = lk;
 }
 
-static double unit_roundoff_b(int prec) {
-  switch (prec) {
-    case GBS_PREC_FP64:
-    case GBS_PREC_FP64P: return ldexp(1.0, -53);
-    case GBS_PREC_DD: return ldexp(1.0, -102);
-    case GBS_PREC_TD: return ldexp(1.0, -152);
-    case GBS_PREC_FP32_DIAG: return ldexp(1.0, -24);
-    case GBS_PREC_FXN: return ldexp(1.0, -108);
-    case GBS_PREC_FX: return ldexp(1.0, -140);
-    case GBS_PREC_FXW: return ldexp(1.0, -158);  // the three-double output, not the 2^-192 resolution, limits it
-  }
-  return 1.0;
-}
-
 // The engine of a precision and basis (fixed64: FP64 in 64-bit fixed point).
 static gbs_status batch_variant(gbs_ctx* ctx, int prec, bool real, bool fixed64, int nt, const BatchTree* tr,
                                 const void* roots, int* status, const TreeFinish& fin) {
@@ -355,7 +341,7 @@ gbs_status batch_eval(gbs_ctx* ctx, int prec, bool real, int ntrees, const Batch
   ProbOut* po = (ProbOut*)ctx->aux_dev.ptr;
   int* status = (int*)((unsigned char*)po + r256(n * sizeof(ProbOut)));  // then the counters
   if ((st = check_cuda(ctx, cudaMemsetAsync(status, 0, 2 * n * sizeof(int), ctx->stream), "memset"))) return st;
-  const double u = unit_roundoff_b(prec), extra = err_factor(prec, 1) - err_factor(GBS_PREC_TD, 1);
+  const double u = unit_of(prec), extra = err_factor(prec, 1) - err_factor(GBS_PREC_TD, 1);
   std::vector<double> scale(n);
   for (size_t t = 0; t < n; ++t) scale[t] = std::exp(-0.5 * logdet[t]);
   // The bounded trees and the others, each on its engine, side by side and with one wait for

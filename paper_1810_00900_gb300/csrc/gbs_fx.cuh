@@ -346,7 +346,7 @@ __device__ __forceinline__ fxn<L, F> rsqrt_(const fxn<L, F>& x) {
     const unsigned long long sq2 = shh + (sm >> 32);         // (e/2)^2 2^(2U - 64 (NC - 2) - 64)
     // (e/2)^2 in units of 2^-U: up by U - (2U - 64 (NC - 2) - 64) = 64 (NC - 1) - U
     constexpr int U = 32 * F + 155 - 32 * (CLO + 1);
-    constexpr int DN = U - 64 * (NC - 1);  // -5 for every F: 64 (NC - 1) - U = 5
+    constexpr int DN = U - 64 * (NC - 1);  // -5 (F = 5, 6) or 27 (F = 4)
     static_assert(DN == -5 || DN == 27, "alignment of the squared residual");
     unsigned long long q2;
     uint32_t q2h;

@@ -280,16 +280,18 @@ GBS_HD_INLINE double err_factor(int prec, int n) {
   return (prec == GBS_PREC_FP64 || prec == GBS_PREC_FP64P || prec == GBS_PREC_FP32_DIAG) ? base + 24.0 : base;
 }
 
-// Unit of the error model of a precision.
+// Unit of the error model of a precision (batches and the sampler).
 GBS_HD_INLINE double unit_of(int prec) {
   switch (prec) {
-    case GBS_PREC_FP64: return 0x1p-53;
+    case GBS_PREC_FP64:
+    case GBS_PREC_FP64P: return 0x1p-53;
     case GBS_PREC_DD: return 0x1p-102;
+    case GBS_PREC_FP32_DIAG: return 0x1p-24;
     case GBS_PREC_FXN: return 0x1p-108;
     case GBS_PREC_FX: return 0x1p-140;
-    case GBS_PREC_FXW: return 0x1p-158;  // limited by the three-double tree output
+    case GBS_PREC_FXW: return 0x1p-158;  // limited by the three-double tree output, not 2^-192
   }
-  return 0x1p-152;
+  return 0x1p-152;  // TD
 }
 
 // Sampler: bound on |delta p0|, half the near-tie threshold, so that a decision can
