@@ -72,8 +72,8 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     s = ctx->side;
     return GBS_OK;
   };
-  // Launched once the others have their workspace: a batch that is evaluated in parts for
-  // want of it has not run its small trees yet.
+  // Launched once the others' plan is known to fit: a batch that goes in parts by its plan has
+  // not run its small trees yet.
   gbs_status st;
   auto launch_small = [&]() -> gbs_status {
     const void* d_small[2] = {};
@@ -179,6 +179,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     ctx->batch_split = true;  // the caller evaluates the batch in parts
     return GBS_ENOMEM;
   }
+  if ((st = launch_small())) return st;  // they run while a context's first call allocates
   // one allocation: a context's first call pays for each
   DevBuf& buf = fin.beside ? ctx->side_nodes : ctx->lvl[0];
   while ((st = dev_reserve(ctx, buf, space.total)) == GBS_ENOMEM) {
@@ -190,7 +191,7 @@ gbs_status fx_batch_run(gbs_ctx* ctx, int ntrees, const BatchTree* in, const voi
     if (less.total >= space.total) return st;
     space = less;
   }
-  if (st || (st = launch_small())) return st;
+  if (st) return st;
   const int d0 = space.d0, cb = space.cb;
   std::vector<long long> off(34 * (size_t)ntrees, 0);
   long long words = 0, selems = 0;
