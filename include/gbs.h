@@ -169,7 +169,12 @@ gbs_status gbs_build_state(gbs_ctx* ctx, int M, const double* U, const double* r
                            gbs_state** st);
 
 /* A state given only by its 2M x 2M complex covariance V (block order, host).
- * Sigma = V + I/2 is inverted once on the device (Gauss-Jordan, FP64).
+ * Sigma = V + I/2 is inverted once on the device (blocked sweep operator, FP64).
+ * V must be Hermitian: of two entries that ought to be conjugates either may be
+ * the one that counts.  Sigma > 0 is all that is asked of it.  The fixed-point
+ * precisions evaluate an unphysical V as well (Sigma not above I/2) while the
+ * entries of (Sigma^-1)_S stay below 2^29, the product of a mode's two diagonal
+ * ones below 2^31 and every pivot's determinant in [2^-20, 2^12).
  * Errors: GBS_EINVAL, GBS_ENOTPD (Sigma not positive definite), GBS_ENOMEM. */
 gbs_status gbs_state_from_V(gbs_ctx* ctx, int M, const double* V, gbs_state** st);
 void gbs_state_free(gbs_state* st);
@@ -317,9 +322,9 @@ typedef struct {
  * 32 M per attempt slot, a probability request only the shared tree
  * workspace) and at most max_active sampling requests run at once.  Each loop
  * iteration evaluates all newly admitted probability requests as one batch and
- * advances every running sampling attempt by one measured mode, all their
- * subset trees batched together, so late arrivals join running work at the
- * next step.  attempt_width (1..64): postselection attempts a sampling request
+ * advances every running sampling attempt: those with few clicks by up to 24
+ * measured modes in one launch, the others by one, their subset trees batched
+ * together; late arrivals join running work at the next iteration.  attempt_width (1..64): postselection attempts a sampling request
  * runs at once (attempts a, a+1, ... on separate trajectories); its result is
  * still the lowest accepted attempt, the one attempts run one after another
  * give, so a result is bitwise the same alone, in any mix and at any width.

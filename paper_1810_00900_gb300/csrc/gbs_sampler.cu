@@ -24,10 +24,11 @@
 // (the paper's Eq. 4a in Sigma form), a rank-2 update of the active block.
 //
 // Precision: the cancellation ratio grows with every click, so each
-// trajectory's tree runs in the cheapest of FP64 / double-double /
-// triple-double whose error bound keeps |delta p0| below 5e-10 (half the 1e-9
-// near-tie threshold), predicted from its previous step and verified
-// (escalated to a full tree at a wider precision) after the fact.
+// trajectory's tree runs in the cheapest of FP64, fixed point with 128, 160 and
+// 192 fraction bits (where the state bounds the tree) and triple-double whose
+// error bound keeps |delta p0| below 5e-10 (half the 1e-9 near-tie threshold),
+// predicted from its previous step and verified (escalated to a full tree at a
+// wider precision) after the fact.
 #include <algorithm>
 #include <chrono>
 #include <cmath>

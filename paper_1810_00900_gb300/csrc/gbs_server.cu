@@ -7,9 +7,10 @@
 // 32 M^2 bytes plus a little), a probability request only the shared tree
 // workspace.  Every iteration of the loop
 //   1. evaluates all newly admitted probability requests as one tree batch, and
-//   2. advances every active sampling trajectory by one measured mode, all of
-//      their subset trees (of whatever state, size and step) in shared batches,
-// so requests that arrive while others are on the GPU join at the next step
+//   2. advances every active sampling trajectory: those with few clicks by up to
+//      kChainSteps measured modes in one launch, the others by one, their subset
+//      trees (of whatever state, size and step) in shared batches,
+// so requests that arrive while others are on the GPU join at the next iteration
 // and their work shares the same kernel launches.  A finished request frees its
 // arena block at once, which admits the next queued one.  gbs_poll waits on a
 // condition variable with a caller-given bound.  No device code ever waits on
