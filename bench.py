@@ -266,7 +266,7 @@ def captured_traffic(args, tuning):
 # (prec, basis, N) -> bytes per launch of the leaf kernel, dram__bytes_read.sum +
 # dram__bytes_write.sum of one ncu capture of the current kernel code
 CAPTURED_TRAFFIC = {
-    ("fp64", "real", 24): 572865024 + 5093632,
+    ("fp64", "real", 24): 570571008 + 233984,
 }
 
 

@@ -632,8 +632,8 @@ __device__ __forceinline__ bool fx_leaf_node(const uint32_t* m, int p, const typ
   } else {
     // Three modes, for the narrow type (registers): the included child's ten entries are
     // formed row by row into local memory, the excluded one is a view.  356 us at N = 24
-    // (64 fraction bits) against 164 + 216 for a level launch that writes them and a
-    // two-mode leaf that reads them back, and a launch less.
+    // (64 fraction bits; 309 now) against 164 + 216 for a level launch that writes them and
+    // a two-mode leaf that reads them back, and a launch less.
     static_assert(Q == 3, "at most three levels per leaf thread");
     constexpr int L = sizeof(E) / 4;
     uint32_t child[10 * L];
