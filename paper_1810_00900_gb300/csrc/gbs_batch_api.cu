@@ -739,7 +739,8 @@ extern "C" gbs_status gbs_get_tuning(gbs_ctx* ctx, int prec, int basis, int* sub
 
 extern "C" gbs_status gbs_set_tuning(gbs_ctx* ctx, int prec, int basis, int sub_e, int d_top, int grid_per_sm,
                                      long long level_threads, int q_drop, int mid_e) {
-  if (!ctx || !valid_shape(prec, basis) || sub_e < 0 || sub_e > 7 || d_top < 0 || d_top > 16 || grid_per_sm < 0 || level_threads < 1 || q_drop < 0 || q_drop > 2 || mid_e < 0 || mid_e > 8)
+  if (!ctx || !valid_shape(prec, basis) || sub_e < 0 || sub_e > 7 || d_top < 0 || d_top > 16 || grid_per_sm < 0 ||
+      level_threads < 1 || q_drop < 0 || q_drop > 2 || mid_e < 0 || mid_e > 8)
     return GBS_EINVAL;
   std::lock_guard<std::mutex> g(ctx->mu);
   BatchTune& t = ctx->tune[prec][basis != GBS_BASIS_COMPLEX ? 1 : 0];
